@@ -382,15 +382,27 @@ __device__ __forceinline__ void ext4(const float* v, float& mx, float& mn)
     }
 }
 
-// Venkatakrishnan ratio of venkat() in two lanes (division as a reciprocal
-// and a product, like fdiv); capped at 1
+// Venkatakrishnan ratio of venkat() in two lanes, uncapped: (d1^2 + eps2 +
+// 2 d1 d2) / (d1^2 + 2 d2^2 + d1 d2 + eps2).  All terms are >= 0 (d1 and d2 have
+// one sign).  The reciprocal flushes subnormal denominators, |f| below 1e-19,
+// where the ratio comes out infinite or NaN and limit2 takes 1.
 __device__ __forceinline__ float2 venkat2(float2 d1, float2 d2, float2 eps2)
 {
-    const float2 d11 = mul2(d1, d1);
-    const float2 num = fma2(mul2(bc2(2.0f), d1), d2, add2(d11, eps2));
-    const float2 den = add2(fma2(d1, d2, fma2(mul2(bc2(2.0f), d2), d2, d11)), eps2);
-    const float2 v = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
-    return make_float2(v.x < 1.0f ? v.x : 1.0f, v.y < 1.0f ? v.y : 1.0f);
+    const float2 u = fma2(d1, d1, eps2), v = mul2(d1, d2);
+    const float2 num = fma2(bc2(2.0f), v, u);
+    const float2 den = fma2(mul2(bc2(2.0f), d2), d2, add2(u, v));
+    return make_float2(num.x * rcp_ftz(den.x), num.y * rcp_ftz(den.y));
+}
+
+// Limiter of a node pair: the smaller of the two sides' ratios, capped at 1.
+// A side without a projection (pp = 0 or nn = 0) has equal numerator and
+// denominator, so it needs no test; NaN (0/0 in the tails) loses to 1 in the
+// three-input minimum.  Against a compare and two selects per side and lane
+// this takes one instruction per lane of the ALU pipe, the kernel's busiest.
+__device__ __forceinline__ float2 limit2(float2 dmax, float2 dmin, float2 pp, float2 nn, float2 eps2)
+{
+    const float2 tp = venkat2(dmax, pp, eps2), tn = venkat2(dmin, nn, eps2);
+    return make_float2(min3f(tp.x, tn.x, 1.0f), min3f(tp.y, tn.y, 1.0f));
 }
 
 template <int D, int NS, int NA>
@@ -421,7 +433,11 @@ __global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int limiter
         gn[0][s] = n >= 0 ? n : i;
         gn[1][s] = sl;
 #pragma unroll
-        for (int d = 0; d < 4; ++d) gs[2][s][d] = (s < ns && d < D) ? An[(size_t)(sl >> 1) * D + d] : 0.0f;
+        for (int d = 0; d < D; ++d) {
+            const float a = s < ns ? An[(size_t)(sl >> 1) * D + d] : 0.0f;
+            gs[2][s][d] = (sl & 1) ? -a : a;
+        }
+        gs[2][s][3] = (sl & 1) ? __int_as_float(1) : 0.0f;
     }
     __syncthreads();
     if (k0 >= Nv) return;
@@ -480,12 +496,7 @@ __global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int limiter
                 ext4<NS>(ey, pp.y, nn.y);
                 // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
                 const float2 e2p = mul2(mul2(bc2(e2), phi[a][p]), phi[a][p]);
-                const float2 tp = venkat2(dmax, pp, e2p);
-                const float2 tn = venkat2(dmin, nn, e2p);
-                if (pp.x > 0.0f) L.x = tp.x;
-                if (pp.y > 0.0f) L.y = tp.y;
-                if (nn.x < 0.0f && tn.x < L.x) L.x = tn.x;
-                if (nn.y < 0.0f && tn.y < L.y) L.y = tn.y;
+                L = limit2(dmax, dmin, pp, nn, e2p);
             }
             if (limiter == 0) L = bc2(0.0f);     // first order: phi_bar = phi_C
 #pragma unroll
@@ -516,21 +527,21 @@ __global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int limiter
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
         if (s >= ns) break;
-        const int sl = gn[1][s];
-        const int fc = sl >> 1;
-        const bool isR = sl & 1;
-        float an[D], rr[D];
-        vec(2, s, an);
+        const int fc = gn[1][s] >> 1;
+        float rr[D];
+        const float4 an = *reinterpret_cast<const float4*>(gs[2][s]);
         vec(1, s, rr);
         bool up[4];
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-            // xi . An as in k_foot: a product, then fused multiply-adds
-            float2 sn = mul2(X[p][0], bc2(an[0]));
-#pragma unroll
-            for (int d = 1; d < D; ++d) sn = fma2(X[p][d], bc2(an[d]), sn);
-            up[2 * p] = isR ? (sn.x < 0.0f) : (sn.x >= 0.0f);
-            up[2 * p + 1] = isR ? (sn.y < 0.0f) : (sn.y >= 0.0f);
+            // xi . An as in k_foot: a product, then fused multiply-adds; the
+            // normal points out of the cell (an exact sign change), so the
+            // face's L cell is upwind at >= 0 and its R cell at > 0, that is,
+            // at or above the smallest subnormal (an.w)
+            float2 sn = fma2(X[p][1], bc2(an.y), mul2(X[p][0], bc2(an.x)));
+            if constexpr (D == 3) sn = fma2(X[p][2], bc2(an.z), sn);
+            up[2 * p] = sn.x >= an.w;
+            up[2 * p + 1] = sn.y >= an.w;
         }
         const bool all = up[0] && up[1] && up[2] && up[3];
         const bool any = up[0] || up[1] || up[2] || up[3];
@@ -1793,12 +1804,7 @@ __global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter
                 ext4<NS>(ey, pp.y, nn.y);
                 // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
                 const float2 e2p = mul2(mul2(bc2(e2), phi[p]), phi[p]);
-                const float2 tp = venkat2(dmax, pp, e2p);
-                const float2 tn = venkat2(dmin, nn, e2p);
-                if (pp.x > 0.0f) L.x = tp.x;
-                if (pp.y > 0.0f) L.y = tp.y;
-                if (nn.x < 0.0f && tn.x < L.x) L.x = tn.x;
-                if (nn.y < 0.0f && tn.y < L.y) L.y = tn.y;
+                L = limit2(dmax, dmin, pp, nn, e2p);
             }
             if (limiter == 0) L = bc2(0.0f);
 #pragma unroll
