@@ -177,9 +177,7 @@ avs_status avs_dt(avs_ctx *ctx, double cfl, double *dt_out);
  * multiscale flux (Eq. equ28), conservative W update, implicit-collision
  * update of f (diagonal of Eq. SGS_phi).  dt from cfl (avs_dt); dt_out
  * nullable.  Does not synchronise; numeric failures surface at the next
- * blocking call as AVS_ENUMERIC, and an asynchronous copy of the FP32 face
- * kernel that did not complete within its bound (about a second) as
- * AVS_ETIMEOUT. */
+ * blocking call as AVS_ENUMERIC. */
 avs_status ugks_step(avs_ctx *ctx, int nsteps, double cfl, double *dt_out);
 avs_status ugks_step_dt(avs_ctx *ctx, int nsteps, double dt);
 
@@ -325,14 +323,15 @@ avs_status avs_paper_parameters(const avs_flow_spec *spec, avs_config *cfg);
  * blocks.  Blocking.  Errors: EINVAL, ENOMEM, ECUDA, ETIMEOUT. */
 avs_status avs_grid_barrier_check(avs_ctx *ctx, int blocks, int rounds, int short_by, int *passed);
 
-/* Self-test of the bounded mbarrier wait that the staged face and cell
- * kernels use for their asynchronous bulk copies: one block initialises an
- * mbarrier; with arrive = 1 one thread issues a 128-byte bulk copy into
- * shared memory that completes it, with arrive = 0 nothing ever does, so the
- * wait gives up after its limit (about a second), sets the error bit of the
- * staged copies and the call returns AVS_ETIMEOUT with the context still
- * usable.  *completed (host) = 1 when the copy arrived and its 128 bytes
- * equal the source's.  Blocking.  Errors: EINVAL, ENOMEM, ECUDA, ETIMEOUT. */
+/* Self-test of the bounded mbarrier wait on an asynchronous bulk copy: one
+ * block initialises an mbarrier; with arrive = 1 one thread issues a 128-byte
+ * bulk copy into shared memory that completes it, with arrive = 0 nothing ever
+ * does, so the wait gives up after its limit (about a second), sets the error
+ * bit of such copies and the call returns AVS_ETIMEOUT with the context still
+ * usable.  (The step kernels' copies are waited for by the copying thread
+ * itself and need no such wait.)  *completed (host) = 1 when the copy arrived
+ * and its 128 bytes equal the source's.  Blocking.  Errors: EINVAL, ENOMEM,
+ * ECUDA, ETIMEOUT. */
 avs_status avs_stage_wait_check(avs_ctx *ctx, int arrive, int *completed);
 
 /* Measured FMA throughput of the current GPU (GFLOP/s, 2 flops per FMA):

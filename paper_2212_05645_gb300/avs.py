@@ -282,9 +282,8 @@ class AVS:
         return out.value
 
     def stage_wait_check(self, arrive=True):
-        """1 when a bulk copy completed the staged kernels' bounded mbarrier
-        wait with the right bytes; raises AVSError(AVS_ETIMEOUT) when nothing
-        arrives (arrive=False)."""
+        """1 when a bulk copy completed a bounded mbarrier wait with the right
+        bytes; raises AVSError(AVS_ETIMEOUT) when nothing arrives (arrive=False)."""
         out = C.c_int()
         self._ck(self.L.avs_stage_wait_check(self.h, int(bool(arrive)), C.byref(out)))
         return out.value

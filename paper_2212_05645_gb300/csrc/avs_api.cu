@@ -53,7 +53,7 @@ void free_all(avs_ctx* c)
     void* ptrs[] = {c->faceL, c->faceR, c->An_d, c->rL_d, c->rR_d, c->An_f, c->rL_f, c->rR_f, c->vol, c->bc,
                     c->slot, c->nslot, c->nbr, c->cg_d, c->r_d, c->eps2_d, c->cg_f, c->r_f, c->eps2_f,
                     c->level, c->base, c->key, c->level2, c->base2, c->key2, c->src, c->kind, c->emit,
-                    c->newidx, c->d_count, c->xi_d, c->w_d, c->xi_f, c->w_f, c->xi_p, c->M, c->Mkey, c->f[0], c->f[1],
+                    c->newidx, c->d_count, c->xi_d, c->w_d, c->xi_f, c->w_f, c->xi_p, c->xi_s, c->M, c->Mkey, c->f[0], c->f[1],
                     c->W[0], c->W[1], c->ncap, c->Wf, c->q, c->pseudo_f, c->pseudo_W, c->crit_cp, c->crit_cp32, c->Mlo, c->Mhi, c->Mthr, c->stage, c->dev_err,
                     c->dt_key, c->gap_d, c->grad, c->flux, c->AFf, c->forder, c->cmom, c->rmom, c->cpar, c->clist, c->cstart_d, c->imp_dW, c->imp_rhs0, c->imp_diag, c->imp_Wta,
                     c->imp_co, c->imp_nint, c->imp_bar, c->mlp_P, c->mlp_Wb, c->mlp_part, c->mlp_grad,
@@ -113,7 +113,7 @@ avs_status read_err(avs_ctx* c)
     CK(cudaStreamSynchronize(c->stream));
     if (e & 4) {
         CK(cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream));
-        return fail(c, AVS_ETIMEOUT, "an asynchronous copy into the face kernel's shared memory did not complete");
+        return fail(c, AVS_ETIMEOUT, "an asynchronous copy into shared memory did not complete");
     }
     if (e & 2) {
         CK(cudaMemsetAsync(c->dev_err, 0, sizeof(int), c->stream));
@@ -404,7 +404,12 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
     std::vector<int> order(Nf);
     for (int f = 0; f < Nf; ++f) order[f] = f;
     auto low = [&](int f) { const int R = m->faceR[f]; return R >= 0 ? std::min(m->faceL[f], R) : m->faceL[f]; };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return low(a) < low(b); });
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        const bool ba = m->faceR[a] < 0, bb = m->faceR[b] < 0;     // interior faces first
+        return ba != bb ? bb : low(a) < low(b);
+    });
+    c->Nfi = 0;
+    for (int f = 0; f < Nf; ++f) c->Nfi += m->faceR[f] >= 0;
     CK(up(c->forder, order, s));
     // greedy colouring in cell order (smallest colour no face neighbour has):
     // cells of one colour share no face (implicit sweeps)
@@ -562,6 +567,8 @@ avs_status avs_create(const avs_config* cfg, const avs_mesh* mesh, void* cuda_st
     AL(c->newidx, 2 * (size_t)capp); AL(c->d_count, 4);
     AL(c->xi_d, (size_t)capp * c->D); AL(c->w_d, capp);
     AL(c->xi_f, (size_t)capp * c->D); AL(c->w_f, capp); AL(c->xi_p, (size_t)capp * c->D);
+    c->xstride = capp;
+    AL(c->xi_s, (size_t)capp * c->D);
     AL(c->M, capp); AL(c->Mkey, capp); AL(c->ncap, capp);
     AL(c->pseudo_f, 2 * (size_t)c->NA * capp); AL(c->pseudo_W, 4 * NW);
     AL(c->crit_cp, 5 * (size_t)std::max(c->Nc, 2)); AL(c->crit_cp32, 8 * (size_t)std::max(c->Nc, 2));
@@ -762,7 +769,7 @@ avs_status avs_stage_wait_check(avs_ctx* c, int arrive, int* completed)
     int* dc = nullptr;
     if (dalloc(&d, 32) != cudaSuccess || dalloc(&dc, 1) != cudaSuccess) {
         cudaFree(d);
-        return fail(c, AVS_ENOMEM, "staged-copy wait check");
+        return fail(c, AVS_ENOMEM, "bulk-copy wait check");
     }
     cudaError_t e = cudaMemcpyAsync(d, src, sizeof(src), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(dc, 0, sizeof(int), c->stream);

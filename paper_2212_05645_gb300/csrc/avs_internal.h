@@ -13,7 +13,6 @@
 #define AVS_NT 256            // threads per block of the per-cell kernels
 #define AVS_CELLPAR_BYTES 256 // bytes per cell of the collision parameters (CellPar)
 #define AVS_CMOM_MAX 17       // carried raw moments per cell (monatomic 11 / 13, Rykov 14 / 17)
-#define AVS_SMALL_ROW_BYTES 8192 // f rows of a cell up to this size: one warp per face in the mixed step
 #define AVS_IMPSLOT_BYTES 96  // bytes per slot record of the implicit macroscopic sweep
 
 // Refinement caps of the velocity nodes (Sec. 3.5), passed to kernels by value.
@@ -64,6 +63,8 @@ struct avs_ctx {
     double *xi_d = nullptr, *w_d = nullptr;          // [cap][D], [cap]
     int *ncap = nullptr;                             // [cap] largest level a node may split to (zones)
     float *xi_f = nullptr, *w_f = nullptr;
+    float *xi_s = nullptr;                           // FP32 node coordinates by components: [D][xstride]
+    size_t xstride = 0;
     float *xi_p = nullptr;                           // FP32 node coordinates by pairs: [cap/2][D][2]
     double *M = nullptr;                             // [cap]
     unsigned long long *Mkey = nullptr;              // [cap]
@@ -85,7 +86,7 @@ struct avs_ctx {
     float *Mthr = nullptr;                           // [cap][4] label thresholds per node
     double *stage = nullptr;                         // FP64 staging [Nc][NA][Nv] for get/set (lazy)
     size_t stage_elems = 0;
-    int *dev_err = nullptr;                          // device error word (1: numeric, 2: grid barrier, 4: staged copy)
+    int *dev_err = nullptr;                          // device error word (1: numeric, 2: grid barrier, 4: bulk copy)
     unsigned long long *dt_key = nullptr;
     double *gap_d = nullptr;                         // correction gap (max over cells)
     double dt_unit = 0.0;
@@ -95,7 +96,8 @@ struct avs_ctx {
     void *flux = nullptr;                            // per-node face flux [Nf][NA][Nvp] of T
     size_t flux_bytes = 0;
     double *AFf = nullptr;                           // area-weighted face flux of W [Nf][D+2]
-    int *forder = nullptr;                           // face processing order (by lower cell index)
+    int *forder = nullptr;                           // face processing order: interior, then boundary faces,
+    int Nfi = 0;                                     //   each by lower cell index; number of interior faces
     double *cmom = nullptr;                          // raw moments of f about U(W) per cell [Nc][NMom]
     double *rmom = nullptr;                          // scratch raw moments [max(Nc,2)][NMom]
     int mom_valid = 0;                               // cmom matches the current f and W

@@ -1,15 +1,15 @@
 // One explicit UGKS step on the global velocity mesh (paper Sec. 2.3, with
 // the explicit readings R1-R4), as four kernels.
 //
-// k_foot: one thread block per (cell, node chunk).  The limited
-//   least-squares gradient L grad phi of the cell (Sec. 2.3.3: weights
-//   1/|d|^2, Venkatakrishnan limiter with epsilon^2 = (K dx)^3 phi_C^2) at
-//   each node, kept in registers, and the
-//   foot values phi_C + (L grad phi)_C . (x_f - xi h - x_C) of every face of
-//   the cell at the nodes where the cell is upwind (sign of xi . An), written
-//   to the face's row: each face node gets its foot value exactly once.
+// k_foot_f2 (FP32 form) / k_foot (FP64 form): per cell and node, the limited
+//   least-squares gradient L grad phi (Sec. 2.3.3: weights 1/|d|^2,
+//   Venkatakrishnan limiter with epsilon^2 = (K dx)^3 phi_C^2), kept in
+//   registers, and the foot values phi_C + (L grad phi)_C . (x_f - xi h - x_C)
+//   of every face of the cell at the nodes where the cell is upwind (sign of
+//   xi . An), written to the face's row: each face node gets its foot value
+//   exactly once.
 //
-// k_face: one thread block per face.  The raw velocity moments of the foot
+// k_face32 (avs_step32.cu) / k_face: the raw velocity moments of a face's foot
 //   values (interface W of Eq. w_interface and heat flux), the interface
 //   Shakhov state (Eqs. 3, equ28, R4), then the interface distribution
 //   phi_ij = tau/(tau+h) phi_bar + h/(tau+h) g_ij per node.  Writes the
@@ -17,10 +17,10 @@
 //   area-weighted flux of W.  Boundaries: diffuse wall with zero net mass
 //   flux, far-field Maxwellian (R8).
 //
-// k_cell_state / k_cell: one thread per cell, then one block per cell.
-//   Lagged heat flux from the moments of f^n (R3), W~ = W - dt/|V| sum_j A F_j
-//   (R2), the cell's Shakhov state and the collision update of every node
-//   from the net flux of its faces (diagonal of Eq. SGS_phi, R1).
+// k_cell_state: one thread per cell.  Lagged heat flux from the moments of f^n
+//   (R3), W~ = W - dt/|V| sum_j A F_j (R2), the cell's Shakhov state.
+// k_cell32 (avs_step32.cu) / k_cell: the collision update of every node of a
+//   cell from the net flux of its faces (diagonal of Eq. SGS_phi, R1).
 //
 // Every face is evaluated once, so the two cells of a face see the same flux
 // and W telescopes exactly.  f^n and W^n are read-only during the step; no
@@ -33,6 +33,7 @@
 
 #include "avs_dev.cuh"
 #include "avs_internal.h"
+#include "avs_step32.h"
 
 namespace avs {
 
@@ -600,40 +601,6 @@ __device__ __forceinline__ void load_nodes(const PP& P, int k0, T (*x)[D], T* w)
     ldv<T, V>(P.w + k0, w);
 }
 
-// FP32 node pair (k, k+1), k even, from the pair layout: X[d] the pair's
-// d-th components (one 8- or 16-byte load each), W2 their weights.
-template <int D, typename PP>
-__device__ __forceinline__ void load_pair(const PP& P, int k, float2 (&X)[D], float2& W2)
-{
-    const float* p = P.xp + (size_t)k * D;
-    if constexpr (D == 2) {
-        const float4 v = *reinterpret_cast<const float4*>(p);
-        X[0] = make_float2(v.x, v.y);
-        X[1] = make_float2(v.z, v.w);
-    } else {
-#pragma unroll
-        for (int d = 0; d < D; ++d) X[d] = *reinterpret_cast<const float2*>(p + 2 * d);
-    }
-    W2 = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(P.w) + k);
-}
-
-// Four FP32 nodes k..k+3, k a multiple of 4, as two pairs from the pair
-// layout (16-byte loads): X[p][d], W2[p] for the pair (k + 2p, k + 2p + 1).
-template <int D>
-__device__ __forceinline__ void load_quad(const float* xp, const float* w, int k, float2 (&X)[2][D],
-                                          float2 (&W2)[2])
-{
-    float xx[4 * D];
-    ldvn<float, 4 * D>(xp + (size_t)k * D, xx);
-#pragma unroll
-    for (int p = 0; p < 2; ++p)
-#pragma unroll
-        for (int d = 0; d < D; ++d) X[p][d] = make_float2(xx[(p * D + d) * 2], xx[(p * D + d) * 2 + 1]);
-    const float4 wv = *reinterpret_cast<const float4*>(w + k);
-    W2[0] = make_float2(wv.x, wv.y);
-    W2[1] = make_float2(wv.z, wv.w);
-}
-
 // ------------------------------------------------------------------ k_face
 template <int D, typename T>
 struct FaceP {
@@ -648,7 +615,6 @@ struct FaceP {
     const double* __restrict__ Win;
     const T* __restrict__ xi;
     const T* __restrict__ w;
-    const float* __restrict__ xp;            // FP32 node coordinates by pairs [Nvp/2][D][2]
     const int* __restrict__ order;
     const int* __restrict__ faceL;
     const int* __restrict__ faceR;
@@ -725,9 +691,8 @@ template <int D, typename T, int NT, bool CACHE, int V>
 __device__ __forceinline__ void face_pass_a(const FaceP<D, T>& P, const FaceSt<T>& S, T* fc, int kb, int ke,
                                             T* acc, int tid, int f)
 {
-    constexpr int NA = NArr<D>::v, NM = NMom<D>::v, NW = D + 2;
+    constexpr int NA = NArr<D>::v, NW = D + 2;
     constexpr int NR = FaceNR<D>::v;
-    constexpr bool PACK = sizeof(T) == 4 && V == 2;      // FP32 pairs in packed arithmetic
     const bool inter = S.kind == 0;
     T An[D], Vt[D];
 #pragma unroll
@@ -739,36 +704,7 @@ __device__ __forceinline__ void face_pass_a(const FaceP<D, T>& P, const FaceSt<T
     const T* fb = P.FB + (size_t)f * NA * Nvp;          // the face's foot values
 #pragma unroll
     for (int m = 0; m < NR; ++m) acc[m] = T(0);
-    bool packed = false;
-    if constexpr (PACK) {
-      if (inter) {
-        packed = true;
-        // FP32 node pairs in packed two-lane arithmetic; per-lane partial sums
-        float2 acc2[NM];
-#pragma unroll
-        for (int m = 0; m < NM; ++m) acc2[m] = bc2(0.0f);
-#pragma unroll 2
-        for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
-            float2 X[D], W2;
-            load_pair<D>(P, k0, X, W2);          // pad nodes carry w = 0 and contribute nothing
-            float2 F[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) F[a] = __ldcg(reinterpret_cast<const float2*>((const float*)fb + a * Nvp + k0));
-            if constexpr (CACHE) {
-#pragma unroll
-                for (int a = 0; a < NA; ++a) *reinterpret_cast<float2*>((float*)fc + a * Nvp + k0) = F[a];
-            }
-            float2 xs[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) xs[d] = add2(X[d], bc2(-(float)Vt[d]));
-            raw_acc2<D>(acc2, xs, mul2(W2, F[0]), NA == 2 ? mul2(W2, F[NA - 1]) : bc2(0.0f));
-        }
-#pragma unroll
-        for (int m = 0; m < NM; ++m) acc[m] = (T)(acc2[m].x + acc2[m].y);
-      }
-    }
-    if (packed) {
-    } else if (inter) {
+    if (inter) {
 #pragma unroll 2
         for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
             T x[V][D], wv[V];
@@ -858,7 +794,6 @@ __device__ __forceinline__ void face_pass_b(const FaceP<D, T>& P, const FaceSt<T
                                             T* acc, int tid, int f)
 {
     constexpr int NA = NArr<D>::v, NW = D + 2;
-    constexpr bool PACK = sizeof(T) == 4 && V == 2;
     const bool inter = S.kind == 0;
     T An[D];
 #pragma unroll
@@ -867,49 +802,7 @@ __device__ __forceinline__ void face_pass_b(const FaceP<D, T>& P, const FaceSt<T
     T* Fo = P.FB + (size_t)f * NA * Nvp;                // foot values in, flux out
 #pragma unroll
     for (int m = 0; m < NW; ++m) acc[m] = T(0);
-    bool packed = false;
-    if constexpr (PACK) {
-      if (inter) {
-        packed = true;
-        const float2 wa = bc2((float)S.wa), wb = bc2((float)S.wb);
-        const EqPar<float> eq = *reinterpret_cast<const EqPar<float>*>(&S.eq);
-        float2 acc2[NW];
-#pragma unroll
-        for (int m = 0; m < NW; ++m) acc2[m] = bc2(0.0f);
-#pragma unroll 2
-        for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
-            float2 X[D], W2;
-            load_pair<D>(P, k0, X, W2);
-            float2 sn = mul2(X[0], bc2(An[0]));
-#pragma unroll
-            for (int d = 1; d < D; ++d) sn = add2(sn, mul2(X[d], bc2(An[d])));
-            float2 F[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a)
-                F[a] = CACHE ? *reinterpret_cast<const float2*>((const float*)fc + a * Nvp + k0)
-                             : __ldcg(reinterpret_cast<const float2*>((const float*)Fo + a * Nvp + k0));
-            float2 gG, gH;
-            eq_eval2<D>(eq, X, gG, gH);
-            const float2 pG = fma2(wb, gG, mul2(wa, F[0]));
-            const float2 pH = NA == 2 ? fma2(wb, gH, mul2(wa, F[NA - 1])) : bc2(0.0f);
-            const float2 t = mul2(W2, sn);
-            float2 x2 = mul2(X[0], X[0]);
-#pragma unroll
-            for (int d = 1; d < D; ++d) x2 = fma2(X[d], X[d], x2);
-            acc2[0] = fma2(t, pG, acc2[0]);
-            const float2 tp = mul2(t, pG);
-#pragma unroll
-            for (int d = 0; d < D; ++d) acc2[1 + d] = fma2(tp, X[d], acc2[1 + d]);
-            acc2[D + 1] = fma2(mul2(t, bc2(0.5f)), fma2(x2, pG, pH), acc2[D + 1]);
-            *reinterpret_cast<float2*>((float*)Fo + k0) = mul2(sn, pG);
-            if (NA == 2) *reinterpret_cast<float2*>((float*)Fo + (size_t)(NA - 1) * Nvp + k0) = mul2(sn, pH);
-        }
-#pragma unroll
-        for (int m = 0; m < NW; ++m) acc[m] = (T)(acc2[m].x + acc2[m].y);
-      }
-    }
-    if (packed) {
-    } else if (inter) {
+    if (inter) {
         const T wa = S.wa, wb = S.wb;
 #pragma unroll 2
         for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
@@ -969,7 +862,7 @@ __device__ __forceinline__ void face_pass_b(const FaceP<D, T>& P, const FaceSt<T
 
 // One block per face, all nodes: setup, pass A, state, pass B.
 template <int D, typename T, int NT, bool CACHE, int VF>
-__global__ void __launch_bounds__(NT, NT == 32 ? 32 : ((sizeof(T) == 4) ? (VF == 4 ? 5 : 7) : 4)) k_face(FaceP<D, T> P)
+__global__ void __launch_bounds__(NT, 4) k_face(FaceP<D, T> P)
 {
     constexpr int NW = D + 2;
     constexpr int NR = FaceNR<D>::v;
@@ -995,239 +888,6 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 32 : ((sizeof(T) == 4) ? (VF ==
     if (S.kind == 0) {
         block_sum_t<NW, NT>(acc, sw, red);
         if (tid < NW) P.AF[(size_t)f * NW + tid] = red[tid];
-    }
-}
-
-// ---- k_face_staged: the FP32 face kernel for rows beyond the shared-memory
-// cache.  Same passes, state and arithmetic as k_face's packed path; the
-// face's foot-value row (and, with SXI, the node coordinates and weights,
-// which otherwise come by direct loads) reach shared memory by asynchronous
-// 1D bulk copies in stages of CH nodes, double-buffered on two mbarriers, so
-// that the loads of stage g+1 (and the first stages of pass B, during the
-// state computation) overlap the work on stage g.  Offsets and sizes are multiples of 16 bytes by construction (rows
-// of Nvp = 32 m nodes, stages of CH = 32 n nodes, the last one cut at Nvp).  Every
-// wait is bounded (about a second); a wait that gives up sets bit 4 of the
-// error word (AVS_ETIMEOUT at the next blocking call) and the block drains its
-// copies, again with a bound, before it leaves.
-template <int D, int CH, bool SXI>
-struct StageFloats { static constexpr int v = (NArr<D>::v + (SXI ? D + 1 : 0)) * CH; };
-constexpr long long kWaitCycles = 2000000000ll;
-
-template <int D, int NT, int CH, bool SXI>
-__global__ void __launch_bounds__(NT, NT == 64 ? 13 : 7) k_face_staged(FaceP<D, float> P)
-{
-    constexpr int NA = NArr<D>::v, NM = NMom<D>::v, NW = D + 2;
-    constexpr int NR = FaceNR<D>::v;
-    static_assert(CH % 32 == 0 && CH % (4 * NT) == 0, "stage: whole node quads per thread, 128-byte rows");
-    // node loop: with the coordinates loaded directly, quads (two 16-byte
-    // pair loads per coordinate block); with them staged, pairs (measured on
-    // GB300: 3D 68.1 against 70.4 ms per UGKS step, 2D 9.92 against 10.0)
-    constexpr bool QUAD = !SXI;
-    __shared__ FaceSt<float> S;
-    __shared__ double sw[(NT / 32) * NR];
-    __shared__ double red[NR];
-    extern __shared__ __align__(128) float stg[];   // two stages of SF floats
-    constexpr int SF = StageFloats<D, CH, SXI>::v;
-    __shared__ __align__(8) unsigned long long full[2];
-    __shared__ int bad, gbad, nissued;           // timeout flag, first stage given up, stages issued
-
-    const int tid = threadIdx.x;
-    const int f = P.order[blockIdx.x];
-    if (tid == 0) {
-        face_setup<D, float>(P, f, S);
-        mbar_init(&full[0], 1);
-        mbar_init(&full[1], 1);
-        mbar_init_fence();
-        bad = 0;
-        gbad = 1 << 30;
-        nissued = 0;
-    }
-    __syncthreads();
-    if (S.kind != 0) {
-        // boundary face: the direct-load passes
-        float acc[NR];
-        face_pass_a<D, float, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
-        block_sum_t<NR, NT>(acc, sw, red);
-        if (tid == 0) face_state<D, float>(P, S, red, P.AF + (size_t)f * NW);
-        __syncthreads();
-        float accb[NW];
-        face_pass_b<D, float, NT, false, 2>(P, S, nullptr, 0, P.Nv, accb, tid, f);
-        return;
-    }
-    const int Nv = P.Nv, Nvp = P.Nvp;
-    const int nst = (Nv + CH - 1) / CH;          // stages per pass
-    const int ng = 2 * nst;                      // pass A stages, then pass B stages
-    float* row = P.FB + (size_t)f * NA * Nvp;
-    auto issue = [&](int g) {                    // thread 0
-        const int b = g & 1;
-        const int k0 = (g < nst ? g : g - nst) * CH;
-        const int n = min(CH, Nvp - k0);         // a multiple of 32 nodes
-        const unsigned bytes = (unsigned)n * 4u;
-        float* dst = stg + b * SF;
-        nissued = g + 1;
-        mbar_arrive_expect_tx(&full[b], bytes * (unsigned)(NA + (SXI ? D + 1 : 0)));
-#pragma unroll
-        for (int a = 0; a < NA; ++a) bulk_g2s(dst + a * CH, row + (size_t)a * Nvp + k0, bytes, &full[b]);
-        if constexpr (SXI) {
-            bulk_g2s(dst + NA * CH, P.xp + (size_t)k0 * D, bytes * D, &full[b]);
-            bulk_g2s(dst + (NA + D) * CH, P.w + k0, bytes, &full[b]);
-        }
-    };
-    // node pair (k, k+1) = stage offsets (kk, kk+1): from the stage, or
-    // direct loads (the coordinates and weights are shared by all faces)
-    auto stage_nodes = [&](const float* st, int k, int kk, float2 (&X)[D], float2& W2) {
-        if constexpr (SXI) {
-            const float* xv = st + NA * CH + kk * D;      // pair layout, as in P.xp
-#pragma unroll
-            for (int d = 0; d < D; ++d) X[d] = *reinterpret_cast<const float2*>(xv + 2 * d);
-            W2 = *reinterpret_cast<const float2*>(st + (NA + D) * CH + kk);
-        } else {
-            load_pair<D>(P, k, X, W2);
-        }
-    };
-    auto wait = [&](int g) {
-        if (bad) return;                         // a wait gave up: no further waits
-        if (!mbar_wait_bounded(&full[g & 1], (unsigned)((g >> 1) & 1), kWaitCycles)) {
-            atomicOr(P.err, 4);
-            atomicMin(&gbad, g);
-            bad = 1;
-        }
-    };
-    if (tid == 0) {
-        // after a wait that gave up anywhere, later blocks issue no copies
-        if (*(volatile int*)P.err & 4) bad = 2;
-        if (!bad) {
-            issue(0);
-            if (ng > 1) issue(1);
-        }
-    }
-    __syncthreads();
-    if (bad) return;
-    float Vt[D], An[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        Vt[d] = S.Vt[d];
-        An[d] = S.An[d];
-    }
-    // ---------------- pass A: raw moments of the foot values about V
-    float2 acc2[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) acc2[m] = bc2(0.0f);
-    for (int g = 0; g < nst; ++g) {
-        wait(g);
-        const float* st = stg + (g & 1) * SF;
-        const int k0 = g * CH;
-        auto bodyA = [&](int kk, const float2 (&X)[D], float2 W2) {
-            float2 F[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) F[a] = *reinterpret_cast<const float2*>(st + a * CH + kk);
-            float2 xs[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) xs[d] = add2(X[d], bc2(-Vt[d]));
-            raw_acc2<D>(acc2, xs, mul2(W2, F[0]), NA == 2 ? mul2(W2, F[NA - 1]) : bc2(0.0f));
-        };
-        if constexpr (QUAD) {
-#pragma unroll 1
-            for (int kq = tid * 4; kq < CH; kq += NT * 4) {
-                if (k0 + kq >= Nv) break;        // the quad's pad nodes carry w = 0
-                float2 XQ[2][D], WQ[2];
-                load_quad<D>(P.xp, P.w, k0 + kq, XQ, WQ);
-                bodyA(kq, XQ[0], WQ[0]);
-                bodyA(kq + 2, XQ[1], WQ[1]);
-            }
-        } else {
-#pragma unroll 4
-            for (int kk = tid * 2; kk < CH; kk += NT * 2) {
-                if (k0 + kk >= Nv) break;
-                float2 X[D], W2;
-                stage_nodes(st, k0 + kk, kk, X, W2);
-                bodyA(kk, X, W2);
-            }
-        }
-        __syncthreads();
-        if (tid == 0 && g + 2 < ng && !bad) {
-            fence_proxy_async_smem();
-            issue(g + 2);
-        }
-    }
-    {
-        float acc[NR];
-#pragma unroll
-        for (int m = 0; m < NR; ++m) acc[m] = m < NM ? acc2[m].x + acc2[m].y : 0.0f;
-        block_sum_t<NR, NT>(acc, sw, red);
-    }
-    if (tid == 0) face_state<D, float>(P, S, red, P.AF + (size_t)f * NW);
-    __syncthreads();
-    // ---------------- pass B: per-node flux of the interface distribution
-    const float2 wa = bc2(S.wa), wb = bc2(S.wb);
-    const EqPar<float> eq = S.eq;
-    float2 accB[NW];
-#pragma unroll
-    for (int m = 0; m < NW; ++m) accB[m] = bc2(0.0f);
-    for (int g = nst; g < ng; ++g) {
-        wait(g);
-        const float* st = stg + (g & 1) * SF;
-        const int k0 = (g - nst) * CH;
-        auto bodyB = [&](int kk, const float2 (&X)[D], float2 W2) {
-            const int k = k0 + kk;
-            float2 F[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) F[a] = *reinterpret_cast<const float2*>(st + a * CH + kk);
-            float2 sn = mul2(X[0], bc2(An[0]));
-#pragma unroll
-            for (int d = 1; d < D; ++d) sn = add2(sn, mul2(X[d], bc2(An[d])));
-            float2 gG, gH;
-            eq_eval2<D>(eq, X, gG, gH);
-            const float2 pG = fma2(wb, gG, mul2(wa, F[0]));
-            const float2 pH = NA == 2 ? fma2(wb, gH, mul2(wa, F[NA - 1])) : bc2(0.0f);
-            const float2 t = mul2(W2, sn);
-            float2 x2 = mul2(X[0], X[0]);
-#pragma unroll
-            for (int d = 1; d < D; ++d) x2 = fma2(X[d], X[d], x2);
-            accB[0] = fma2(t, pG, accB[0]);
-            const float2 tp = mul2(t, pG);
-#pragma unroll
-            for (int d = 0; d < D; ++d) accB[1 + d] = fma2(tp, X[d], accB[1 + d]);
-            accB[D + 1] = fma2(mul2(t, bc2(0.5f)), fma2(x2, pG, pH), accB[D + 1]);
-            *reinterpret_cast<float2*>(row + k) = mul2(sn, pG);
-            if (NA == 2) *reinterpret_cast<float2*>(row + (size_t)(NA - 1) * Nvp + k) = mul2(sn, pH);
-        };
-        if constexpr (QUAD) {
-#pragma unroll 1
-            for (int kq = tid * 4; kq < CH; kq += NT * 4) {
-                if (k0 + kq >= Nv) break;        // the quad's pad nodes carry w = 0 and xi = 0
-                float2 XQ[2][D], WQ[2];
-                load_quad<D>(P.xp, P.w, k0 + kq, XQ, WQ);
-                bodyB(kq, XQ[0], WQ[0]);
-                bodyB(kq + 2, XQ[1], WQ[1]);
-            }
-        } else {
-#pragma unroll 4
-            for (int kk = tid * 2; kk < CH; kk += NT * 2) {
-                if (k0 + kk >= Nv) break;
-                float2 X[D], W2;
-                stage_nodes(st, k0 + kk, kk, X, W2);
-                bodyB(kk, X, W2);
-            }
-        }
-        __syncthreads();
-        if (tid == 0 && g + 2 < ng && !bad) {
-            fence_proxy_async_smem();
-            issue(g + 2);
-        }
-    }
-    {
-        float acc[NW];
-#pragma unroll
-        for (int m = 0; m < NW; ++m) acc[m] = accB[m].x + accB[m].y;
-        block_sum_t<NW, NT>(acc, sw, red);
-        if (tid < NW) P.AF[(size_t)f * NW + tid] = red[tid];
-    }
-    // a wait that gave up leaves copies in flight: drain them (bounded) before
-    // the block's shared memory is released
-    if (bad && tid == 0) {
-        for (int g = gbad; g < nissued; ++g)
-            mbar_wait_bounded(&full[g & 1], (unsigned)((g >> 1) & 1), kWaitCycles);
     }
 }
 
@@ -1258,7 +918,6 @@ struct CellP {
     CellPar<T>* par;         // [cell]
     const T* __restrict__ xi;
     const T* __restrict__ w;
-    const float* __restrict__ xp;            // FP32 node coordinates by pairs [Nvp/2][D][2]
     const int* __restrict__ slot;
     const unsigned char* __restrict__ nslot;
     const double* __restrict__ vol;
@@ -1276,44 +935,19 @@ __device__ __forceinline__ void cell_raw_moments(const CellP<D, T>& P, int i, in
 #pragma unroll
     for (int d = 0; d < D; ++d) Vct[d] = (T)P.Win[(size_t)i * NW + 1 + d] / (T)P.Win[(size_t)i * NW];
     const T* fi = P.fin + (size_t)i * P.cstride;
-    if constexpr (sizeof(T) == 4 && V == 4) {
-        // FP32: the four nodes as two lane pairs in packed arithmetic (the
-        // same pairing and order as cell_update's carried sums)
-        float2 acc2[NM];
 #pragma unroll
-        for (int m = 0; m < NM; ++m) acc2[m] = bc2(0.0f);
-        for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
-            float2 X[2][D], W2[2];
-            float f0[V], f1[V];
-            load_quad<D>(P.xp, P.w, k0, X, W2);
-            ldv<T, V>(fi + k0, f0);
-            if (NA == 2) ldv<T, V>(fi + P.Nvp + k0, f1);
+    for (int m = 0; m < NM; ++m) acc[m] = T(0);
+    for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
+        T x[V][D], wv[V], f0[V], f1[V];
+        load_nodes<D, V>(P, k0, x, wv);
+        ldv<T, V>(fi + k0, f0);
+        if (NA == 2) ldv<T, V>(fi + P.Nvp + k0, f1);
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                float2 xs[D];
+        for (int v = 0; v < V; ++v) {
+            T xs[D];
 #pragma unroll
-                for (int d = 0; d < D; ++d) xs[d] = add2(X[p][d], bc2(-Vct[d]));
-                raw_acc2<D>(acc2, xs, mul2(W2[p], make_float2(f0[2 * p], f0[2 * p + 1])),
-                            NA == 2 ? mul2(W2[p], make_float2(f1[2 * p], f1[2 * p + 1])) : bc2(0.0f));
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < NM; ++m) acc[m] = acc2[m].x + acc2[m].y;
-    } else {
-#pragma unroll
-        for (int m = 0; m < NM; ++m) acc[m] = T(0);
-        for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
-            T x[V][D], wv[V], f0[V], f1[V];
-            load_nodes<D, V>(P, k0, x, wv);
-            ldv<T, V>(fi + k0, f0);
-            if (NA == 2) ldv<T, V>(fi + P.Nvp + k0, f1);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                T xs[D];
-#pragma unroll
-                for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vct[d];
-                raw_acc<D>(acc, xs, wv[v] * f0[v], NA == 2 ? wv[v] * f1[v] : T(0));
-            }
+            for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vct[d];
+            raw_acc<D>(acc, xs, wv[v] * f0[v], NA == 2 ? wv[v] * f1[v] : T(0));
         }
     }
 }
@@ -1334,6 +968,26 @@ __global__ void __launch_bounds__(NT) k_raw_moments(CellP<D, T> P)
     if (threadIdx.x < NM) P.mom[(size_t)i * NM + threadIdx.x] = red[threadIdx.x];
 }
 
+// Cell record of the FP32 kernels: out = k0 f + k1 g~ + kN N.
+__device__ __forceinline__ Cell32Par cell32_par(const EqPar<float>& e, float k0, float k1, float kN, const float* V,
+                                                float diag)
+{
+    Cell32Par z;
+    for (int d = 0; d < 3; ++d) {
+        z.U[d] = e.U[d];
+        z.al[d] = e.alpha[d];
+        z.V[d] = V[d];
+    }
+    z.k2 = e.k2;
+    z.l2 = e.l2pref + log2f(k1);
+    z.k0 = k0;
+    z.RTH = e.RTH;
+    z.kN = kN;
+    z.pad = 0.0f;
+    z.diag = diag;
+    return z;
+}
+
 // One thread per cell: lagged heat flux q~ from the raw moments of f^n (R3),
 // W~ = W - dt/|V| sum_j sgn_j A F_j (R2), tau~ and the Shakhov parameters.
 template <int D, typename T>
@@ -1344,7 +998,10 @@ __global__ void k_cell_state(CellP<D, T> P)
     if (i >= P.Nc) return;
     const double* Wi = P.Win + (size_t)i * NW;
     double Vc[3] = {0.0, 0.0, 0.0}, m[NM];
-    for (int d = 0; d < D; ++d) Vc[d] = (double)((T)Wi[1 + d] / (T)Wi[0]);
+    for (int d = 0; d < D; ++d) {
+        if constexpr (sizeof(T) == 4) Vc[d] = (double)reinterpret_cast<const Cell32Par*>(P.par)[i].V[d];
+        else Vc[d] = Wi[1 + d] / Wi[0];
+    }
     for (int k = 0; k < NM; ++k) m[k] = P.mom[(size_t)i * NM + k];
     T rn, Un[3], RTn, qn[3];
     state_from_raw<D, T>(m, Vc, rn, Un, RTn, qn);
@@ -1372,6 +1029,12 @@ __global__ void k_cell_state(CellP<D, T> P)
     const T tau = tau_vhs<T>(rho, RT, (T)P.R, (T)P.mu_ref, (T)P.T_ref, (T)P.omega);
     cp.eq = make_eq_a<D, T, T>(rho, U, RT, qn, (T)P.Pr);
     const T idt = (T)(1.0 / P.dt), itau = T(1) / tau;
+    if constexpr (sizeof(T) == 4) {
+        const float u3 = 1.0f / (idt + itau);
+        reinterpret_cast<Cell32Par*>(P.par)[i] =
+            cell32_par(cp.eq, idt * u3, itau * u3, -(float)(1.0 / P.vol[i]) * u3, U, 0.0f);
+        return;
+    }
     cp.upd[0] = idt;
     cp.upd[1] = itau;
     cp.upd[2] = (T)(1.0 / P.vol[i]);
@@ -1397,116 +1060,52 @@ __device__ __forceinline__ void cell_update(const CellP<D, T>& P, int i, int ns,
     T Vnt[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) Vnt[d] = cp.Vn[d];
-    if constexpr (sizeof(T) == 4 && V == 4) {
-        // FP32: the four nodes as two lane pairs in packed arithmetic
-        float2 acc2[NM];
 #pragma unroll
-        for (int m = 0; m < NM; ++m) acc2[m] = bc2(0.0f);
-        const float2 U0 = bc2(u0), U1 = bc2(u1), U2n = bc2(-u2), U3 = bc2(u3);
-        const EqPar<float> eq = cp.eq;
-        for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
-            float2 XX[2][D], W2[2];
-            load_quad<D>(P.xp, P.w, k0, XX, W2);
-            float fv[NA][V];
-            float2 Nn[NA][2];
+    for (int m = 0; m < NM; ++m) acc[m] = T(0);
+    for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
+        T x[V][D], wv[V];
+        load_nodes<D, V>(P, k0, x, wv);
+        T Nn[NA][V], fv[NA][V], out[NA][V];
 #pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                ldv_cg<T, V>(fi + (size_t)a * P.Nvp + k0, fv[a]);
-                Nn[a][0] = Nn[a][1] = bc2(0.0f);
-            }
+        for (int a = 0; a < NA; ++a) {
+            ldv_cg<T, V>(fi + (size_t)a * P.Nvp + k0, fv[a]);
 #pragma unroll
-            for (int s = 0; s < AVS_MAXS; ++s) {
-                if (s >= ns) break;
-                const float* Fs = P.F + (size_t)fs[s] * NA * P.Nvp + k0;
-                const float2 g = bc2(sg[s]);
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    float t[V];
-                    ldv_cg<T, V>(Fs + (size_t)a * P.Nvp, t);
-                    Nn[a][0] = fma2(g, make_float2(t[0], t[1]), Nn[a][0]);
-                    Nn[a][1] = fma2(g, make_float2(t[2], t[3]), Nn[a][1]);
-                }
-            }
-            float out[NA][V];
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                const float2* X = XX[p];
-                float2 gG, gH;
-                eq_eval2<D>(eq, X, gG, gH);
-                const bool r0 = k0 + 2 * p < P.Nv, r1 = k0 + 2 * p + 1 < P.Nv;
-                float2 o[NA];
-                o[0] = mul2(fma2(Nn[0][p], U2n, fma2(make_float2(fv[0][2 * p], fv[0][2 * p + 1]), U0, mul2(gG, U1))),
-                            U3);
-                if (NA == 2)
-                    o[NA - 1] = mul2(fma2(Nn[NA - 1][p], U2n,
-                                          fma2(make_float2(fv[NA - 1][2 * p], fv[NA - 1][2 * p + 1]), U0,
-                                               mul2(gH, U1))),
-                                     U3);
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    out[a][2 * p] = r0 ? o[a].x : 0.0f;
-                    out[a][2 * p + 1] = r1 ? o[a].y : 0.0f;
-                }
-                float2 xs[D];
-#pragma unroll
-                for (int d = 0; d < D; ++d) xs[d] = add2(X[d], bc2(-Vnt[d]));
-                raw_acc2<D>(acc2, xs, mul2(W2[p], make_float2(out[0][2 * p], out[0][2 * p + 1])),
-                            NA == 2 ? mul2(W2[p], make_float2(out[NA - 1][2 * p], out[NA - 1][2 * p + 1]))
-                                    : bc2(0.0f));
-            }
-#pragma unroll
-            for (int a = 0; a < NA; ++a) stv<T, V>(fo + (size_t)a * P.Nvp + k0, out[a]);
+            for (int v = 0; v < V; ++v) Nn[a][v] = T(0);
         }
 #pragma unroll
-        for (int m = 0; m < NM; ++m) acc[m] = acc2[m].x + acc2[m].y;
-    } else {
-#pragma unroll
-        for (int m = 0; m < NM; ++m) acc[m] = T(0);
-        for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
-            T x[V][D], wv[V];
-            load_nodes<D, V>(P, k0, x, wv);
-            T Nn[NA][V], fv[NA][V], out[NA][V];
+        for (int s = 0; s < AVS_MAXS; ++s) {
+            if (s >= ns) break;
+            const T* Fs = P.F + (size_t)fs[s] * NA * P.Nvp + k0;
+            const T g = sg[s];
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
-                ldv_cg<T, V>(fi + (size_t)a * P.Nvp + k0, fv[a]);
+                T t[V];
+                ldv_cg<T, V>(Fs + (size_t)a * P.Nvp, t);
 #pragma unroll
-                for (int v = 0; v < V; ++v) Nn[a][v] = T(0);
+                for (int v = 0; v < V; ++v) Nn[a][v] += g * t[v];
             }
-#pragma unroll
-            for (int s = 0; s < AVS_MAXS; ++s) {
-                if (s >= ns) break;
-                const T* Fs = P.F + (size_t)fs[s] * NA * P.Nvp + k0;
-                const T g = sg[s];
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    T t[V];
-                    ldv_cg<T, V>(Fs + (size_t)a * P.Nvp, t);
-#pragma unroll
-                    for (int v = 0; v < V; ++v) Nn[a][v] += g * t[v];
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                T gG, gH;
-                eq_eval<D>(cp.eq, x[v], gG, gH);
-                const bool real = k0 + v < P.Nv;
-                out[0][v] = real ? (fv[0][v] * u0 + gG * u1 - Nn[0][v] * u2) * u3 : T(0);
-                if (NA == 2)
-                    out[NA - 1][v] = real ? (fv[NA - 1][v] * u0 + gH * u1 - Nn[NA - 1][v] * u2) * u3 : T(0);
-                T xs[D];
-#pragma unroll
-                for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vnt[d];
-                raw_acc<D>(acc, xs, wv[v] * out[0][v], NA == 2 ? wv[v] * out[NA - 1][v] : T(0));
-            }
-#pragma unroll
-            for (int a = 0; a < NA; ++a) stv<T, V>(fo + (size_t)a * P.Nvp + k0, out[a]);
         }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            T gG, gH;
+            eq_eval<D>(cp.eq, x[v], gG, gH);
+            const bool real = k0 + v < P.Nv;
+            out[0][v] = real ? (fv[0][v] * u0 + gG * u1 - Nn[0][v] * u2) * u3 : T(0);
+            if (NA == 2)
+                out[NA - 1][v] = real ? (fv[NA - 1][v] * u0 + gH * u1 - Nn[NA - 1][v] * u2) * u3 : T(0);
+            T xs[D];
+#pragma unroll
+            for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vnt[d];
+            raw_acc<D>(acc, xs, wv[v] * out[0][v], NA == 2 ? wv[v] * out[NA - 1][v] : T(0));
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) stv<T, V>(fo + (size_t)a * P.Nvp + k0, out[a]);
     }
 }
 
 // One block per cell, all nodes; the raw moments of f^{n+1} to P.mom.
 template <int D, typename T, int NT, int VC>
-__global__ void __launch_bounds__(NT, NT == 32 ? 28 : ((sizeof(T) == 4) ? (VC == 4 ? 7 : 7) : 4)) k_cell(CellP<D, T> P)
+__global__ void __launch_bounds__(NT, 4) k_cell(CellP<D, T> P)
 {
     constexpr int NM = NMom<D>::v;
     __shared__ int fs[AVS_MAXS];
@@ -1527,198 +1126,6 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 28 : ((sizeof(T) == 4) ? (VC ==
     __syncthreads();
     T acc[NM];
     cell_update<D, T, NT, VC>(P, i, ns, fs, sg, cp, 0, P.Nv, acc);
-    block_sum_t<NM, NT>(acc, sw, red);
-    if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
-}
-
-// ---- k_cell_staged: the FP32 cell kernel with the cell's own f row and its
-// faces' flux rows streamed through shared memory in stages of CH nodes by
-// asynchronous 1D bulk copies, double-buffered on two mbarriers (the direct
-// form waits on its loads: eleven 16-byte rows per four nodes and warp).
-// Same arithmetic as cell_update's packed form.  Nodes by pairs, pair kk/2 of
-// a stage to thread (kk/2) mod NT, up to the quad boundary Nvq of the real
-// nodes (pad nodes written as zero); k_raw_moments_pairs repeats that order,
-// so that the carried raw moments equal recomputed ones bit for bit.  nrow:
-// rows per stage, NA (1 + largest face count).  Copies start on 128-byte row
-// boundaries (Nvp = 32 m) and are multiples of 128 bytes.  Waits are bounded
-// as in k_face_staged (bit 4 of the error word).
-constexpr int kCellStageMin = 1024;              // nodes above which the 3D cell kernel stages its rows
-template <int D, int NT, int CH>
-__global__ void __launch_bounds__(NT, 7) k_cell_staged(CellP<D, float> P, int nrow)
-{
-    constexpr int NA = NArr<D>::v, NM = NMom<D>::v;
-    static_assert(CH % 32 == 0 && CH % (2 * NT) == 0, "stage: whole node pairs per thread, 128-byte rows");
-    extern __shared__ __align__(128) float stg[];
-    __shared__ int fs[AVS_MAXS];
-    __shared__ float sg[AVS_MAXS];
-    __shared__ double sw[(NT / 32) * NM];
-    __shared__ double red[NM];
-    __shared__ CellPar<float> cp;
-    __shared__ __align__(8) unsigned long long full[2];
-    __shared__ int bad, gbad, nissued;           // timeout flag, first stage given up, stages issued
-
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x;
-    const int ns = P.nslot[i];
-    if (tid < ns) {
-        const int sl = P.slot[i * AVS_MAXS + tid];
-        fs[tid] = sl >> 1;
-        sg[tid] = (sl & 1) ? -1.0f : 1.0f;
-    }
-    if (tid == NT - 1) cp = P.par[i];
-    if (tid == 0) {
-        mbar_init(&full[0], 1);
-        mbar_init(&full[1], 1);
-        mbar_init_fence();
-        bad = 0;
-        gbad = 1 << 30;
-        nissued = 0;
-    }
-    __syncthreads();
-    const int Nv = P.Nv, Nvp = P.Nvp, Nvq = (Nv + 3) & ~3;
-    const int nst = (Nvq + CH - 1) / CH;
-    const size_t SF = (size_t)nrow * CH;
-    const float* fi = P.fin + (size_t)i * P.cstride;
-    float* fo = P.fout + (size_t)i * P.cstride;
-    auto issue = [&](int g) {                    // thread 0
-        const int b = g & 1;
-        const int k0 = g * CH;
-        const int n = min(CH, Nvp - k0);         // a multiple of 32 nodes
-        const unsigned bytes = (unsigned)n * 4u;
-        float* dst = stg + b * SF;
-        nissued = g + 1;
-        mbar_arrive_expect_tx(&full[b], bytes * (unsigned)(NA * (1 + ns)));
-#pragma unroll
-        for (int a = 0; a < NA; ++a) bulk_g2s(dst + a * CH, fi + (size_t)a * Nvp + k0, bytes, &full[b]);
-        for (int s = 0; s < ns; ++s)
-#pragma unroll
-            for (int a = 0; a < NA; ++a)
-                bulk_g2s(dst + (size_t)(NA * (1 + s) + a) * CH, P.F + ((size_t)fs[s] * NA + a) * Nvp + k0, bytes,
-                         &full[b]);
-    };
-    auto wait = [&](int g) {
-        if (bad) return;                         // a wait gave up: no further waits
-        if (!mbar_wait_bounded(&full[g & 1], (unsigned)((g >> 1) & 1), kWaitCycles)) {
-            atomicOr(P.err, 4);
-            atomicMin(&gbad, g);
-            bad = 1;
-        }
-    };
-    if (tid == 0) {
-        // after a wait that gave up anywhere, later blocks issue no copies
-        if (*(volatile int*)P.err & 4) bad = 2;
-        if (!bad) {
-            issue(0);
-            if (nst > 1) issue(1);
-        }
-    }
-    __syncthreads();
-    if (bad) return;
-    const float2 U0 = bc2(cp.upd[0]), U1 = bc2(cp.upd[1]), U2n = bc2(-cp.upd[2]), U3 = bc2(cp.upd[3]);
-    const EqPar<float> eq = cp.eq;
-    float Vnt[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) Vnt[d] = cp.Vn[d];
-    float2 acc2[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) acc2[m] = bc2(0.0f);
-    for (int g = 0; g < nst; ++g) {
-        wait(g);
-        const float* st = stg + (g & 1) * SF;
-        const int k0 = g * CH;
-        for (int kk = tid * 2; kk < CH; kk += NT * 2) {
-            const int k = k0 + kk;
-            if (k >= Nvq) break;
-            float2 X[D], W2;
-            load_pair<D>(P, k, X, W2);
-            float2 fv[NA], Nn[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                fv[a] = *reinterpret_cast<const float2*>(st + a * CH + kk);
-                Nn[a] = bc2(0.0f);
-            }
-#pragma unroll
-            for (int s = 0; s < AVS_MAXS; ++s) {
-                if (s >= ns) break;
-                const float2 gs = bc2(sg[s]);
-#pragma unroll
-                for (int a = 0; a < NA; ++a)
-                    Nn[a] = fma2(gs, *reinterpret_cast<const float2*>(st + (NA * (1 + s) + a) * CH + kk), Nn[a]);
-            }
-            float2 gG, gH;
-            eq_eval2<D>(eq, X, gG, gH);
-            const bool r0 = k < Nv, r1 = k + 1 < Nv;
-            float2 o[NA];
-            o[0] = mul2(fma2(Nn[0], U2n, fma2(fv[0], U0, mul2(gG, U1))), U3);
-            if (NA == 2) o[NA - 1] = mul2(fma2(Nn[NA - 1], U2n, fma2(fv[NA - 1], U0, mul2(gH, U1))), U3);
-#pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                o[a] = make_float2(r0 ? o[a].x : 0.0f, r1 ? o[a].y : 0.0f);
-                *reinterpret_cast<float2*>(fo + (size_t)a * Nvp + k) = o[a];
-            }
-            float2 xs[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) xs[d] = add2(X[d], bc2(-Vnt[d]));
-            raw_acc2<D>(acc2, xs, mul2(W2, o[0]), NA == 2 ? mul2(W2, o[NA - 1]) : bc2(0.0f));
-        }
-        __syncthreads();
-        if (tid == 0 && g + 2 < nst && !bad) {
-            fence_proxy_async_smem();
-            issue(g + 2);
-        }
-    }
-    float acc[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) acc[m] = acc2[m].x + acc2[m].y;
-    block_sum_t<NM, NT>(acc, sw, red);
-    if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
-    // a wait that gave up leaves copies in flight: drain them (bounded) before
-    // the block's shared memory is released
-    if (bad && tid == 0) {
-        for (int g = gbad; g < nissued; ++g)
-            mbar_wait_bounded(&full[g & 1], (unsigned)((g >> 1) & 1), kWaitCycles);
-    }
-}
-
-// Raw moments of the own FP32 f of every cell about its U(W) in the node
-// order of k_cell_staged (pairs kk/2 of each CH-node stage to thread
-// (kk/2) mod NT, up to the quad boundary), one block per cell.
-template <int D, int NT, int CH>
-__global__ void __launch_bounds__(NT) k_raw_moments_pairs(CellP<D, float> P)
-{
-    constexpr int NA = NArr<D>::v, NM = NMom<D>::v, NW = D + 2;
-    __shared__ double sw[(NT / 32) * NM];
-    __shared__ double red[NM];
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x;
-    float Vct[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) Vct[d] = (float)P.Win[(size_t)i * NW + 1 + d] / (float)P.Win[(size_t)i * NW];
-    const int Nv = P.Nv, Nvp = P.Nvp, Nvq = (Nv + 3) & ~3;
-    const int nst = (Nvq + CH - 1) / CH;
-    const float* fi = P.fin + (size_t)i * P.cstride;
-    float2 acc2[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) acc2[m] = bc2(0.0f);
-    for (int g = 0; g < nst; ++g) {
-        const int k0 = g * CH;
-        for (int kk = tid * 2; kk < CH; kk += NT * 2) {
-            const int k = k0 + kk;
-            if (k >= Nvq) break;
-            float2 X[D], W2;
-            load_pair<D>(P, k, X, W2);
-            float2 fv[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) fv[a] = *reinterpret_cast<const float2*>(fi + (size_t)a * Nvp + k);
-            float2 xs[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) xs[d] = add2(X[d], bc2(-Vct[d]));
-            raw_acc2<D>(acc2, xs, mul2(W2, fv[0]), NA == 2 ? mul2(W2, fv[NA - 1]) : bc2(0.0f));
-        }
-    }
-    float acc[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) acc[m] = acc2[m].x + acc2[m].y;
     block_sum_t<NM, NT>(acc, sw, red);
     if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
 }
@@ -1907,6 +1314,7 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
         }
         c->launches += 1;
     }
+    if constexpr (sizeof(T) == 4) return launch_face32(c, Win, dt);
     FaceP<D, T> P;
     P.Nv = c->Nv;
     P.Nvp = c->Nvp;
@@ -1923,7 +1331,6 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
     P.Win = Win;
     P.xi = xi;
     P.w = w;
-    P.xp = c->xi_p;
     P.order = c->forder;
     P.faceL = c->faceL;
     P.faceR = c->faceR;
@@ -1937,50 +1344,16 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
     // the default dynamic allowance (48 KB); otherwise pass B re-reads the
     // face's row
     const size_t cache_bytes = (size_t)NA * c->Nvp * sizeof(T);
-    // two nodes per thread per iteration (8-byte FP32 / 16-byte FP64 vectors):
-    // fewer registers and more resident warps than 16-byte FP32 vectors, which
-    // the latency-bound face passes prefer; the node loops are unrolled twice
-    // so that two iterations' loads are in flight together
-    constexpr int VF = 2;
-    // small velocity meshes (the Sec. 3.5 spaces): one warp per face, so that
-    // threads are not left idle and the block's serial state section holds no
-    // other warp; the foot cache then stays small enough for 28+ blocks per SM.
-    // Above 256 nodes only with faces enough to fill every SM with such
-    // blocks (on fewer faces, 128-thread blocks keep more nodes in flight).
-    bool done = false;
-    if constexpr (sizeof(T) == 4) {
-        if (cache_bytes <= AVS_SMALL_ROW_BYTES && (c->Nv <= 256 || c->Nf >= 32 * c->nsm)) {
-            k_face<D, T, 32, true, VF><<<c->Nf, 32, cache_bytes, c->stream>>>(P);
-            done = true;
-        }
-    }
+    constexpr int VF = 2;            // nodes per thread and iteration: 16-byte vectors
     // the default allowance covers static and dynamic shared memory together:
     // the block's own arrays (state, reductions: under 2 KB) come first
     constexpr size_t kStaticFace = 2048;
     static_assert(sizeof(FaceSt<T>) + (NT / 32 + 1) * FaceNR<D>::v * sizeof(double) <= kStaticFace,
                   "static shared memory of the face block");
-    if (done) {
-    } else if (cache_bytes + kStaticFace <= 48 * 1024) {
+    if (cache_bytes + kStaticFace <= 48 * 1024)
         k_face<D, T, NT, true, VF><<<c->Nf, NT, cache_bytes, c->stream>>>(P);
-    } else if constexpr (sizeof(T) == 4) {
-        // rows beyond the cache: bulk-copy stages in shared memory (rows of
-        // Nvp = 32 m FP32 values keep every copy 16-byte aligned)
-        // measured on GB300 (2D wedge, 12k nodes; 3D sphere, 21k nodes):
-        // 2D: stages of 1024 nodes with the node coordinates and weights;
-        // 3D: stages of 2048 nodes, coordinates and weights loaded directly
-        constexpr int CH = D == 2 ? 1024 : 2048;
-        constexpr bool SXI = D == 2;
-        constexpr int NTs = D == 2 ? NT : 64;    // 3D: 64-thread face blocks, 13 per SM
-        constexpr size_t smem = 2 * sizeof(float) * StageFloats<D, CH, SXI>::v;
-        if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(k_face_staged<D, NTs, CH, SXI>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        k_face_staged<D, NTs, CH, SXI><<<c->Nf, NTs, smem, c->stream>>>(P);
-    } else {
+    else
         k_face<D, T, NT, false, VF><<<c->Nf, NT, 0, c->stream>>>(P);
-    }
     c->launches += 1;
 
     return cudaGetLastError();
@@ -2018,59 +1391,29 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
     Q.par = (CellPar<T>*)c->cpar;
     Q.xi = xi;
     Q.w = w;
-    Q.xp = c->xi_p;
     Q.slot = c->slot;
     Q.nslot = c->nslot;
     Q.vol = c->vol;
     Q.err = c->dev_err;
-    // 16-byte vectors (4 FP32 / 2 FP64 nodes per thread) in the cell kernel: it
-    // streams f and the face fluxes, and more bytes in flight per warp beat the
-    // extra warps of narrower vectors; k_raw_moments uses the same node mapping
-    // so that its sums equal the carried ones bit for bit
-    constexpr int VC = VW<T>::v;
-    // one warp per cell wherever the cells fill every SM with such blocks (and
-    // on small velocity meshes): the cell kernel streams its rows, so a warp
-    // per cell keeps as many loads in flight and ends with a warp-only
-    // reduction; the raw-moment kernel takes the same node mapping (the sums
-    // stay the carried ones bit for bit; an adaptation drops them)
-    auto cell_stage = [&](auto ntc) {
-        constexpr int NTc = decltype(ntc)::value;
-        if (!c->mom_valid) {
-            k_raw_moments<D, T, NTc, VC><<<c->Nc, NTc, 0, c->stream>>>(Q);
+    if (!c->mom_valid) {
+        if constexpr (sizeof(T) == 4) {
+            e = launch_raw32(c, fin, Win);
+            if (e != cudaSuccess) return e;
+        } else {
+            k_raw_moments<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
             c->launches += 1;
         }
-        k_cell_state<D, T><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(Q);
-        k_cell<D, T, NTc, VC><<<c->Nc, NTc, 0, c->stream>>>(Q);
-        c->launches += 2;
-    };
+    }
+    k_cell_state<D, T><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(Q);
+    c->launches += 1;
     if constexpr (sizeof(T) == 4) {
-        if (D == 3 && c->Nv > kCellStageMin) {
-            // 3D rows beyond a thousand nodes: the staged cell kernel and the
-            // raw-moment kernel of its node order (measured on GB300: 1 %
-            // faster on the 21.8k-node sphere; slower in 2D, where the two
-            // arrays and four faces take 40 KB of shared memory per block)
-            constexpr int NTs = 128, CHs = 512;
-            const int nrow = NA * (1 + c->max_ns);
-            const size_t smem = 2 * sizeof(float) * (size_t)nrow * CHs;
-            if (smem > 48 * 1024) {
-                const cudaError_t e = cudaFuncSetAttribute(k_cell_staged<D, NTs, CHs>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-            }
-            if (!c->mom_valid) {
-                k_raw_moments_pairs<D, NTs, CHs><<<c->Nc, NTs, 0, c->stream>>>(Q);
-                c->launches += 1;
-            }
-            k_cell_state<D, T><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(Q);
-            k_cell_staged<D, NTs, CHs><<<c->Nc, NTs, smem, c->stream>>>(Q, nrow);
-            c->launches += 2;
-        } else if (c->Nv <= 256 || c->Nc >= 28 * c->nsm) {
-            cell_stage(std::integral_constant<int, 32>{});
-        } else {
-            cell_stage(std::integral_constant<int, NT>{});
-        }
+        e = launch_cell32(c, fin, fout, false);
+        if (e != cudaSuccess) return e;
     } else {
-        cell_stage(std::integral_constant<int, NT>{});
+        // 16-byte vectors of nodes per thread; k_raw_moments takes the same
+        // node mapping, so that its sums equal the carried ones bit for bit
+        k_cell<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+        c->launches += 1;
     }
     c->mom_valid = 1;          // the raw moments of fout about U(Wout) are in cmom
     return cudaGetLastError();
@@ -2235,7 +1578,8 @@ cudaError_t launch_grid_barrier_check(avs_ctx* c, int blocks, int rounds, int sh
     return e;
 }
 
-// Self-test of the bounded mbarrier wait of the staged kernels: with `arrive`
+constexpr long long kWaitCycles = 2000000000ll;
+// Self-test of a bounded mbarrier wait on a bulk copy: with `arrive`
 // one 128-byte bulk copy completes the barrier and the copied bytes are
 // compared with the source; without, no arrival ever comes and every thread's
 // wait gives up after kWaitCycles, setting bit 4 of the error word.
@@ -2351,7 +1695,10 @@ __global__ void k_imp_state(CellP<D, T> P, const double* Wt)
     if (i >= P.Nc) return;
     const double* Wi = P.Win + (size_t)i * NW;
     double Vc[3] = {0.0, 0.0, 0.0}, m[NM];
-    for (int d = 0; d < D; ++d) Vc[d] = (double)((T)Wi[1 + d] / (T)Wi[0]);
+    for (int d = 0; d < D; ++d) {
+        if constexpr (sizeof(T) == 4) Vc[d] = (double)reinterpret_cast<const Cell32Par*>(P.par)[i].V[d];
+        else Vc[d] = Wi[1 + d] / Wi[0];
+    }
     for (int k = 0; k < NM; ++k) m[k] = P.mom[(size_t)i * NM + k];
     T rn, Un[3], RTn, qn[3];
     state_from_raw<D, T>(m, Vc, rn, Un, RTn, qn);
@@ -2365,6 +1712,12 @@ __global__ void k_imp_state(CellP<D, T> P, const double* Wt)
     const T tau = tau_vhs<T>(rho, RT, (T)P.R, (T)P.mu_ref, (T)P.T_ref, (T)P.omega);
     cp.eq = make_eq_a<D, T, T>(rho, U, RT, qn, (T)P.Pr);
     const T V = (T)P.vol[i];
+    if constexpr (sizeof(T) == 4) {
+        const float zero[3] = {0.0f, 0.0f, 0.0f};
+        reinterpret_cast<Cell32Par*>(P.par)[i] =
+            cell32_par(cp.eq, -V / tau, V / tau, -1.0f, zero, V / (float)P.dt + V / tau);
+        return;
+    }
     cp.upd[0] = V / (T)P.dt + V / tau;
     cp.upd[1] = tau;
     cp.upd[2] = V;
@@ -2457,7 +1810,9 @@ __global__ void __launch_bounds__(NT) k_imp_micro(CellP<D, T> P, const T* __rest
     __syncthreads();
     const int k0 = (blockIdx.y * NT + tid) * V;
     if (k0 >= P.Nv) return;
-    const T u0 = P.par[i].upd[0];
+    T u0;
+    if constexpr (sizeof(T) == 4) u0 = reinterpret_cast<const Cell32Par*>(P.par)[i].diag;
+    else u0 = P.par[i].upd[0];
     T x[V][D], wv[V];
     load_nodes<D, V>(P, k0, x, wv);
     T sn[AVS_MAXS][V], dg[V];
@@ -2599,19 +1954,29 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
     Q.par = (CellPar<T>*)c->cpar;
     Q.xi = xi;
     Q.w = w;
-    Q.xp = c->xi_p;
     Q.slot = c->slot;
     Q.nslot = c->nslot;
     Q.vol = c->vol;
     Q.err = c->dev_err;
     constexpr int NT = 128;
     if (!c->mom_valid) {
-        k_raw_moments<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
-        c->launches += 1;
+        if constexpr (sizeof(T) == 4) {
+            e = launch_raw32(c, fin, Win);
+            if (e != cudaSuccess) return e;
+        } else {
+            k_raw_moments<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+            c->launches += 1;
+        }
     }
     k_imp_state<D, T><<<cb, 128, 0, c->stream>>>(Q, Wout);
-    k_imp_res<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
-    c->launches += 2;
+    c->launches += 1;
+    if constexpr (sizeof(T) == 4) {
+        e = launch_cell32(c, fin, fout, true);
+        if (e != cudaSuccess) return e;
+    } else {
+        k_imp_res<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+        c->launches += 1;
+    }
     T* dphi = (T*)c->flux;                    // the face flux has been used: its buffer holds dphi
     e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);
     if (e != cudaSuccess) return e;
