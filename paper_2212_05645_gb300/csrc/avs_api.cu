@@ -51,7 +51,7 @@ size_t elem_size(const avs_ctx* c) { return c->mixed ? sizeof(float) : sizeof(do
 void free_all(avs_ctx* c)
 {
     void* ptrs[] = {c->faceL, c->faceR, c->An_d, c->rL_d, c->rR_d, c->An_f, c->rL_f, c->rR_f, c->vol, c->bc,
-                    c->slot, c->nslot, c->nbr, c->cg_d, c->r_d, c->eps2_d, c->cg_f, c->r_f, c->eps2_f,
+                    c->slot, c->nslot, c->nbr, c->cg_d, c->r_d, c->eps2_d, c->eps2_f, c->geo32, c->iorder,
                     c->level, c->base, c->key, c->level2, c->base2, c->key2, c->src, c->kind, c->emit,
                     c->newidx, c->d_count, c->xi_d, c->w_d, c->xi_f, c->w_f, c->xi_p, c->xi_s, c->M, c->Mkey, c->f[0], c->f[1],
                     c->W[0], c->W[1], c->ncap, c->Wf, c->q, c->pseudo_f, c->pseudo_W, c->crit_cp, c->crit_cp32, c->Mlo, c->Mhi, c->Mthr, c->stage, c->dev_err,
@@ -372,8 +372,9 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
         dalloc(&c->rR_d, nfd) || dalloc(&c->An_f, nfd) || dalloc(&c->rL_f, nfd) || dalloc(&c->rR_f, nfd) ||
         dalloc(&c->vol, Nc) || dalloc(&c->bc, (size_t)std::max(1, c->nbc) * 6) || dalloc(&c->slot, ncs) ||
         dalloc(&c->nslot, Nc) || dalloc(&c->nbr, ncs) || dalloc(&c->cg_d, ncsd) || dalloc(&c->r_d, ncsd) ||
-        dalloc(&c->eps2_d, Nc) || dalloc(&c->cg_f, ncsd) || dalloc(&c->r_f, ncsd) || dalloc(&c->eps2_f, Nc) ||
-        dalloc(&c->AFf, (size_t)Nf * c->NW) || dalloc(&c->forder, Nf) || dalloc(&c->cmom, (size_t)Nc * AVS_CMOM_MAX) ||
+        dalloc(&c->eps2_d, Nc) || dalloc(&c->eps2_f, Nc) ||
+        dalloc(&c->geo32, ncs * 12) ||
+        dalloc(&c->AFf, (size_t)Nf * c->NW) || dalloc(&c->forder, Nf) || dalloc(&c->iorder, Nf) || dalloc(&c->cmom, (size_t)Nc * AVS_CMOM_MAX) ||
         dalloc((unsigned char**)&c->cpar, (size_t)Nc * AVS_CELLPAR_BYTES) || dalloc(&c->clist, Nc) ||
         dalloc(&c->imp_dW, (size_t)Nc * c->NW) || dalloc(&c->imp_rhs0, (size_t)Nc * c->NW) ||
         dalloc(&c->imp_diag, Nc) || dalloc(&c->imp_Wta, (size_t)Nc * c->NW) ||
@@ -396,21 +397,42 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
     CK(up(c->cg_d, cg, s));
     CK(up(c->r_d, r, s));
     CK(up(c->eps2_d, eps2, s));
-    CK(up(c->cg_f, tof(cg.data(), ncsd), s));
-    CK(up(c->r_f, tof(r.data(), ncsd), s));
     CK(up(c->eps2_f, tof(eps2.data(), Nc), s));
+    // FP32 geometry records, one contiguous block per cell: per slot the
+    // least-squares weights with the neighbour (the cell itself where there is
+    // none), the face offset with the face (-1: no further slot), and the
+    // outward normal with the least normal velocity at which the cell is upwind
+    // (0 for the face's L cell, the smallest subnormal for its R cell: > 0)
+    std::vector<float> geo(ncs * 12, 0.0f);
+    for (int i = 0; i < Nc; ++i)
+        for (int q = 0; q < AVS_MAXS; ++q) {
+            const size_t o = (size_t)i * AVS_MAXS + q;
+            float* g = geo.data() + o * 12;
+            const int sl = slot[o], j = q < ns[i] && nbr[o] >= 0 ? nbr[o] : i, fc = q < ns[i] ? sl >> 1 : -1;
+            memcpy(g + 3, &j, 4);
+            memcpy(g + 7, &fc, 4);
+            if (fc < 0) continue;
+            const uint32_t above = (sl & 1) ? 1u : 0u;
+            memcpy(g + 11, &above, 4);
+            for (int a = 0; a < D; ++a) {
+                g[a] = (float)cg[o * D + a];
+                g[4 + a] = (float)r[o * D + a];
+                const float an = (float)m->An[(size_t)fc * D + a];
+                g[8 + a] = (sl & 1) ? -an : an;
+            }
+        }
+    CK(up(c->geo32, geo, s));
     // faces in the order of their lower cell index, so that the face blocks in
     // flight together read the f and gradient rows of nearby cells (L2 reuse)
     std::vector<int> order(Nf);
     for (int f = 0; f < Nf; ++f) order[f] = f;
     auto low = [&](int f) { const int R = m->faceR[f]; return R >= 0 ? std::min(m->faceL[f], R) : m->faceL[f]; };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        const bool ba = m->faceR[a] < 0, bb = m->faceR[b] < 0;     // interior faces first
-        return ba != bb ? bb : low(a) < low(b);
-    });
-    c->Nfi = 0;
-    for (int f = 0; f < Nf; ++f) c->Nfi += m->faceR[f] >= 0;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return low(a) < low(b); });
     CK(up(c->forder, order, s));
+    std::vector<int> iorder(order);
+    c->Nfi = (int)(std::stable_partition(iorder.begin(), iorder.end(), [&](int f) { return m->faceR[f] >= 0; }) -
+                   iorder.begin());
+    CK(up(c->iorder, iorder, s));
     // greedy colouring in cell order (smallest colour no face neighbour has):
     // cells of one colour share no face (implicit sweeps)
     {

@@ -50,7 +50,8 @@ struct avs_ctx {
     int max_ns = 0;                                  // largest face count of a cell
     int *nbr = nullptr;                              // [Nc][MAXS]
     double *cg_d = nullptr, *r_d = nullptr, *eps2_d = nullptr;
-    float *cg_f = nullptr, *r_f = nullptr, *eps2_f = nullptr;
+    float *eps2_f = nullptr;
+    float *geo32 = nullptr;                          // [Nc][MAXS][3][4] FP32 geometry record of a cell (k_foot_f2)
 
     // ---- velocity tree (device), capacity `cap` nodes
     int Nv = 0, Nvp = 0, cap = 0;
@@ -96,8 +97,9 @@ struct avs_ctx {
     void *flux = nullptr;                            // per-node face flux [Nf][NA][Nvp] of T
     size_t flux_bytes = 0;
     double *AFf = nullptr;                           // area-weighted face flux of W [Nf][D+2]
-    int *forder = nullptr;                           // face processing order: interior, then boundary faces,
-    int Nfi = 0;                                     //   each by lower cell index; number of interior faces
+    int *forder = nullptr;                           // face processing order (by lower cell index)
+    int *iorder = nullptr;                           // the same, interior faces before the boundary faces
+    int Nfi = 0;                                     // number of interior faces
     double *cmom = nullptr;                          // raw moments of f about U(W) per cell [Nc][NMom]
     double *rmom = nullptr;                          // scratch raw moments [max(Nc,2)][NMom]
     int mom_valid = 0;                               // cmom matches the current f and W

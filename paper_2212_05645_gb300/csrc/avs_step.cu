@@ -406,166 +406,156 @@ __device__ __forceinline__ float2 limit2(float2 dmax, float2 dmin, float2 pp, fl
     return make_float2(min3f(tp.x, tn.x, 1.0f), min3f(tp.y, tn.y, 1.0f));
 }
 
+// The cell's geometry from its record (Geo32): per slot least-squares weights
+// and neighbour cell, face offset and face, outward normal and upwind threshold
+// as three 16-byte vectors, copied once per block to shared memory.
+template <int NS>
+__device__ __forceinline__ void load_geo32(const float4* __restrict__ geo, int i, float4* gs)
+{
+    if (threadIdx.x < 3 * NS) gs[threadIdx.x] = geo[(size_t)i * (3 * AVS_MAXS) + threadIdx.x];
+    __syncthreads();
+}
+template <int D>
+__device__ __forceinline__ void vec3(const float4& v, float (&o)[D])
+{
+    o[0] = v.x;
+    o[1] = v.y;
+    if constexpr (D == 3) o[2] = v.z;
+}
+
+// Thread block (cell i, nodes of one chunk), the thread's quads one after the
+// other: the block's start (launch, geometry, barrier) is paid once for up to
+// four quads per thread.
 template <int D, int NS, int NA>
-__global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int limiter, float h, const float* __restrict__ f,
-                                                 float* __restrict__ FB, CellGeo<float> geo,
-                                                 const int* __restrict__ slot, const float* __restrict__ An,
-                                                 const float* __restrict__ xp)
+__global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
+                                                    const float* __restrict__ f, float* __restrict__ FB,
+                                                    const float4* __restrict__ geo, const float* __restrict__ eps2,
+                                                    const float* __restrict__ xs, size_t xstride)
 {
     constexpr int VG = 4;
+    __shared__ float4 gs[3 * NS];
     const int i = blockIdx.x;
-    const int t = threadIdx.x;
-    const int k0 = (blockIdx.y * blockDim.x + t) * VG;
-    const int ns = geo.ns[i];
-    // the cell's geometry, once per block: least-squares weights, face
-    // offsets and face normals per slot (padded to four floats, read back as
-    // one 16-byte vector), neighbour cells and slot codes
-    __shared__ __align__(16) float gs[3][NS][4];
-    __shared__ int gn[2][NS];
-    if (t < NS * 4) {
-        const int s = t >> 2, d = t & 3;
-        const bool on = s < ns && d < D;
-        gs[0][s][d] = on ? geo.cg[(size_t)(i * AVS_MAXS + s) * D + d] : 0.0f;
-        gs[1][s][d] = on ? geo.r[(size_t)(i * AVS_MAXS + s) * D + d] : 0.0f;
-    } else if (t >= 32 && t < 32 + NS) {
-        const int s = t - 32;
-        const int n = s < ns ? geo.nbr[i * AVS_MAXS + s] : -1;
-        const int sl = s < ns ? slot[i * AVS_MAXS + s] : 0;
-        gn[0][s] = n >= 0 ? n : i;
-        gn[1][s] = sl;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            const float a = s < ns ? An[(size_t)(sl >> 1) * D + d] : 0.0f;
-            gs[2][s][d] = (sl & 1) ? -a : a;
-        }
-        gs[2][s][3] = (sl & 1) ? __int_as_float(1) : 0.0f;
-    }
-    __syncthreads();
-    if (k0 >= Nv) return;
+    load_geo32<NS>(geo, i, gs);
     const size_t cstride = (size_t)NA * Nvp;
-    auto vec = [&](int q, int s, float (&o)[D]) {
-        const float4 v = *reinterpret_cast<const float4*>(gs[q][s]);
-        o[0] = v.x;
-        o[1] = v.y;
-        if constexpr (D == 3) o[2] = v.z;
-    };
-    const float e2 = geo.eps2[i];
-    float2 phi[NA][2], G[NA][D][2];
-#pragma unroll
-    for (int a = 0; a < NA; ++a) {
-        const float* fa = f + (size_t)a * Nvp + k0;
-        const float4 c4 = __ldg(reinterpret_cast<const float4*>(fa + (size_t)i * cstride));
-        phi[a][0] = lo2(c4);
-        phi[a][1] = hi2(c4);
-        float4 n4[NS];
-#pragma unroll
-        for (int s = 0; s < NS; ++s) n4[s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)gn[0][s] * cstride));
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float2 g[D], dd[NS];
-#pragma unroll
-            for (int d = 0; d < D; ++d) g[d] = bc2(0.0f);
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                float cg[D];
-                vec(0, s, cg);
-                dd[s] = sub2(p ? hi2(n4[s]) : lo2(n4[s]), phi[a][p]);
-#pragma unroll
-                for (int d = 0; d < D; ++d) g[d] = fma2(bc2(cg[d]), dd[s], g[d]);
-            }
-            float2 L = bc2(1.0f);
-            if (limiter == 1) {
-                float2 d2[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    float rr[D];
-                    vec(1, s, rr);
-                    d2[s] = mul2(g[0], bc2(rr[0]));
-#pragma unroll
-                    for (int d = 1; d < D; ++d) d2[s] = fma2(g[d], bc2(rr[d]), d2[s]);
-                }
-                float dx[NS], dy[NS], ex[NS], ey[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    dx[s] = dd[s].x; dy[s] = dd[s].y;
-                    ex[s] = d2[s].x; ey[s] = d2[s].y;
-                }
-                float2 dmax, dmin, pp, nn;
-                ext4<NS>(dx, dmax.x, dmin.x);
-                ext4<NS>(dy, dmax.y, dmin.y);
-                ext4<NS>(ex, pp.x, nn.x);
-                ext4<NS>(ey, pp.y, nn.y);
-                // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
-                const float2 e2p = mul2(mul2(bc2(e2), phi[a][p]), phi[a][p]);
-                L = limit2(dmax, dmin, pp, nn, e2p);
-            }
-            if (limiter == 0) L = bc2(0.0f);     // first order: phi_bar = phi_C
-#pragma unroll
-            for (int d = 0; d < D; ++d) G[a][d][p] = mul2(L, g[d]);
-        }
-    }
-    // node coordinates of the thread's nodes, as lane pairs (xp: the pair layout)
-    float2 X[2][D];
-    {
-        float xx[VG * D];
-        ldvn<float, VG * D>(xp + (size_t)k0 * D, xx);
-#pragma unroll
-        for (int p = 0; p < 2; ++p)
-#pragma unroll
-            for (int d = 0; d < D; ++d) X[p][d] = make_float2(xx[(p * D + d) * 2], xx[(p * D + d) * 2 + 1]);
-    }
-    // phi_bar = A + G . r_s with A = phi - h G . xi, the part common to the faces
-    float2 A[NA][2];
-#pragma unroll
-    for (int a = 0; a < NA; ++a)
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float2 gx = mul2(G[a][0][p], X[p][0]);
-#pragma unroll
-            for (int d = 1; d < D; ++d) gx = fma2(G[a][d][p], X[p][d], gx);
-            A[a][p] = fma2(bc2(-h), gx, phi[a][p]);
-        }
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        if (s >= ns) break;
-        const int fc = gn[1][s] >> 1;
-        float rr[D];
-        const float4 an = *reinterpret_cast<const float4*>(gs[2][s]);
-        vec(1, s, rr);
-        bool up[4];
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            // xi . An as in k_foot: a product, then fused multiply-adds; the
-            // normal points out of the cell (an exact sign change), so the
-            // face's L cell is upwind at >= 0 and its R cell at > 0, that is,
-            // at or above the smallest subnormal (an.w)
-            float2 sn = fma2(X[p][1], bc2(an.y), mul2(X[p][0], bc2(an.x)));
-            if constexpr (D == 3) sn = fma2(X[p][2], bc2(an.z), sn);
-            up[2 * p] = sn.x >= an.w;
-            up[2 * p + 1] = sn.y >= an.w;
-        }
-        const bool all = up[0] && up[1] && up[2] && up[3];
-        const bool any = up[0] || up[1] || up[2] || up[3];
-        if (!any) continue;
-        float* row = FB + (size_t)fc * NA * Nvp + k0;
+    const float e2 = eps2[i];
+    const int kend = min(Nv, (int)(blockIdx.y + 1) * chunk);
+#pragma unroll 1
+    for (int k0 = blockIdx.y * chunk + threadIdx.x * VG; k0 < kend; k0 += blockDim.x * VG) {
+        float2 phi[NA][2], G[NA][D][2];
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
-            float2 o[2];
+            const float* fa = f + (size_t)a * Nvp + k0;
+            const float4 c4 = __ldg(reinterpret_cast<const float4*>(fa + (size_t)i * cstride));
+            phi[a][0] = lo2(c4);
+            phi[a][1] = hi2(c4);
+            float4 n4[NS];
+#pragma unroll
+            for (int s = 0; s < NS; ++s) n4[s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)__float_as_int(gs[3 * s].w) * cstride));
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                float2 val = A[a][p];
+                float2 g[D], dd[NS];
 #pragma unroll
-                for (int d = 0; d < D; ++d) val = fma2(G[a][d][p], bc2(rr[d]), val);
-                o[p] = val;
+                for (int d = 0; d < D; ++d) g[d] = bc2(0.0f);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    float cg[D];
+                    vec3<D>(gs[3 * s], cg);
+                    dd[s] = sub2(p ? hi2(n4[s]) : lo2(n4[s]), phi[a][p]);
+#pragma unroll
+                    for (int d = 0; d < D; ++d) g[d] = fma2(bc2(cg[d]), dd[s], g[d]);
+                }
+                float2 L = bc2(1.0f);
+                if (limiter == 1) {
+                    float2 d2[NS];
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        float rr[D];
+                        vec3<D>(gs[3 * s + 1], rr);
+                        d2[s] = mul2(g[0], bc2(rr[0]));
+#pragma unroll
+                        for (int d = 1; d < D; ++d) d2[s] = fma2(g[d], bc2(rr[d]), d2[s]);
+                    }
+                    float dx[NS], dy[NS], ex[NS], ey[NS];
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        dx[s] = dd[s].x; dy[s] = dd[s].y;
+                        ex[s] = d2[s].x; ey[s] = d2[s].y;
+                    }
+                    float2 dmax, dmin, pp, nn;
+                    ext4<NS>(dx, dmax.x, dmin.x);
+                    ext4<NS>(dy, dmax.y, dmin.y);
+                    ext4<NS>(ex, pp.x, nn.x);
+                    ext4<NS>(ey, pp.y, nn.y);
+                    // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
+                    const float2 e2p = mul2(mul2(bc2(e2), phi[a][p]), phi[a][p]);
+                    L = limit2(dmax, dmin, pp, nn, e2p);
+                }
+                if (limiter == 0) L = bc2(0.0f);     // first order: phi_bar = phi_C
+#pragma unroll
+                for (int d = 0; d < D; ++d) G[a][d][p] = mul2(L, g[d]);
             }
-            float* ra = row + (size_t)a * Nvp;
-            if (all) {
-                *reinterpret_cast<float4*>(ra) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
-            } else {
-                if (up[0]) ra[0] = o[0].x;
-                if (up[1]) ra[1] = o[0].y;
-                if (up[2]) ra[2] = o[1].x;
-                if (up[3]) ra[3] = o[1].y;
+        }
+        // node coordinates of the thread's nodes, as lane pairs
+        float2 X[2][D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(xs + d * xstride + k0));
+            X[0][d] = lo2(v);
+            X[1][d] = hi2(v);
+        }
+        // phi_bar = A + G . r_s with A = phi - h G . xi, the part common to the faces
+        float2 A[NA][2];
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                float2 gx = mul2(G[a][0][p], X[p][0]);
+#pragma unroll
+                for (int d = 1; d < D; ++d) gx = fma2(G[a][d][p], X[p][d], gx);
+                A[a][p] = fma2(bc2(-h), gx, phi[a][p]);
+            }
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const float4 r4 = gs[3 * s + 1], an = gs[3 * s + 2];
+            const int fc = __float_as_int(r4.w);
+            if (fc < 0) break;                       // no further faces
+            float rr[D];
+            vec3<D>(r4, rr);
+            bool up[4];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                // xi . An as in k_foot: a product, then fused multiply-adds; the
+                // normal points out of the cell (an exact sign change), so the
+                // face's L cell is upwind at >= 0 and its R cell at > 0, that is,
+                // at or above the smallest subnormal (an.w)
+                float2 sn = fma2(X[p][1], bc2(an.y), mul2(X[p][0], bc2(an.x)));
+                if constexpr (D == 3) sn = fma2(X[p][2], bc2(an.z), sn);
+                up[2 * p] = sn.x >= an.w;
+                up[2 * p + 1] = sn.y >= an.w;
+            }
+            const bool all = up[0] && up[1] && up[2] && up[3];
+            const bool any = up[0] || up[1] || up[2] || up[3];
+            if (!any) continue;
+            float* row = FB + (size_t)fc * NA * Nvp + k0;
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                float2 o[2];
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    float2 val = A[a][p];
+#pragma unroll
+                    for (int d = 0; d < D; ++d) val = fma2(G[a][d][p], bc2(rr[d]), val);
+                    o[p] = val;
+                }
+                float* ra = row + (size_t)a * Nvp;
+                if (all) {
+                    *reinterpret_cast<float4*>(ra) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+                } else {
+                    if (up[0]) ra[0] = o[0].x;
+                    if (up[1]) ra[1] = o[0].y;
+                    if (up[2]) ra[2] = o[1].x;
+                    if (up[3]) ra[3] = o[1].y;
+                }
             }
         }
     }
@@ -968,9 +958,9 @@ __global__ void __launch_bounds__(NT) k_raw_moments(CellP<D, T> P)
     if (threadIdx.x < NM) P.mom[(size_t)i * NM + threadIdx.x] = red[threadIdx.x];
 }
 
-// Cell record of the FP32 kernels: out = k0 f + k1 g~ + kN N.
-__device__ __forceinline__ Cell32Par cell32_par(const EqPar<float>& e, float k0, float k1, float kN, const float* V,
-                                                float diag)
+// Cell record of the FP32 kernels: out = (u0 f + u1 g~ + un N) u3.
+__device__ __forceinline__ Cell32Par cell32_par(const EqPar<float>& e, float u0, float u1, float un, float u3,
+                                                const float* V, float diag)
 {
     Cell32Par z;
     for (int d = 0; d < 3; ++d) {
@@ -979,12 +969,15 @@ __device__ __forceinline__ Cell32Par cell32_par(const EqPar<float>& e, float k0,
         z.V[d] = V[d];
     }
     z.k2 = e.k2;
-    z.l2 = e.l2pref + log2f(k1);
-    z.k0 = k0;
+    z.l2 = e.l2pref;
+    z.u0 = u0;
+    z.u1 = u1;
+    z.un = un;
+    z.u3 = u3;
+    z.irt = e.invRT;
     z.RTH = e.RTH;
-    z.kN = kN;
-    z.pad = 0.0f;
     z.diag = diag;
+    z.pad[0] = z.pad[1] = 0.0f;
     return z;
 }
 
@@ -1030,9 +1023,8 @@ __global__ void k_cell_state(CellP<D, T> P)
     cp.eq = make_eq_a<D, T, T>(rho, U, RT, qn, (T)P.Pr);
     const T idt = (T)(1.0 / P.dt), itau = T(1) / tau;
     if constexpr (sizeof(T) == 4) {
-        const float u3 = 1.0f / (idt + itau);
         reinterpret_cast<Cell32Par*>(P.par)[i] =
-            cell32_par(cp.eq, idt * u3, itau * u3, -(float)(1.0 / P.vol[i]) * u3, U, 0.0f);
+            cell32_par(cp.eq, idt, itau, -(float)(1.0 / P.vol[i]), 1.0f / (idt + itau), U, 0.0f);
         return;
     }
     cp.upd[0] = idt;
@@ -1136,35 +1128,17 @@ __global__ void __launch_bounds__(NT, 4) k_cell(CellP<D, T> P)
 // them ([cell][array][D][Nvp]).  128-thread blocks, eight per SM.
 template <int D, int NS, int NA>
 __global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter, const float* __restrict__ f,
-                                                    float* __restrict__ Gout, CellGeo<float> geo)
+                                                    float* __restrict__ Gout, const float4* __restrict__ geo,
+                                                    const float* __restrict__ eps2)
 {
     constexpr int VG = 4;
+    __shared__ float4 gs[3 * NS];
     const int i = blockIdx.x;
-    const int t = threadIdx.x;
-    const int k0 = (blockIdx.y * blockDim.x + t) * VG;
-    const int ns = geo.ns[i];
-    __shared__ __align__(16) float gs[2][NS][4];      // LSQ weights, face offsets per slot
-    __shared__ int gn[NS];                            // neighbour cells (the cell itself where none)
-    if (t < NS * 4) {
-        const int s = t >> 2, d = t & 3;
-        const bool on = s < ns && d < D;
-        gs[0][s][d] = on ? geo.cg[(size_t)(i * AVS_MAXS + s) * D + d] : 0.0f;
-        gs[1][s][d] = on ? geo.r[(size_t)(i * AVS_MAXS + s) * D + d] : 0.0f;
-    } else if (t >= 32 && t < 32 + NS) {
-        const int s = t - 32;
-        const int n = s < ns ? geo.nbr[i * AVS_MAXS + s] : -1;
-        gn[s] = n >= 0 ? n : i;
-    }
-    __syncthreads();
+    load_geo32<NS>(geo, i, gs);
+    const int k0 = (blockIdx.y * blockDim.x + threadIdx.x) * VG;
     if (k0 >= Nv) return;
     const size_t cstride = (size_t)NA * Nvp;
-    auto vec = [&](int q, int s, float (&o)[D]) {
-        const float4 v = *reinterpret_cast<const float4*>(gs[q][s]);
-        o[0] = v.x;
-        o[1] = v.y;
-        if constexpr (D == 3) o[2] = v.z;
-    };
-    const float e2 = geo.eps2[i];
+    const float e2 = eps2[i];
 #pragma unroll
     for (int a = 0; a < NA; ++a) {
         const float* fa = f + (size_t)a * Nvp + k0;
@@ -1172,7 +1146,7 @@ __global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter
         const float2 phi[2] = {lo2(c4), hi2(c4)};
         float4 n4[NS];
 #pragma unroll
-        for (int s = 0; s < NS; ++s) n4[s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)gn[s] * cstride));
+        for (int s = 0; s < NS; ++s) n4[s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)__float_as_int(gs[3 * s].w) * cstride));
         float2 G[D][2];
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -1182,7 +1156,7 @@ __global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
                 float cg[D];
-                vec(0, s, cg);
+                vec3<D>(gs[3 * s], cg);
                 dd[s] = sub2(p ? hi2(n4[s]) : lo2(n4[s]), phi[p]);
 #pragma unroll
                 for (int d = 0; d < D; ++d) g[d] = fma2(bc2(cg[d]), dd[s], g[d]);
@@ -1193,7 +1167,7 @@ __global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter
 #pragma unroll
                 for (int s = 0; s < NS; ++s) {
                     float rr[D];
-                    vec(1, s, rr);
+                    vec3<D>(gs[3 * s + 1], rr);
                     d2[s] = mul2(g[0], bc2(rr[0]));
 #pragma unroll
                     for (int d = 1; d < D; ++d) d2[s] = fma2(g[d], bc2(rr[d]), d2[s]);
@@ -1224,29 +1198,37 @@ __global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter
     }
 }
 
+// geometry of the FP64 kernels (the FP32 ones read geo32)
+template <typename T>
+static CellGeo<T> cell_geo(const avs_ctx* c)
+{
+    CellGeo<T> geo;
+    geo.nbr = c->nbr;
+    geo.cg = (const T*)c->cg_d;
+    geo.r = (const T*)c->r_d;
+    geo.eps2 = (const T*)c->eps2_d;
+    geo.ns = c->nslot;
+    return geo;
+}
+
 // Limited gradients of every array of every cell into c->grad (allocated by the caller).
 template <int D, typename T, int NA>
 static void grad_t(avs_ctx* c, const void* fin)
 {
-    const bool f32 = sizeof(T) == 4;
-    CellGeo<T> geo;
-    geo.nbr = c->nbr;
-    geo.cg = f32 ? (const T*)c->cg_f : (const T*)c->cg_d;
-    geo.r = f32 ? (const T*)c->r_f : (const T*)c->r_d;
-    geo.eps2 = f32 ? (const T*)c->eps2_f : (const T*)c->eps2_d;
-    geo.ns = c->nslot;
     constexpr int VG = 4;
     if constexpr (sizeof(T) == 4) {
         const dim3 g2(c->Nc, (c->Nv + 128 * VG - 1) / (128 * VG));
         if (D == 2 && c->max_ns <= 4)
             k_grad_f2<D, 4, NA><<<g2, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const float*)fin,
-                                                          (float*)c->grad, geo);
+                                                          (float*)c->grad, (const float4*)c->geo32, c->eps2_f);
         else
             k_grad_f2<D, AVS_MAXS, NA><<<g2, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const float*)fin,
-                                                                 (float*)c->grad, geo);
+                                                                 (float*)c->grad, (const float4*)c->geo32,
+                                                                 c->eps2_f);
         c->launches += 1;
         return;
     }
+    const CellGeo<T> geo = cell_geo<T>(c);
     dim3 g(c->Nc, (c->Nv + 256 * VG - 1) / (256 * VG));
     if (D == 2 && c->max_ns <= 4)
         k_grad<D, T, VG, 4, NA><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const T*)fin, (T*)c->grad, geo);
@@ -1283,34 +1265,34 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
     const T* An = f32 ? (const T*)c->An_f : (const T*)c->An_d;
     const double hd = 0.5 * dt;
     {
-        CellGeo<T> geo;
-        geo.nbr = c->nbr;
-        geo.cg = f32 ? (const T*)c->cg_f : (const T*)c->cg_d;
-        geo.r = f32 ? (const T*)c->r_f : (const T*)c->r_d;
-        geo.eps2 = f32 ? (const T*)c->eps2_f : (const T*)c->eps2_d;
-        geo.ns = c->nslot;
         constexpr int VG = 4;
-        const dim3 g(c->Nc, (c->Nv + 256 * VG - 1) / (256 * VG));
         if constexpr (sizeof(T) == 4) {
-            // 128-thread blocks, eight per SM (measured on GB300: 1-2 % faster
-            // per UGKS step than 256-thread blocks, four per SM)
-            const dim3 g2(c->Nc, (c->Nv + 128 * VG - 1) / (128 * VG));
-            if (D == 2 && c->max_ns <= 4)
-                k_foot_f2<D, 4, NArr<D>::v><<<g2, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (float)hd,
-                                                                      (const float*)fin, (float*)c->flux, geo,
-                                                                      c->slot, An, c->xi_p);
-            else
-                k_foot_f2<D, AVS_MAXS, NArr<D>::v><<<g2, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter,
-                                                                             (float)hd, (const float*)fin,
-                                                                             (float*)c->flux, geo, c->slot, An,
-                                                                             c->xi_p);
-        } else if (D == 2 && c->max_ns <= 4) {
-            k_foot<D, T, VG, 4, NArr<D>::v><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (T)hd,
-                                                                      (const T*)fin, (T*)c->flux, geo, c->slot, An, xi);
+            // 128 threads, or 64 where a row has no more quads (190 nodes,
+            // 12288 cells: 41 -> 25 us), with up to four quads per thread while
+            // that leaves 32 blocks per SM (21k nodes, 36864 cells: 5.41 ->
+            // 4.46 ms; chunks of 2048 nodes still let the rows of a cell's
+            // neighbours be reused from L2)
+            const int nquad = (c->Nv + VG - 1) / VG;
+            const int nt = nquad <= 64 ? 64 : 128;
+            const int per = (int)std::max(1ll, std::min(4ll, (long long)c->Nc * nquad / nt / (32 * std::max(1, c->nsm))));
+            const int ny = (nquad + nt * per - 1) / (nt * per);
+            const int chunk = (nquad + ny - 1) / ny * VG;
+            auto go = [&](auto ns) {
+                k_foot_f2<D, decltype(ns)::value, NArr<D>::v><<<dim3(c->Nc, ny), nt, 0, c->stream>>>(
+                    c->Nv, c->Nvp, chunk, c->cfg.limiter, (float)hd, (const float*)fin, (float*)c->flux,
+                    (const float4*)c->geo32, c->eps2_f, c->xi_s, c->xstride);
+            };
+            if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
+            else go(std::integral_constant<int, AVS_MAXS>{});
         } else {
-            k_foot<D, T, VG, AVS_MAXS, NArr<D>::v><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (T)hd,
-                                                                             (const T*)fin, (T*)c->flux, geo, c->slot,
-                                                                             An, xi);
+            const CellGeo<T> geo = cell_geo<T>(c);
+            const dim3 g(c->Nc, (c->Nv + 256 * VG - 1) / (256 * VG));
+            if (D == 2 && c->max_ns <= 4)
+                k_foot<D, T, VG, 4, NArr<D>::v><<<g, 256, 0, c->stream>>>(
+                    c->Nv, c->Nvp, c->cfg.limiter, (T)hd, (const T*)fin, (T*)c->flux, geo, c->slot, An, xi);
+            else
+                k_foot<D, T, VG, AVS_MAXS, NArr<D>::v><<<g, 256, 0, c->stream>>>(
+                    c->Nv, c->Nvp, c->cfg.limiter, (T)hd, (const T*)fin, (T*)c->flux, geo, c->slot, An, xi);
         }
         c->launches += 1;
     }
@@ -1715,7 +1697,7 @@ __global__ void k_imp_state(CellP<D, T> P, const double* Wt)
     if constexpr (sizeof(T) == 4) {
         const float zero[3] = {0.0f, 0.0f, 0.0f};
         reinterpret_cast<Cell32Par*>(P.par)[i] =
-            cell32_par(cp.eq, -V / tau, V / tau, -1.0f, zero, V / (float)P.dt + V / tau);
+            cell32_par(cp.eq, -V / tau, V / tau, -1.0f, 1.0f, zero, V / (float)P.dt + V / tau);
         return;
     }
     cp.upd[0] = V / (T)P.dt + V / tau;

@@ -76,16 +76,35 @@ __device__ __forceinline__ float2 dot2(const float2* x, const float* a)
     return s;
 }
 
-// Equilibrium at a node pair: e = 2^(l2 + k2 c^2) and the Shakhov factors of G
-// and H (pG, pH), so that G = e pG and H = RTH e pH; c = xi - U, c2 = |c|^2.
+// Equilibrium G and H at a node pair as eq_eval2 forms them; c = xi - U.
 template <int D>
-__device__ __forceinline__ void eq2(const float2* x, const float* U, const float* al, float k2, float l2, float2& e,
-                                    float2& pG, float2& pH, float2* c, float2& c2)
+__device__ __forceinline__ void eq2(const float2* x, const float* U, const float* al, float k2, float l2, float irt,
+                                    float RTH, float2& gG, float2& gH, float2* c)
 {
 #pragma unroll
     for (int d = 0; d < D; ++d) c[d] = add2(x[d], bc2(-U[d]));
-    c2 = mul2(c[0], c[0]);
-    float2 cq = mul2(c[0], bc2(al[0]));
+    float2 c2 = mul2(c[0], c[0]), cq = mul2(c[0], bc2(al[0]));
+#pragma unroll
+    for (int d = 1; d < D; ++d) {
+        c2 = fma2(c[d], c[d], c2);
+        cq = fma2(c[d], bc2(al[d]), cq);
+    }
+    const float2 a = fma2(c2, bc2(k2), bc2(l2));
+    const float2 e = make_float2(ex2_approx(a.x), ex2_approx(a.y));
+    const float2 s = mul2(c2, bc2(irt));
+    gG = mul2(e, fma2(cq, add2(s, bc2(-(float)(D + 2))), bc2(1.0f)));
+    gH = D == 2 ? mul2(mul2(bc2(RTH), e), fma2(cq, add2(s, bc2(-(float)D)), bc2(1.0f))) : bc2(0.0f);
+}
+// the same with the prefactor wb within the exponent: e = 2^(l2 + k2 c^2) and
+// the Shakhov factors, so that wb g^G = e pG and wb g^H = RTH e pH
+template <int D>
+__device__ __forceinline__ void eq2f(const float2* x, const float* U, const float* al, float k2, float l2, float2& e,
+                                    float2& pG, float2& pH)
+{
+    float2 c[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) c[d] = add2(x[d], bc2(-U[d]));
+    float2 c2 = mul2(c[0], c[0]), cq = mul2(c[0], bc2(al[0]));
 #pragma unroll
     for (int d = 1; d < D; ++d) {
         c2 = fma2(c[d], c[d], c2);
@@ -97,13 +116,6 @@ __device__ __forceinline__ void eq2(const float2* x, const float* U, const float
     const float2 s = fma2(c2, bc2(irt), bc2(-(float)(D + 2)));
     pG = fma2(cq, s, bc2(1.0f));
     pH = D == 2 ? fma2(cq, add2(s, bc2(2.0f)), bc2(1.0f)) : bc2(0.0f);
-}
-template <int D>
-__device__ __forceinline__ void eq2(const float2* x, const float* U, const float* al, float k2, float l2, float2& e,
-                                    float2& pG, float2& pH)
-{
-    float2 c[D], c2;
-    eq2<D>(x, U, al, k2, l2, e, pG, pH, c, c2);
 }
 
 // raw moments of a node pair (values o) about V, y = xi - V
@@ -520,20 +532,22 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 128 ? (FPT > 2 ? 3 : 4) :
                     float2 o[NA][2];
 #pragma unroll
                     for (int p = 0; p < 2; ++p) {
-                        float2 x[D], ex, pG, pH;
+                        float2 x[D];
 #pragma unroll
                         for (int d = 0; d < D; ++d) x[d] = X[d][p];
-                        eq2<D>(x, e[j].U, e[j].al, e[j].k2, e[j].l2, ex, pG, pH);
                         const float2 sn = dot2<D>(x, An[j]);
-                        o[0][p] = mul2(sn, fma2(ex, pG, mul2(bc2(e[j].wa), F[j][0][p])));
+                        float2 ex, pG, pH;
+                        eq2f<D>(x, e[j].U, e[j].al, e[j].k2, e[j].l2, ex, pG, pH);
+                        const float2 G = fma2(ex, pG, mul2(bc2(e[j].wa), F[j][0][p]));
+                        o[0][p] = mul2(sn, G);
                         const float2 q = mul2(W2[p], o[0][p]);
                         m[j][0] = add2(m[j][0], q);
 #pragma unroll
                         for (int d = 0; d < D; ++d) m[j][1 + d] = fma2(q, x[d], m[j][1 + d]);
                         m[j][D + 1] = fma2(q, hx2[p], m[j][D + 1]);   // twice the energy moment
                         if constexpr (NA == 2) {
-                            o[NA - 1][p] = mul2(
-                                sn, fma2(mul2(bc2(e[j].RTH), ex), pH, mul2(bc2(e[j].wa), F[j][NA - 1][p])));
+                            const float2 H = fma2(mul2(bc2(e[j].RTH), ex), pH, mul2(bc2(e[j].wa), F[j][NA - 1][p]));
+                            o[NA - 1][p] = mul2(sn, H);
                             m[j][D + 1] = fma2(W2[p], o[NA - 1][p], m[j][D + 1]);
                         }
                     }
@@ -560,16 +574,19 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 128 ? (FPT > 2 ? 3 : 4) :
 }
 
 // ------------------------------------------------------------------ k_cell32
-// One block of NT threads per cell.  out = k0 f + k1 g~ + kN N per node, N the
+// One block of NT threads per cell.  out = (u0 f + u1 g~ + un N) u3 per node, N the
 // net flux of the cell's faces: the collision update (diagonal of Eq. SGS_phi)
-// with k0, k1, -kN |V| = (1/dt, 1/tau~, 1) / (1/dt + 1/tau~), or the residual of
-// the implicit step with k0, k1, kN = -|V|/tau~, |V|/tau~, -1 (RES).  Each thread
+// with 1/dt, 1/tau~, -1/|V| and 1 / (1/dt + 1/tau~), or the residual of the
+// implicit step with -|V|/tau~, |V|/tau~, -1 and 1 (RES).  Each thread
 // takes node quads, the rows of its next quads on their way into its own ring of
 // STG slots in shared memory, as in k_face32.  The kernel moves one row of f in
 // and out and the flux rows of the cell's faces (2D: four faces of two arrays,
 // 3D: six faces).  RES = false also sums the raw moments of the new f about U(W~) (P.mom), on the
 // same c = xi - U as the equilibrium, in the node order that k_raw32 repeats, so
-// that carried and recomputed moments are equal bit for bit.
+// that carried and recomputed moments are equal bit for bit.  (The update with
+// u0 u3, u1 u3 and un u3 formed first takes two instructions less per value, no
+// time, and rounds f differently: the heat flux of a gas near equilibrium, a
+// small difference of large sums, moved by 2e-5 of itself.)
 template <int D>
 struct Cell32P {
     int Nc, Nv, Nvp;
@@ -606,8 +623,9 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<D> P, 
     if (t < ns) {
         const int sl = P.slot[i * AVS_MAXS + t];
         fs[t] = sl >> 1;
-        sg[t] = (sl & 1) ? -P.par[i].kN : P.par[i].kN;
+        sg[t] = (sl & 1) ? -1.0f : 1.0f;
     }
+    static_assert(sizeof(Cell32Par) / 4 <= 32, "copied by one warp");
     if (t < (int)(sizeof(Cell32Par) / 4)) reinterpret_cast<float*>(&cp)[t] = reinterpret_cast<const float*>(P.par + i)[t];
     group_bar<NT>(1);
     const int nq = (Nv - 4 * t + CH - 1) / CH;
@@ -643,39 +661,38 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<D> P, 
         const int k = q * CH + t * 4;
         cp_wait<STG - 2>();
         const float* src = my + (size_t)slot * nrow * RS;
-        float2 X[D][2], W2[2], o[NA][2];
+        float2 X[D][2], W2[2], f0[NA][2], N[NA][2], o[NA][2];
 #pragma unroll
         for (int d = 0; d < D; ++d) lds4(src + d * RS, X[d]);
         if constexpr (!RES) lds4(src + D * RS, W2);
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
-            float2 F[2];
-            lds4(src + (D + 1 + a) * RS, F);
-#pragma unroll
-            for (int p = 0; p < 2; ++p) o[a][p] = mul2(bc2(cp.k0), F[p]);
+            lds4(src + (D + 1 + a) * RS, f0[a]);
+            N[a][0] = N[a][1] = bc2(0.0f);
         }
 #pragma unroll
         for (int s = 0; s < AVS_MAXS; ++s) {
             if (s >= ns) break;
-            const float2 kn = bc2(sg[s]);
+            const float2 g = bc2(sg[s]);
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
                 float2 F[2];
                 lds4(src + (D + 1 + NA * (1 + s) + a) * RS, F);
 #pragma unroll
-                for (int p = 0; p < 2; ++p) o[a][p] = fma2(kn, F[p], o[a][p]);
+                for (int p = 0; p < 2; ++p) N[a][p] = fma2(g, F[p], N[a][p]);
             }
         }
         fetch(q + STG - 1, slot == 0 ? STG - 1 : slot - 1);
         slot = slot + 1 == STG ? 0 : slot + 1;
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-            float2 x[D], c[D], ex, pG, pH, c2;
+            float2 x[D], c[D], g[2];
 #pragma unroll
             for (int d = 0; d < D; ++d) x[d] = X[d][p];
-            eq2<D>(x, cp.U, cp.al, cp.k2, cp.l2, ex, pG, pH, c, c2);
-            o[0][p] = fma2(ex, pG, o[0][p]);
-            if constexpr (NA == 2) o[NA - 1][p] = fma2(mul2(bc2(cp.RTH), ex), pH, o[NA - 1][p]);
+            eq2<D>(x, cp.U, cp.al, cp.k2, cp.l2, cp.irt, cp.RTH, g[0], g[1], c);
+#pragma unroll
+            for (int a = 0; a < NA; ++a)
+                o[a][p] = mul2(fma2(N[a][p], bc2(cp.un), fma2(f0[a][p], bc2(cp.u0), mul2(g[a], bc2(cp.u1)))), bc2(cp.u3));
             if (k + 4 > Nv) {                    // the last quad's pad nodes are stored as zero
                 const bool r0 = k + 2 * p < Nv, r1 = k + 2 * p + 1 < Nv;
 #pragma unroll
@@ -770,7 +787,7 @@ static cudaError_t face32_t(avs_ctx* c, const double* Win, double dt)
     P.xs = c->xi_s;
     P.w = c->w_f;
     P.xstride = c->xstride;
-    P.order = c->forder;
+    P.order = c->iorder;
     P.faceL = c->faceL;
     P.faceR = c->faceR;
     P.An = c->An_f;

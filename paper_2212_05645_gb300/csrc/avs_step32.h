@@ -5,14 +5,15 @@
 
 namespace avs {
 
-// A cell's collision update out = k0 f + k1 g~ + kN N (k1 inside l2), and the
+// A cell's update out = (u0 f + u1 g~ + un N) u3 with g~ the Shakhov equilibrium
+// 2^(l2 + k2 |c|^2) (1 + (c . al)(|c|^2 / RT - D - 2)), c = xi - U, and the
 // reference velocity V of its raw moments.
 struct alignas(16) Cell32Par {
     float U[3], k2;
     float al[3], l2;
-    float k0, RTH, kN, pad;
-    float V[3];
-    float diag;              // implicit step: |V|/dt + |V|/tau~
+    float u0, u1, un, u3;
+    float V[3], irt;
+    float RTH, diag, pad[2];     // diag, implicit step: |V|/dt + |V|/tau~
 };
 static_assert(sizeof(Cell32Par) <= AVS_CELLPAR_BYTES, "cell parameter buffer");
 
