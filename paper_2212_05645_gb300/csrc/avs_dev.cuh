@@ -448,11 +448,14 @@ constexpr float kCritScale = 0x1p64f;
 __device__ __forceinline__ float crit_scaled(float G) { return G * kCritScale; }
 __device__ __forceinline__ float crit_scaled(double G) { return (float)(G * 0x1p64); }
 
-__device__ __forceinline__ void crit32(int D, float Gs, float wk, const float* x, const float* c32, float& m, float& B)
+// (c32: 1/rho, U, 0.5/e_int; D a compile-time constant, so that x and c32 stay in registers)
+template <int D>
+__device__ __forceinline__ void crit32(float Gs, float wk, const float* x, const float* c32, float& m, float& B)
 {
     const float wg = wk * Gs;
     const float m1 = wg * c32[0];
     float c2 = 0.0f, ac = 0.0f, a2 = 0.0f;
+#pragma unroll
     for (int d = 0; d < D; ++d) {
         const float cc = x[d] - c32[1 + d];
         const float aa = fabsf(x[d]) + fabsf(c32[1 + d]);
