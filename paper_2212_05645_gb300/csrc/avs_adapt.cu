@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(NT) k_cell_moments(int Nv, int Nvp, const T* _
     const T* fi = f + (size_t)i * NA * Nvp;
     double acc[NM];
     cell_raw_sums<D, T, NT>(Nv, Nvp, fi, xi, w, Vt, acc);
-    block_sum<NM, NT>(acc, sw, mom);
+    block_sum_t<NM, NT>(acc, sw, mom);
     if (threadIdx.x < NM) rmom[(size_t)i * NM + threadIdx.x] = mom[threadIdx.x];
 }
 
@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(NT) k_correct(int Nv, int Nvp, T* f, const T* 
         // moments of the current f' (nodes per thread as in the update below)
         double acc[NM];
         cell_raw_sums<D, T, NT>(Nv, Nvp, fi, xi, w, Vt, acc);
-        block_sum<NM, NT>(acc, sw, mom);
+        block_sum_t<NM, NT>(acc, sw, mom);
         if (it == iters) {
             if (threadIdx.x == 0) {
                 double Wp[5];

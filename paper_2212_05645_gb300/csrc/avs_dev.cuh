@@ -588,28 +588,37 @@ __device__ __forceinline__ void eq_eval2(const EqPar<float>& p, const float2* X,
 }
 
 // ---------------------------------------------------------------- reductions
-// Deterministic block reduction of N doubles per thread: warp tree with
-// shuffles, then a fixed-order sum over warps.  Result in out[0..N-1] (smem),
-// visible to all threads after return.
-template <int N, int NT>
-__device__ __forceinline__ void block_sum(double* v, double* sred, double* out)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Sum of N values per lane over the warp by halves: at each of the five steps a
+// lane keeps one half of its values and hands the other to its partner, so N
+// values take about N + 4 shuffles and additions instead of 5 N (on the FP64
+// pipe, where each costs 16 cycles of an SM, that was most of a short row's
+// time).  Afterwards v[0] of a lane with cnt > 0 is the sum of value idx (start
+// with idx = 0, cnt = N).  Fixed order, so deterministic.
+template <typename T, int N, int O>
+struct WarpSum {
+    static constexpr int H = (N + 1) / 2;
+    __device__ static __forceinline__ void run(T* v, int& idx, int& cnt)
+    {
+        if constexpr (N == 1) {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+        } else {
+            const bool up = (threadIdx.x & O) != 0;
 #pragma unroll
-    for (int m = 0; m < N; ++m) {
-        double x = v[m];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sred[warp * N + m] = x;
+            for (int i = 0; i < H; ++i) {
+                const T lo = v[i], hi = i + H < N ? v[i + H] : T(0);
+                const T r = __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
+                v[i] = (up ? hi : lo) + r;
+            }
+            idx += up ? H : 0;
+            cnt = up ? cnt - H : min(cnt, H);
+        }
+        WarpSum<T, H, O / 2>::run(v, idx, cnt);
     }
-    __syncthreads();
-    if (threadIdx.x < N) {
-        double s = 0.0;
-        for (int w = 0; w < NT / 32; ++w) s += sred[w * N + threadIdx.x];
-        out[threadIdx.x] = s;
-    }
-    __syncthreads();
-}
+};
+template <typename T, int N>
+struct WarpSum<T, N, 0> {
+    __device__ static __forceinline__ void run(T*, int&, int&) {}
+};
 
 // float -> double by bit manipulation on the integer pipe (exact for normal
 // numbers; subnormals, far below any partial sum here, become signed zero).
@@ -633,21 +642,17 @@ __device__ __forceinline__ double to_double(float x)
     return __hiloint2double((int)hi, (int)lo);
 }
 
-// Block reduction of N values per thread kept in the element type: warp tree
-// with shuffles in T, then a fixed-order FP64 sum of the per-warp results.
-// Deterministic.  out[0..N-1] (smem, double) is visible to all threads after
-// return.  sw must hold (NT/32)*N doubles.
+// Block reduction of N values per thread: warp sums in the element type, then a
+// fixed-order FP64 sum of the per-warp results.  Deterministic.  out[0..N-1]
+// (smem, double) is visible to all threads after return.  sw must hold
+// (NT/32)*N doubles.
 template <int N, int NT, typename T>
 __device__ __forceinline__ void block_sum_t(T* v, double* sw, double* out)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int m = 0; m < N; ++m) {
-        T x = v[m];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sw[warp * N + m] = to_double(x);
-    }
+    static_assert(N <= 32, "one value per lane at most");
+    int idx = 0, cnt = N;
+    WarpSum<T, N, 16>::run(v, idx, cnt);
+    if (cnt > 0) sw[(threadIdx.x >> 5) * N + idx] = to_double(v[0]);
     __syncthreads();
     for (int m = threadIdx.x; m < N; m += NT) {
         double s = 0.0;

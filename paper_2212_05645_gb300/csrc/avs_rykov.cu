@@ -161,7 +161,7 @@ __device__ void rk_cell_mom(const T* fi, int Nv, int Nvp, const double* __restri
         acc[D + 1] += wk * (0.5 * (x2 * G + H) + Rr);
         acc[D + 2] += wk * Rr;
     }
-    block_sum<NW, RK_NT>(acc, sred, sout);
+    block_sum_t<NW, RK_NT>(acc, sred, sout);
 #pragma unroll
     for (int m = 0; m < NW; ++m) W[m] = sout[m];
     if (!qt) return;
@@ -187,7 +187,7 @@ __device__ void rk_cell_mom(const T* fi, int Nv, int Nvp, const double* __restri
             a[D + d] += wk * c[d] * Rr;
         }
     }
-    block_sum<2 * D, RK_NT>(a, sred, sout);
+    block_sum_t<2 * D, RK_NT>(a, sred, sout);
     for (int d = 0; d < D; ++d) {
         qt[d] = sout[d];
         qr[d] = sout[D + d];
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(RK_NT) rk_face(RkP<T> P)
             }
         }
     }
-    block_sum<NW, RK_NT>(acc, sred, sout);
+    block_sum_t<NW, RK_NT>(acc, sred, sout);
     if (R >= 0) {
         double W[NW];
 #pragma unroll
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(RK_NT) rk_face(RkP<T> P)
                 a2[D + d] += wk * c[d] * Rr;
             }
         }
-        block_sum<2 * D, RK_NT>(a2, sred, sout);
+        block_sum_t<2 * D, RK_NT>(a2, sred, sout);
         if (threadIdx.x == 0) {
             double rho, Uu[3], RTt, RTr, RT;
             rk_prim<D>(W, rho, Uu, RTt, RTr, RT);
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(RK_NT) rk_face(RkP<T> P)
         af[D + 1] += wk * (0.5 * (x2 * Fd[0] + (D == 2 ? Fd[1] : 0.0)) + Fd[NA - 1]);
         af[D + 2] += wk * Fd[NA - 1];
     }
-    block_sum<NW, RK_NT>(af, sred, sout);
+    block_sum_t<NW, RK_NT>(af, sred, sout);
     if (threadIdx.x < NW) P.AF[(size_t)f * NW + threadIdx.x] = sout[threadIdx.x];
 }
 

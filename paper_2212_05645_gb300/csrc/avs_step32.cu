@@ -126,36 +126,6 @@ __device__ __forceinline__ void pair_moments(float2* m, const float2* y, float2 
 }
 
 // ---------------------------------------------------------------- reductions
-// Sum of N floats per lane over the warp by halves: at each of the five steps a
-// lane keeps one half of its values and hands the other to its partner, so N
-// values take about N + 4 shuffles instead of 5 N.  On return lane l holds in
-// v[0] the sum of value `idx` (-1: none).  Fixed order, so deterministic.
-template <int N, int O>
-struct WarpSum {
-    static constexpr int H = (N + 1) / 2;
-    __device__ static __forceinline__ void run(float* v, int& idx, int& cnt)
-    {
-        if constexpr (N == 1) {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-        } else {
-            const bool up = (threadIdx.x & O) != 0;
-#pragma unroll
-            for (int i = 0; i < H; ++i) {
-                const float lo = v[i], hi = i + H < N ? v[i + H] : 0.0f;
-                const float r = __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
-                v[i] = (up ? hi : lo) + r;
-            }
-            idx += up ? H : 0;
-            cnt = up ? cnt - H : min(cnt, H);
-        }
-        WarpSum<H, O / 2>::run(v, idx, cnt);
-    }
-};
-template <int N>
-struct WarpSum<N, 0> {
-    __device__ static __forceinline__ void run(float*, int&, int&) {}
-};
-
 // Per-thread floats v[N] of a group of NT threads (NT a multiple of 32, its
 // warps consecutive) summed into out[N] (shared memory, FP64 across warps).
 // sw: (NT / 32) * N floats.  gsync synchronises the group.
@@ -164,7 +134,7 @@ __device__ __forceinline__ void group_sum(float* v, int t, float* sw, double* ou
 {
     static_assert(N <= 32, "one value per lane at most");
     int idx = 0, cnt = N;
-    WarpSum<N, 16>::run(v, idx, cnt);
+    WarpSum<float, N, 16>::run(v, idx, cnt);
     if constexpr (NT == 32) {
         if (cnt > 0) out[idx] = to_double(v[0]);
     } else {
