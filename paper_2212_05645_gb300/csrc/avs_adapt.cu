@@ -40,7 +40,8 @@ __device__ int zone_cap(const ZoneSet& Z, int D, const double* x)
 __global__ void k_geom(int D, int Nv, int Nvp, const int* __restrict__ level, const int* __restrict__ base,
                        const uint32_t* __restrict__ key, int nb0, int nb1, int nb2, double vlo0, double vlo1,
                        double vlo2, double hb0, double hb1, double hb2, double* xi_d, double* w_d, float* xi_f,
-                       float* w_f, float* xi_p, float* xi_s, size_t xstride, ZoneSet Z, int* ncap)
+                       float* w_f, float* xi_p, float* xi_s, size_t xstride, unsigned short* tix, int t0, int t1,
+                       ZoneSet Z, int* ncap)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= Nvp) return;
@@ -52,6 +53,7 @@ __global__ void k_geom(int D, int Nv, int Nvp, const int* __restrict__ level, co
             xi_f[(size_t)k * D + d] = 0.0f;
             xp[2 * d] = 0.0f;
             xi_s[d * xstride + k] = 0.0f;
+            if (tix) tix[d * xstride + k] = 0;
         }
         w_d[k] = 0.0;
         w_f[k] = 0.0f;
@@ -81,6 +83,10 @@ __global__ void k_geom(int D, int Nv, int Nvp, const int* __restrict__ level, co
         xi_f[(size_t)k * D + d] = (float)x;
         xp[2 * d] = (float)x;
         xi_s[d * xstride + k] = (float)x;
+        if (tix) {
+            const int start = d == 0 ? 0 : d == 1 ? t0 : t1;
+            tix[d * xstride + k] = (unsigned short)(start + nb[d] * ((1 << l) - 1) + (bi << l) + (int)o);
+        }
         wk = __dmul_rn(wk, hb[d]);
     }
     const double wv = ldexp(wk, -D * l);
@@ -89,13 +95,36 @@ __global__ void k_geom(int D, int Nv, int Nvp, const int* __restrict__ level, co
     ncap[k] = zone_cap(Z, D, xc);
 }
 
+// Coordinates of an axis in the order level, base element, offset, formed as in k_geom.
+__global__ void k_axis_table(int n, int start, int nb, double vlo, double hb, double* xtab)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    int l = 0;
+    while (j >= nb * ((2 << l) - 1)) ++l;
+    const int r = j - nb * ((1 << l) - 1), bi = r >> l, o = r & ((1 << l) - 1);
+    const double frac = (double)(2 * o + 1) / (double)(1u << (l + 1));
+    xtab[start + j] = __dadd_rn(vlo, __dmul_rn(hb, __dadd_rn((double)bi, frac)));
+}
+
+cudaError_t launch_axis_table(avs_ctx* c)
+{
+    for (int d = 0; d < c->D; ++d) {
+        const int start = d ? c->tab_end[d - 1] : 0, n = c->tab_end[d] - start;
+        k_axis_table<<<(n + 127) / 128, 128, 0, c->stream>>>(n, start, c->cfg.base[d], c->cfg.vlo[d], c->hb[d], c->xtab);
+        c->launches += 1;
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_geom(avs_ctx* c)
 {
     const int n = c->Nvp;
     k_geom<<<(n + 255) / 256, 256, 0, c->stream>>>(c->D, c->Nv, c->Nvp, c->level, c->base, c->key, c->cfg.base[0],
                                                    c->cfg.base[1], c->cfg.base[2], c->cfg.vlo[0], c->cfg.vlo[1],
                                                    c->cfg.vlo[2], c->hb[0], c->hb[1], c->hb[2], c->xi_d, c->w_d,
-                                                   c->xi_f, c->w_f, c->xi_p, c->xi_s, c->xstride, c->zs, c->ncap);
+                                                   c->xi_f, c->w_f, c->xi_p, c->xi_s, c->xstride, c->tix, c->tab_end[0],
+                                                   c->tab_end[1], c->zs, c->ncap);
     c->launches += 1;
     return cudaGetLastError();
 }

@@ -53,7 +53,7 @@ void free_all(avs_ctx* c)
     void* ptrs[] = {c->faceL, c->faceR, c->An_d, c->rL_d, c->rR_d, c->An_f, c->rL_f, c->rR_f, c->vol, c->bc,
                     c->slot, c->nslot, c->nbr, c->cg_d, c->r_d, c->eps2_d, c->eps2_f, c->geo32, c->iorder,
                     c->level, c->base, c->key, c->level2, c->base2, c->key2, c->src, c->kind, c->emit,
-                    c->newidx, c->d_count, c->xi_d, c->w_d, c->xi_f, c->w_f, c->xi_p, c->xi_s, c->M, c->Mkey, c->f[0], c->f[1],
+                    c->newidx, c->d_count, c->xi_d, c->w_d, c->xi_f, c->w_f, c->xi_p, c->xi_s, c->xtab, c->tix, c->M, c->Mkey, c->f[0], c->f[1],
                     c->W[0], c->W[1], c->ncap, c->Wf, c->q, c->pseudo_f, c->pseudo_W, c->crit_cp, c->crit_cp32, c->Mlo, c->Mhi, c->Mthr, c->stage, c->dev_err,
                     c->dt_key, c->gap_d, c->grad, c->flux, c->AFf, c->forder, c->cmom, c->rmom, c->cpar, c->clist, c->cstart_d, c->imp_dW, c->imp_rhs0, c->imp_diag, c->imp_Wta,
                     c->imp_co, c->imp_nint, c->imp_bar, c->mlp_P, c->mlp_Wb, c->mlp_part, c->mlp_grad,
@@ -591,6 +591,18 @@ avs_status avs_create(const avs_config* cfg, const avs_mesh* mesh, void* cuda_st
     AL(c->xi_f, (size_t)capp * c->D); AL(c->w_f, capp); AL(c->xi_p, (size_t)capp * c->D);
     c->xstride = capp;
     AL(c->xi_s, (size_t)capp * c->D);
+    if (!c->mixed && c->model == AVS_SHAKHOV) {
+        long long n = 0;
+        for (int d = 0; d < c->D; ++d) {
+            n += (long long)c->cfg.base[d] * ((2ll << c->cfg.max_refine) - 1);
+            c->tab_end[d] = (int)std::min<long long>(n, AVS_TAB_MAX + 1);
+        }
+        if (n <= AVS_TAB_MAX) {
+            c->tab_n = (int)n;
+            AL(c->xtab, n);
+            AL(c->tix, (size_t)capp * c->D);
+        }
+    }
     AL(c->M, capp); AL(c->Mkey, capp); AL(c->ncap, capp);
     AL(c->pseudo_f, 2 * (size_t)c->NA * capp); AL(c->pseudo_W, 4 * NW);
     AL(c->crit_cp, 5 * (size_t)std::max(c->Nc, 2)); AL(c->crit_cp32, 8 * (size_t)std::max(c->Nc, 2));
@@ -606,6 +618,10 @@ avs_status avs_create(const avs_config* cfg, const avs_mesh* mesh, void* cuda_st
     }
     st = setup_mesh(c, mesh);
     if (st != AVS_OK) goto bad;
+    if (c->tab_n > 0 && launch_axis_table(c) != cudaSuccess) {
+        st = fail(c, AVS_ECUDA, "axis table");
+        goto bad;
+    }
     st = initial_tree(c);
     if (st != AVS_OK) goto bad;
     {

@@ -129,6 +129,13 @@ __device__ __forceinline__ float min3f(float a, float b, float c)
     return r;
 }
 
+// Venkatakrishnan limiter function, uncapped (FP64).
+__device__ __forceinline__ double venkat_ratio(double d1, double d2, double eps2)
+{
+    const double u = d1 * d1 + eps2, v = d1 * d2;
+    return (u + 2.0 * v) / (u + v + 2.0 * d2 * d2);
+}
+
 // Venkatakrishnan limiter function, capped at 1.
 template <typename T>
 __device__ __forceinline__ T venkat(T d1, T d2, T eps2)

@@ -12,6 +12,7 @@
 
 #define AVS_NT 256            // threads per block of the per-cell kernels
 #define AVS_CELLPAR_BYTES 256 // bytes per cell of the collision parameters (CellPar)
+#define AVS_TAB_MAX 3072      // entries of the axes' coordinate tables (32 bytes each in shared memory)
 #define AVS_CMOM_MAX 17       // carried raw moments per cell (monatomic 11 / 13, Rykov 14 / 17)
 #define AVS_IMPSLOT_BYTES 96  // bytes per slot record of the implicit macroscopic sweep
 
@@ -66,6 +67,12 @@ struct avs_ctx {
     float *xi_f = nullptr, *w_f = nullptr;
     float *xi_s = nullptr;                           // FP32 node coordinates by components: [D][xstride]
     size_t xstride = 0;
+    // FP64 form: the coordinates a node can have per axis, all levels up to
+    // max_refine (axis d: entries tab_end[d-1]..tab_end[d]), and each node's
+    // entries; tab_n = 0 where there are more than AVS_TAB_MAX
+    double *xtab = nullptr;                          // [tab_n]
+    unsigned short *tix = nullptr;                   // [D][xstride]
+    int tab_end[3] = {0, 0, 0}, tab_n = 0;
     float *xi_p = nullptr;                           // FP32 node coordinates by pairs: [cap/2][D][2]
     double *M = nullptr;                             // [cap]
     unsigned long long *Mkey = nullptr;              // [cap]
@@ -158,6 +165,7 @@ cudaError_t launch_step_implicit(avs_ctx* c, const void* fin, void* fout, const 
                                  int k_macro, int k_micro);
 
 // ---- launchers (avs_adapt.cu)
+cudaError_t launch_axis_table(avs_ctx* c);                 // coordinates a node can have per axis
 cudaError_t launch_geom(avs_ctx* c);                       // xi, w of the current tree
 cudaError_t launch_dt_unit(avs_ctx* c);                    // min |V|/sum max(xi.n,0) -> c->dt_key
 cudaError_t launch_maxwell(avs_ctx* c, const double* Wp, int Ncells, double amp, uint64_t seed,

@@ -188,169 +188,187 @@ __global__ void __launch_bounds__(256) k_grad(int Nv, int Nvp, int limiter, cons
     }
 }
 
+// The cell's geometry from its record (Geo32): per slot least-squares weights
+// and neighbour cell, face offset and face, outward normal and upwind threshold
+// as three 16-byte vectors, copied once per block to shared memory.
+template <int NS>
+__device__ __forceinline__ void load_geo32(const float4* __restrict__ geo, int i, float4* gs)
+{
+    if (threadIdx.x < 3 * NS) gs[threadIdx.x] = geo[(size_t)i * (3 * AVS_MAXS) + threadIdx.x];
+    __syncthreads();
+}
+template <int D>
+__device__ __forceinline__ void vec3(const float4& v, float (&o)[D])
+{
+    o[0] = v.x;
+    o[1] = v.y;
+    if constexpr (D == 3) o[2] = v.z;
+}
+
 // ------------------------------------------------------------------ k_foot
-// Cell-centric reconstruction (Sec. 2.3.3).  Thread block (cell i, 256 x VG
-// nodes): the limited gradient of every array of cell i (as k_grad, kept in
-// registers), then for every face slot s of the cell the foot values
+// Cell-centric reconstruction (Sec. 2.3.3), FP64 form.  Thread block (cell i,
+// nodes of one chunk, two per thread and iteration): the limited gradient of
+// every array of cell i (as k_grad, kept in registers), then for every face
+// slot s of the cell the foot values
 //   phi_bar = phi_i + (L grad phi)_i . (x_f - x_i - xi h)
+//           = phi_i - h L (g . xi) + L (g . r_s)
 // at the nodes where i is that face's upwind cell (xi . An >= 0 for the face's
 // L cell, < 0 for its R cell; xi . An summed without contraction, the same
 // value the face kernel tests), written to the face's row of
 // FB [face][array][Nvp].  Every node of an interior face is written exactly
 // once, by its upwind cell; of a boundary face only the outgoing half.  The
 // gradient itself is never stored.
-template <int D, typename T, int VG, int NS, int NA>
-__global__ void __launch_bounds__(256) k_foot(int Nv, int Nvp, int limiter, T h, const T* __restrict__ f,
-                                              T* __restrict__ FB, CellGeo<T> geo, const int* __restrict__ slot,
-                                              const T* __restrict__ An, const T* __restrict__ xi)
+//
+// The FP64 pipe is the bound (one warp instruction in 16 cycles of an SM, 1/32
+// of the integer and FP32 rates), so what need not run on it does not: the
+// extremes compare bit patterns as integers, the upwind choice is an FP32 dot
+// product unless that lies within its rounding bound of zero, and g . r_s
+// serves the limiter and the foot value.  160 -> about 90 FP64 instructions
+// per cell and node in 3D; per step 181 -> 99 us on the 32 x 32 cavity (298
+// nodes), 4.30 -> 2.24 ms on 1000 cells x 13824 nodes in 3D, where the pipe is
+// full.
+__device__ __noinline__ bool upwind_exact(int D, const double* __restrict__ x, const double* __restrict__ a, bool isR)
 {
-    static_assert((VG * sizeof(T)) % 16 == 0, "whole 16-byte vectors per thread");
+    double s = dadd(dmul(x[0], a[0]), dmul(x[1], a[1]));
+    if (D == 3) s = dadd(s, dmul(x[2], a[2]));
+    return isR ? s < 0.0 : s >= 0.0;
+}
+
+// Largest value of v[0..N-1] and 0, and smallest of them and 0, by integer
+// comparison: as signed integers the positive doubles order as their values
+// and negative ones lie below zero; as unsigned integers the negative ones
+// order by magnitude, above every positive one.
+template <int N>
+__device__ __forceinline__ void ext_bits(const double* v, double& mx, double& mn)
+{
+    long long hi = 0;
+    unsigned long long lo = 0;
+#pragma unroll
+    for (int s = 0; s < N; ++s) {
+        const long long b = __double_as_longlong(v[s]);
+        hi = b > hi ? b : hi;
+        lo = (unsigned long long)b > lo ? (unsigned long long)b : lo;
+    }
+    mx = __longlong_as_double(hi);
+    mn = (long long)lo < 0 ? __longlong_as_double((long long)lo) : 0.0;
+}
+
+template <int D, int NS, int NA>
+__global__ void __launch_bounds__(128) k_foot(int Nv, int Nvp, int chunk, int limiter, double h,
+                                              const double* __restrict__ f, double* __restrict__ FB,
+                                              CellGeo<double> geo, const int* __restrict__ slot,
+                                              const double* __restrict__ An, const double* __restrict__ xi,
+                                              const float4* __restrict__ geo32, const float* __restrict__ xs,
+                                              size_t xstride)
+{
+    constexpr int VG = 2;
+    __shared__ double sc[NS][D], sr[NS][D];      // least-squares weights, face offsets
+    __shared__ float4 g32[3 * NS];               // FP32 record: neighbours, faces, outward normals
     const int i = blockIdx.x;
-    const int k0 = (blockIdx.y * blockDim.x + threadIdx.x) * VG;
-    if (k0 >= Nv) return;
+    for (int e = threadIdx.x; e < NS * D; e += blockDim.x) {
+        const int q = e / D, d = e % D;
+        const bool on = q < geo.ns[i];
+        sc[q][d] = on ? geo.cg[(size_t)(i * AVS_MAXS + q) * D + d] : 0.0;
+        sr[q][d] = on ? geo.r[(size_t)(i * AVS_MAXS + q) * D + d] : 0.0;
+    }
+    load_geo32<NS>(geo32, i, g32);
     const size_t cstride = (size_t)NA * Nvp;
-    const int ns = geo.ns[i];
-    int nb[NS];
-    T cg[NS][D], rr[NS][D];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const int n = s < ns ? geo.nbr[i * AVS_MAXS + s] : -1;
-        nb[s] = n >= 0 ? n : i;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            cg[s][d] = s < ns ? geo.cg[(size_t)(i * AVS_MAXS + s) * D + d] : T(0);
-            rr[s][d] = s < ns ? geo.r[(size_t)(i * AVS_MAXS + s) * D + d] : T(0);
-        }
-    }
-    const T e2 = geo.eps2[i];
-    T phi[NA][VG], G[NA][D][VG];
-#pragma unroll
-    for (int a = 0; a < NA; ++a) {
-        const T* fa = f + (size_t)a * Nvp + k0;
-        T nv[NS][VG];
-        ldvn<T, VG>(fa + (size_t)i * cstride, phi[a]);
-#pragma unroll
-        for (int s = 0; s < NS; ++s) ldvn<T, VG>(fa + (size_t)nb[s] * cstride, nv[s]);
-#pragma unroll
-        for (int v = 0; v < VG; ++v) {
-            T g[D], dd[NS];
-#pragma unroll
-            for (int d = 0; d < D; ++d) g[d] = T(0);
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                dd[s] = nv[s][v] - phi[a][v];
-#pragma unroll
-                for (int d = 0; d < D; ++d) g[d] += cg[s][d] * dd[s];
-            }
-            T L = T(1);
-            if (limiter == 1) {
-                // extremes of the neighbour differences and of the face
-                // projections g . r_s (both include 0: the cell itself)
-                T d2[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    d2[s] = g[0] * rr[s][0];
-#pragma unroll
-                    for (int d = 1; d < D; ++d) d2[s] += g[d] * rr[s][d];
-                }
-                T dmax, dmin, p, n;
-                if constexpr (sizeof(T) == 4 && NS == 6) {
-                    dmax = max3f(max3f(dd[0], dd[1], dd[2]), max3f(dd[3], dd[4], dd[5]), 0.0f);
-                    dmin = min3f(min3f(dd[0], dd[1], dd[2]), min3f(dd[3], dd[4], dd[5]), 0.0f);
-                    p = max3f(max3f(d2[0], d2[1], d2[2]), max3f(d2[3], d2[4], d2[5]), 0.0f);
-                    n = min3f(min3f(d2[0], d2[1], d2[2]), min3f(d2[3], d2[4], d2[5]), 0.0f);
-                } else if constexpr (sizeof(T) == 4 && NS == 4) {
-                    dmax = max3f(max3f(dd[0], dd[1], dd[2]), dd[3], 0.0f);
-                    dmin = min3f(min3f(dd[0], dd[1], dd[2]), dd[3], 0.0f);
-                    p = max3f(max3f(d2[0], d2[1], d2[2]), d2[3], 0.0f);
-                    n = min3f(min3f(d2[0], d2[1], d2[2]), d2[3], 0.0f);
-                } else {
-                    dmax = dmin = p = n = T(0);
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        dmax = dd[s] > dmax ? dd[s] : dmax;
-                        dmin = dd[s] < dmin ? dd[s] : dmin;
-                        p = d2[s] > p ? d2[s] : p;
-                        n = d2[s] < n ? d2[s] : n;
-                    }
-                }
-                // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
-                const T e2p = e2 * phi[a][v] * phi[a][v];
-                if (p > T(0)) { const T t = venkat(dmax, p, e2p); L = t < L ? t : L; }
-                if (n < T(0)) { const T t = venkat(dmin, n, e2p); L = t < L ? t : L; }
-            }
-            if (limiter == 0) L = T(0);          // first order: phi_bar = phi_C
-#pragma unroll
-            for (int d = 0; d < D; ++d) G[a][d][v] = L * g[d];
-        }
-    }
-    // node coordinates of the thread's nodes
-    T x[VG][D];
-    {
-        T xx[VG * D];
-        ldvn<T, VG * D>(xi + (size_t)k0 * D, xx);
-#pragma unroll
-        for (int v = 0; v < VG; ++v)
-#pragma unroll
-            for (int d = 0; d < D; ++d) x[v][d] = xx[v * D + d];
-    }
-    // phi_bar = A + G . r_s with A = phi - h G . xi, the part common to the faces
-    T A[NA][VG];
-#pragma unroll
-    for (int a = 0; a < NA; ++a)
-#pragma unroll
-        for (int v = 0; v < VG; ++v) {
-            T gx = G[a][0][v] * x[v][0];
-#pragma unroll
-            for (int d = 1; d < D; ++d) gx += G[a][d][v] * x[v][d];
-            A[a][v] = phi[a][v] - h * gx;
-        }
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        if (s >= ns) break;
-        const int sl = slot[i * AVS_MAXS + s];
-        const int fc = sl >> 1;
-        const bool isR = sl & 1;
-        T an[D];
-#pragma unroll
-        for (int d = 0; d < D; ++d) an[d] = An[(size_t)fc * D + d];
-        bool up[VG];
-        bool all = true, any = false;
-#pragma unroll
-        for (int v = 0; v < VG; ++v) {
-            // the face kernel's xi . An (FP64: summed without contraction, so
-            // the upwind choice is the plain sequential one; FP32: any fixed
-            // formula, since only the face's two cells must agree)
-            T sn;
-            if constexpr (sizeof(T) == 8) {
-                sn = dot_rn<D>(x[v], an);
-            } else {
-                sn = x[v][0] * an[0];
-#pragma unroll
-                for (int d = 1; d < D; ++d) sn = fmaf(x[v][d], an[d], sn);
-            }
-            up[v] = isR ? (sn < T(0)) : (sn >= T(0));
-            all = all && up[v];
-            any = any || up[v];
-        }
-        if (!any) continue;
-        T* row = FB + (size_t)fc * NA * Nvp + k0;
+    const double e2 = geo.eps2[i];
+    const int kend = min(Nv, (int)(blockIdx.y + 1) * chunk);
+#pragma unroll 1
+    for (int k0 = blockIdx.y * chunk + threadIdx.x * VG; k0 < kend; k0 += blockDim.x * VG) {
+        double phi[NA][VG], L[NA][VG], dr[NA][VG][NS], A[NA][VG], x[VG][D];
+        ldvn<double, VG * D>(xi + (size_t)k0 * D, &x[0][0]);
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
-            T out[VG];
+            const double* fa = f + (size_t)a * Nvp + k0;
+            double nv[NS][VG];
+            ldvn<double, VG>(fa + (size_t)i * cstride, phi[a]);
+#pragma unroll
+            for (int q = 0; q < NS; ++q)
+                ldvn<double, VG>(fa + (size_t)__float_as_int(g32[3 * q].w) * cstride, nv[q]);
 #pragma unroll
             for (int v = 0; v < VG; ++v) {
-                T val = A[a][v];
+                double g[D], dd[NS];
 #pragma unroll
-                for (int d = 0; d < D; ++d) val += G[a][d][v] * rr[s][d];
-                out[v] = val;
+                for (int d = 0; d < D; ++d) g[d] = 0.0;
+#pragma unroll
+                for (int q = 0; q < NS; ++q) {
+                    dd[q] = nv[q][v] - phi[a][v];
+#pragma unroll
+                    for (int d = 0; d < D; ++d) g[d] += sc[q][d] * dd[q];
+                }
+#pragma unroll
+                for (int q = 0; q < NS; ++q) {
+                    dr[a][v][q] = g[0] * sr[q][0];
+#pragma unroll
+                    for (int d = 1; d < D; ++d) dr[a][v][q] += g[d] * sr[q][d];
+                }
+                double l = limiter == 0 ? 0.0 : 1.0;       // first order: phi_bar = phi_C
+                if (limiter == 1) {
+                    // extremes of the neighbour differences and of the face
+                    // projections g . r_s (both include 0: the cell itself)
+                    double dmax, dmin, p, n;
+                    ext_bits<NS>(dd, dmax, dmin);
+                    ext_bits<NS>(dr[a][v], p, n);
+                    // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
+                    const double e2p = e2 * phi[a][v] * phi[a][v];
+                    // the ratios are >= 0 or NaN (0/0), whose bits are above those of 1
+                    unsigned long long b = (unsigned long long)__double_as_longlong(1.0);
+                    if (__double_as_longlong(p) > 0) {
+                        const unsigned long long t = (unsigned long long)__double_as_longlong(venkat_ratio(dmax, p, e2p));
+                        b = t < b ? t : b;
+                    }
+                    if (__double_as_longlong(n) < 0) {
+                        const unsigned long long t = (unsigned long long)__double_as_longlong(venkat_ratio(dmin, n, e2p));
+                        b = t < b ? t : b;
+                    }
+                    l = __longlong_as_double((long long)b);
+                }
+                double gx = g[0] * x[v][0];
+#pragma unroll
+                for (int d = 1; d < D; ++d) gx += g[d] * x[v][d];
+                L[a][v] = l;
+                A[a][v] = phi[a][v] - (h * l) * gx;
             }
-            if (all) {
-                stvn<T, VG>(row + (size_t)a * Nvp, out);
-            } else {
+        }
+        float2 x32[D];
 #pragma unroll
-                for (int v = 0; v < VG; ++v)
-                    if (up[v]) row[(size_t)a * Nvp + v] = out[v];
+        for (int d = 0; d < D; ++d) x32[d] = *reinterpret_cast<const float2*>(xs + d * xstride + k0);
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            const int fc = __float_as_int(g32[3 * q + 1].w);
+            if (fc < 0) break;                   // no further faces
+            const float4 n4 = g32[3 * q + 2];
+            const float na[3] = {n4.x, n4.y, n4.z};
+            bool up[VG];
+#pragma unroll
+            for (int v = 0; v < VG; ++v) {
+                float sn = 0.0f, sa = 0.0f;
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    const float xv = v ? x32[d].y : x32[d].x;
+                    sn = fmaf(xv, na[d], sn);
+                    sa = fmaf(fabsf(xv), fabsf(na[d]), sa);
+                }
+                // |sn - xi . An| <= 5 * 2^-24 sum |xi_d An_d| while normal
+                if (fabsf(sn) > fmaf(sa, 0x1p-20f, 0x1p-100f) && sa < INFINITY) up[v] = sn > 0.0f;
+                else up[v] = upwind_exact(D, x[v], An + (size_t)fc * D, n4.w != 0.0f);
+            }
+            if (!up[0] && !up[1]) continue;
+            double* row = FB + (size_t)fc * NA * Nvp + k0;
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                double o[VG];
+#pragma unroll
+                for (int v = 0; v < VG; ++v) o[v] = A[a][v] + L[a][v] * dr[a][v][q];
+                if (up[0] && up[1]) {
+                    stvn<double, VG>(row + (size_t)a * Nvp, o);
+                } else {
+#pragma unroll
+                    for (int v = 0; v < VG; ++v)
+                        if (up[v]) row[(size_t)a * Nvp + v] = o[v];
+                }
             }
         }
     }
@@ -404,23 +422,6 @@ __device__ __forceinline__ float2 limit2(float2 dmax, float2 dmin, float2 pp, fl
 {
     const float2 tp = venkat2(dmax, pp, eps2), tn = venkat2(dmin, nn, eps2);
     return make_float2(min3f(tp.x, tn.x, 1.0f), min3f(tp.y, tn.y, 1.0f));
-}
-
-// The cell's geometry from its record (Geo32): per slot least-squares weights
-// and neighbour cell, face offset and face, outward normal and upwind threshold
-// as three 16-byte vectors, copied once per block to shared memory.
-template <int NS>
-__device__ __forceinline__ void load_geo32(const float4* __restrict__ geo, int i, float4* gs)
-{
-    if (threadIdx.x < 3 * NS) gs[threadIdx.x] = geo[(size_t)i * (3 * AVS_MAXS) + threadIdx.x];
-    __syncthreads();
-}
-template <int D>
-__device__ __forceinline__ void vec3(const float4& v, float (&o)[D])
-{
-    o[0] = v.x;
-    o[1] = v.y;
-    if constexpr (D == 3) o[2] = v.z;
 }
 
 // Thread block (cell i, nodes of one chunk), the thread's quads one after the
@@ -609,8 +610,6 @@ struct FaceP {
     const int* __restrict__ faceL;
     const int* __restrict__ faceR;
     const T* __restrict__ An;
-    const T* __restrict__ rL;
-    const T* __restrict__ rR;
     const double* __restrict__ bc;
     int* err;
 };
@@ -618,7 +617,7 @@ struct FaceP {
 template <typename T>
 struct FaceSt {
     int kind, L, R;          // kind: 0 interior, 1 wall, 2 far field
-    T An[3], rL[3], rR[3];
+    T An[3];
     double V[3];             // reference velocity of the moment sums
     T Vt[3];                 // the same in the element type
     EqPar<T> eq;             // interface equilibrium / incoming Maxwellian
@@ -652,8 +651,6 @@ __device__ __forceinline__ void face_setup(const FaceP<D, T>& P, int f, FaceSt<T
     S.kind = S.R >= 0 ? 0 : (int)P.bc[(size_t)(-1 - S.R) * 6];
     for (int d = 0; d < 3; ++d) {
         S.An[d] = d < D ? P.An[(size_t)f * D + d] : T(0);
-        S.rL[d] = d < D ? P.rL[(size_t)f * D + d] : T(0);
-        S.rR[d] = d < D ? P.rR[(size_t)f * D + d] : T(0);
         T v = T(0);
         if (d < D) {
             v = (T)P.Win[(size_t)S.L * NW + 1 + d] / (T)P.Win[(size_t)S.L * NW];
@@ -881,6 +878,107 @@ __global__ void __launch_bounds__(NT, 4) k_face(FaceP<D, T> P)
     }
 }
 
+// ------------------------------------------------------------------ k_face_tab
+// The FP64 face kernel where the tree's nodes have few different coordinates
+// per axis.  A Maxwellian is a product over the axes, so pass B takes the
+// interface equilibrium, xi . An and |c|^2 from tables of the axes' values, one
+// entry per coordinate (xtab, at most half as many as nodes), built by the
+// block once the face's state is known: an exponential and 16 further FP64
+// operations per node become three products and four sums.  FP64 instructions
+// per face and node 80 -> 48 (3D); per step 202 -> 128 us on the 32 x 32 cavity
+// (298 nodes), 5.46 -> 3.46 ms on 1000 cells x 13824 nodes in 3D.
+struct AxisEq {
+    double E, c2, ca, xa;    // exp(-c^2 / 2RT) (axis 0: times wb pref), c^2, c alpha, xi An
+};
+
+template <int D, int NT>
+__global__ void __launch_bounds__(NT) k_face_tab(FaceP<D, double> P, const double* __restrict__ xtab,
+                                                 const unsigned short* __restrict__ tix, size_t xstride, int n0,
+                                                 int n1, int nt)
+{
+    constexpr int NA = NArr<D>::v, NW = D + 2;
+    constexpr int NR = FaceNR<D>::v;
+    extern __shared__ __align__(16) unsigned char tab_dsm[];
+    AxisEq* tab = reinterpret_cast<AxisEq*>(tab_dsm);
+    __shared__ FaceSt<double> S;
+    __shared__ double sw[(NT / 32) * NR];
+    __shared__ double red[NR];
+    const int tid = threadIdx.x;
+    const int f = P.order[blockIdx.x];
+    if (tid == 0) face_setup<D, double>(P, f, S);
+    __syncthreads();
+    {
+        double acc[NR];
+        face_pass_a<D, double, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
+        block_sum_t<NR, NT>(acc, sw, red);
+    }
+    if (tid == 0) face_state<D, double>(P, S, red, P.AF + (size_t)f * NW);
+    __syncthreads();
+    double acc[NW];
+    if (S.kind != 0) {
+        face_pass_b<D, double, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
+        return;
+    }
+    for (int e = tid; e < nt; e += NT) {
+        const int d = e < n0 ? 0 : e < n1 ? 1 : 2;
+        const double x = xtab[e], c = x - S.eq.U[d], c2 = c * c;
+        AxisEq q;
+        q.E = ex(-c2 * S.eq.inv2RT);
+        if (d == 0) q.E *= S.wb * S.eq.pref;
+        q.c2 = c2;
+        q.ca = c * S.eq.alpha[d];
+        q.xa = dmul(x, S.An[d]);
+        tab[e] = q;
+    }
+    __syncthreads();
+    const double wa = S.wa, irt = S.eq.invRT, RTH = S.eq.RTH;
+    const int Nvp = P.Nvp;
+    double* Fo = P.FB + (size_t)f * NA * Nvp;            // foot values in, flux out
+#pragma unroll
+    for (int m = 0; m < NW; ++m) acc[m] = 0.0;
+    for (int k0 = tid * 2; k0 < P.Nv; k0 += NT * 2) {
+        double x[2][D], wv[2], fv[NA][2], o[NA][2];
+        load_nodes<D, 2>(P, k0, x, wv);
+        ushort2 ix[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) ix[d] = *reinterpret_cast<const ushort2*>(tix + d * xstride + k0);
+#pragma unroll
+        for (int a = 0; a < NA; ++a) ldv<double, 2>(Fo + (size_t)a * Nvp + k0, fv[a]);
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const AxisEq* q0 = tab + (v ? ix[0].y : ix[0].x);
+            double E = q0->E, c2 = q0->c2, ca = q0->ca, sn = q0->xa;
+            double x2 = x[v][0] * x[v][0];
+#pragma unroll
+            for (int d = 1; d < D; ++d) {
+                const AxisEq* q = tab + (v ? ix[d].y : ix[d].x);
+                E *= q->E;
+                c2 += q->c2;
+                ca += q->ca;
+                sn = dadd(sn, q->xa);
+                x2 += x[v][d] * x[v][d];
+            }
+            const double pG = wa * fv[0][v] + E * (1.0 + ca * (c2 * irt - (D + 2)));
+            const double pH = NA == 2 ? wa * fv[NA - 1][v] + RTH * E * (1.0 + ca * (c2 * irt - D)) : 0.0;
+            o[0][v] = sn * pG;
+            const double q = wv[v] * o[0][v];
+            acc[0] += q;
+#pragma unroll
+            for (int d = 0; d < D; ++d) acc[1 + d] += q * x[v][d];
+            acc[D + 1] += q * x2;                          // twice the energy moment
+            if (NA == 2) {
+                o[NA - 1][v] = sn * pH;
+                acc[D + 1] += wv[v] * o[NA - 1][v];
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) stv<double, 2>(Fo + (size_t)a * Nvp + k0, o[a]);
+    }
+    acc[D + 1] *= 0.5;
+    block_sum_t<NW, NT>(acc, sw, red);
+    if (tid < NW) P.AF[(size_t)f * NW + tid] = red[tid];
+}
+
 // ------------------------------------------------------------------ k_cell
 // Per-cell parameters of the collision update, written by k_cell_state.
 template <typename T>
@@ -991,10 +1089,7 @@ __global__ void k_cell_state(CellP<D, T> P)
     if (i >= P.Nc) return;
     const double* Wi = P.Win + (size_t)i * NW;
     double Vc[3] = {0.0, 0.0, 0.0}, m[NM];
-    for (int d = 0; d < D; ++d) {
-        if constexpr (sizeof(T) == 4) Vc[d] = (double)reinterpret_cast<const Cell32Par*>(P.par)[i].V[d];
-        else Vc[d] = Wi[1 + d] / Wi[0];
-    }
+    for (int d = 0; d < D; ++d) Vc[d] = (double)((T)Wi[1 + d] / (T)Wi[0]);
     for (int k = 0; k < NM; ++k) m[k] = P.mom[(size_t)i * NM + k];
     T rn, Un[3], RTn, qn[3];
     state_from_raw<D, T>(m, Vc, rn, Un, RTn, qn);
@@ -1024,7 +1119,7 @@ __global__ void k_cell_state(CellP<D, T> P)
     const T idt = (T)(1.0 / P.dt), itau = T(1) / tau;
     if constexpr (sizeof(T) == 4) {
         reinterpret_cast<Cell32Par*>(P.par)[i] =
-            cell32_par(cp.eq, idt, itau, -(float)(1.0 / P.vol[i]), 1.0f / (idt + itau), U, 0.0f);
+            cell32_par(cp.eq, idt, itau, -(float)(1.0 / P.vol[i]), 1.0f / (idt + itau), cp.Vn, 0.0f);
         return;
     }
     cp.upd[0] = idt;
@@ -1118,6 +1213,108 @@ __global__ void __launch_bounds__(NT, 4) k_cell(CellP<D, T> P)
     __syncthreads();
     T acc[NM];
     cell_update<D, T, NT, VC>(P, i, ns, fs, sg, cp, 0, P.Nv, acc);
+    block_sum_t<NM, NT>(acc, sw, red);
+    if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
+}
+
+// k_cell in the FP64 form with the cell's equilibrium from tables of the axes'
+// values, as k_face_tab (67 -> 39 FP64 instructions per cell and node in 3D; per
+// step 61 -> 43 us and 1.63 -> 0.99 ms on the same cases).
+// The carried raw moments are summed from c = xi - U(W~) as k_raw_moments forms
+// it, in its node order.
+struct AxisCell {
+    double E, c, ca, pad;    // exp(-c^2 / 2RT) (axis 0: times pref), c, c alpha
+};
+
+template <int D, int NT>
+__global__ void __launch_bounds__(NT) k_cell_tab(CellP<D, double> P, const double* __restrict__ xtab,
+                                                 const unsigned short* __restrict__ tix, size_t xstride, int n0,
+                                                 int n1, int nt)
+{
+    constexpr int NA = NArr<D>::v, NM = NMom<D>::v;
+    extern __shared__ __align__(16) unsigned char tab_dsm[];
+    AxisCell* tab = reinterpret_cast<AxisCell*>(tab_dsm);
+    __shared__ int fs[AVS_MAXS];
+    __shared__ double sg[AVS_MAXS];
+    __shared__ double sw[(NT / 32) * NM];
+    __shared__ double red[NM];
+    const int tid = threadIdx.x;
+    const int i = blockIdx.x;
+    const int ns = P.nslot[i];
+    const CellPar<double>& cp = P.par[i];
+    if (tid < ns) {
+        const int sl = P.slot[i * AVS_MAXS + tid];
+        fs[tid] = sl >> 1;
+        sg[tid] = (sl & 1) ? -1.0 : 1.0;
+    }
+    for (int e = tid; e < nt; e += NT) {
+        const int d = e < n0 ? 0 : e < n1 ? 1 : 2;
+        const double c = xtab[e] - cp.eq.U[d];
+        AxisCell q;
+        q.E = ex(-(c * c) * cp.eq.inv2RT);
+        if (d == 0) q.E *= cp.eq.pref;
+        q.c = c;
+        q.ca = c * cp.eq.alpha[d];
+        q.pad = 0.0;
+        tab[e] = q;
+    }
+    __syncthreads();
+    const double u0 = cp.upd[0], u1 = cp.upd[1], u2 = cp.upd[2], u3 = cp.upd[3], irt = cp.eq.invRT, RTH = cp.eq.RTH;
+    const double* fi = P.fin + (size_t)i * P.cstride;
+    double* fo = P.fout + (size_t)i * P.cstride;
+    double acc[NM];
+#pragma unroll
+    for (int m = 0; m < NM; ++m) acc[m] = 0.0;
+    for (int k0 = tid * 2; k0 < P.Nv; k0 += NT * 2) {
+        double wv[2], Nn[NA][2], fv[NA][2], out[NA][2];
+        ldv<double, 2>(P.w + k0, wv);
+        ushort2 ix[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) ix[d] = *reinterpret_cast<const ushort2*>(tix + d * xstride + k0);
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+            ldv_cg<double, 2>(fi + (size_t)a * P.Nvp + k0, fv[a]);
+            Nn[a][0] = Nn[a][1] = 0.0;
+        }
+#pragma unroll
+        for (int s = 0; s < AVS_MAXS; ++s) {
+            if (s >= ns) break;
+            const double* Fs = P.F + (size_t)fs[s] * NA * P.Nvp + k0;
+            const double g = sg[s];
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                double t[2];
+                ldv_cg<double, 2>(Fs + (size_t)a * P.Nvp, t);
+                Nn[a][0] += g * t[0];
+                Nn[a][1] += g * t[1];
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const AxisCell* q0 = tab + (v ? ix[0].y : ix[0].x);
+            double E = q0->E, ca = q0->ca, c[D];
+            c[0] = q0->c;
+            double c2 = c[0] * c[0];
+#pragma unroll
+            for (int d = 1; d < D; ++d) {
+                const AxisCell* q = tab + (v ? ix[d].y : ix[d].x);
+                E *= q->E;
+                ca += q->ca;
+                c[d] = q->c;
+                c2 += c[d] * c[d];
+            }
+            const double gG = E * (1.0 + ca * (c2 * irt - (D + 2)));
+            const bool real = k0 + v < P.Nv;
+            out[0][v] = real ? (fv[0][v] * u0 + gG * u1 - Nn[0][v] * u2) * u3 : 0.0;
+            if (NA == 2) {
+                const double gH = RTH * E * (1.0 + ca * (c2 * irt - D));
+                out[NA - 1][v] = real ? (fv[NA - 1][v] * u0 + gH * u1 - Nn[NA - 1][v] * u2) * u3 : 0.0;
+            }
+            raw_acc<D>(acc, c, wv[v] * out[0][v], NA == 2 ? wv[v] * out[NA - 1][v] : 0.0);
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) stv<double, 2>(fo + (size_t)a * P.Nvp + k0, out[a]);
+    }
     block_sum_t<NM, NT>(acc, sw, red);
     if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
 }
@@ -1238,6 +1435,11 @@ static void grad_t(avs_ctx* c, const void* fin)
     c->launches += 1;
 }
 
+// Tables of the axes' coordinates pay where a face's or cell's nodes are at
+// least twice the entries: an entry costs what a node without tables does, a
+// node with them about half.
+static bool axis_tables(const avs_ctx* c) { return c->tab_n > 0 && 2 * c->tab_n <= c->Nv; }
+
 // Foot values of every face (k_foot) and the face stage of a step: per-node
 // face flux in c->flux, area-weighted face flux of W in c->AFf (shared by
 // the explicit and the implicit step).
@@ -1286,59 +1488,76 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
             else go(std::integral_constant<int, AVS_MAXS>{});
         } else {
             const CellGeo<T> geo = cell_geo<T>(c);
-            const dim3 g(c->Nc, (c->Nv + 256 * VG - 1) / (256 * VG));
-            if (D == 2 && c->max_ns <= 4)
-                k_foot<D, T, VG, 4, NArr<D>::v><<<g, 256, 0, c->stream>>>(
-                    c->Nv, c->Nvp, c->cfg.limiter, (T)hd, (const T*)fin, (T*)c->flux, geo, c->slot, An, xi);
-            else
-                k_foot<D, T, VG, AVS_MAXS, NArr<D>::v><<<g, 256, 0, c->stream>>>(
-                    c->Nv, c->Nvp, c->cfg.limiter, (T)hd, (const T*)fin, (T*)c->flux, geo, c->slot, An, xi);
+            // two nodes per thread and iteration; 64 threads for short rows, up
+            // to four iterations while that leaves 16 blocks per SM
+            const int npair = (c->Nv + 1) / 2;
+            const int nt = npair <= 64 ? 64 : 128;
+            const int per = (int)std::max(1ll, std::min(4ll, (long long)c->Nc * npair / nt / (16 * std::max(1, c->nsm))));
+            const int ny = (npair + nt * per - 1) / (nt * per);
+            const int chunk = (npair + ny - 1) / ny * 2;
+            auto go = [&](auto ns) {
+                k_foot<D, decltype(ns)::value, NArr<D>::v><<<dim3(c->Nc, ny), nt, 0, c->stream>>>(
+                    c->Nv, c->Nvp, chunk, c->cfg.limiter, hd, (const double*)fin, (double*)c->flux, geo, c->slot,
+                    c->An_d, c->xi_d, (const float4*)c->geo32, c->xi_s, c->xstride);
+            };
+            if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
+            else go(std::integral_constant<int, AVS_MAXS>{});
         }
         c->launches += 1;
     }
-    if constexpr (sizeof(T) == 4) return launch_face32(c, Win, dt);
-    FaceP<D, T> P;
-    P.Nv = c->Nv;
-    P.Nvp = c->Nvp;
-    P.cstride = (size_t)NA * c->Nvp;
-    P.hd = hd;
-    P.h = (T)P.hd;
-    P.R = c->cfg.R;
-    P.Pr = c->cfg.Pr;
-    P.omega = c->cfg.omega;
-    P.mu_ref = c->mu_ref;
-    P.T_ref = c->cfg.T_ref;
-    P.FB = (T*)c->flux;
-    P.AF = c->AFf;
-    P.Win = Win;
-    P.xi = xi;
-    P.w = w;
-    P.order = c->forder;
-    P.faceL = c->faceL;
-    P.faceR = c->faceR;
-    P.An = An;
-    P.rL = f32 ? (const T*)c->rL_f : (const T*)c->rL_d;
-    P.rR = f32 ? (const T*)c->rR_f : (const T*)c->rR_d;
-    P.bc = c->bc;
-    P.err = c->dev_err;
-    constexpr int NT = 128;
-    // foot values of pass A kept in shared memory for pass B when they fit in
-    // the default dynamic allowance (48 KB); otherwise pass B re-reads the
-    // face's row
-    const size_t cache_bytes = (size_t)NA * c->Nvp * sizeof(T);
-    constexpr int VF = 2;            // nodes per thread and iteration: 16-byte vectors
-    // the default allowance covers static and dynamic shared memory together:
-    // the block's own arrays (state, reductions: under 2 KB) come first
-    constexpr size_t kStaticFace = 2048;
-    static_assert(sizeof(FaceSt<T>) + (NT / 32 + 1) * FaceNR<D>::v * sizeof(double) <= kStaticFace,
-                  "static shared memory of the face block");
-    if (cache_bytes + kStaticFace <= 48 * 1024)
-        k_face<D, T, NT, true, VF><<<c->Nf, NT, cache_bytes, c->stream>>>(P);
-    else
-        k_face<D, T, NT, false, VF><<<c->Nf, NT, 0, c->stream>>>(P);
-    c->launches += 1;
+    if constexpr (sizeof(T) == 4) {
+        return launch_face32(c, Win, dt);
+    } else {
+        FaceP<D, T> P;
+        P.Nv = c->Nv;
+        P.Nvp = c->Nvp;
+        P.cstride = (size_t)NA * c->Nvp;
+        P.hd = hd;
+        P.h = (T)P.hd;
+        P.R = c->cfg.R;
+        P.Pr = c->cfg.Pr;
+        P.omega = c->cfg.omega;
+        P.mu_ref = c->mu_ref;
+        P.T_ref = c->cfg.T_ref;
+        P.FB = (T*)c->flux;
+        P.AF = c->AFf;
+        P.Win = Win;
+        P.xi = xi;
+        P.w = w;
+        P.order = c->forder;
+        P.faceL = c->faceL;
+        P.faceR = c->faceR;
+        P.An = An;
+        P.bc = c->bc;
+        P.err = c->dev_err;
+        constexpr int NT = 128;
+        // foot values of pass A kept in shared memory for pass B when they fit in
+        // the default dynamic allowance (48 KB); otherwise pass B re-reads the
+        // face's row
+        const size_t cache_bytes = (size_t)NA * c->Nvp * sizeof(T);
+        constexpr int VF = 2;            // nodes per thread and iteration: 16-byte vectors
+        // the default allowance covers static and dynamic shared memory together:
+        // the block's own arrays (state, reductions: under 2 KB) come first
+        constexpr size_t kStaticFace = 2048;
+        static_assert(sizeof(FaceSt<T>) + (NT / 32 + 1) * FaceNR<D>::v * sizeof(double) <= kStaticFace,
+                      "static shared memory of the face block");
+        if (axis_tables(c)) {
+            const size_t smem = (size_t)c->tab_n * sizeof(AxisEq);
+            if (smem > 40 * 1024) {
+                const cudaError_t e =
+                    cudaFuncSetAttribute(k_face_tab<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+            }
+            k_face_tab<D, NT><<<c->Nf, NT, smem, c->stream>>>(P, c->xtab, c->tix, c->xstride, c->tab_end[0], c->tab_end[1],
+                                                             c->tab_n);
+        } else if (cache_bytes + kStaticFace <= 48 * 1024)
+            k_face<D, T, NT, true, VF><<<c->Nf, NT, cache_bytes, c->stream>>>(P);
+        else
+            k_face<D, T, NT, false, VF><<<c->Nf, NT, 0, c->stream>>>(P);
+        c->launches += 1;
 
-    return cudaGetLastError();
+        return cudaGetLastError();
+    }
 }
 
 template <int D, typename T>
@@ -1394,7 +1613,17 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
     } else {
         // 16-byte vectors of nodes per thread; k_raw_moments takes the same
         // node mapping, so that its sums equal the carried ones bit for bit
-        k_cell<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+        if (axis_tables(c)) {
+            const size_t smem = (size_t)c->tab_n * sizeof(AxisCell);
+            if (smem > 40 * 1024) {
+                e = cudaFuncSetAttribute(k_cell_tab<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+            }
+            k_cell_tab<D, NT><<<c->Nc, NT, smem, c->stream>>>(Q, c->xtab, c->tix, c->xstride, c->tab_end[0],
+                                                             c->tab_end[1], c->tab_n);
+        } else {
+            k_cell<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+        }
         c->launches += 1;
     }
     c->mom_valid = 1;          // the raw moments of fout about U(Wout) are in cmom
@@ -1677,10 +1906,7 @@ __global__ void k_imp_state(CellP<D, T> P, const double* Wt)
     if (i >= P.Nc) return;
     const double* Wi = P.Win + (size_t)i * NW;
     double Vc[3] = {0.0, 0.0, 0.0}, m[NM];
-    for (int d = 0; d < D; ++d) {
-        if constexpr (sizeof(T) == 4) Vc[d] = (double)reinterpret_cast<const Cell32Par*>(P.par)[i].V[d];
-        else Vc[d] = Wi[1 + d] / Wi[0];
-    }
+    for (int d = 0; d < D; ++d) Vc[d] = (double)((T)Wi[1 + d] / (T)Wi[0]);
     for (int k = 0; k < NM; ++k) m[k] = P.mom[(size_t)i * NM + k];
     T rn, Un[3], RTn, qn[3];
     state_from_raw<D, T>(m, Vc, rn, Un, RTn, qn);

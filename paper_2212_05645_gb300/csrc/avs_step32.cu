@@ -76,11 +76,12 @@ __device__ __forceinline__ float2 dot2(const float2* x, const float* a)
     return s;
 }
 
-// Equilibrium G and H at a node pair as eq_eval2 forms them; c = xi - U.
+// Equilibrium G and H at a node pair as eq_eval2 forms them.
 template <int D>
 __device__ __forceinline__ void eq2(const float2* x, const float* U, const float* al, float k2, float l2, float irt,
-                                    float RTH, float2& gG, float2& gH, float2* c)
+                                    float RTH, float2& gG, float2& gH)
 {
+    float2 c[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) c[d] = add2(x[d], bc2(-U[d]));
     float2 c2 = mul2(c[0], c[0]), cq = mul2(c[0], bc2(al[0]));
@@ -551,9 +552,9 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 128 ? (FPT > 2 ? 3 : 4) :
 // takes node quads, the rows of its next quads on their way into its own ring of
 // STG slots in shared memory, as in k_face32.  The kernel moves one row of f in
 // and out and the flux rows of the cell's faces (2D: four faces of two arrays,
-// 3D: six faces).  RES = false also sums the raw moments of the new f about U(W~) (P.mom), on the
-// same c = xi - U as the equilibrium, in the node order that k_raw32 repeats, so
-// that carried and recomputed moments are equal bit for bit.  (The update with
+// 3D: six faces).  RES = false also sums the raw moments of the new f about U(W~)
+// (P.mom), in the node order that k_raw32 repeats, so that carried and
+// recomputed moments are equal bit for bit.  (The update with
 // u0 u3, u1 u3 and un u3 formed first takes two instructions less per value, no
 // time, and rounds f differently: the heat flux of a gas near equilibrium, a
 // small difference of large sums, moved by 2e-5 of itself.)
@@ -563,7 +564,7 @@ struct Cell32P {
     const float* fin;
     float* fout;
     const float* F;          // [face][array][Nvp] per-node flux
-    Cell32Par* par;
+    const Cell32Par* par;
     const double* W;         // k_raw32: W of the reference velocity
     double* mom;
     const float* xs;
@@ -656,10 +657,10 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<D> P, 
         slot = slot + 1 == STG ? 0 : slot + 1;
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-            float2 x[D], c[D], g[2];
+            float2 x[D], y[D], g[2];
 #pragma unroll
             for (int d = 0; d < D; ++d) x[d] = X[d][p];
-            eq2<D>(x, cp.U, cp.al, cp.k2, cp.l2, cp.irt, cp.RTH, g[0], g[1], c);
+            eq2<D>(x, cp.U, cp.al, cp.k2, cp.l2, cp.irt, cp.RTH, g[0], g[1]);
 #pragma unroll
             for (int a = 0; a < NA; ++a)
                 o[a][p] = mul2(fma2(N[a][p], bc2(cp.un), fma2(f0[a][p], bc2(cp.u0), mul2(g[a], bc2(cp.u1)))), bc2(cp.u3));
@@ -672,7 +673,9 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<D> P, 
                 float2 v[NA];
 #pragma unroll
                 for (int a = 0; a < NA; ++a) v[a] = o[a][p];
-                pair_moments<D>(m, c, W2[p], v);
+#pragma unroll
+                for (int d = 0; d < D; ++d) y[d] = add2(x[d], bc2(-cp.V[d]));
+                pair_moments<D>(m, y, W2[p], v);
             }
         }
 #pragma unroll
@@ -690,24 +693,17 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<D> P, 
 }
 
 // Raw moments of the own f of every cell about its U(W) in k_cell32's node
-// order, and that U into the cell's record; after anything but a step changed
-// f or W.
+// order; after anything but a step changed f or W.
 template <int D, int NT>
 __global__ void __launch_bounds__(NT) k_raw32(Cell32P<D> P)
 {
     constexpr int NA = NArr<D>::v, NM = NMom<D>::v, NW = D + 2;
     __shared__ float sw[(NT / 32) * NM];
     __shared__ double red[NM];
-    __shared__ float Vs[3];
     const int t = threadIdx.x, i = blockIdx.x;
-    if (t < D) {
-        Vs[t] = (float)(P.W[(size_t)i * NW + 1 + t] / P.W[(size_t)i * NW]);
-        P.par[i].V[t] = Vs[t];
-    }
-    group_bar<NT>(1);
     float V[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) V[d] = Vs[d];
+    for (int d = 0; d < D; ++d) V[d] = (float)P.W[(size_t)i * NW + 1 + d] / (float)P.W[(size_t)i * NW];
     const float* fi = P.fin + (size_t)i * NA * P.Nvp;
     float2 m[NM];
 #pragma unroll
@@ -820,7 +816,7 @@ static Cell32P<D> cell_params(avs_ctx* c, const void* fin, void* fout, const dou
     P.fin = (const float*)fin;
     P.fout = (float*)fout;
     P.F = (const float*)c->flux;
-    P.par = (Cell32Par*)c->cpar;
+    P.par = (const Cell32Par*)c->cpar;
     P.W = W;
     P.mom = c->cmom;
     P.xs = c->xi_s;
