@@ -55,7 +55,7 @@ void free_all(avs_ctx* c)
                     c->level, c->base, c->key, c->level2, c->base2, c->key2, c->src, c->kind, c->emit,
                     c->newidx, c->d_count, c->xi_d, c->w_d, c->xi_f, c->w_f, c->xi_p, c->xi_s, c->xtab, c->tix, c->M, c->Mkey, c->f[0], c->f[1],
                     c->W[0], c->W[1], c->ncap, c->Wf, c->q, c->pseudo_f, c->pseudo_W, c->crit_cp, c->crit_cp32, c->Mlo, c->Mhi, c->Mthr, c->stage, c->dev_err,
-                    c->dt_key, c->gap_d, c->grad, c->flux, c->AFf, c->forder, c->cmom, c->rmom, c->cpar, c->clist, c->cstart_d, c->imp_dW, c->imp_rhs0, c->imp_diag, c->imp_Wta,
+                    c->dt_key, c->gap_d, c->grad, c->flux, c->AFf, c->forder, c->cmom, c->rmom, c->cpar, c->colour, c->clist, c->cstart_d, c->imp_dW, c->imp_rhs0, c->imp_diag, c->imp_Wta,
                     c->imp_co, c->imp_nint, c->imp_bar, c->mlp_P, c->mlp_Wb, c->mlp_part, c->mlp_grad,
                     c->mlp_X, c->mlp_Y, c->mlp_logits, c->mlp_list, c->mlp_count, c->M_alt};
     for (void* p : ptrs)
@@ -375,7 +375,7 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
         dalloc(&c->eps2_d, Nc) || dalloc(&c->eps2_f, Nc) ||
         dalloc(&c->geo32, ncs * 12) ||
         dalloc(&c->AFf, (size_t)Nf * c->NW) || dalloc(&c->forder, Nf) || dalloc(&c->iorder, Nf) || dalloc(&c->cmom, (size_t)Nc * AVS_CMOM_MAX) ||
-        dalloc((unsigned char**)&c->cpar, (size_t)Nc * AVS_CELLPAR_BYTES) || dalloc(&c->clist, Nc) ||
+        dalloc((unsigned char**)&c->cpar, (size_t)Nc * AVS_CELLPAR_BYTES) || dalloc(&c->clist, Nc) || dalloc(&c->colour, Nc) ||
         dalloc(&c->imp_dW, (size_t)Nc * c->NW) || dalloc(&c->imp_rhs0, (size_t)Nc * c->NW) ||
         dalloc(&c->imp_diag, Nc) || dalloc(&c->imp_Wta, (size_t)Nc * c->NW) ||
         dalloc(&c->imp_co, ncs * AVS_IMPSLOT_BYTES) || dalloc(&c->imp_nint, Nc) || dalloc(&c->imp_bar, 1))
@@ -455,6 +455,7 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
         std::vector<int> pos(c->cstart.begin(), c->cstart.end() - 1), cl(Nc);
         for (int i = 0; i < Nc; ++i) cl[pos[col[i]]++] = i;
         CK(up(c->clist, cl, s));
+        CK(up(c->colour, std::vector<unsigned char>(col.begin(), col.end()), s));
         if (dalloc(&c->cstart_d, c->ncolor + 1)) return fail(c, AVS_ENOMEM, "colour offsets");
         CK(up(c->cstart_d, c->cstart, s));
     }

@@ -685,10 +685,58 @@ __host__ __device__ inline double dkey_inv(unsigned long long k)
     return x;
 }
 
-// Grid-wide barrier of a cooperative launch, bounded: the block's thread 0
-// counts in and waits for the target count at most kGridSpin polls; a timeout
-// (or one seen in another block) sets error bit 2 and makes the block leave.
-// Monotone counter: the n-th barrier waits for n * gridDim.x arrivals.
+// A row of N values that other blocks may have written before the last grid
+// barrier (read past L1): vectors of 16 bytes where the row is made of them.
+template <int N, typename A>
+__device__ __forceinline__ void ld_row(const A* p, A (&o)[N])
+{
+    if constexpr (sizeof(A) == 4 && N % 4 == 0) {
+#pragma unroll
+        for (int v = 0; v < N; v += 4) {
+            const float4 u = __ldcg(reinterpret_cast<const float4*>(p + v));
+            o[v] = u.x;
+            o[v + 1] = u.y;
+            o[v + 2] = u.z;
+            o[v + 3] = u.w;
+        }
+    } else if constexpr (sizeof(A) == 8 && N % 2 == 0) {
+#pragma unroll
+        for (int v = 0; v < N; v += 2) {
+            const double2 u = __ldcg(reinterpret_cast<const double2*>(p + v));
+            o[v] = u.x;
+            o[v + 1] = u.y;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < N; ++c) o[c] = __ldcg(p + c);
+    }
+}
+
+template <int N, typename A>
+__device__ __forceinline__ void st_row(A* p, const A (&v)[N])
+{
+    if constexpr (sizeof(A) == 4 && N % 4 == 0) {
+#pragma unroll
+        for (int c = 0; c < N; c += 4)
+            __stcg(reinterpret_cast<float4*>(p + c), make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]));
+    } else if constexpr (sizeof(A) == 8 && N % 2 == 0) {
+#pragma unroll
+        for (int c = 0; c < N; c += 2) __stcg(reinterpret_cast<double2*>(p + c), make_double2(v[c], v[c + 1]));
+    } else {
+#pragma unroll
+        for (int c = 0; c < N; ++c) __stcg(p + c, v[c]);
+    }
+}
+
+// Grid-wide barrier of a cooperative launch, bounded, in two halves between
+// which a block may do work that no other block's depends on: every thread's
+// accesses before grid_arrive are seen by every thread after the grid_wait of
+// that target.  Thread 0 counts the block in, and waits for the target count at
+// most kGridSpin polls; a timeout (or one seen in another block) sets error
+// bit 2 and makes the block leave.  Monotone counter: the n-th barrier waits
+// for n * gridDim.x arrivals.  The block barrier before the release arrival
+// and after the acquire load orders the other threads' accesses: no further
+// fence (a fence on both sides and a sleep between polls took 1.3 us a barrier).
 constexpr long long kGridSpin = 1ll << 21;
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p)
@@ -697,14 +745,20 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void red_release_u32(unsigned* p, unsigned v)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 
-__device__ __forceinline__ bool grid_sync_bounded(unsigned* bar, unsigned target, int* err)
+__device__ __forceinline__ void grid_arrive(unsigned* bar)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) red_release_u32(bar, 1u);
+}
+__device__ __forceinline__ bool grid_wait(unsigned* bar, unsigned target, int* err)
 {
     __shared__ int ok;
-    __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
         int good = 1;
         for (long long it = 0; ld_acquire_u32(bar) < target; ++it) {
             if (it >= kGridSpin || ((it & 255) == 255 && (*(volatile int*)err & 2))) {
@@ -712,13 +766,16 @@ __device__ __forceinline__ bool grid_sync_bounded(unsigned* bar, unsigned target
                 good = 0;
                 break;
             }
-            __nanosleep(64);
         }
-        __threadfence();
         ok = good;
     }
     __syncthreads();
     return ok != 0;
+}
+__device__ __forceinline__ bool grid_sync_bounded(unsigned* bar, unsigned target, int* err)
+{
+    grid_arrive(bar);
+    return grid_wait(bar, target, err);
 }
 
 }  // namespace avs

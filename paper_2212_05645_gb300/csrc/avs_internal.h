@@ -115,6 +115,7 @@ struct avs_ctx {
     // ---- implicit step (Sec. 2.3.1): cell colouring and the macroscopic system
     int ncolor = 0;
     std::vector<int> cstart;                         // [ncolor+1] offsets into clist (host)
+    unsigned char *colour = nullptr;                 // [Nc]
     int *clist = nullptr;                            // [Nc] cells by colour, ascending within a colour
     int *cstart_d = nullptr;                         // [ncolor+1] the same offsets on the device
     double *imp_dW = nullptr, *imp_rhs0 = nullptr;   // [Nc][NW] (dW and -sum sgn A F, in the sweep type)

@@ -15,6 +15,7 @@
 
 #include "avs_dev.cuh"
 #include "avs_internal.h"
+#include "avs_step32.h"
 
 namespace avs {
 namespace {
@@ -1409,17 +1410,25 @@ __device__ __forceinline__ void rk_imp_cell(const RkImpP<A>& P, int q)
     A rhs[NW];
 #pragma unroll
     for (int c = 0; c < NW; ++c) rhs[c] = P.rhs[(size_t)q * NW + c];
-    for (int s = 0; s < n; ++s) {
-        const RkImpSlot<A> sc = P.co[(size_t)q * AVS_MAXS + s];
-        A Wj[NW], dWj[NW], G[NW];
+    // loads before the arithmetic, as imp_macro_cell
+    int j[AVS_MAXS];
+    A Wj[AVS_MAXS][NW], dWj[AVS_MAXS][NW];
 #pragma unroll
-        for (int c = 0; c < NW; ++c) {
-            Wj[c] = __ldcg(P.Wta + (size_t)sc.j * NW + c);
-            dWj[c] = __ldcg(P.dWa + (size_t)sc.j * NW + c);
+    for (int s = 0; s < AVS_MAXS; ++s) j[s] = s < n ? P.co[(size_t)q * AVS_MAXS + s].j : i;
+#pragma unroll
+    for (int s = 0; s < AVS_MAXS; ++s)
+        if (s < n) {
+            ld_row<NW>(P.Wta + (size_t)j[s] * NW, Wj[s]);
+            ld_row<NW>(P.dWa + (size_t)j[s] * NW, dWj[s]);
         }
-        rk_euler_flux<D, A>(Wj, sc.n, G);
 #pragma unroll
-        for (int c = 0; c < NW; ++c) rhs[c] += sc.nhA * (G[c] - sc.Gn[c]) + sc.hr * dWj[c];
+    for (int s = 0; s < AVS_MAXS; ++s) {
+        if (s >= n) break;
+        const RkImpSlot<A> sc = P.co[(size_t)q * AVS_MAXS + s];
+        A G[NW];
+        rk_euler_flux<D, A>(Wj[s], sc.n, G);
+#pragma unroll
+        for (int c = 0; c < NW; ++c) rhs[c] += sc.nhA * (G[c] - sc.Gn[c]) + sc.hr * dWj[s][c];
     }
     const A dg = P.dg[q];
     A dgr = dg;
@@ -1657,7 +1666,7 @@ __global__ void __launch_bounds__(RK_NT) rk_imp_micro(int Nv, int Nvp, const T* 
                                                       const int* __restrict__ faceL, const int* __restrict__ faceR,
                                                       const int* __restrict__ clist, int c0)
 {
-    static_assert(sizeof(T) == 8, "the mixed form uses rk_imp_micro32");
+    static_assert(sizeof(T) == 8, "the mixed form uses k_micro32");
     constexpr int NA = RkNA<D>::v;
     __shared__ double sAd[AVS_MAXS][3];
     __shared__ int snb[AVS_MAXS];
@@ -1693,94 +1702,6 @@ __global__ void __launch_bounds__(RK_NT) rk_imp_micro(int Nv, int Nvp, const T* 
         for (int s = 0; s < ns; ++s)
             if (snb[s] >= 0 && sn[s] < T(0)) acc -= sn[s] * dphi[((size_t)snb[s] * NA + a) * Nvp + k];
         dphi[((size_t)i * NA + a) * Nvp + k] = acc / dg;
-    }
-}
-
-// One colour of a microscopic sweep in the mixed form: as rk_imp_micro, four
-// nodes per thread in 16-byte vectors; a neighbour's dphi row is read only
-// when one of the four nodes is downwind of it.
-template <int D>
-__global__ void __launch_bounds__(RK_NT) rk_imp_micro32(int Nv, int Nvp, const float* __restrict__ res, float* dphi,
-                                                        const double* __restrict__ u0, const float* __restrict__ xif,
-                                                        const float* __restrict__ An, const int* __restrict__ slot,
-                                                        const unsigned char* __restrict__ nslot,
-                                                        const int* __restrict__ faceL, const int* __restrict__ faceR,
-                                                        const int* __restrict__ clist, int c0)
-{
-    constexpr int NA = RkNA<D>::v, V = 4;
-    __shared__ float sA[AVS_MAXS][D];
-    __shared__ int snb[AVS_MAXS];
-    __shared__ float su0;
-    const int tid = threadIdx.x;
-    const int i = clist[c0 + blockIdx.x];
-    const int ns = nslot[i];
-    if (tid < ns) {
-        const int sl = slot[i * AVS_MAXS + tid];
-        const int f = sl >> 1;
-#pragma unroll
-        for (int d = 0; d < D; ++d) sA[tid][d] = (sl & 1) ? -An[(size_t)f * D + d] : An[(size_t)f * D + d];
-        snb[tid] = (sl & 1) ? faceL[f] : faceR[f];
-    }
-    if (tid == 32) su0 = (float)u0[i];
-    __syncthreads();
-    const int k0 = (blockIdx.y * RK_NT + tid) * V;
-    if (k0 >= Nv) return;                          // pad nodes keep the zero of the initial dphi
-    float x[V][D];
-    {
-        float t[V * D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(xif + (size_t)k0 * D) + j);
-            t[4 * j] = q.x;
-            t[4 * j + 1] = q.y;
-            t[4 * j + 2] = q.z;
-            t[4 * j + 3] = q.w;
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-#pragma unroll
-            for (int d = 0; d < D; ++d) x[v][d] = t[v * D + d];
-    }
-    float sn[AVS_MAXS][V], idg[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) idg[v] = 0.0f;
-#pragma unroll
-    for (int s = 0; s < AVS_MAXS; ++s) {
-        if (s >= ns) break;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            float p = 0.0f;
-#pragma unroll
-            for (int d = 0; d < D; ++d) p += x[v][d] * sA[s][d];
-            sn[s][v] = p;
-            if (p >= 0.0f) idg[v] += p;
-        }
-    }
-    const float u = su0;
-#pragma unroll
-    for (int v = 0; v < V; ++v) idg[v] = 1.0f / (u + idg[v]);
-#pragma unroll
-    for (int a = 0; a < NA; ++a) {
-        const float4 r4 = __ldcg(reinterpret_cast<const float4*>(res + ((size_t)i * NA + a) * Nvp + k0));
-        float acc[V] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-        for (int s = 0; s < AVS_MAXS; ++s) {
-            if (s >= ns) break;
-            const int j = snb[s];
-            bool in = false;
-#pragma unroll
-            for (int v = 0; v < V; ++v) in |= sn[s][v] < 0.0f;
-            if (j < 0 || !in) continue;
-            const float4 t4 = __ldcg(reinterpret_cast<const float4*>(dphi + ((size_t)j * NA + a) * Nvp + k0));
-            const float t[V] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                if (sn[s][v] < 0.0f) acc[v] -= sn[s][v] * t[v];
-        }
-        float o[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) o[v] = k0 + v < Nv ? acc[v] * idg[v] : 0.0f;
-        *reinterpret_cast<float4*>(dphi + ((size_t)i * NA + a) * Nvp + k0) = make_float4(o[0], o[1], o[2], o[3]);
     }
 }
 
@@ -1935,7 +1856,7 @@ cudaError_t rk_step_implicit_t(avs_ctx* c, const void* fin, void* fout, const do
     c->launches += 1;
     const int nc = c->ncolor;
     if (k_macro > 0) {
-        constexpr int NTM = 128;
+        constexpr int NTM = 64;        // small blocks on many SMs: as the monatomic sweep
         int maxcol = 0;
         for (int k = 0; k < nc; ++k) maxcol = std::max(maxcol, c->cstart[k + 1] - c->cstart[k]);
         int dev = 0, nsm = 0, occ = 0;
@@ -1964,35 +1885,32 @@ cudaError_t rk_step_implicit_t(avs_ctx* c, const void* fin, void* fout, const do
     else
         rk_imp_res<D, T><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_d, c->w_d, u0);
     c->launches += 1;
-    T* dphi = (T*)c->flux;              // the face flux has been used
-    e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);
-    if (e != cudaSuccess) return e;
-    const int nyb = (c->Nvp + 127) / 128;
-    int prev = -1;
-    for (int it = 0; it < k_micro; ++it)
-        for (int dir = 0; dir < 2; ++dir)
-            for (int q = 0; q < nc; ++q) {
-                const int col = dir == 0 ? q : nc - 1 - q;
-                if (col == prev) continue;      // same inputs as the pass before: same values
-                prev = col;
-                const int c0 = c->cstart[col], c1 = c->cstart[col + 1];
-                if (c1 <= c0) continue;
-                if constexpr (sizeof(T) == 4) {
-                    rk_imp_micro32<D><<<dim3(c1 - c0, (c->Nv + RK_NT * 4 - 1) / (RK_NT * 4)), RK_NT, 0, c->stream>>>(
-                        c->Nv, c->Nvp, (const float*)fout, (float*)dphi, u0, c->xi_f, c->An_f, c->slot, c->nslot,
+    if constexpr (sizeof(T) == 4) {
+        e = launch_micro32(c, fin, fout, u0, k_micro);
+        if (e != cudaSuccess) return e;
+    } else {
+        T* dphi = (T*)c->flux;          // the face flux has been used
+        e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);
+        if (e != cudaSuccess) return e;
+        const int nyb = (c->Nvp + 127) / 128;
+        int prev = -1;
+        for (int it = 0; it < k_micro; ++it)
+            for (int dir = 0; dir < 2; ++dir)
+                for (int q = 0; q < nc; ++q) {
+                    const int col = dir == 0 ? q : nc - 1 - q;
+                    if (col == prev) continue;      // same inputs as the pass before: same values
+                    prev = col;
+                    const int c0 = c->cstart[col], c1 = c->cstart[col + 1];
+                    if (c1 <= c0) continue;
+                    rk_imp_micro<D, T><<<dim3(c1 - c0, nyb), 128, 0, c->stream>>>(
+                        c->Nv, c->Nvp, (const T*)fout, dphi, u0, c->xi_d, c->xi_d, c->An_d, c->An_d, c->slot, c->nslot,
                         c->faceL, c->faceR, c->clist, c0);
                     c->launches += 1;
-                } else {
-                    rk_imp_micro<D, T><<<dim3(c1 - c0, nyb), 128, 0, c->stream>>>(
-                        c->Nv, c->Nvp, (const T*)fout, dphi, u0, f32 ? (const T*)c->xi_f : (const T*)c->xi_d,
-                        c->xi_d, c->An_d, f32 ? (const T*)c->An_f : (const T*)c->An_d, c->slot, c->nslot, c->faceL,
-                        c->faceR, c->clist, c0);
-                    c->launches += 1;
                 }
-            }
-    dim3 gf(c->Nc * NA, std::min(8, (c->Nvp + 255) / 256));
-    rk_imp_finish<T><<<gf, 256, 0, c->stream>>>(c->Nv, c->Nvp, (const T*)fin, dphi, (T*)fout);
-    c->launches += 1;
+        dim3 gf(c->Nc * NA, std::min(8, (c->Nvp + 255) / 256));
+        rk_imp_finish<T><<<gf, 256, 0, c->stream>>>(c->Nv, c->Nvp, (const T*)fin, dphi, (T*)fout);
+        c->launches += 1;
+    }
     c->mom_valid = 0;          // no carried moments of fout
     return cudaGetLastError();
 }

@@ -1660,7 +1660,7 @@ __device__ __forceinline__ void euler_flux_n(const A* W, const A* n, A* G)
 // n, -A/2, A r/2 (r the face's spectral radius) and the Euler flux of the
 // neighbour's W^n through n, so that a sweep only evaluates G(W~_j).
 template <typename A>
-struct ImpSlot {
+struct alignas(16) ImpSlot {
     A n[3];
     A nhA;
     A hr;
@@ -1830,70 +1830,120 @@ cudaError_t launch_stage_wait_check(avs_ctx* c, const float* src, bool arrive, i
     return cudaGetLastError();
 }
 
-// One cell of a macroscopic sweep: dW_i = (Res_i(W~) + 1/2 sum A r dW_j) / diag_i,
+// One cell of a macroscopic sweep: dW_i = (Res_i + 1/2 sum A r dW_j) / dg_i,
 // Res_i = -sum sgn A F - 1/2 sum A (G(W~_j) - G(W^n_j)) over the interior faces.
 // Arithmetic in A (FP32 in the mixed form, where dW is a small correction of
-// the FP64 W^n); W~ = W^n + dW in FP64.  The neighbours' values are read past
-// L1: other blocks wrote them before the last grid barrier.
-template <int D, typename A>
-__device__ __forceinline__ void imp_macro_cell(const ImpP<A>& P, int q)
-{
-    constexpr int NW = D + 2;
-    const int i = P.clist[q];
-    const int n = P.nint[q];
-    A rhs[NW];
+// the FP64 W^n); W~ = W^n + dW in FP64.  What no sweep changes is loaded by
+// load() ahead of the grid barrier (FP32; in FP64 the slot records would not
+// fit the registers and are read in update()), the neighbours' values after it,
+// all before the arithmetic and past L1: other blocks wrote them.
+template <int D, typename A, int NS>
+struct ImpCell {
+    static constexpr int NW = D + 2;
+    static constexpr bool PRE = sizeof(A) == 4;
+    int i, n, j[NS];
+    A rhs[NW], dg;
+    double Wn[NW];
+    ImpSlot<A> s[PRE ? NS : 1];
+
+    __device__ __forceinline__ void load(const ImpP<A>& P, int q)
+    {
+        i = P.clist[q];
+        n = P.nint[q];
+        dg = P.dg[q];
 #pragma unroll
-    for (int c = 0; c < NW; ++c) rhs[c] = P.rhs[(size_t)q * NW + c];
-    for (int s = 0; s < n; ++s) {
-        const ImpSlot<A> sc = P.co[(size_t)q * AVS_MAXS + s];
-        A Wj[NW], dWj[NW], G[NW];
+        for (int c = 0; c < NW; ++c) rhs[c] = P.rhs[(size_t)q * NW + c];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            if (k >= n) break;
+            if constexpr (PRE) {
+                s[k] = P.co[(size_t)q * AVS_MAXS + k];
+                j[k] = s[k].j;
+            } else {
+                j[k] = P.co[(size_t)q * AVS_MAXS + k].j;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NW; ++c) Wn[c] = P.Wn[(size_t)i * NW + c];
+    }
+
+    __device__ __forceinline__ void update(const ImpP<A>& P, int q)
+    {
+        A Wj[NS][NW], dWj[NS][NW];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            if (k >= n) break;
+            ld_row<NW>(P.Wta + (size_t)j[k] * NW, Wj[k]);
+            ld_row<NW>(P.dWa + (size_t)j[k] * NW, dWj[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            if (k >= n) break;
+            if constexpr (!PRE) s[0] = P.co[(size_t)q * AVS_MAXS + k];
+            const ImpSlot<A>& sc = s[PRE ? k : 0];
+            A G[NW];
+            euler_flux_n<D, A>(Wj[k], sc.n, G);
+#pragma unroll
+            for (int c = 0; c < NW; ++c) rhs[c] += sc.nhA * (G[c] - sc.Gn[c]) + sc.hr * dWj[k][c];
+        }
+        A d[NW], wt[NW];
 #pragma unroll
         for (int c = 0; c < NW; ++c) {
-            Wj[c] = __ldcg(P.Wta + (size_t)sc.j * NW + c);
-            dWj[c] = __ldcg(P.dWa + (size_t)sc.j * NW + c);
+            d[c] = rhs[c] / dg;
+            wt[c] = (A)(Wn[c] + (double)d[c]);
         }
-        euler_flux_n<D, A>(Wj, sc.n, G);
-#pragma unroll
-        for (int c = 0; c < NW; ++c) rhs[c] += sc.nhA * (G[c] - sc.Gn[c]) + sc.hr * dWj[c];
+        st_row<NW>(P.dWa + (size_t)i * NW, d);
+        st_row<NW>(P.Wta + (size_t)i * NW, wt);
     }
-    const A dg = P.dg[q];
-#pragma unroll
-    for (int c = 0; c < NW; ++c) {
-        const A d = rhs[c] / dg;
-        const double wt = P.Wn[(size_t)i * NW + c] + (double)d;
-        __stcg(P.dWa + (size_t)i * NW + c, d);
-        if constexpr (sizeof(A) == sizeof(double)) {
-            __stcg(P.Wt + (size_t)i * NW + c, wt);
-        } else {
-            P.Wt[(size_t)i * NW + c] = wt;
-            __stcg(P.Wta + (size_t)i * NW + c, (A)wt);
-        }
-    }
-}
+};
 
 // The whole macroscopic solve in one cooperative launch: k_macro symmetric
 // Gauss-Seidel iterations, each colour a grid-stride pass, a grid barrier
-// between passes.  A colour that follows itself (the turn of a symmetric
+// between passes; the next pass's first cell is loaded while the barrier
+// collects its arrivals.  A colour that follows itself (the turn of a symmetric
 // sweep) is skipped: its neighbours have not changed, so the pass would
-// rewrite the same values.
-template <int D, typename A, int NT>
+// rewrite the same values.  Bounded by latency (barrier, one trip to L2, the
+// arithmetic of one cell per thread), so small blocks on many SMs: the 121
+// passes of 6144 cells (cylinder) took 690 us with the loads face by face after
+// the barrier, 368 us now.
+template <int D, typename A, int NT, int NS>
 __global__ void __launch_bounds__(NT) k_imp_macro(ImpP<A> P, int k_macro, int ncolor, const int* __restrict__ cstart,
                                                   unsigned* bar)
 {
+    constexpr int NW = D + 2;
     const unsigned nb = gridDim.x;
     unsigned gen = 0;
-    int prev = -1;
-    for (int it = 0; it < k_macro; ++it)
-        for (int dir = 0; dir < 2; ++dir)
-            for (int qq = 0; qq < ncolor; ++qq) {
-                const int col = dir == 0 ? qq : ncolor - 1 - qq;
-                if (col == prev) continue;
-                if (prev >= 0 && !grid_sync_bounded(bar, ++gen * nb, P.err)) return;
-                prev = col;
-                const int c1 = cstart[col + 1];
-                for (int q = cstart[col] + blockIdx.x * NT + threadIdx.x; q < c1; q += nb * NT)
-                    imp_macro_cell<D, A>(P, q);
+    const int q0 = blockIdx.x * NT + threadIdx.x, dq = nb * NT;
+    ImpCell<D, A, NS> C;
+    int col = 0, q = cstart[0] + q0, c1 = cstart[1];
+    if (q < c1) C.load(P, q);
+    for (int it = 0, r = 0;;) {                  // r: place in the symmetric sweep
+        while (q < c1) {
+            C.update(P, q);
+            q += dq;
+            if (q < c1) C.load(P, q);
+        }
+        int nx = col;
+        while (nx == col && it < k_macro) {
+            if (++r == 2 * ncolor) r = 0, ++it;
+            nx = r < ncolor ? r : 2 * ncolor - 1 - r;
+        }
+        if (it >= k_macro) break;
+        col = nx;
+        grid_arrive(bar);
+        q = cstart[col] + q0;
+        c1 = cstart[col + 1];
+        if (q < c1) C.load(P, q);
+        if (!grid_wait(bar, ++gen * nb, P.err)) return;
+    }
+    if constexpr (sizeof(A) == 4) {              // W~ in FP64, by the thread that updated the cell
+        for (col = 0; col < ncolor; ++col)
+            for (q = cstart[col] + q0; q < cstart[col + 1]; q += dq) {
+                const size_t o = (size_t)P.clist[q] * NW;
+#pragma unroll
+                for (int c = 0; c < NW; ++c) P.Wt[o + c] = P.Wn[o + c] + (double)__ldcg(P.dWa + o + c);
             }
+    }
 }
 
 // Per cell: Shakhov state of W~ with the lagged heat flux of f^n (R3);
@@ -2018,9 +2068,7 @@ __global__ void __launch_bounds__(NT) k_imp_micro(CellP<D, T> P, const T* __rest
     __syncthreads();
     const int k0 = (blockIdx.y * NT + tid) * V;
     if (k0 >= P.Nv) return;
-    T u0;
-    if constexpr (sizeof(T) == 4) u0 = reinterpret_cast<const Cell32Par*>(P.par)[i].diag;
-    else u0 = P.par[i].upd[0];
+    const T u0 = P.par[i].upd[0];
     T x[V][D], wv[V];
     load_nodes<D, V>(P, k0, x, wv);
     T sn[AVS_MAXS][V], dg[V];
@@ -2118,13 +2166,15 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
     if (k_macro > 0) {
         // one cooperative launch: every block resident, so the bounded grid
         // barriers between colour passes can complete
-        constexpr int NTM = 128;
+        constexpr int NTM = 64;
         int maxcol = 0;
         for (int k = 0; k < nc; ++k) maxcol = std::max(maxcol, c->cstart[k + 1] - c->cstart[k]);
+        const void* kern = D == 2 && c->max_ns <= 4 ? (const void*)k_imp_macro<D, A, NTM, D == 2 ? 4 : AVS_MAXS>
+                                                    : (const void*)k_imp_macro<D, A, NTM, AVS_MAXS>;
         int dev = 0, nsm = 0, occ = 0;
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_imp_macro<D, A, NTM>, NTM, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NTM, 0);
         if (e != cudaSuccess) return e;
         const int nblk = std::max(1, std::min(nsm * std::max(occ, 1), (maxcol + NTM - 1) / NTM));
         e = cudaMemsetAsync(c->imp_bar, 0, sizeof(unsigned), c->stream);
@@ -2133,8 +2183,7 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
         const int* cs = c->cstart_d;
         unsigned* bar = c->imp_bar;
         void* args[] = {&I, &km, &ncol, &cs, &bar};
-        e = cudaLaunchCooperativeKernel((const void*)k_imp_macro<D, A, NTM>, dim3(nblk), dim3(NTM), args, 0,
-                                        c->stream);
+        e = cudaLaunchCooperativeKernel(kern, dim3(nblk), dim3(NTM), args, 0, c->stream);
         if (e != cudaSuccess) return e;
         c->launches += 1;
     }
@@ -2180,35 +2229,35 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
     c->launches += 1;
     if constexpr (sizeof(T) == 4) {
         e = launch_cell32(c, fin, fout, true);
+        if (e == cudaSuccess) e = launch_micro32(c, fin, fout, nullptr, k_micro);
         if (e != cudaSuccess) return e;
     } else {
         k_imp_res<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
         c->launches += 1;
-    }
-    T* dphi = (T*)c->flux;                    // the face flux has been used: its buffer holds dphi
-    e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);
-    if (e != cudaSuccess) return e;
-    constexpr int VM = VW<T>::v;
-    const int nyb = (c->Nv + NT * VM - 1) / (NT * VM);
-    const T* Anv = f32 ? (const T*)c->An_f : (const T*)c->An_d;
-    int prev = -1;
-    for (int it = 0; it < k_micro; ++it)
-        for (int dir = 0; dir < 2; ++dir)
-            for (int q = 0; q < nc; ++q) {
-                const int col = dir == 0 ? q : nc - 1 - q;
-                if (col == prev) continue;      // the turn of a symmetric sweep: same inputs, same values
-                prev = col;
-                const int c0 = c->cstart[col], c1 = c->cstart[col + 1];
-                if (c1 > c0) {
-                    dim3 g(c1 - c0, nyb);
-                    k_imp_micro<D, T, NT, VM><<<g, NT, 0, c->stream>>>(Q, (const T*)fout, dphi, Anv, c->faceL,
-                                                                        c->faceR, c->clist, c0);
-                    c->launches += 1;
+        T* dphi = (T*)c->flux;                // the face flux has been used: its buffer holds dphi
+        e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);
+        if (e != cudaSuccess) return e;
+        constexpr int VM = VW<T>::v;
+        const int nyb = (c->Nv + NT * VM - 1) / (NT * VM);
+        int prev = -1;
+        for (int it = 0; it < k_micro; ++it)
+            for (int dir = 0; dir < 2; ++dir)
+                for (int q = 0; q < nc; ++q) {
+                    const int col = dir == 0 ? q : nc - 1 - q;
+                    if (col == prev) continue;      // the turn of a symmetric sweep: same inputs, same values
+                    prev = col;
+                    const int c0 = c->cstart[col], c1 = c->cstart[col + 1];
+                    if (c1 > c0) {
+                        dim3 g(c1 - c0, nyb);
+                        k_imp_micro<D, T, NT, VM><<<g, NT, 0, c->stream>>>(Q, (const T*)fout, dphi, c->An_d, c->faceL,
+                                                                            c->faceR, c->clist, c0);
+                        c->launches += 1;
+                    }
                 }
-            }
-    dim3 gf(c->Nc * NA, (c->Nvp + 255) / 256 < 8 ? (c->Nvp + 255) / 256 : 8);
-    k_imp_finish<T><<<gf, 256, 0, c->stream>>>(c->Nc * NA, c->Nv, c->Nvp, (const T*)fin, dphi, (T*)fout);
-    c->launches += 1;
+        dim3 gf(c->Nc * NA, (c->Nvp + 255) / 256 < 8 ? (c->Nvp + 255) / 256 : 8);
+        k_imp_finish<T><<<gf, 256, 0, c->stream>>>(c->Nc * NA, c->Nv, c->Nvp, (const T*)fin, dphi, (T*)fout);
+        c->launches += 1;
+    }
     c->mom_valid = 0;          // the carried moments are of f^n
     (void)NW;
     return cudaGetLastError();

@@ -15,6 +15,7 @@
 // spares the stores but takes 126 more FP32 operations per cell and node in 3D
 // and was no gain (29.2 + 27.2 and 2.63 + 4.51 ms).
 #include <algorithm>
+#include <vector>
 
 #include "avs_dev.cuh"
 #include "avs_internal.h"
@@ -732,6 +733,122 @@ __global__ void __launch_bounds__(NT) k_raw32(Cell32P<D> P)
     if (t < NM) P.mom[(size_t)i * NM + t] = red[t];
 }
 
+// ------------------------------------------------------------------ k_micro32
+// One colour of a microscopic sweep of the implicit step, FP32 form of either
+// gas: dphi_i = (Res_i - sum_{xi.n<0} (xi.n) dphi_j) / (diag_i + sum_{xi.n>=0} xi.n)
+// at every node of every array, by quads.  A neighbour's row is read only where
+// one of the quad's nodes flows in from it, and only once its colour has been
+// visited (`below`: colours that have; dphi is zero before), so dphi needs no
+// clearing and the first pass reads no neighbour.  The last visit of a colour
+// writes f^{n+1} = f^n + dphi over the residual (`finish`), and dphi itself only
+// where another colour still follows (`keep`).  Against a pass for every step
+// (clearing, sweeps of four-node threads, one addition at the end), per implicit
+// step of the cylinder (12288 cells, 3522 nodes): 1.43 -> 0.60 ms.
+template <int D, int NA>
+struct Micro32P {
+    int Nv, Nvp, chunk, c0, below;
+    bool finish, keep;
+    const float* fin;
+    float* fout;             // the residual; f^{n+1} after the last visit
+    float* dphi;
+    const float4* geo;
+    const Cell32Par* par;    // diag of the monatomic gas,
+    const double* diag;      // or (par = nullptr) per cell
+    const float* xs;
+    size_t xstride;
+    const int* nbr;
+    const int* clist;
+    const unsigned char* colour;
+};
+
+template <int D, int NS, int NA>
+__global__ void __launch_bounds__(128, 8) k_micro32(Micro32P<D, NA> P)
+{
+    __shared__ float4 sA[NS];                    // outward normal, neighbour to read (-1: none)
+    __shared__ float su;
+    __shared__ int sn_;
+    const int i = P.clist[P.c0 + blockIdx.x];
+    const int t = threadIdx.x;
+    if (t < NS) {
+        const float4* r = P.geo + (size_t)i * (3 * AVS_MAXS) + 3 * t;
+        const int j = P.nbr[i * AVS_MAXS + t], f = __float_as_int(r[1].w);
+        float4 n = r[2];
+        n.w = __int_as_float(f >= 0 && j >= 0 && P.colour[j] < P.below ? j : -1);
+        sA[t] = n;
+        const unsigned has = __ballot_sync((1u << NS) - 1u, f >= 0);
+        if (t == 0) sn_ = __popc(has);
+    } else if (t == 32) {
+        su = P.par ? P.par[i].diag : (float)P.diag[i];
+    }
+    __syncthreads();
+    const int ns = sn_;
+    const float u = su;
+    const int Nv = P.Nv, Nvp = P.Nvp;
+    const size_t own = (size_t)i * NA * Nvp;
+    const int kend = min(Nvp, (int)(blockIdx.y + 1) * P.chunk);
+#pragma unroll 1
+    for (int k = blockIdx.y * P.chunk + t * 4; k < kend; k += blockDim.x * 4) {
+        float2 X[D][2], acc[NA][2], dg[2];
+#pragma unroll
+        for (int a = 0; a < NA; ++a) ld4cg(P.fout + own + (size_t)a * Nvp + k, acc[a]);
+#pragma unroll
+        for (int d = 0; d < D; ++d) ld4(P.xs + d * P.xstride + k, X[d]);
+        dg[0] = dg[1] = bc2(0.0f);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            if (s >= ns) break;
+            const float4 n4 = sA[s];
+            const float An[3] = {n4.x, n4.y, n4.z};
+            const int j = __float_as_int(n4.w);
+            float2 in[2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                float2 x[D];
+#pragma unroll
+                for (int d = 0; d < D; ++d) x[d] = X[d][p];
+                const float2 sn = dot2<D>(x, An);
+                dg[p] = add2(dg[p], make_float2(fmaxf(sn.x, 0.0f), fmaxf(sn.y, 0.0f)));
+                in[p] = make_float2(fmaxf(-sn.x, 0.0f), fmaxf(-sn.y, 0.0f));
+            }
+            if (j < 0 || (in[0].x + in[0].y) + (in[1].x + in[1].y) == 0.0f) continue;
+            const float* dj = P.dphi + (size_t)j * NA * Nvp + k;
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                float2 v[2];
+                ld4cg(dj + (size_t)a * Nvp, v);
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    // a node that flows out takes nothing, whatever the neighbour holds
+                    const float2 w = make_float2(in[p].x > 0.0f ? v[p].x : 0.0f, in[p].y > 0.0f ? v[p].y : 0.0f);
+                    acc[a][p] = fma2(in[p], w, acc[a][p]);
+                }
+            }
+        }
+        const float2 inv[2] = {make_float2(1.0f / (u + dg[0].x), 1.0f / (u + dg[0].y)),
+                               make_float2(1.0f / (u + dg[1].x), 1.0f / (u + dg[1].y))};
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+            float2 o0 = mul2(acc[a][0], inv[0]), o1 = mul2(acc[a][1], inv[1]);
+            if (k + 4 > Nv) {                    // pad nodes: zero
+                if (k >= Nv) o0.x = 0.0f;
+                if (k + 1 >= Nv) o0.y = 0.0f;
+                if (k + 2 >= Nv) o1.x = 0.0f;
+                o1.y = 0.0f;
+            }
+            if (P.keep)
+                *reinterpret_cast<float4*>(P.dphi + own + (size_t)a * Nvp + k) = make_float4(o0.x, o0.y, o1.x, o1.y);
+            if (P.finish) {
+                float2 f[2];
+                ld4cg(P.fin + own + (size_t)a * Nvp + k, f);
+                f[0] = add2(f[0], o0);
+                f[1] = add2(f[1], o1);
+                *reinterpret_cast<float4*>(P.fout + own + (size_t)a * Nvp + k) =
+                    make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------ launchers
 template <int D>
 static cudaError_t face32_t(avs_ctx* c, const double* Win, double dt)
@@ -871,6 +988,65 @@ cudaError_t launch_raw32(avs_ctx* c, const void* fin, const double* W)
     }
     c->launches += 1;
     return cudaGetLastError();
+}
+
+// k_micro symmetric Gauss-Seidel iterations over the colours, then f^{n+1}.  A
+// colour that follows itself (the turn of a symmetric sweep) would write the
+// same values and is skipped.
+template <int D, int NA>
+static cudaError_t micro32_t(avs_ctx* c, const void* fin, void* fout, const double* diag, int k_micro)
+{
+    std::vector<int> seq;
+    for (int it = 0; it < k_micro; ++it)
+        for (int dir = 0; dir < 2; ++dir)
+            for (int q = 0; q < c->ncolor; ++q) {
+                const int col = dir == 0 ? q : c->ncolor - 1 - q;
+                if ((seq.empty() || col != seq.back()) && c->cstart[col + 1] > c->cstart[col]) seq.push_back(col);
+            }
+    if (seq.empty())
+        return cudaMemcpyAsync(fout, fin, (size_t)c->Nc * NA * c->Nvp * sizeof(float), cudaMemcpyDeviceToDevice,
+                               c->stream);
+    std::vector<int> last(c->ncolor, -1);
+    for (int p = 0; p < (int)seq.size(); ++p) last[seq[p]] = p;
+    std::vector<char> seen(c->ncolor, 0);
+    const int nquad = c->Nvp / 4;
+    const int nt = nquad <= 64 ? 64 : 128;
+    for (int p = 0; p < (int)seq.size(); ++p) {
+        const int col = seq[p], cells = c->cstart[col + 1] - c->cstart[col];
+        const int per = (int)std::max(1ll, std::min(4ll, (long long)cells * nquad / nt / (32 * std::max(1, c->nsm))));
+        const int ny = (nquad + nt * per - 1) / (nt * per);
+        Micro32P<D, NA> P;
+        P.Nv = c->Nv;
+        P.Nvp = c->Nvp;
+        P.chunk = (nquad + ny - 1) / ny * 4;
+        P.c0 = c->cstart[col];
+        P.below = seen[col] ? c->ncolor : col;     // the first forward sweep visits the colours in order
+        P.finish = last[col] == p;
+        P.keep = p + 1 < (int)seq.size();
+        P.fin = (const float*)fin;
+        P.fout = (float*)fout;
+        P.dphi = (float*)c->flux;                  // the face flux has been used
+        P.geo = (const float4*)c->geo32;
+        P.par = diag ? nullptr : (const Cell32Par*)c->cpar;
+        P.diag = diag;
+        P.xs = c->xi_s;
+        P.xstride = c->xstride;
+        P.nbr = c->nbr;
+        P.clist = c->clist;
+        P.colour = c->colour;
+        seen[col] = 1;
+        if (D == 2 && c->max_ns <= 4) k_micro32<D, 4, NA><<<dim3(cells, ny), nt, 0, c->stream>>>(P);
+        else k_micro32<D, AVS_MAXS, NA><<<dim3(cells, ny), nt, 0, c->stream>>>(P);
+        c->launches += 1;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_micro32(avs_ctx* c, const void* fin, void* fout, const double* diag, int k_micro)
+{
+    if (c->model == AVS_RYKOV)
+        return c->D == 2 ? micro32_t<2, 3>(c, fin, fout, diag, k_micro) : micro32_t<3, 2>(c, fin, fout, diag, k_micro);
+    return c->D == 2 ? micro32_t<2, 2>(c, fin, fout, diag, k_micro) : micro32_t<3, 1>(c, fin, fout, diag, k_micro);
 }
 
 }  // namespace avs
