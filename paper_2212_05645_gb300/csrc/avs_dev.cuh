@@ -685,6 +685,30 @@ __host__ __device__ inline double dkey_inv(unsigned long long k)
     return x;
 }
 
+// Upwind choice of a node where its FP32 normal velocity cannot tell: xi . An
+// summed in FP64 without contraction, >= 0 for the face's L cell, < 0 for its R
+// cell.  Out of line: inlined, its FP64 instructions are issued predicated off
+// at every node and still occupy the scarce FP64 pipe.
+template <int D>
+__device__ __noinline__ bool upwind_exact(const double* __restrict__ x, const double* __restrict__ a, bool isR)
+{
+    double s = dadd(dmul(x[0], a[0]), dmul(x[1], a[1]));
+    if (D == 3) s = dadd(s, dmul(x[2], a[2]));
+    return isR ? s < 0.0 : s >= 0.0;
+}
+
+// Whether the sign of sn, the FP32 sum of x_d n_d by fused multiply-adds from the
+// FP32 roundings of xi and An, is that of the FP64 sum:
+// |sn - xi . An| <= 5 * 2^-24 sum |xi_d An_d| while normal.
+template <int D>
+__device__ __forceinline__ bool upwind_sure(const float* x, const float* n, float sn)
+{
+    float sa = 0.0f;
+#pragma unroll
+    for (int d = 0; d < D; ++d) sa = fmaf(fabsf(x[d]), fabsf(n[d]), sa);
+    return fabsf(sn) > fmaf(sa, 0x1p-20f, 0x1p-100f) && sa < INFINITY;
+}
+
 // A row of N values that other blocks may have written before the last grid
 // barrier (read past L1): vectors of 16 bytes where the row is made of them.
 template <int N, typename A>

@@ -15,7 +15,7 @@
 
 #include "avs_dev.cuh"
 #include "avs_internal.h"
-#include "avs_step32.h"
+#include "avs_step32.cuh"
 
 namespace avs {
 namespace {
@@ -637,293 +637,6 @@ __device__ __forceinline__ float rk_tau32(const RkGas& g, float rho, float RTt)
     return (float)g.mu_ref * powa(T / (float)g.T_ref, (float)g.omega) / (rho * RTt);
 }
 
-// The FP64 upwind decision (the oracle's) for the nodes inside the FP32
-// rounding bound.  Not inlined: inlined, the compiler predicates it into every
-// node's instruction stream, and an FP64 instruction issued with its predicate
-// off still occupies the scarce FP64 pipe (out of line, the face kernel's FP64
-// pipe went from 52 % to 4 % busy and the kernel ran 12 % faster).
-template <int D>
-__device__ __noinline__ bool rk_upwind_exact(const double* __restrict__ xi, int k, const double* An)
-{
-    double xd[3] = {0, 0, 0};
-    for (int d = 0; d < D; ++d) xd[d] = xi[(size_t)k * D + d];
-    return dot_rn<D>(xd, An) >= 0.0;
-}
-
-// Upwind side of a node: xi . A n >= 0 decided in FP32 when the FP32 sum is
-// farther from zero than its rounding bound, else in FP64 without
-// contraction, so the decision always equals the FP64 one.
-template <int D>
-__device__ __forceinline__ bool rk_upwind_L(const float* x, const float* Af, const double* __restrict__ xi, int k,
-                                            const double* An, float& s)
-{
-    float a = 0.0f;
-    s = 0.0f;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        const float p = __fmul_rn(x[d], Af[d]);
-        s = __fadd_rn(s, p);
-        a += fabsf(p);
-    }
-    if (fabsf(s) > a * 0x1p-20f) return s >= 0.0f;
-    return rk_upwind_exact<D>(xi, k, An);
-}
-
-// rk_face for the FP32 form (same steps; sums as above).
-template <int D>
-__global__ void __launch_bounds__(RK_NT, D == 2 ? 8 : 7) rk_face32(RkP<float> P, const float* __restrict__ xif,
-                                                   const float* __restrict__ wf, const float* __restrict__ Anf,
-                                                   const float* __restrict__ rLf, const float* __restrict__ rRf)
-{
-    using T = float;
-    constexpr int NA = RkNA<D>::v, NW = D + 3, NR = RkNR<D>::v;
-    __shared__ double sw[(RK_NT / 32) * RkNR<3>::v], sout[RkNR<3>::v];
-    __shared__ RkEq<T> eq;
-    __shared__ float blend[2];
-    // per-face constants, converted from FP64 once by thread 0 (an FP64
-    // conversion or division in every thread costs as much as the node work)
-    __shared__ float cAf[3], crl[3], crr[3], cV[3], cUb[3], cpw, ci2b, ch;
-    __shared__ double An[3], Vd[3], cRTb, crb;
-    __shared__ int cbt;
-    const int f = P.order[blockIdx.x];
-    const int L = P.faceL[f], R = P.faceR[f];
-    const int Nv = P.Nv, Nvp = P.Nvp;
-    if (threadIdx.x == 0) {
-        for (int d = 0; d < 3; ++d) {
-            An[d] = d < D ? P.An[(size_t)f * D + d] : 0.0;
-            cAf[d] = d < D ? Anf[(size_t)f * D + d] : 0.0f;
-            crl[d] = d < D ? rLf[(size_t)f * D + d] : 0.0f;
-            crr[d] = d < D && R >= 0 ? rRf[(size_t)f * D + d] : 0.0f;
-        }
-        int btype = 0;
-        double rb = 0.0, Ub[3] = {0, 0, 0}, RTb = 1.0;
-        if (R < 0) {
-            const double* B = P.bc + (size_t)(-1 - R) * 6;
-            btype = (int)B[0];
-            rb = B[1];
-            for (int d = 0; d < 3; ++d) Ub[d] = B[2 + d];
-            RTb = P.g.R * B[5];
-        }
-        cbt = btype;
-        crb = rb;
-        cRTb = RTb;
-        // reference velocity of the sums: the left cell's mean velocity in
-        // FP32 (any V gives the same moments; Vd is its exact FP64 value)
-        const double* WL = P.Win + (size_t)L * NW;
-        const float irL = 1.0f / (float)WL[0];
-        for (int d = 0; d < 3; ++d) {
-            cV[d] = d < D ? (float)WL[1 + d] * irL : 0.0f;
-            Vd[d] = (double)cV[d];
-            cUb[d] = (float)Ub[d];
-        }
-        // wall Maxwellian prefactor (2 pi RT_w)^(-D/2) and 1/(2 RT_w) in FP32
-        const float xb = 2.0f * (float)AVS_PI * (float)RTb;
-        cpw = D == 2 ? 1.0f / xb : 1.0f / (xb * sqrtf(xb));
-        ci2b = 0.5f / (float)RTb;
-        ch = (float)P.h;
-    }
-    __syncthreads();
-    T Af[D], rl[D], rr[D], V[D], Ubf[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        Af[d] = cAf[d];
-        rl[d] = crl[d];
-        rr[d] = crr[d];
-        V[d] = cV[d];
-        Ubf[d] = cUb[d];
-    }
-    const int btype = cbt;
-    const T pw = cpw, i2b = ci2b;
-    T* fx = P.FX + (size_t)f * NA * Nvp;
-    const size_t cs = (size_t)NA * Nvp;
-    const T h = ch;
-    T racc[NR], wacc[2] = {T(0), T(0)};
-#pragma unroll
-    for (int m = 0; m < NR; ++m) racc[m] = T(0);
-    // pass A: foot values and their raw moments (or the wall balance); the
-    // interior and boundary loops are separate so that neither carries the
-    // other's instructions predicated off
-    const int Rc = R >= 0 ? R : L;
-    const float* fLp = P.f + (size_t)L * cs;
-    const float* fRp = P.f + (size_t)Rc * cs;
-    const float* gLp = P.G ? P.G + (size_t)L * NA * D * Nvp : nullptr;
-    const float* gRp = P.G ? P.G + (size_t)Rc * NA * D * Nvp : nullptr;
-    if (R >= 0) {
-        for (int k = threadIdx.x; k < Nv; k += RK_NT) {
-            T x[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) x[d] = xif[(size_t)k * D + d];
-            T s;
-            const bool up = rk_upwind_L<D>(x, Af, P.xi, k, An, s);
-            const float* fb = (up ? fLp : fRp) + k;
-            T ph[NA];
-            if (gLp) {
-                const float* gb = (up ? gLp : gRp) + k;
-                T off[D];
-#pragma unroll
-                for (int d = 0; d < D; ++d) off[d] = (up ? rl[d] : rr[d]) - x[d] * h;
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    T v = fb[a * Nvp];
-#pragma unroll
-                    for (int d = 0; d < D; ++d) v += gb[(a * D + d) * Nvp] * off[d];
-                    ph[a] = v;
-                }
-            } else {
-#pragma unroll
-                for (int a = 0; a < NA; ++a) ph[a] = fb[a * Nvp];
-            }
-#pragma unroll
-            for (int a = 0; a < NA; ++a) fx[(size_t)a * Nvp + k] = ph[a];
-            const T wk = wf[k];
-            T c[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) c[d] = x[d] - V[d];
-            rk_raw_acc<D>(racc, c, wk * ph[0], D == 2 ? wk * ph[1] : T(0), wk * ph[NA - 1]);
-        }
-    } else {
-        for (int k = threadIdx.x; k < Nv; k += RK_NT) {
-            T x[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) x[d] = xif[(size_t)k * D + d];
-            T s;
-            const bool up = rk_upwind_L<D>(x, Af, P.xi, k, An, s);
-            T ph[NA];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) ph[a] = T(0);
-            if (up) {
-                T off[D];
-#pragma unroll
-                for (int d = 0; d < D; ++d) off[d] = rl[d] - x[d] * h;
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    T v = fLp[a * Nvp + k];
-                    if (gLp)
-#pragma unroll
-                        for (int d = 0; d < D; ++d) v += gLp[(a * D + d) * Nvp + k] * off[d];
-                    ph[a] = v;
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < NA; ++a) fx[(size_t)a * Nvp + k] = ph[a];
-            if (btype == AVS_BC_WALL) {
-                const T wk = wf[k];
-                if (up) {
-                    wacc[0] += wk * s * ph[0];
-                } else {
-                    T c2 = T(0);
-#pragma unroll
-                    for (int d = 0; d < D; ++d) c2 += (x[d] - Ubf[d]) * (x[d] - Ubf[d]);
-                    wacc[1] += wk * (-s) * (pw * ex(-c2 * i2b));
-                }
-            }
-        }
-    }
-    if (R >= 0) {
-        block_sum_t<NR, RK_NT>(racc, sw, sout);
-        if (threadIdx.x == 0) {
-            // the interface state in FP32 (as the monatomic mixed form): no FP64 pow or division here
-            float rho, Uu[3] = {0, 0, 0}, et, r0, qb[3] = {0, 0, 0}, qrb[3] = {0, 0, 0};
-            rk_state_raw32<D>(sout, Vd, rho, Uu, et, r0, qb, qrb);
-            float RTt = et / (1.5f * rho), RT = (et + r0) / (2.5f * rho);
-            if (!(rho > 0.0f) || !(RTt > 0.0f) || !(RT > 0.0f)) atomicOr(P.err, 1);
-            const float tau = rk_tau32(P.g, rho, RTt), hf = (float)P.h, Z = (float)P.g.Z;
-            const float az = hf / (Z * tau);
-            const float RTr = (r0 + az * rho * RT) / (1.0f + az) / rho;
-            RTt = (5.0f * RT - 2.0f * RTr) * (1.0f / 3.0f);
-            const float lt = 2.0f / 3.0f + (1.0f - (float)P.g.om0) / (3.0f * Z);
-            const float lr = 1.0f - (1.0f - (float)P.g.dl) * ((1.0f - 1.0f / Z) * RTr / RTt + (float)P.g.om1 / Z);
-            float qt[3] = {0, 0, 0}, qr[3] = {0, 0, 0};
-            for (int d = 0; d < D; ++d) {
-                qt[d] = tau * qb[d] / (tau + hf * lt);
-                qr[d] = tau * qrb[d] / (tau + hf * lr);
-            }
-            eq = rk_make32<D>(P.g, rho, Uu, RTt, RTr, qt, qr);
-            blend[0] = tau / (tau + hf);
-            blend[1] = hf / (tau + hf);
-        }
-    } else {
-        block_sum_t<2, RK_NT>(wacc, sw, sout);
-        if (threadIdx.x == 0) {
-            const double rho_b = btype == AVS_BC_WALL ? (sout[1] > 0.0 ? sout[0] / sout[1] : 0.0) : crb;
-            const double z[3] = {0, 0, 0};
-            const double* B = P.bc + (size_t)(-1 - R) * 6;
-            const double Ub[3] = {B[2], B[3], B[4]};
-            RkGas g0 = P.g;
-            g0.iz = 0.0;
-            eq = rk_make<D, T>(g0, rho_b, Ub, cRTb, cRTb, z, z);
-            blend[0] = 1.0;
-            blend[1] = 0.0;
-        }
-    }
-    __syncthreads();
-    // pass B: phi_ij, per-node flux (xi . A n) phi and its moments
-    const T wa = (T)blend[0], wb = (T)blend[1];
-    T af[NW];
-#pragma unroll
-    for (int m = 0; m < NW; ++m) af[m] = T(0);
-    // interior: phi = wa phi_bar + wb g at every node; boundary: the
-    // incoming nodes take g (wall or far-field Maxwellian)
-    const bool inter = R >= 0;
-    for (int k = threadIdx.x; k < Nv; k += RK_NT) {
-        T x[D], x2 = T(0);
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            x[d] = xif[(size_t)k * D + d];
-            x2 += x[d] * x[d];
-        }
-        T s;
-        const bool up = rk_upwind_L<D>(x, Af, P.xi, k, An, s);
-        T ph[NA];
-#pragma unroll
-        for (int a = 0; a < NA; ++a) ph[a] = fx[(size_t)a * Nvp + k];
-        if (inter) {
-            T gv[NA];
-            rk_eval<D, T>(eq, x, gv);
-#pragma unroll
-            for (int a = 0; a < NA; ++a) ph[a] = wa * ph[a] + wb * gv[a];
-        } else if (!up) {
-            T gv[NA];
-            rk_eval<D, T>(eq, x, gv);
-#pragma unroll
-            for (int a = 0; a < NA; ++a) ph[a] = gv[a];
-        }
-        T F[NA];
-#pragma unroll
-        for (int a = 0; a < NA; ++a) {
-            F[a] = s * ph[a];
-            fx[(size_t)a * Nvp + k] = F[a];
-        }
-        const T wk = wf[k];
-        af[0] += wk * F[0];
-#pragma unroll
-        for (int d = 0; d < D; ++d) af[1 + d] += wk * x[d] * F[0];
-        af[D + 1] += wk * (T(0.5) * (x2 * F[0] + (D == 2 ? F[1] : T(0))) + F[NA - 1]);
-        af[D + 2] += wk * F[NA - 1];
-    }
-    block_sum_t<NW, RK_NT>(af, sw, sout);
-    if (threadIdx.x < NW) P.AF[(size_t)f * NW + threadIdx.x] = sout[threadIdx.x];
-}
-
-// ---------------------------------------------------------------- mixed-form cell stage
-// As the monatomic mixed form: the raw moments of f^{n+1} that the next step
-// needs for its lagged heat fluxes are summed while f^{n+1} is written and
-// carried per cell ([cell][NR] FP64, about V(W^{n+1})); all per-cell FP64
-// work (the balance of W, the rotational relaxation) runs one thread per
-// cell in rk_cell_state32; the cell kernel streams f, the face fluxes and
-// f^{n+1} RK_VC nodes per thread in vector loads.
-
-// Per-cell parameters of the Rykov collision update (mixed form).
-struct RkCellPar {
-    RkEq<float> eq;          // Rykov equilibrium of (W~ with relaxed E_rot, q~)
-    float upd[4];            // 1/dt, 1/tau~, 1/|V|, 1/(1/dt + 1/tau~)
-    float Vn[3];             // reference velocity of the next raw moments: V(W^{n+1})
-};
-static_assert(sizeof(RkCellPar) <= AVS_CELLPAR_BYTES, "RkCellPar buffer size");
-static_assert(RkNR<3>::v <= AVS_CMOM_MAX, "carried moments buffer size");
-
-constexpr int RK_VC = 2;     // nodes per thread per iteration of the cell kernels (2 or 4)
-
 // Reference velocity of the raw sums of a cell from a carried W (FP32; the
 // same expression wherever carried moments are taken or used).
 template <int D>
@@ -933,6 +646,135 @@ __device__ __forceinline__ void rk_vref(const double* W, float* V)
 #pragma unroll
     for (int d = 0; d < 3; ++d) V[d] = d < D ? (float)W[1 + d] * ir : 0.0f;
 }
+
+// The Rykov equilibrium of one state for node pairs: with c = xi - U, the
+// Maxwellians e_t = At 2^(kt c^2) and e_r = Ar 2^(kr c^2) at T_t and T, their
+// heat-flux factors in c . at and c . bt (the ones at T are ra and rb times
+// those at T_t), and scale s of the whole: At = s (1 - 1/Z) rho / (2 pi R T_t)^(D/2),
+// Ar = s / Z rho / (2 pi R T)^(D/2).
+struct RkEq2 {
+    float U[3], kt;
+    float at[3], kr;
+    float bt[3], ra;
+    float rb, At, Ar, RTt;
+    float RTr, RT;
+};
+template <int D>
+__device__ __forceinline__ RkEq2 rk_make2(const RkGas& g, float s, float rho, const float* U, float RTt, float RTr,
+                                          const float* qt, const float* qr)
+{
+    const RkEq<float> e = rk_make32<D>(g, rho, U, RTt, RTr, qt, qr);
+    const float z = RTt / e.RT, zz = z * z;
+    RkEq2 r;
+    for (int d = 0; d < 3; ++d) {
+        r.U[d] = e.U[d];
+        r.at[d] = e.at[d];
+        r.bt[d] = e.bt[d];
+    }
+    r.kt = (float)(-0.5 * kLog2e) * e.iRTt;
+    r.kr = (float)(-0.5 * kLog2e) * e.iRT;
+    r.ra = (float)g.om0 * zz;
+    r.rb = (float)g.om1 * zz;
+    r.At = s * ((1.0f - e.iz) * e.pt);
+    r.Ar = s * (e.iz * e.pr);
+    r.RTt = RTt;
+    r.RTr = RTr;
+    r.RT = e.RT;
+    return r;
+}
+template <int D>
+__device__ __forceinline__ void rk_eval2(const RkEq2& e, const float2* x, float2* out)
+{
+    float2 c = add2(x[0], bc2(-e.U[0])), c2 = mul2(c, c), cat = mul2(c, bc2(e.at[0])), cbt = mul2(c, bc2(e.bt[0]));
+#pragma unroll
+    for (int d = 1; d < D; ++d) {
+        c = add2(x[d], bc2(-e.U[d]));
+        c2 = fma2(c, c, c2);
+        cat = fma2(c, bc2(e.at[d]), cat);
+        cbt = fma2(c, bc2(e.bt[d]), cbt);
+    }
+    // c^2 / R T = -2 ln 2 k c^2
+    const float2 ut = mul2(c2, bc2(e.kt)), ur = mul2(c2, bc2(e.kr));
+    const float2 gt = mul2(bc2(e.At), make_float2(ex2_approx(ut.x), ex2_approx(ut.y)));
+    const float2 gr = mul2(bc2(e.Ar), make_float2(ex2_approx(ur.x), ex2_approx(ur.y)));
+    const float2 car = mul2(cat, bc2(e.ra)), cbr = mul2(cbt, bc2(e.rb));
+    const float2 pt = fma2(cat, fma2(ut, bc2(-kTwoLn2), bc2(-(float)(D + 2))), bc2(1.0f));
+    const float2 pr = fma2(car, fma2(ur, bc2(-kTwoLn2), bc2(-(float)(D + 2))), bc2(1.0f));
+    const float2 Gt = mul2(gt, pt), Gr = mul2(gr, pr);
+    out[0] = add2(Gt, Gr);
+    if constexpr (D == 2)
+        out[1] = fma2(mul2(bc2(e.RTt), gt), fma2(bc2(2.0f), cat, pt),
+                      mul2(mul2(bc2(e.RT), gr), fma2(bc2(2.0f), car, pr)));
+    out[RkNA<D>::v - 1] = fma2(bc2(e.RTr), fma2(cbt, gt, Gt), mul2(bc2(e.RT), fma2(cbr, gr, Gr)));
+}
+
+// Rykov gas of the FP32 face and cell kernels (avs_step32.cuh): the upwind choice
+// is the FP64 one, as the plain FP64 code takes it.
+template <int D_>
+struct Rykov {
+    static constexpr int D = D_, NA = RkNA<D>::v, NM = RkNR<D>::v, NW = D + 3;
+    static constexpr bool ROT = true, EXACT = true;
+    using Consts = RkGas;
+    struct Eq {
+        RkEq2 e;                 // scaled with h / (tau + h)
+        float wa;
+    };
+    // collision update out = (u0 f + u1 g + un N) u3, V the reference velocity of the next raw moments
+    struct Par : RkEq2 {
+        float u0, u1, un, u3, V[3];
+    };
+
+    // interface state (reading R27) in FP32 from a face's raw moments about V
+    static __device__ __forceinline__ Eq face_eq(const Consts& g, double hd, const double* red, const double* Vd, int* err)
+    {
+        float rho, U[3] = {0, 0, 0}, et, r0, qb[3] = {0, 0, 0}, qrb[3] = {0, 0, 0};
+        rk_state_raw32<D>(red, Vd, rho, U, et, r0, qb, qrb);
+        float RTt = et / (1.5f * rho), RT = (et + r0) / (2.5f * rho);
+        if (!(rho > 0.0f) || !(RTt > 0.0f) || !(RT > 0.0f)) atomicOr(err, 1);
+        const float tau = rk_tau32(g, rho, RTt), hf = (float)hd, Z = (float)g.Z;
+        const float az = hf / (Z * tau);
+        const float RTr = (r0 + az * rho * RT) / (1.0f + az) / rho;
+        RTt = (5.0f * RT - 2.0f * RTr) * (1.0f / 3.0f);
+        const float lt = 2.0f / 3.0f + (1.0f - (float)g.om0) / (3.0f * Z);
+        const float lr = 1.0f - (1.0f - (float)g.dl) * ((1.0f - 1.0f / Z) * RTr / RTt + (float)g.om1 / Z);
+        float qt[3] = {0, 0, 0}, qr[3] = {0, 0, 0};
+        for (int d = 0; d < D; ++d) {
+            qt[d] = tau * qb[d] / (tau + hf * lt);
+            qr[d] = tau * qrb[d] / (tau + hf * lr);
+        }
+        Eq q;
+        q.e = rk_make2<D>(g, hf / (tau + hf), rho, U, RTt, RTr, qt, qr);
+        q.wa = tau / (tau + hf);
+        return q;
+    }
+    static __device__ __forceinline__ void face_phi(const Eq& e, const float2* x, const float2* F, float2* phi)
+    {
+        float2 g[NA];
+        rk_eval2<D>(e.e, x, g);
+#pragma unroll
+        for (int a = 0; a < NA; ++a) phi[a] = fma2(bc2(e.wa), F[a], g[a]);
+    }
+    static __device__ __forceinline__ void cell_eq(const Par& c, const float2* x, float2* g) { rk_eval2<D>(c, x, g); }
+    static __device__ __forceinline__ float vref(const double* W, int d)
+    {
+        float V[3];
+        rk_vref<D>(W, V);
+        return V[d];
+    }
+};
+
+// ---------------------------------------------------------------- mixed-form cell stage
+// As the monatomic mixed form: the raw moments of f^{n+1} that the next step
+// needs for its lagged heat fluxes are summed while f^{n+1} is written and
+// carried per cell ([cell][NR] FP64, about V(W^{n+1})); all per-cell FP64
+// work (the balance of W, the rotational relaxation) runs one thread per
+// cell in rk_cell_state32; the cell kernel streams f, the face fluxes and
+// f^{n+1} RK_VC nodes per thread in vector loads.
+
+static_assert(sizeof(Rykov<3>::Par) <= AVS_CELLPAR_BYTES, "cell parameter buffer");
+static_assert(RkNR<3>::v <= AVS_CMOM_MAX, "carried moments buffer size");
+
+constexpr int RK_VC = 2;     // nodes per thread per iteration of the cell kernels (2 or 4)
 
 // V = RK_VC consecutive nodes of an FP32 row in one vector load (L2 only).
 __device__ __forceinline__ void rk_ldv(const float* p, float* o)
@@ -948,14 +790,6 @@ __device__ __forceinline__ void rk_ldv(const float* p, float* o)
         o[0] = t.x;
         o[1] = t.y;
     }
-}
-
-__device__ __forceinline__ void rk_stv(float* p, const float* o)
-{
-    if constexpr (RK_VC == 4)
-        *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
-    else
-        *reinterpret_cast<float2*>(p) = make_float2(o[0], o[1]);
 }
 
 // xi (D per node) and w of the RK_VC nodes from k0 (rows padded to 32 nodes;
@@ -984,46 +818,11 @@ __device__ __forceinline__ void rk_ld_nodes(const float* __restrict__ xif, const
     }
 }
 
-// Raw moments of the own f^n of every cell about V(W^n), when the previous
-// step did not leave them (after init, set_f, an adaptation or an implicit
-// step).  Same nodes per thread and order as rk_cell32, so the sums are the
-// carried ones bit for bit.
-template <int D>
-__global__ void __launch_bounds__(RK_NT) rk_raw_moments32(RkP<float> P, const float* __restrict__ xif,
-                                                          const float* __restrict__ wf, double* mom)
-{
-    constexpr int NA = RkNA<D>::v, NW = D + 3, NR = RkNR<D>::v;
-    __shared__ double sw[(RK_NT / 32) * NR], red[NR];
-    const int i = blockIdx.x;
-    const int Nvp = P.Nvp;
-    float V[3];
-    rk_vref<D>(P.Win + (size_t)i * NW, V);
-    const float* fi = P.f + (size_t)i * NA * Nvp;
-    float acc[NR];
-#pragma unroll
-    for (int m = 0; m < NR; ++m) acc[m] = 0.0f;
-    for (int k0 = threadIdx.x * RK_VC; k0 < P.Nv; k0 += RK_NT * RK_VC) {
-        float x[RK_VC][D], wv[RK_VC], fv[NA][RK_VC];
-        rk_ld_nodes<D>(xif, wf, k0, x, wv);
-#pragma unroll
-        for (int a = 0; a < NA; ++a) rk_ldv(fi + (size_t)a * Nvp + k0, fv[a]);
-#pragma unroll
-        for (int v = 0; v < RK_VC; ++v) {
-            float c[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) c[d] = x[v][d] - V[d];
-            rk_raw_acc<D>(acc, c, wv[v] * fv[0][v], D == 2 ? wv[v] * fv[1][v] : 0.0f, wv[v] * fv[NA - 1][v]);
-        }
-    }
-    block_sum_t<NR, RK_NT>(acc, sw, red);
-    if (threadIdx.x < NR) mom[(size_t)i * NR + threadIdx.x] = red[threadIdx.x];
-}
-
 // One thread per cell: lagged q_t, q_r of f^n from its carried moments,
 // W~ = W - dt/|V| sum_j sgn_j A F_j (FP64), the implicit rotational relaxation
 // of E_rot over dt with tau~ (reading R28), and the collision parameters.
 template <int D>
-__global__ void rk_cell_state32(RkP<float> P, const double* __restrict__ mom, RkCellPar* par)
+__global__ void rk_cell_state32(RkP<float> P, const double* __restrict__ mom, typename Rykov<D>::Par* par)
 {
     constexpr int NW = D + 3, NR = RkNR<D>::v;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1061,98 +860,16 @@ __global__ void rk_cell_state32(RkP<float> P, const double* __restrict__ mom, Rk
     Wt[D + 2] = (Wt[D + 2] + az * rho * RT) / (1.0 + az);
     const double RTr = Wt[D + 2] * ir;
     for (int c = 0; c < NW; ++c) P.Wout[(size_t)i * NW + c] = Wt[c];
-    RkCellPar cp;
-    cp.eq = rk_make32<D>(P.g, (float)rho, U, (float)((5.0 * RT - 2.0 * RTr) * (1.0 / 3.0)), (float)RTr, qt, qr);
-    const float dtf = (float)P.dt, idt = 1.0f / dtf, itau = 1.0f / tau;
-    cp.upd[0] = idt;
-    cp.upd[1] = itau;
-    cp.upd[2] = 1.0f / (float)P.vol[i];
-    cp.upd[3] = dtf * tau / (dtf + tau);
-    rk_vref<D>(Wt, cp.Vn);
+    typename Rykov<D>::Par cp;
+    static_cast<RkEq2&>(cp) = rk_make2<D>(P.g, 1.0f, (float)rho, U, (float)((5.0 * RT - 2.0 * RTr) * (1.0 / 3.0)),
+                                          (float)RTr, qt, qr);
+    const float dtf = (float)P.dt;
+    cp.u0 = 1.0f / dtf;
+    cp.u1 = 1.0f / tau;
+    cp.un = -1.0f / (float)P.vol[i];
+    cp.u3 = dtf * tau / (dtf + tau);
+    rk_vref<D>(Wt, cp.V);
     par[i] = cp;
-}
-
-// One block per cell: net flux N = sum_j sgn_j F_j per node, the collision
-// update (Eq. SGS_phi's diagonal, R1) with the Rykov equilibrium, pad nodes
-// written as zero, and the raw moments of f^{n+1} about V(W^{n+1}) for the
-// next step.
-template <int D>
-__global__ void __launch_bounds__(RK_NT, 7) rk_cell32(RkP<float> P, const float* __restrict__ xif,
-                                                   const float* __restrict__ wf, double* mom,
-                                                   const RkCellPar* __restrict__ par)
-{
-    constexpr int NA = RkNA<D>::v, NR = RkNR<D>::v, V = RK_VC;
-    __shared__ double sw[(RK_NT / 32) * NR], red[NR];
-    __shared__ RkCellPar cp;
-    __shared__ int fs[AVS_MAXS];
-    __shared__ float sg[AVS_MAXS];
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x;
-    const int ns = P.nslot[i];
-    const int Nv = P.Nv, Nvp = P.Nvp;
-    if (tid < ns) {
-        const int sl = P.slot[i * AVS_MAXS + tid];
-        fs[tid] = sl >> 1;
-        sg[tid] = (sl & 1) ? -1.0f : 1.0f;
-    }
-    if (tid == 32) cp = par[i];
-    __syncthreads();
-    const size_t cs = (size_t)NA * Nvp;
-    const float* fi = P.f + (size_t)i * cs;
-    float* fo = P.fout + (size_t)i * cs;
-    const float u0 = cp.upd[0], u1 = cp.upd[1], u2 = cp.upd[2], u3 = cp.upd[3];
-    float Vn[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) Vn[d] = cp.Vn[d];
-    float acc[NR];
-#pragma unroll
-    for (int m = 0; m < NR; ++m) acc[m] = 0.0f;
-    for (int k0 = tid * V; k0 < Nv; k0 += RK_NT * V) {
-        float x[V][D], wv[V], fv[NA][V], Nn[NA][V];
-        rk_ld_nodes<D>(xif, wf, k0, x, wv);
-#pragma unroll
-        for (int a = 0; a < NA; ++a) {
-            rk_ldv(fi + (size_t)a * Nvp + k0, fv[a]);
-#pragma unroll
-            for (int v = 0; v < V; ++v) Nn[a][v] = 0.0f;
-        }
-#pragma unroll
-        for (int q = 0; q < AVS_MAXS; ++q) {
-            if (q >= ns) break;
-            const float* Fq = P.FX + (size_t)fs[q] * cs + k0;
-            const float g = sg[q];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                float t[V];
-                rk_ldv(Fq + (size_t)a * Nvp, t);
-#pragma unroll
-                for (int v = 0; v < V; ++v) Nn[a][v] += g * t[v];
-            }
-        }
-        float out[NA][V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            float gv[NA];
-            rk_eval<D, float>(cp.eq, x[v], gv);
-            const bool real = k0 + v < Nv;
-#pragma unroll
-            for (int a = 0; a < NA; ++a) out[a][v] = real ? (fv[a][v] * u0 + gv[a] * u1 - Nn[a][v] * u2) * u3 : 0.0f;
-            float c[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) c[d] = x[v][d] - Vn[d];
-            rk_raw_acc<D>(acc, c, wv[v] * out[0][v], D == 2 ? wv[v] * out[1][v] : 0.0f, wv[v] * out[NA - 1][v]);
-        }
-#pragma unroll
-        for (int a = 0; a < NA; ++a) rk_stv(fo + (size_t)a * Nvp + k0, out[a]);
-    }
-    // rows are padded to a multiple of 32 nodes and every thread's k0 is a
-    // multiple of V, so the loop above wrote every node below the first k0 >= Nv;
-    // the pad nodes from there to Nvp are zeroed here
-    for (int k = ((Nv + V - 1) / V) * V + tid; k < Nvp; k += RK_NT)
-#pragma unroll
-        for (int a = 0; a < NA; ++a) fo[(size_t)a * Nvp + k] = 0.0f;
-    block_sum_t<NR, RK_NT>(acc, sw, red);
-    if (tid < NR) mom[(size_t)i * NR + tid] = red[tid];
 }
 
 // W (and the total heat flux q_t + q_r) of every cell.
@@ -1487,111 +1204,36 @@ __global__ void __launch_bounds__(NT) rk_imp_macro(RkImpP<A> P, int k_macro, int
                     rk_imp_cell<D, A>(P, q);
             }
 }
-// rk_imp_res for the mixed form: the raw moments of f^n and the residual
-// RK_VC nodes per thread in vector loads (the cell kernel's layout), the
-// state of W~ by thread 0 (FP64 W~, FP32 tau~ and equilibrium).
+// Mixed form: the Rykov state of W~ with the lagged q_t, q_r of f^n (its raw
+// moments in mom), as the parameters of the residual V (g~ - phi^n) / tau~ - N,
+// and u0 = V/dt + V/tau~ for the sweeps.
 template <int D>
-__global__ void __launch_bounds__(RK_NT, 7) rk_imp_res32(RkP<float> P, const float* __restrict__ xif,
-                                                         const float* __restrict__ wf, double* u0)
+__global__ void rk_imp_state32(RkP<float> P, const double* __restrict__ mom, typename Rykov<D>::Par* par, double* u0)
 {
-    constexpr int NA = RkNA<D>::v, NW = D + 3, NR = RkNR<D>::v, V = RK_VC;
-    __shared__ double sw[(RK_NT / 32) * NR], red[NR];
-    __shared__ RkEq<float> eq;
-    __shared__ float ctau, cvol, cV[3];
-    __shared__ double Vd[3];
-    __shared__ int fs[AVS_MAXS];
-    __shared__ float sg[AVS_MAXS];
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x;
-    const int ns = P.nslot[i];
-    const int Nv = P.Nv, Nvp = P.Nvp;
-    if (tid < ns) {
-        const int sl = P.slot[i * AVS_MAXS + tid];
-        fs[tid] = sl >> 1;
-        sg[tid] = (sl & 1) ? -1.0f : 1.0f;
-    }
-    if (tid == 32) {
-        rk_vref<D>(P.Win + (size_t)i * NW, cV);
-        for (int d = 0; d < 3; ++d) Vd[d] = cV[d];
-        cvol = (float)P.vol[i];
-    }
-    __syncthreads();
-    const size_t cs = (size_t)NA * Nvp;
-    const float* fi = P.f + (size_t)i * cs;
-    float Vr[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) Vr[d] = cV[d];
-    float acc[NR];
-#pragma unroll
-    for (int m = 0; m < NR; ++m) acc[m] = 0.0f;
-    for (int k0 = tid * V; k0 < Nv; k0 += RK_NT * V) {
-        float x[V][D], wv[V], fv[NA][V];
-        rk_ld_nodes<D>(xif, wf, k0, x, wv);
-#pragma unroll
-        for (int a = 0; a < NA; ++a) rk_ldv(fi + (size_t)a * Nvp + k0, fv[a]);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            float c[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) c[d] = x[v][d] - Vr[d];
-            rk_raw_acc<D>(acc, c, wv[v] * fv[0][v], D == 2 ? wv[v] * fv[1][v] : 0.0f, wv[v] * fv[NA - 1][v]);
-        }
-    }
-    block_sum_t<NR, RK_NT>(acc, sw, red);
-    if (tid == 0) {
-        float rn, Un[3], etn, r0n, qt[3] = {0, 0, 0}, qr[3] = {0, 0, 0};
-        rk_state_raw32<D>(red, Vd, rn, Un, etn, r0n, qt, qr);
-        double rho, U[3], RTt, RTr, RT;
-        rk_prim<D>(P.Wout + (size_t)i * NW, rho, U, RTt, RTr, RT);
-        if (!(rho > 0.0) || !(RTt > 0.0) || !(RT > 0.0)) atomicOr(P.err, 1);
-        const float tau = rk_tau32(P.g, (float)rho, (float)RTt);
-        float Uf[3] = {0, 0, 0};
-        for (int d = 0; d < D; ++d) Uf[d] = (float)U[d];
-        eq = rk_make32<D>(P.g, (float)rho, Uf, (float)RTt, (float)RTr, qt, qr);
-        ctau = tau;
-        u0[i] = P.vol[i] / P.dt + P.vol[i] / (double)tau;
-    }
-    __syncthreads();
-    const float Vc = cvol, vit = cvol / ctau;
-    float* ro = P.fout + (size_t)i * cs;
-    for (int k0 = tid * V; k0 < Nv; k0 += RK_NT * V) {
-        float x[V][D], wv[V], fv[NA][V], Nn[NA][V];
-        rk_ld_nodes<D>(xif, wf, k0, x, wv);
-#pragma unroll
-        for (int a = 0; a < NA; ++a) {
-            rk_ldv(fi + (size_t)a * Nvp + k0, fv[a]);
-#pragma unroll
-            for (int v = 0; v < V; ++v) Nn[a][v] = 0.0f;
-        }
-#pragma unroll
-        for (int q = 0; q < AVS_MAXS; ++q) {
-            if (q >= ns) break;
-            const float* Fq = P.FX + (size_t)fs[q] * cs + k0;
-            const float g = sg[q];
-#pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                float t[V];
-                rk_ldv(Fq + (size_t)a * Nvp, t);
-#pragma unroll
-                for (int v = 0; v < V; ++v) Nn[a][v] += g * t[v];
-            }
-        }
-        float out[NA][V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            float gv[NA];
-            rk_eval<D, float>(eq, x[v], gv);
-            const bool real = k0 + v < Nv;
-#pragma unroll
-            for (int a = 0; a < NA; ++a) out[a][v] = real ? (gv[a] - fv[a][v]) * vit - Nn[a][v] : 0.0f;
-        }
-#pragma unroll
-        for (int a = 0; a < NA; ++a) rk_stv(ro + (size_t)a * Nvp + k0, out[a]);
-    }
-    for (int k = ((Nv + V - 1) / V) * V + tid; k < Nvp; k += RK_NT)
-#pragma unroll
-        for (int a = 0; a < NA; ++a) ro[(size_t)a * Nvp + k] = 0.0f;
-    (void)Vc;
+    constexpr int NW = D + 3, NR = RkNR<D>::v;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= P.Nc) return;
+    float V[3];
+    rk_vref<D>(P.Win + (size_t)i * NW, V);
+    const double Vd[3] = {V[0], V[1], V[2]};
+    float rn, Un[3], etn, r0n, qt[3] = {0, 0, 0}, qr[3] = {0, 0, 0};
+    rk_state_raw32<D>(mom + (size_t)i * NR, Vd, rn, Un, etn, r0n, qt, qr);
+    double rho, U[3], RTt, RTr, RT;
+    rk_prim<D>(P.Wout + (size_t)i * NW, rho, U, RTt, RTr, RT);
+    if (!(rho > 0.0) || !(RTt > 0.0) || !(RT > 0.0)) atomicOr(P.err, 1);
+    const float tau = rk_tau32(P.g, (float)rho, (float)RTt);
+    float Uf[3] = {0, 0, 0};
+    for (int d = 0; d < D; ++d) Uf[d] = (float)U[d];
+    typename Rykov<D>::Par cp;
+    static_cast<RkEq2&>(cp) = rk_make2<D>(P.g, 1.0f, (float)rho, Uf, (float)RTt, (float)RTr, qt, qr);
+    const float vit = (float)P.vol[i] / tau;
+    cp.u0 = -vit;
+    cp.u1 = vit;
+    cp.un = -1.0f;
+    cp.u3 = 1.0f;
+    for (int d = 0; d < 3; ++d) cp.V[d] = 0.0f;      // the residual carries no moments
+    par[i] = cp;
+    u0[i] = P.vol[i] / P.dt + P.vol[i] / (double)tau;
 }
 
 // Per cell: Rykov state of W~ with the lagged q_t, q_r of f^n, and the
@@ -1601,7 +1243,7 @@ template <int D, typename T>
 __global__ void __launch_bounds__(RK_NT) rk_imp_res(RkP<T> P, const T* __restrict__ xiT,
                                                     const T* __restrict__ wT, double* u0)
 {
-    static_assert(sizeof(T) == 8, "the mixed form uses rk_imp_res32");
+    static_assert(sizeof(T) == 8, "the mixed form uses k_cell32");
     constexpr int NA = RkNA<D>::v, NW = D + 3;
     __shared__ double sred[(RK_NT / 32) * RkNR<3>::v], sout[RkNR<3>::v];
     __shared__ RkEq<T> eq;
@@ -1746,7 +1388,7 @@ cudaError_t rk_face_stage(avs_ctx* c, const void* fin, const double* Win, double
 {
     constexpr int NA = RkNA<D>::v;
     const size_t rows = (size_t)std::max(c->fcap, c->Nvp);
-    const bool grad = c->cfg.limiter != 0;
+    const bool grad = c->cfg.limiter != 0 && sizeof(T) == 8;   // the FP32 form never stores gradients
     cudaError_t e;
     if (grad) {
         e = ensure_bytes(&c->grad, &c->grad_bytes, (size_t)c->Nc * NA * D * rows * sizeof(T));
@@ -1782,13 +1424,15 @@ cudaError_t rk_face_stage(avs_ctx* c, const void* fin, const double* Win, double
     P.Wout = nullptr;
     P.fout = nullptr;
     P.err = c->dev_err;
-    if (grad) launch_grad_rykov(c, fin);     // the monatomic gradient kernel over NA arrays
-    if constexpr (sizeof(T) == 4)
-        rk_face32<D><<<c->Nf, RK_NT, 0, c->stream>>>(P, c->xi_f, c->w_f, c->An_f, c->rL_f, c->rR_f);
-    else
+    if constexpr (sizeof(T) == 4) {
+        launch_foot32(c, fin, 0.5 * dt);
+        return face32_t<Rykov<D>>(c, Win, dt, P.g);
+    } else {
+        if (grad) launch_grad_rykov(c, fin);     // the monatomic gradient kernel over NA arrays
         rk_face<D, T><<<c->Nf, RK_NT, 0, c->stream>>>(P);
-    c->launches += 1;
-    return cudaGetLastError();
+        c->launches += 1;
+        return cudaGetLastError();
+    }
 }
 
 template <int D, typename T>
@@ -1800,14 +1444,13 @@ cudaError_t rk_step_t(avs_ctx* c, const void* fin, void* fout, const double* Win
     P.Wout = Wout;
     P.fout = (T*)fout;
     if constexpr (sizeof(T) == 4) {
-        RkCellPar* par = reinterpret_cast<RkCellPar*>(c->cpar);
-        if (!c->mom_valid) {
-            rk_raw_moments32<D><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_f, c->w_f, c->cmom);
-            c->launches += 1;
-        }
+        auto* par = reinterpret_cast<typename Rykov<D>::Par*>(c->cpar);
+        if (!c->mom_valid) e = raw32_t<Rykov<D>>(c, fin, Win);
+        if (e != cudaSuccess) return e;
         rk_cell_state32<D><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(P, c->cmom, par);
-        rk_cell32<D><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_f, c->w_f, c->cmom, par);
-        c->launches += 2;
+        c->launches += 1;
+        e = cell32_t<Rykov<D>, false>(c, fin, fout);
+        if (e != cudaSuccess) return e;
         c->mom_valid = 1;      // the raw moments of fout about V(Wout) are in cmom
     } else {
         rk_cell<D, T><<<c->Nc, RK_NT, 0, c->stream>>>(P);
@@ -1880,15 +1523,18 @@ cudaError_t rk_step_implicit_t(avs_ctx* c, const void* fin, void* fout, const do
     P.Wout = Wout;                      // W~
     P.fout = (T*)fout;                  // holds the residual until the finish
     double* u0 = c->imp_diag;           // the macroscopic diagonal is no longer needed
-    if constexpr (sizeof(T) == 4)
-        rk_imp_res32<D><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_f, c->w_f, u0);
-    else
-        rk_imp_res<D, T><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_d, c->w_d, u0);
-    c->launches += 1;
     if constexpr (sizeof(T) == 4) {
-        e = launch_micro32(c, fin, fout, u0, k_micro);
+        auto* par = reinterpret_cast<typename Rykov<D>::Par*>(c->cpar);
+        if (!c->mom_valid) e = raw32_t<Rykov<D>>(c, fin, Win);
+        if (e != cudaSuccess) return e;
+        rk_imp_state32<D><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(P, c->cmom, par, u0);
+        c->launches += 1;
+        e = cell32_t<Rykov<D>, true>(c, fin, fout);
+        if (e == cudaSuccess) e = launch_micro32(c, fin, fout, u0, k_micro);
         if (e != cudaSuccess) return e;
     } else {
+        rk_imp_res<D, T><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_d, c->w_d, u0);
+        c->launches += 1;
         T* dphi = (T*)c->flux;          // the face flux has been used
         e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);
         if (e != cudaSuccess) return e;

@@ -227,13 +227,6 @@ __device__ __forceinline__ void vec3(const float4& v, float (&o)[D])
 // per cell and node in 3D; per step 181 -> 99 us on the 32 x 32 cavity (298
 // nodes), 4.30 -> 2.24 ms on 1000 cells x 13824 nodes in 3D, where the pipe is
 // full.
-__device__ __noinline__ bool upwind_exact(int D, const double* __restrict__ x, const double* __restrict__ a, bool isR)
-{
-    double s = dadd(dmul(x[0], a[0]), dmul(x[1], a[1]));
-    if (D == 3) s = dadd(s, dmul(x[2], a[2]));
-    return isR ? s < 0.0 : s >= 0.0;
-}
-
 // Largest value of v[0..N-1] and 0, and smallest of them and 0, by integer
 // comparison: as signed integers the positive doubles order as their values
 // and negative ones lie below zero; as unsigned integers the negative ones
@@ -344,16 +337,14 @@ __global__ void __launch_bounds__(128) k_foot(int Nv, int Nvp, int chunk, int li
             bool up[VG];
 #pragma unroll
             for (int v = 0; v < VG; ++v) {
-                float sn = 0.0f, sa = 0.0f;
+                float xv[D], sn = 0.0f;
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
-                    const float xv = v ? x32[d].y : x32[d].x;
-                    sn = fmaf(xv, na[d], sn);
-                    sa = fmaf(fabsf(xv), fabsf(na[d]), sa);
+                    xv[d] = v ? x32[d].y : x32[d].x;
+                    sn = fmaf(xv[d], na[d], sn);
                 }
-                // |sn - xi . An| <= 5 * 2^-24 sum |xi_d An_d| while normal
-                if (fabsf(sn) > fmaf(sa, 0x1p-20f, 0x1p-100f) && sa < INFINITY) up[v] = sn > 0.0f;
-                else up[v] = upwind_exact(D, x[v], An + (size_t)fc * D, n4.w != 0.0f);
+                if (upwind_sure<D>(xv, na, sn)) up[v] = sn > 0.0f;
+                else up[v] = upwind_exact<D>(x[v], An + (size_t)fc * D, n4.w != 0.0f);
             }
             if (!up[0] && !up[1]) continue;
             double* row = FB + (size_t)fc * NA * Nvp + k0;
@@ -427,11 +418,15 @@ __device__ __forceinline__ float2 limit2(float2 dmax, float2 dmin, float2 pp, fl
 // Thread block (cell i, nodes of one chunk), the thread's quads one after the
 // other: the block's start (launch, geometry, barrier) is paid once for up to
 // four quads per thread.
-template <int D, int NS, int NA>
-__global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
+// EXACT: the upwind choice is the FP64 one; only a quad with a normal velocity
+// within one bound of zero recomputes it (a bound per node: 565 us for the Rykov
+// cylinder's 12288 cells x 3216 nodes, one per quad: 476).
+template <int D, int NS, int NA, bool EXACT>
+__global__ void __launch_bounds__(128, EXACT ? 6 : 8) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
                                                     const float* __restrict__ f, float* __restrict__ FB,
                                                     const float4* __restrict__ geo, const float* __restrict__ eps2,
-                                                    const float* __restrict__ xs, size_t xstride)
+                                                    const float* __restrict__ xs, size_t xstride,
+                                                    const double* __restrict__ xi, const double* __restrict__ An)
 {
     constexpr int VG = 4;
     __shared__ float4 gs[3 * NS];
@@ -504,6 +499,13 @@ __global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int chunk, 
             X[0][d] = lo2(v);
             X[1][d] = hi2(v);
         }
+        float xmax = 0.0f;
+        if constexpr (EXACT) {
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int d = 0; d < D; ++d) xmax = max3f(xmax, fabsf(X[p][d].x), fabsf(X[p][d].y));
+        }
         // phi_bar = A + G . r_s with A = phi - h G . xi, the part common to the faces
         float2 A[NA][2];
 #pragma unroll
@@ -523,6 +525,7 @@ __global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int chunk, 
             float rr[D];
             vec3<D>(r4, rr);
             bool up[4];
+            float near = INFINITY;
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 // xi . An as in k_foot: a product, then fused multiply-adds; the
@@ -533,6 +536,18 @@ __global__ void __launch_bounds__(128, 8) k_foot_f2(int Nv, int Nvp, int chunk, 
                 if constexpr (D == 3) sn = fma2(X[p][2], bc2(an.z), sn);
                 up[2 * p] = sn.x >= an.w;
                 up[2 * p + 1] = sn.y >= an.w;
+                if constexpr (EXACT) near = min3f(near, fabsf(sn.x), fabsf(sn.y));
+            }
+            if constexpr (EXACT) {
+                // one bound for the quad: 2^-20 max |xi| sum |An_d| is above every node's in upwind_sure
+                float na = fabsf(an.x) + fabsf(an.y);
+                if constexpr (D == 3) na += fabsf(an.z);
+                if (!(near > fmaf(xmax * 0x1p-20f, na, 0x1p-100f))) {
+#pragma unroll
+                    for (int z = 0; z < 4; ++z)
+                        if (k0 + z < Nv)
+                            up[z] = upwind_exact<D>(xi + (size_t)(k0 + z) * D, An + (size_t)fc * D, an.w != 0.0f);
+                }
             }
             const bool all = up[0] && up[1] && up[2] && up[3];
             const bool any = up[0] || up[1] || up[2] || up[3];
@@ -1319,82 +1334,6 @@ __global__ void __launch_bounds__(NT) k_cell_tab(CellP<D, double> P, const doubl
     if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
 }
 
-// k_grad for the FP32 form in packed two-lane arithmetic: four nodes per
-// thread as two pairs; the cell's geometry staged once per block in shared
-// memory; the gradient and limiter of k_foot_f2, stored as k_grad stores
-// them ([cell][array][D][Nvp]).  128-thread blocks, eight per SM.
-template <int D, int NS, int NA>
-__global__ void __launch_bounds__(128, 8) k_grad_f2(int Nv, int Nvp, int limiter, const float* __restrict__ f,
-                                                    float* __restrict__ Gout, const float4* __restrict__ geo,
-                                                    const float* __restrict__ eps2)
-{
-    constexpr int VG = 4;
-    __shared__ float4 gs[3 * NS];
-    const int i = blockIdx.x;
-    load_geo32<NS>(geo, i, gs);
-    const int k0 = (blockIdx.y * blockDim.x + threadIdx.x) * VG;
-    if (k0 >= Nv) return;
-    const size_t cstride = (size_t)NA * Nvp;
-    const float e2 = eps2[i];
-#pragma unroll
-    for (int a = 0; a < NA; ++a) {
-        const float* fa = f + (size_t)a * Nvp + k0;
-        const float4 c4 = __ldg(reinterpret_cast<const float4*>(fa + (size_t)i * cstride));
-        const float2 phi[2] = {lo2(c4), hi2(c4)};
-        float4 n4[NS];
-#pragma unroll
-        for (int s = 0; s < NS; ++s) n4[s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)__float_as_int(gs[3 * s].w) * cstride));
-        float2 G[D][2];
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float2 g[D], dd[NS];
-#pragma unroll
-            for (int d = 0; d < D; ++d) g[d] = bc2(0.0f);
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                float cg[D];
-                vec3<D>(gs[3 * s], cg);
-                dd[s] = sub2(p ? hi2(n4[s]) : lo2(n4[s]), phi[p]);
-#pragma unroll
-                for (int d = 0; d < D; ++d) g[d] = fma2(bc2(cg[d]), dd[s], g[d]);
-            }
-            float2 L = bc2(1.0f);
-            if (limiter == 1) {
-                float2 d2[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    float rr[D];
-                    vec3<D>(gs[3 * s + 1], rr);
-                    d2[s] = mul2(g[0], bc2(rr[0]));
-#pragma unroll
-                    for (int d = 1; d < D; ++d) d2[s] = fma2(g[d], bc2(rr[d]), d2[s]);
-                }
-                float dx[NS], dy[NS], ex[NS], ey[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    dx[s] = dd[s].x; dy[s] = dd[s].y;
-                    ex[s] = d2[s].x; ey[s] = d2[s].y;
-                }
-                float2 dmax, dmin, pp, nn;
-                ext4<NS>(dx, dmax.x, dmin.x);
-                ext4<NS>(dy, dmax.y, dmin.y);
-                ext4<NS>(ex, pp.x, nn.x);
-                ext4<NS>(ey, pp.y, nn.y);
-                // epsilon^2 = (K dx)^3 phi_C^2: scaled to the limited value (R6)
-                const float2 e2p = mul2(mul2(bc2(e2), phi[p]), phi[p]);
-                L = limit2(dmax, dmin, pp, nn, e2p);
-            }
-            if (limiter == 0) L = bc2(0.0f);
-#pragma unroll
-            for (int d = 0; d < D; ++d) G[d][p] = mul2(L, g[d]);
-        }
-        float* o = Gout + ((size_t)i * NA + a) * D * Nvp + k0;
-#pragma unroll
-        for (int d = 0; d < D; ++d)
-            *reinterpret_cast<float4*>(o + (size_t)d * Nvp) = make_float4(G[d][0].x, G[d][0].y, G[d][1].x, G[d][1].y);
-    }
-}
-
 // geometry of the FP64 kernels (the FP32 ones read geo32)
 template <typename T>
 static CellGeo<T> cell_geo(const avs_ctx* c)
@@ -1408,31 +1347,53 @@ static CellGeo<T> cell_geo(const avs_ctx* c)
     return geo;
 }
 
-// Limited gradients of every array of every cell into c->grad (allocated by the caller).
-template <int D, typename T, int NA>
+// Limited gradients of every array of every cell into c->grad (allocated by the
+// caller), FP64 form of the Rykov gas.
+template <int D, int NA>
 static void grad_t(avs_ctx* c, const void* fin)
 {
     constexpr int VG = 4;
-    if constexpr (sizeof(T) == 4) {
-        const dim3 g2(c->Nc, (c->Nv + 128 * VG - 1) / (128 * VG));
-        if (D == 2 && c->max_ns <= 4)
-            k_grad_f2<D, 4, NA><<<g2, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const float*)fin,
-                                                          (float*)c->grad, (const float4*)c->geo32, c->eps2_f);
-        else
-            k_grad_f2<D, AVS_MAXS, NA><<<g2, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const float*)fin,
-                                                                 (float*)c->grad, (const float4*)c->geo32,
-                                                                 c->eps2_f);
-        c->launches += 1;
-        return;
-    }
-    const CellGeo<T> geo = cell_geo<T>(c);
+    const CellGeo<double> geo = cell_geo<double>(c);
     dim3 g(c->Nc, (c->Nv + 256 * VG - 1) / (256 * VG));
     if (D == 2 && c->max_ns <= 4)
-        k_grad<D, T, VG, 4, NA><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const T*)fin, (T*)c->grad, geo);
+        k_grad<D, double, VG, 4, NA><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const double*)fin,
+                                                               (double*)c->grad, geo);
     else
-        k_grad<D, T, VG, AVS_MAXS, NA><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const T*)fin,
-                                                                  (T*)c->grad, geo);
+        k_grad<D, double, VG, AVS_MAXS, NA><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->cfg.limiter, (const double*)fin,
+                                                                      (double*)c->grad, geo);
     c->launches += 1;
+}
+
+// Foot values of the FP32 form into c->flux, either gas (the
+// Rykov form takes the FP64 upwind choice).
+template <int D, int NA, bool EXACT>
+static void foot32_t(avs_ctx* c, const void* fin, double hd)
+{
+    constexpr int VG = 4;
+    // 128 threads, or 64 where a row has no more quads (190 nodes,
+    // 12288 cells: 41 -> 25 us), with up to four quads per thread while
+    // that leaves 32 blocks per SM (21k nodes, 36864 cells: 5.41 ->
+    // 4.46 ms; chunks of 2048 nodes still let the rows of a cell's
+    // neighbours be reused from L2)
+    const int nquad = (c->Nv + VG - 1) / VG;
+    const int nt = nquad <= 64 ? 64 : 128;
+    const int per = (int)std::max(1ll, std::min(4ll, (long long)c->Nc * nquad / nt / (32 * std::max(1, c->nsm))));
+    const int ny = (nquad + nt * per - 1) / (nt * per);
+    const int chunk = (nquad + ny - 1) / ny * VG;
+    auto go = [&](auto ns) {
+        k_foot_f2<D, decltype(ns)::value, NA, EXACT><<<dim3(c->Nc, ny), nt, 0, c->stream>>>(
+            c->Nv, c->Nvp, chunk, c->cfg.limiter, (float)hd, (const float*)fin, (float*)c->flux, (const float4*)c->geo32,
+            c->eps2_f, c->xi_s, c->xstride, c->xi_d, c->An_d);
+    };
+    if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
+    else go(std::integral_constant<int, AVS_MAXS>{});
+    c->launches += 1;
+}
+
+void launch_foot32(avs_ctx* c, const void* fin, double hd)
+{
+    if (c->model == AVS_RYKOV) c->D == 2 ? foot32_t<2, 3, true>(c, fin, hd) : foot32_t<3, 2, true>(c, fin, hd);
+    else c->D == 2 ? foot32_t<2, 2, false>(c, fin, hd) : foot32_t<3, 1, false>(c, fin, hd);
 }
 
 // Tables of the axes' coordinates pay where a face's or cell's nodes are at
@@ -1467,25 +1428,8 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
     const T* An = f32 ? (const T*)c->An_f : (const T*)c->An_d;
     const double hd = 0.5 * dt;
     {
-        constexpr int VG = 4;
         if constexpr (sizeof(T) == 4) {
-            // 128 threads, or 64 where a row has no more quads (190 nodes,
-            // 12288 cells: 41 -> 25 us), with up to four quads per thread while
-            // that leaves 32 blocks per SM (21k nodes, 36864 cells: 5.41 ->
-            // 4.46 ms; chunks of 2048 nodes still let the rows of a cell's
-            // neighbours be reused from L2)
-            const int nquad = (c->Nv + VG - 1) / VG;
-            const int nt = nquad <= 64 ? 64 : 128;
-            const int per = (int)std::max(1ll, std::min(4ll, (long long)c->Nc * nquad / nt / (32 * std::max(1, c->nsm))));
-            const int ny = (nquad + nt * per - 1) / (nt * per);
-            const int chunk = (nquad + ny - 1) / ny * VG;
-            auto go = [&](auto ns) {
-                k_foot_f2<D, decltype(ns)::value, NArr<D>::v><<<dim3(c->Nc, ny), nt, 0, c->stream>>>(
-                    c->Nv, c->Nvp, chunk, c->cfg.limiter, (float)hd, (const float*)fin, (float*)c->flux,
-                    (const float4*)c->geo32, c->eps2_f, c->xi_s, c->xstride);
-            };
-            if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
-            else go(std::integral_constant<int, AVS_MAXS>{});
+            launch_foot32(c, fin, hd);
         } else {
             const CellGeo<T> geo = cell_geo<T>(c);
             // two nodes per thread and iteration; 64 threads for short rows, up
@@ -2275,13 +2219,7 @@ cudaError_t launch_step_implicit(avs_ctx* c, const void* fin, void* fout, const 
 
 void launch_grad_rykov(avs_ctx* c, const void* fin)
 {
-    if (c->D == 2) {
-        if (c->mixed) grad_t<2, float, 3>(c, fin);
-        else grad_t<2, double, 3>(c, fin);
-    } else {
-        if (c->mixed) grad_t<3, float, 2>(c, fin);
-        else grad_t<3, double, 2>(c, fin);
-    }
+    c->D == 2 ? grad_t<2, 3>(c, fin) : grad_t<3, 2>(c, fin);
 }
 
 cudaError_t launch_face_stage(avs_ctx* c, const void* fin, const double* Win, double dt)

@@ -17,10 +17,13 @@ struct alignas(16) Cell32Par {
 };
 static_assert(sizeof(Cell32Par) <= AVS_CELLPAR_BYTES, "cell parameter buffer");
 
+// foot values of every face into c->flux, either gas; hd = dt / 2
+void launch_foot32(avs_ctx* c, const void* fin, double hd);
+// the monatomic gas
 cudaError_t launch_face32(avs_ctx* c, const double* Win, double dt);
 cudaError_t launch_cell32(avs_ctx* c, const void* fin, void* fout, bool residual);
-// diag: per cell, or nullptr for the one in the cells' records
-cudaError_t launch_micro32(avs_ctx* c, const void* fin, void* fout, const double* diag, int k_micro);
 cudaError_t launch_raw32(avs_ctx* c, const void* fin, const double* W);
+// either gas; diag: per cell, or nullptr for the one in the cells' records (monatomic)
+cudaError_t launch_micro32(avs_ctx* c, const void* fin, void* fout, const double* diag, int k_micro);
 
 }  // namespace avs
