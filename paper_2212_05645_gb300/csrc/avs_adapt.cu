@@ -484,8 +484,12 @@ template <int D, typename T>
 static cudaError_t cell_moments_t(avs_ctx* c, const T* f, const T* xi, const T* w, int Ncells, int Nvp,
                                   const double* Wref, double* Wc, double* q)
 {
-    k_cell_moments<D, T, 128><<<Ncells, 128, 0, c->stream>>>(c->Nv, Nvp, f, xi, w, Wref, c->rmom);
-    k_moments_finish<D, T><<<(Ncells + 127) / 128, 128, 0, c->stream>>>(Ncells, c->rmom, Wref, Wc, q);
+    // one warp per cell for short rows, where the sums over the threads, in
+    // FP64, are most of the work (12288 cells, 190 nodes: 131 us with 128
+    // threads, 36 with 32)
+    if (c->Nv <= 512) k_cell_moments<D, T, 32><<<Ncells, 32, 0, c->stream>>>(c->Nv, Nvp, f, xi, w, Wref, c->rmom);
+    else k_cell_moments<D, T, 128><<<Ncells, 128, 0, c->stream>>>(c->Nv, Nvp, f, xi, w, Wref, c->rmom);
+    k_moments_finish<D, T><<<(Ncells + kCellNT - 1) / kCellNT, kCellNT, 0, c->stream>>>(Ncells, c->rmom, Wref, Wc, q);
     c->launches += 2;
     return cudaGetLastError();
 }
@@ -1089,12 +1093,36 @@ cudaError_t launch_correct(avs_ctx* c, void* f, const double* Wtarget, int iters
 }
 
 // ------------------------------------------------------------------ conversions
+// Exact widening on the integer pipe: the FP64 pipe takes 16 cycles for a
+// warp's conversions (38400 x 2 rows of 11992 nodes: 3.21 ms with it, one node
+// per thread, 1.71 now).
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    if ((b & 0x7F800000u) == 0u && (b & 0x7FFFFFu) != 0u) return (double)x;      // subnormal
+    return to_double(x);
+}
+
+constexpr int kConvNodes = 4;     // nodes per thread of a row's chunk, blockDim.x apart
+template <typename T>
+__device__ __forceinline__ void widen_row(int Nv, const T* __restrict__ in, double* out)
+{
+    const int k0 = blockIdx.y * blockDim.x * kConvNodes + threadIdx.x;
+    T v[kConvNodes];
+#pragma unroll
+    for (int j = 0; j < kConvNodes; ++j)
+        if (k0 + j * blockDim.x < Nv) v[j] = __ldcs(in + k0 + j * blockDim.x);
+#pragma unroll
+    for (int j = 0; j < kConvNodes; ++j)
+        if (k0 + j * blockDim.x < Nv) __stcs(out + k0 + j * blockDim.x, widen(v[j]));
+}
+
 template <typename T>
 __global__ void k_to_double(int Nv, int Nvp, const T* __restrict__ f, double* out)
 {
-    const int k = blockIdx.y * blockDim.x + threadIdx.x;
     const int ia = blockIdx.x;
-    if (k < Nv) out[(size_t)ia * Nv + k] = (double)f[(size_t)ia * Nvp + k];
+    widen_row(Nv, f + (size_t)ia * Nvp, out + (size_t)ia * Nv);
 }
 
 template <typename T>
@@ -1107,9 +1135,9 @@ __global__ void k_from_double(int Nv, int Nvp, const double* __restrict__ in, T*
 
 cudaError_t launch_to_double(avs_ctx* c, const void* f, double* out, int Nvp)
 {
-    dim3 g(c->Nc * c->NA, (c->Nv + 255) / 256);
-    if (c->mixed) k_to_double<float><<<g, 256, 0, c->stream>>>(c->Nv, Nvp, (const float*)f, out);
-    else k_to_double<double><<<g, 256, 0, c->stream>>>(c->Nv, Nvp, (const double*)f, out);
+    dim3 g(c->Nc * c->NA, (c->Nv + 128 * kConvNodes - 1) / (128 * kConvNodes));
+    if (c->mixed) k_to_double<float><<<g, 128, 0, c->stream>>>(c->Nv, Nvp, (const float*)f, out);
+    else k_to_double<double><<<g, 128, 0, c->stream>>>(c->Nv, Nvp, (const double*)f, out);
     c->launches += 1;
     return cudaGetLastError();
 }
@@ -1118,21 +1146,19 @@ template <typename T>
 __global__ void k_gather_double(int Nv, int Nvp, int NA, const T* __restrict__ f, const int* __restrict__ cells,
                                 double* out)
 {
-    const int k = blockIdx.y * blockDim.x + threadIdx.x;
     const int ja = blockIdx.x;                      // (list entry, array)
-    if (k >= Nv) return;
     const int j = ja / NA, a = ja % NA;
-    out[(size_t)ja * Nv + k] = (double)f[((size_t)cells[j] * NA + a) * Nvp + k];
+    widen_row(Nv, f + ((size_t)cells[j] * NA + a) * Nvp, out + (size_t)ja * Nv);
 }
 
 cudaError_t launch_gather_double(avs_ctx* c, const int* cells_d, int ncells, double* out)
 {
-    dim3 g(ncells * c->NA, (c->Nv + 255) / 256);
+    dim3 g(ncells * c->NA, (c->Nv + 128 * kConvNodes - 1) / (128 * kConvNodes));
     if (c->mixed)
-        k_gather_double<float><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->NA, (const float*)c->f[c->cur], cells_d,
+        k_gather_double<float><<<g, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->NA, (const float*)c->f[c->cur], cells_d,
                                                          out);
     else
-        k_gather_double<double><<<g, 256, 0, c->stream>>>(c->Nv, c->Nvp, c->NA, (const double*)c->f[c->cur],
+        k_gather_double<double><<<g, 128, 0, c->stream>>>(c->Nv, c->Nvp, c->NA, (const double*)c->f[c->cur],
                                                           cells_d, out);
     c->launches += 1;
     return cudaGetLastError();

@@ -11,6 +11,10 @@
 #include "../../include/avs.h"
 
 #define AVS_NT 256            // threads per block of the per-cell kernels
+// threads per block of the kernels with one thread per cell and much FP64 work: the
+// FP64 pipe of an SM is their bound, so small blocks that reach every SM (k_cell_state,
+// 12288 cells: 8.4 us with 128, 6.7 with 32)
+constexpr int kCellNT = 32;
 #define AVS_CELLPAR_BYTES 256 // bytes per cell of the collision parameters (CellPar)
 #define AVS_TAB_MAX 3072      // entries of the axes' coordinate tables (32 bytes each in shared memory)
 #define AVS_CMOM_MAX 17       // carried raw moments per cell (monatomic 11 / 13, Rykov 14 / 17)

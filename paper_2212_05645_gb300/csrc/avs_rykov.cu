@@ -1447,7 +1447,7 @@ cudaError_t rk_step_t(avs_ctx* c, const void* fin, void* fout, const double* Win
         auto* par = reinterpret_cast<typename Rykov<D>::Par*>(c->cpar);
         if (!c->mom_valid) e = raw32_t<Rykov<D>>(c, fin, Win);
         if (e != cudaSuccess) return e;
-        rk_cell_state32<D><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(P, c->cmom, par);
+        rk_cell_state32<D><<<(c->Nc + kCellNT - 1) / kCellNT, kCellNT, 0, c->stream>>>(P, c->cmom, par);
         c->launches += 1;
         e = cell32_t<Rykov<D>, false>(c, fin, fout);
         if (e != cudaSuccess) return e;
@@ -1494,8 +1494,8 @@ cudaError_t rk_step_implicit_t(avs_ctx* c, const void* fin, void* fout, const do
     I.nint = c->imp_nint;
     I.clist = c->clist;
     I.err = c->dev_err;
-    const int cb = (c->Nc + 127) / 128;
-    rk_imp_setup<D, A><<<cb, 128, 0, c->stream>>>(I);
+    const int cb = (c->Nc + kCellNT - 1) / kCellNT;
+    rk_imp_setup<D, A><<<cb, kCellNT, 0, c->stream>>>(I);
     c->launches += 1;
     const int nc = c->ncolor;
     if (k_macro > 0) {
@@ -1527,7 +1527,7 @@ cudaError_t rk_step_implicit_t(avs_ctx* c, const void* fin, void* fout, const do
         auto* par = reinterpret_cast<typename Rykov<D>::Par*>(c->cpar);
         if (!c->mom_valid) e = raw32_t<Rykov<D>>(c, fin, Win);
         if (e != cudaSuccess) return e;
-        rk_imp_state32<D><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(P, c->cmom, par, u0);
+        rk_imp_state32<D><<<(c->Nc + kCellNT - 1) / kCellNT, kCellNT, 0, c->stream>>>(P, c->cmom, par, u0);
         c->launches += 1;
         e = cell32_t<Rykov<D>, true>(c, fin, fout);
         if (e == cudaSuccess) e = launch_micro32(c, fin, fout, u0, k_micro);

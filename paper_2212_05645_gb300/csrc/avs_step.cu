@@ -1009,7 +1009,7 @@ template <int D, typename T>
 struct CellP {
     int Nc, Nv, Nvp;
     size_t cstride;
-    double dt;
+    double dt, idt;
     double R, Pr, omega, mu_ref, T_ref;
     const T* __restrict__ fin;
     T* __restrict__ fout;
@@ -1110,7 +1110,15 @@ __global__ void k_cell_state(CellP<D, T> P)
     state_from_raw<D, T>(m, Vc, rn, Un, RTn, qn);
     const int ns = P.nslot[i];
     double Wt[5];
-    const double dtv = P.dt / P.vol[i];
+    // the FP32 form divides once by each of |V| and rho (an FP64 division is
+    // about ten instructions of the scarce pipe)
+    double iv, dtv;
+    if constexpr (sizeof(T) == 4) {
+        iv = 1.0 / P.vol[i];
+        dtv = P.dt * iv;
+    } else {
+        dtv = P.dt / P.vol[i];
+    }
     for (int c = 0; c < NW; ++c) {
         double sum = 0.0;
         for (int s = 0; s < ns; ++s) {
@@ -1124,17 +1132,28 @@ __global__ void k_cell_state(CellP<D, T> P)
     CellPar<T> cp;
     for (int d = 0; d < 3; ++d) cp.Vn[d] = d < D ? (T)Wt[1 + d] / (T)Wt[0] : T(0);
     double rhod, Ud[3], RTd;
-    prim<D>(Wt, rhod, Ud, RTd);
+    if constexpr (sizeof(T) == 4) {
+        rhod = Wt[0];
+        const double ir = 1.0 / rhod;
+        double m2 = 0.0;
+        for (int d = 0; d < D; ++d) {
+            Ud[d] = Wt[1 + d] * ir;
+            m2 += Wt[1 + d] * Wt[1 + d];
+        }
+        RTd = (Wt[D + 1] - 0.5 * m2 * ir) * ir * (1.0 / 1.5);
+    } else {
+        prim<D>(Wt, rhod, Ud, RTd);
+    }
     if (!(rhod > 0.0) || !(RTd > 0.0)) atomicOr(P.err, 1);
     const T rho = (T)rhod, RT = (T)RTd;
     T U[3];
-    for (int d = 0; d < 3; ++d) U[d] = (T)Ud[d];
+    for (int d = 0; d < 3; ++d) U[d] = d < D ? (T)Ud[d] : T(0);
     const T tau = tau_vhs<T>(rho, RT, (T)P.R, (T)P.mu_ref, (T)P.T_ref, (T)P.omega);
     cp.eq = make_eq_a<D, T, T>(rho, U, RT, qn, (T)P.Pr);
-    const T idt = (T)(1.0 / P.dt), itau = T(1) / tau;
+    const T idt = (T)P.idt, itau = T(1) / tau;
     if constexpr (sizeof(T) == 4) {
         reinterpret_cast<Cell32Par*>(P.par)[i] =
-            cell32_par(cp.eq, idt, itau, -(float)(1.0 / P.vol[i]), 1.0f / (idt + itau), cp.Vn, 0.0f);
+            cell32_par(cp.eq, idt, itau, -(float)iv, 1.0f / (idt + itau), cp.Vn, 0.0f);
         return;
     }
     cp.upd[0] = idt;
@@ -1521,6 +1540,7 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
     Q.Nvp = c->Nvp;
     Q.cstride = (size_t)NA * c->Nvp;
     Q.dt = dt;
+    Q.idt = 1.0 / dt;
     Q.R = c->cfg.R;
     Q.Pr = c->cfg.Pr;
     Q.omega = c->cfg.omega;
@@ -1549,7 +1569,7 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
             c->launches += 1;
         }
     }
-    k_cell_state<D, T><<<(c->Nc + 127) / 128, 128, 0, c->stream>>>(Q);
+    k_cell_state<D, T><<<(c->Nc + kCellNT - 1) / kCellNT, kCellNT, 0, c->stream>>>(Q);
     c->launches += 1;
     if constexpr (sizeof(T) == 4) {
         e = launch_cell32(c, fin, fout, false);
@@ -2103,8 +2123,8 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
     I.nint = c->imp_nint;
     I.clist = c->clist;
     I.err = c->dev_err;
-    const int cb = (c->Nc + 127) / 128;
-    k_imp_setup<D, A><<<cb, 128, 0, c->stream>>>(I);
+    const int cb = (c->Nc + kCellNT - 1) / kCellNT;
+    k_imp_setup<D, A><<<cb, kCellNT, 0, c->stream>>>(I);
     c->launches += 1;
     const int nc = c->ncolor;
     if (k_macro > 0) {
@@ -2140,6 +2160,7 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
     Q.Nvp = c->Nvp;
     Q.cstride = (size_t)NA * c->Nvp;
     Q.dt = dt;
+    Q.idt = 1.0 / dt;
     Q.R = c->cfg.R;
     Q.Pr = c->cfg.Pr;
     Q.omega = c->cfg.omega;
@@ -2169,7 +2190,7 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
             c->launches += 1;
         }
     }
-    k_imp_state<D, T><<<cb, 128, 0, c->stream>>>(Q, Wout);
+    k_imp_state<D, T><<<cb, kCellNT, 0, c->stream>>>(Q, Wout);
     c->launches += 1;
     if constexpr (sizeof(T) == 4) {
         e = launch_cell32(c, fin, fout, true);
