@@ -76,10 +76,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, u
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity)
 {
     unsigned ok;
@@ -89,12 +85,6 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned 
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     return ok != 0;
-}
-// orders this thread's earlier generic-proxy accesses of shared memory before
-// later asynchronous-proxy writes (a buffer refilled after it was read)
-__device__ __forceinline__ void fence_proxy_async_smem()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar)
 {
@@ -570,28 +560,6 @@ __device__ __forceinline__ void raw_acc2(float2* m, const float2* xs, float2 wg,
         m[11] = fma2(t1, s, m[11]);
         m[12] = fma2(t2, s, m[12]);
     }
-}
-
-// eq_eval for a pair of nodes (X[d] = the pair's d-th velocity components)
-template <int D>
-__device__ __forceinline__ void eq_eval2(const EqPar<float>& p, const float2* X, float2& gG, float2& gH)
-{
-    float2 c[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) c[d] = add2(X[d], bc2(-p.U[d]));
-    float2 c2 = mul2(c[0], c[0]), cq = mul2(c[0], bc2(p.alpha[0]));
-#pragma unroll
-    for (int d = 1; d < D; ++d) {
-        c2 = fma2(c[d], c[d], c2);
-        cq = fma2(c[d], bc2(p.alpha[d]), cq);
-    }
-    // pref exp(-c^2 / 2RT) as 2^(log2 pref - c^2 log2(e) / 2RT): one fused
-    // multiply-add for the exponent of both lanes
-    const float2 a = fma2(c2, bc2(p.k2), bc2(p.l2pref));
-    const float2 e = make_float2(ex2_approx(a.x), ex2_approx(a.y));
-    const float2 s = mul2(c2, bc2(p.invRT));
-    gG = mul2(e, fma2(cq, add2(s, bc2(-(float)(D + 2))), bc2(1.0f)));
-    gH = (D == 2) ? mul2(mul2(bc2(p.RTH), e), fma2(cq, add2(s, bc2(-(float)D)), bc2(1.0f))) : bc2(0.0f);
 }
 
 // ---------------------------------------------------------------- reductions

@@ -77,7 +77,6 @@ struct avs_ctx {
     double *xtab = nullptr;                          // [tab_n]
     unsigned short *tix = nullptr;                   // [D][xstride]
     int tab_end[3] = {0, 0, 0}, tab_n = 0;
-    float *xi_p = nullptr;                           // FP32 node coordinates by pairs: [cap/2][D][2]
     double *M = nullptr;                             // [cap]
     unsigned long long *Mkey = nullptr;              // [cap]
 

@@ -7,10 +7,10 @@
 // rho E_rot = int R = rho R T_r, (3/2) rho R T_t = rho E - rho U^2/2 - rho E_rot,
 // and the equilibrium temperature T = (3 T_t + 2 T_r) / 5.
 //
-// The kernels take one block per face or cell.  The FP64 form sums over the
-// nodes in FP64 directly; the FP32 (mixed) form sums raw moments in FP32 per
-// thread and in FP64 across warps.  The equilibrium is evaluated in the
-// element type.
+// The FP64 form takes one block per face or cell and sums over the nodes in
+// FP64 directly.  The FP32 (mixed) form is the gas Rykov<D> of the kernels in
+// avs_step32.cuh: raw moments in FP32 per thread and in FP64 across warps.  The
+// equilibrium is evaluated in the element type.
 #include <algorithm>
 
 #include "avs_dev.cuh"
@@ -768,13 +768,12 @@ struct Rykov {
 // needs for its lagged heat fluxes are summed while f^{n+1} is written and
 // carried per cell ([cell][NR] FP64, about V(W^{n+1})); all per-cell FP64
 // work (the balance of W, the rotational relaxation) runs one thread per
-// cell in rk_cell_state32; the cell kernel streams f, the face fluxes and
-// f^{n+1} RK_VC nodes per thread in vector loads.
+// cell in rk_cell_state32.
 
 static_assert(sizeof(Rykov<3>::Par) <= AVS_CELLPAR_BYTES, "cell parameter buffer");
 static_assert(RkNR<3>::v <= AVS_CMOM_MAX, "carried moments buffer size");
 
-constexpr int RK_VC = 2;     // nodes per thread per iteration of the cell kernels (2 or 4)
+constexpr int RK_VC = 2;     // nodes per thread per iteration of rk_moments32 (2 or 4)
 
 // V = RK_VC consecutive nodes of an FP32 row in one vector load (L2 only).
 __device__ __forceinline__ void rk_ldv(const float* p, float* o)

@@ -43,13 +43,7 @@ template <typename T> struct VW { static constexpr int v = 16 / sizeof(T); };
 template <typename T, int V>
 __device__ __forceinline__ void ldv(const T* __restrict__ p, T* o)
 {
-    if constexpr (sizeof(T) == 4 && V == 4) {
-        const float4 q = *reinterpret_cast<const float4*>(p);
-        o[0] = q.x; o[1] = q.y; o[2] = q.z; o[3] = q.w;
-    } else if constexpr (sizeof(T) == 4 && V == 2) {
-        const float2 q = *reinterpret_cast<const float2*>(p);
-        o[0] = q.x; o[1] = q.y;
-    } else if constexpr (sizeof(T) == 8 && V == 2) {
+    if constexpr (sizeof(T) == 8 && V == 2) {
         const double2 q = *reinterpret_cast<const double2*>(p);
         o[0] = q.x; o[1] = q.y;
     } else {
@@ -62,13 +56,7 @@ __device__ __forceinline__ void ldv(const T* __restrict__ p, T* o)
 template <typename T, int V>
 __device__ __forceinline__ void ldv_cg(const T* __restrict__ p, T* o)
 {
-    if constexpr (sizeof(T) == 4 && V == 4) {
-        const float4 q = __ldcg(reinterpret_cast<const float4*>(p));
-        o[0] = q.x; o[1] = q.y; o[2] = q.z; o[3] = q.w;
-    } else if constexpr (sizeof(T) == 4 && V == 2) {
-        const float2 q = __ldcg(reinterpret_cast<const float2*>(p));
-        o[0] = q.x; o[1] = q.y;
-    } else if constexpr (sizeof(T) == 8 && V == 2) {
+    if constexpr (sizeof(T) == 8 && V == 2) {
         const double2 q = __ldcg(reinterpret_cast<const double2*>(p));
         o[0] = q.x; o[1] = q.y;
     } else {
@@ -80,11 +68,7 @@ __device__ __forceinline__ void ldv_cg(const T* __restrict__ p, T* o)
 template <typename T, int V>
 __device__ __forceinline__ void stv(T* p, const T* o)
 {
-    if constexpr (sizeof(T) == 4 && V == 4) {
-        *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
-    } else if constexpr (sizeof(T) == 4 && V == 2) {
-        *reinterpret_cast<float2*>(p) = make_float2(o[0], o[1]);
-    } else if constexpr (sizeof(T) == 8 && V == 2) {
+    if constexpr (sizeof(T) == 8 && V == 2) {
         *reinterpret_cast<double2*>(p) = make_double2(o[0], o[1]);
     } else {
 #pragma unroll
@@ -592,10 +576,6 @@ __device__ __forceinline__ void load_nodes(const PP& P, int k0, T (*x)[D], T* w)
         constexpr int PER = 16 / sizeof(T);
 #pragma unroll
         for (int j = 0; j < V * D / PER; ++j) ldv<T, PER>(P.xi + (size_t)k0 * D + j * PER, xx + j * PER);
-    } else if constexpr (sizeof(T) == 4 && (V * D) % 2 == 0) {
-        // 8-byte pairs (k0 is a multiple of V, so k0 D is even)
-#pragma unroll
-        for (int j = 0; j < V * D / 2; ++j) ldv<T, 2>(P.xi + (size_t)k0 * D + 2 * j, xx + 2 * j);
     } else {
 #pragma unroll
         for (int j = 0; j < V * D; ++j) xx[j] = P.xi[(size_t)k0 * D + j];
@@ -1426,7 +1406,6 @@ static bool axis_tables(const avs_ctx* c) { return c->tab_n > 0 && 2 * c->tab_n 
 template <int D, typename T>
 static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, double dt)
 {
-    const bool f32 = sizeof(T) == 4;
     const int NA = NArr<D>::v;
     const size_t rows = (size_t)std::max(c->fcap, c->Nvp);   // sized for the f capacity: no reallocation
     {
@@ -1442,9 +1421,6 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
             c->flux_bytes = need;
         }
     }
-    const T* xi = f32 ? (const T*)c->xi_f : (const T*)c->xi_d;
-    const T* w = f32 ? (const T*)c->w_f : (const T*)c->w_d;
-    const T* An = f32 ? (const T*)c->An_f : (const T*)c->An_d;
     const double hd = 0.5 * dt;
     {
         if constexpr (sizeof(T) == 4) {
@@ -1465,8 +1441,8 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
             };
             if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
             else go(std::integral_constant<int, AVS_MAXS>{});
+            c->launches += 1;
         }
-        c->launches += 1;
     }
     if constexpr (sizeof(T) == 4) {
         return launch_face32(c, Win, dt);
@@ -1485,12 +1461,12 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
         P.FB = (T*)c->flux;
         P.AF = c->AFf;
         P.Win = Win;
-        P.xi = xi;
-        P.w = w;
+        P.xi = c->xi_d;
+        P.w = c->w_d;
         P.order = c->forder;
         P.faceL = c->faceL;
         P.faceR = c->faceR;
-        P.An = An;
+        P.An = c->An_d;
         P.bc = c->bc;
         P.err = c->dev_err;
         constexpr int NT = 128;

@@ -8,7 +8,7 @@ namespace avs {
 
 namespace {
 
-// Equilibrium G and H at a node pair as eq_eval2 forms them.
+// Equilibrium G and H at a node pair.
 template <int D>
 __device__ __forceinline__ void eq2(const float2* x, const float* U, const float* al, float k2, float l2, float irt,
                                     float RTH, float2& gG, float2& gH)
