@@ -78,7 +78,7 @@ __global__ void k_geom(int D, int Nv, int Nvp, const int* __restrict__ level, co
         xc[d] = x;
         xi_d[(size_t)k * D + d] = x;
         xi_f[(size_t)k * D + d] = (float)x;
-        xi_s[d * xstride + k] = (float)x;
+        xi_s[d * xstride + k] = f32_nz(x);
         if (tix) {
             const int start = d == 0 ? 0 : d == 1 ? t0 : t1;
             tix[d * xstride + k] = (unsigned short)(start + nb[d] * ((1 << l) - 1) + (bi << l) + (int)o);

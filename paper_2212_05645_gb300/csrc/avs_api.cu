@@ -386,7 +386,11 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
     CK(up(c->An_d, std::vector<double>(m->An, m->An + nfd), s));
     CK(up(c->rL_d, std::vector<double>(m->rL, m->rL + nfd), s));
     CK(up(c->rR_d, std::vector<double>(m->rR, m->rR + nfd), s));
-    CK(up(c->An_f, tof(m->An, nfd), s));
+    {
+        std::vector<float> an(nfd);
+        for (size_t e = 0; e < nfd; ++e) an[e] = f32_nz(m->An[e]);
+        CK(up(c->An_f, an, s));
+    }
     CK(up(c->rL_f, tof(m->rL, nfd), s));
     CK(up(c->rR_f, tof(m->rR, nfd), s));
     CK(up(c->vol, std::vector<double>(m->vol, m->vol + Nc), s));
@@ -417,7 +421,7 @@ avs_status setup_mesh(avs_ctx* c, const avs_mesh* m)
             for (int a = 0; a < D; ++a) {
                 g[a] = (float)cg[o * D + a];
                 g[4 + a] = (float)r[o * D + a];
-                const float an = (float)m->An[(size_t)fc * D + a];
+                const float an = f32_nz(m->An[(size_t)fc * D + a]);
                 g[8 + a] = (sl & 1) ? -an : an;
             }
         }

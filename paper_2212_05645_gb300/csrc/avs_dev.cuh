@@ -676,6 +676,17 @@ __device__ __forceinline__ bool upwind_sure(const float* x, const float* n, floa
     for (int d = 0; d < D; ++d) sa = fmaf(fabsf(x[d]), fabsf(n[d]), sa);
     return fabsf(sn) > fmaf(sa, 0x1p-20f, 0x1p-100f) && sa < INFINITY;
 }
+// Whether every product xi_d An_d is zero (a node on the axis of an axis-aligned
+// face), so that the FP64 sum is zero as sn is: xi_s and the FP32 normals are
+// zero only where the FP64 values are (f32_nz).
+template <int D>
+__device__ __forceinline__ bool upwind_zero(const float* x, const float* n)
+{
+    bool z = true;
+#pragma unroll
+    for (int d = 0; d < D; ++d) z = z && (x[d] == 0.0f || n[d] == 0.0f);
+    return z;
+}
 
 // A row of N values that other blocks may have written before the last grid
 // barrier (read past L1): vectors of 16 bytes where the row is made of them.

@@ -15,6 +15,15 @@
 // FP64 pipe of an SM is their bound, so small blocks that reach every SM (k_cell_state,
 // 12288 cells: 8.4 us with 128, 6.7 with 32)
 constexpr int kCellNT = 32;
+// FP32 rounding that is zero only for zero
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline float f32_nz(double x)
+{
+    const float f = (float)x;
+    return f == 0.0f && x != 0.0 ? (x > 0.0 ? 0x1p-149f : -0x1p-149f) : f;
+}
 #define AVS_CELLPAR_BYTES 256 // bytes per cell of the collision parameters (CellPar)
 #define AVS_TAB_MAX 3072      // entries of the axes' coordinate tables (32 bytes each in shared memory)
 #define AVS_CMOM_MAX 17       // carried raw moments per cell (monatomic 11 / 13, Rykov 14 / 17)

@@ -328,6 +328,7 @@ __global__ void __launch_bounds__(128) k_foot(int Nv, int Nvp, int chunk, int li
                     sn = fmaf(xv[d], na[d], sn);
                 }
                 if (upwind_sure<D>(xv, na, sn)) up[v] = sn > 0.0f;
+                else if (upwind_zero<D>(xv, na)) up[v] = n4.w == 0.0f;
                 else up[v] = upwind_exact<D>(x[v], An + (size_t)fc * D, n4.w != 0.0f);
             }
             if (!up[0] && !up[1]) continue;
@@ -400,13 +401,20 @@ __device__ __forceinline__ float2 limit2(float2 dmax, float2 dmin, float2 pp, fl
 }
 
 // Thread block (cell i, nodes of one chunk), the thread's quads one after the
-// other: the block's start (launch, geometry, barrier) is paid once for up to
-// four quads per thread.
+// other: the block's start (launch, geometry, barrier) is paid once for them.
+// Bounded by the latency of the rows' loads at the warps that the registers
+// allow: all rows of a quad are loaded before its arithmetic (12288 cells x 3522
+// nodes, 2D: array by array 294 us, all at once 270; Rykov, 3216 nodes, 476 and
+// 398), seven blocks of 128 threads per SM in 2D, 18 of 64 in 3D; rings of
+// copies in shared memory as in the face kernel leave too few warps (311 us).
 // EXACT: the upwind choice is the FP64 one; only a quad with a normal velocity
-// within one bound of zero recomputes it (a bound per node: 565 us for the Rykov
-// cylinder's 12288 cells x 3216 nodes, one per quad: 476).
+// within one bound of zero recomputes it (a bound per node cost the Rykov
+// cylinder 90 us more).
+// Warps per SM, by the vectors a quad loads (own and neighbours', every array):
+// the most that do not spill more than a few registers.
+constexpr int foot_warps(int D, int rows) { return D == 3 ? (rows <= 7 ? 36 : 16) : rows <= 10 ? 28 : rows <= 15 ? 24 - 4 * (rows < 15) : 16; }
 template <int D, int NS, int NA, bool EXACT>
-__global__ void __launch_bounds__(128, EXACT ? 6 : 8) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
+__global__ void __launch_bounds__(D == 3 ? 64 : 128, foot_warps(D, NA * (NS + 1)) / (D == 3 ? 2 : 4)) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
                                                     const float* __restrict__ f, float* __restrict__ FB,
                                                     const float4* __restrict__ geo, const float* __restrict__ eps2,
                                                     const float* __restrict__ xs, size_t xstride,
@@ -422,15 +430,20 @@ __global__ void __launch_bounds__(128, EXACT ? 6 : 8) k_foot_f2(int Nv, int Nvp,
 #pragma unroll 1
     for (int k0 = blockIdx.y * chunk + threadIdx.x * VG; k0 < kend; k0 += blockDim.x * VG) {
         float2 phi[NA][2], G[NA][D][2];
+        float4 n4a[NA][NS];
+        float4 c4a[NA];
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
             const float* fa = f + (size_t)a * Nvp + k0;
-            const float4 c4 = __ldg(reinterpret_cast<const float4*>(fa + (size_t)i * cstride));
-            phi[a][0] = lo2(c4);
-            phi[a][1] = hi2(c4);
-            float4 n4[NS];
+            c4a[a] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)i * cstride));
 #pragma unroll
-            for (int s = 0; s < NS; ++s) n4[s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)__float_as_int(gs[3 * s].w) * cstride));
+            for (int s = 0; s < NS; ++s) n4a[a][s] = __ldg(reinterpret_cast<const float4*>(fa + (size_t)__float_as_int(gs[3 * s].w) * cstride));
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+            phi[a][0] = lo2(c4a[a]);
+            phi[a][1] = hi2(c4a[a]);
+            float4* n4 = n4a[a];
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 float2 g[D], dd[NS];
@@ -528,9 +541,17 @@ __global__ void __launch_bounds__(128, EXACT ? 6 : 8) k_foot_f2(int Nv, int Nvp,
                 if constexpr (D == 3) na += fabsf(an.z);
                 if (!(near > fmaf(xmax * 0x1p-20f, na, 0x1p-100f))) {
 #pragma unroll
-                    for (int z = 0; z < 4; ++z)
-                        if (k0 + z < Nv)
+                    for (int z = 0; z < 4; ++z) {
+                        float xz[D], nz[D], sn = 0.0f;
+                        vec3<D>(an, nz);
+#pragma unroll
+                        for (int d = 0; d < D; ++d) {
+                            xz[d] = z & 1 ? X[z >> 1][d].y : X[z >> 1][d].x;
+                            sn = d == 0 ? xz[0] * nz[0] : fmaf(xz[d], nz[d], sn);
+                        }
+                        if (!upwind_sure<D>(xz, nz, sn) && !upwind_zero<D>(xz, nz) && k0 + z < Nv)
                             up[z] = upwind_exact<D>(xi + (size_t)(k0 + z) * D, An + (size_t)fc * D, an.w != 0.0f);
+                    }
                 }
             }
             const bool all = up[0] && up[1] && up[2] && up[3];
@@ -1369,14 +1390,17 @@ template <int D, int NA, bool EXACT>
 static void foot32_t(avs_ctx* c, const void* fin, double hd)
 {
     constexpr int VG = 4;
-    // 128 threads, or 64 where a row has no more quads (190 nodes,
-    // 12288 cells: 41 -> 25 us), with up to four quads per thread while
-    // that leaves 32 blocks per SM (21k nodes, 36864 cells: 5.41 ->
-    // 4.46 ms; chunks of 2048 nodes still let the rows of a cell's
-    // neighbours be reused from L2)
+    // 2D: 128 threads, or 64 where a row has no more quads (190 nodes, 12288
+    // cells: 41 -> 25 us), with up to eight quads per thread (3.5k nodes, 12288
+    // cells: 252 us, four 270; 12k nodes, 38400 cells: 2.48 ms, 2.56).  3D: 64
+    // threads and up to four quads, as chunks of 1024 nodes let the rows of six
+    // neighbours be reused from the caches (21k nodes, 36864 cells: 4.00 ms; 128
+    // threads of up to eight 4.09, of up to four 4.24).  One block per cell and
+    // chunk while that leaves 32 blocks per SM.
     const int nquad = (c->Nv + VG - 1) / VG;
-    const int nt = nquad <= 64 ? 64 : 128;
-    const int per = (int)std::max(1ll, std::min(4ll, (long long)c->Nc * nquad / nt / (32 * std::max(1, c->nsm))));
+    const int nt = D == 3 || nquad <= 64 ? 64 : 128;
+    const long long most = D == 3 ? 4 : 8;
+    const int per = (int)std::max(1ll, std::min(most, (long long)c->Nc * nquad / nt / (32 * std::max(1, c->nsm))));
     const int ny = (nquad + nt * per - 1) / (nt * per);
     const int chunk = (nquad + ny - 1) / ny * VG;
     auto go = [&](auto ns) {
@@ -1384,9 +1408,10 @@ static void foot32_t(avs_ctx* c, const void* fin, double hd)
             c->Nv, c->Nvp, chunk, c->cfg.limiter, (float)hd, (const float*)fin, (float*)c->flux, (const float4*)c->geo32,
             c->eps2_f, c->xi_s, c->xstride, c->xi_d, c->An_d);
     };
-    if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
-    else go(std::integral_constant<int, AVS_MAXS>{});
     c->launches += 1;
+    if constexpr (D == 2)
+        if (c->max_ns <= 4) return go(std::integral_constant<int, 4>{});
+    go(std::integral_constant<int, AVS_MAXS>{});
 }
 
 void launch_foot32(avs_ctx* c, const void* fin, double hd)

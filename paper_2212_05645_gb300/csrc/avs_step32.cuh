@@ -84,6 +84,17 @@ __device__ __forceinline__ float2 dot2(const float2* x, const float* a)
     for (int d = 1; d < D; ++d) s = fma2(x[d], bc2(a[d]), s);
     return s;
 }
+// xi . An of the flux, every product and sum rounded: the heat flux of a gas near
+// equilibrium, a small difference of large sums, follows the rounding of each
+// node's flux
+template <int D>
+__device__ __forceinline__ float2 dot2r(const float2* x, const float* a)
+{
+    float2 s = mul2(x[0], bc2(a[0]));
+#pragma unroll
+    for (int d = 1; d < D; ++d) s = add2(s, mul2(x[d], bc2(a[d])));
+    return s;
+}
 
 // raw moments of a node pair (values o of the gas's arrays: G, in 2D H, for a
 // gas with rotation R) about V, y = xi - V
@@ -203,7 +214,7 @@ struct Face32S {
 };
 
 template <class G, int FPT, int NT, int HG, int STG>
-__global__ void __launch_bounds__(NT * HG, (NT * HG == 128 ? (FPT > 2 ? 3 : 4) : 2)) k_face32(Face32P<G> P)
+__global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ? (FPT > 2 ? 3 : 4) : 2)) k_face32(Face32P<G> P)
 {
     constexpr int D = G::D, NA = G::NA, NM = G::NM, NW = G::NW, CH = 4 * NT;
     constexpr int NR = FPT * NA + D + 1;         // rows of a slot: foot values, coordinates, weights
@@ -260,7 +271,7 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 128 ? (FPT > 2 ? 3 : 4) :
 #pragma unroll
                         for (int d = 0; d < D; ++d) xz[d] = z ? x[d].y : x[d].x;
                         const int kn = k + 2 * p + z;
-                        if (!upwind_sure<D>(xz, An, z ? sn[p].y : sn[p].x) && kn < Nv)
+                        if (!upwind_sure<D>(xz, An, z ? sn[p].y : sn[p].x) && !upwind_zero<D>(xz, An) && kn < Nv)
                             up[2 * p + z] = upwind_exact<D>(P.xid + (size_t)kn * D, P.And + (size_t)f * D, false);
                     }
                 }
@@ -488,7 +499,7 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 128 ? (FPT > 2 ? 3 : 4) :
                         float2 x[D];
 #pragma unroll
                         for (int d = 0; d < D; ++d) x[d] = X[d][p];
-                        const float2 sn = dot2<D>(x, An[j]);
+                        const float2 sn = dot2r<D>(x, An[j]);
                         float2 F1[NA], o1[NA];
 #pragma unroll
                         for (int a = 0; a < NA; ++a) F1[a] = F[j][a][p];
@@ -750,26 +761,32 @@ cudaError_t face32_t(avs_ctx* c, const double* Win, double dt, const typename G:
     using I2 = integral_constant<int, 2>;
     using I4 = integral_constant<int, 4>;
     using N32 = integral_constant<int, 32>;
+    using N64 = integral_constant<int, 64>;
     using N128 = integral_constant<int, 128>;
     using I3 = integral_constant<int, 3>;
     // Short rows (a few quads per lane): one warp per group, so that a group's
-    // reductions and serial state hold no other warp; 128 threads per group
-    // beyond.  Two faces per group where that leaves groups enough to fill the
-    // SMs (190 nodes, 24672 faces, 20 steps: 0.73 ms, one face 1.04 ms).
-    // Slots of the ring: three, or four in 3D and for long 2D rows, where the
-    // larger ring also keeps fewer rows in flight, so that pass B finds them in
-    // L2 (12k nodes in 2D, four steps: 10.9 against 12.5 ms; 21k in 3D, five
-    // steps: 24.0 against 25.7 ms; 3.5k in 2D, ten steps: 3.04 against 2.74 ms,
-    // with three arrays, 39 kB a row, 4.11 against 3.67 ms).
+    // reductions and serial state hold no other warp.  Beyond, 64 threads, eight
+    // groups per SM, so that some are in their loops while others wait for their
+    // states (3D, 6783 cells x 2197 nodes, ten steps: 1.17 ms, 128 threads 1.53;
+    // 2D, 12288 x 3522: 2.63 against 2.74); for rows over 48 KB 128 threads, whose
+    // fewer rows in flight pass B still finds in L2 (2D, 12k nodes, four steps:
+    // 10.9 against 12.8 ms; 3D, 21k, five steps: 24.0 against 24.2).  Two faces per
+    // group where that leaves groups enough to fill the SMs (190 nodes, 24672
+    // faces, 20 steps: 0.73 ms, one face 1.04 ms).  Slots of the ring: three, or
+    // four in 3D and for long rows, again for L2 (12k nodes in 2D 10.9 against
+    // 12.5 ms; 21k in 3D 24.0 against 25.7; 2D, 39 kB a row, 4.11 with four, 3.67
+    // with three).
     if (c->Nv <= 512 || (c->Nv <= 1024 && c->Nf >= 32 * c->nsm)) {
         if (c->Nf >= 16 * c->nsm) go(I2{}, N32{}, I4{}, I3{});
         else go(I1{}, N32{}, I4{}, I3{});
     } else if (c->Nf < 4 * c->nsm) {
         go(I1{}, N128{}, I1{}, I3{});
-    } else if (D == 3 || (size_t)NA * c->Nvp * sizeof(float) > 49152) {
+    } else if ((size_t)NA * c->Nvp * sizeof(float) > 49152) {
         go(I2{}, N128{}, I1{}, I4{});
+    } else if (D == 3) {
+        go(I2{}, N64{}, I1{}, I4{});
     } else {
-        go(I2{}, N128{}, I1{}, I3{});
+        go(I2{}, N64{}, I1{}, I3{});
     }
     if (e != cudaSuccess) return e;
     c->launches += 1;
