@@ -582,14 +582,14 @@ __device__ __forceinline__ void crit_row(const float4* c8, int j, float (&c32)[5
 // loads: 1.00 ms for 18432 cells x 21372 nodes, now 0.49; k_criterion, two nodes
 // per thread, 1.32 and 0.88 ms.)
 template <int D, typename T>
-__global__ void __launch_bounds__(128) k_crit_screen(int NA, int Nv, int Nvp, int ncells, const T* __restrict__ f,
+__global__ void __launch_bounds__(128) k_crit_screen(int NA, int Nv, int Nvp, int ncells, int per, const T* __restrict__ f,
                                                      const float* __restrict__ xs, size_t xstride,
                                                      const float* __restrict__ w, const float* __restrict__ cp32,
                                                      const int* __restrict__ cells, unsigned* Mlo, unsigned* Mhi)
 {
     __shared__ int ci[kCritCells];
     __shared__ float4 c8[2 * kCritCells];
-    const int j0 = blockIdx.y * kCritCells, n = min(kCritCells, ncells - j0);
+    const int j0 = blockIdx.y * per, n = min(per, ncells - j0);
     crit_stage(j0, n, cells, cp32, ci, c8);
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (k >= Nv) return;                           // rows are padded to 32 nodes: whole vectors
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(128) k_crit_screen(int NA, int Nv, int Nvp, in
 // relative) is left to k_decode_M, which stores lo as its value; the tests
 // give the same answers for it as for the exact M_k.
 template <int D, typename T>
-__global__ void __launch_bounds__(128) k_criterion(int NA, int Nv, int Nvp, int ncells, const T* __restrict__ f,
+__global__ void __launch_bounds__(128) k_criterion(int NA, int Nv, int Nvp, int ncells, int per, const T* __restrict__ f,
                                                    const double* __restrict__ xi, const double* __restrict__ w,
                                                    const double* __restrict__ cp, const float* __restrict__ xs,
                                                    size_t xstride, const float* __restrict__ w32,
@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(128) k_criterion(int NA, int Nv, int Nvp, int 
     __shared__ int ci[kCritCells];
     __shared__ float4 c8[2 * kCritCells];
     constexpr int V = 2;                           // nodes per thread
-    const int j0 = blockIdx.y * kCritCells, n = min(kCritCells, ncells - j0);
+    const int j0 = blockIdx.y * per, n = min(per, ncells - j0);
     crit_stage(j0, n, cells, cp32, ci, c8);
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (k >= Nv) return;
@@ -760,14 +760,22 @@ cudaError_t launch_criterion(avs_ctx* c, const void* f, int f_is_double, int Nce
     const bool dbl = f_is_double || !c->mixed;
     const float s32 = (float)c->s_norm, C1s = (float)c->cfg.C1 * kCritScale, C2s = (float)c->cfg.C2 * kCritScale;
     if (n > 0) {
-        const int ny = (n + kCritCells - 1) / kCritCells;
+        // cells per block: 64, fewer where that would leave less than eight
+        // blocks per SM (884 cells, 3310 nodes: k_criterion 45 us with 64, 18 now)
+        auto cells_per = [&](int nx) {
+            int per = kCritCells;
+            while (per > 8 && (long long)nx * ((n + per - 1) / per) < 8ll * std::max(1, c->nsm)) per /= 2;
+            return per;
+        };
         auto go = [&](auto dim, auto* fp) {
             constexpr int D = decltype(dim)::value;
             using T = std::remove_cv_t<std::remove_pointer_t<decltype(fp)>>;
-            k_crit_screen<D, T><<<dim3((c->Nv + 511) / 512, ny), 128, 0, c->stream>>>(
-                c->NA, c->Nv, Nvp, n, fp, c->xi_s, c->xstride, c->w_f, c->crit_cp32, cells, c->Mlo, c->Mhi);
-            k_criterion<D, T><<<dim3((c->Nv + 255) / 256, ny), 128, 0, c->stream>>>(
-                c->NA, c->Nv, Nvp, n, fp, c->xi_d, c->w_d, cp, c->xi_s, c->xstride, c->w_f, c->crit_cp32, c->Mlo,
+            const int nx1 = (c->Nv + 511) / 512, nx2 = (c->Nv + 255) / 256;
+            const int per1 = cells_per(nx1), per2 = cells_per(nx2);
+            k_crit_screen<D, T><<<dim3(nx1, (n + per1 - 1) / per1), 128, 0, c->stream>>>(
+                c->NA, c->Nv, Nvp, n, per1, fp, c->xi_s, c->xstride, c->w_f, c->crit_cp32, cells, c->Mlo, c->Mhi);
+            k_criterion<D, T><<<dim3(nx2, (n + per2 - 1) / per2), 128, 0, c->stream>>>(
+                c->NA, c->Nv, Nvp, n, per2, fp, c->xi_d, c->w_d, cp, c->xi_s, c->xstride, c->w_f, c->crit_cp32, c->Mlo,
                 c->Mhi, decide, s32, C1s, C2s, cells, c->Mkey);
         };
         using D2 = std::integral_constant<int, 2>;
