@@ -200,6 +200,24 @@ def _peaks():
     return 6800.0, "fallback"
 
 
+def _step_kernels(w, implicit, fp64):
+    """The step's kernels, as a label of the roofline entry."""
+    ryk = w.model == "rykov"
+    if fp64:
+        foot, face, res, micro = ("k_grad", "rk_face", "rk_imp_res", "rk_imp_micro + rk_imp_finish") if ryk else \
+            ("k_foot", "k_face", "k_imp_res", "k_imp_micro + k_imp_finish")
+        cell = "rk_cell" if ryk else "k_cell_state + k_cell"
+    else:
+        foot, face, res, micro = "k_foot_f2", "k_face32", "k_raw32 + k_cell32", "k_micro32"
+        cell = ("rk_cell_state32" if ryk else "k_cell_state") + " + k_cell32"
+    if implicit:
+        p = "rk_" if ryk else "k_"
+        state = "" if ryk and fp64 else f"{p}imp_state{'32' if ryk else ''} + "
+        cell = f"{p}imp_setup + {p}imp_macro + {state}{res} + {micro}"
+    return (f"{'implicit ' if implicit else ''}{'Rykov ' if ryk else ''}UGKS step: {foot} + {face} + {cell} "
+            f"<{w.D},{'double' if fp64 else 'float'}>")
+
+
 def _traffic(family, Nc, Nv):
     """DRAM bytes per UGKS step (the step kernels, one ncu pass) from the
     committed record of this workload family, scaled to this step by
@@ -212,7 +230,7 @@ def _traffic(family, Nc, Nv):
     with open(p) as fh:
         d = json.load(fh)
     h = hashlib.sha256()
-    for f in ("avs_step.cu", "avs_dev.cuh"):
+    for f in ("avs_step.cu", "avs_step32.cu", "avs_step32.cuh", "avs_dev.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2212_05645_gb300", "csrc", f), "rb").read())
     sha = h.hexdigest()[:16]
     e = d.get(family)
@@ -407,12 +425,7 @@ def run_gpu(args):
                if family and args.implicit <= 0 and w.model == "shakhov" else None)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": traffic,
-            "kernel": (f"implicit Rykov UGKS step: k_grad + rk_face + rk_imp_setup + rk_imp_macro + rk_imp_res"
-                       f" + rk_imp_micro + rk_imp_finish <{w.D},float>" if args.implicit > 0 and w.model == "rykov" else
-                       f"implicit UGKS step: k_foot + k_face + k_imp_setup + k_imp_macro + k_imp_state + k_imp_res"
-                       f" + k_imp_micro + k_imp_finish <{w.D},float>" if args.implicit > 0 else
-                       f"Rykov UGKS step: k_grad + rk_face + rk_cell <{w.D},float>" if w.model == "rykov" else
-                       f"UGKS step: k_foot + k_face + k_cell_state + k_cell <{w.D},{'double' if main_fp64 else 'float'}>"),
+            "kernel": _step_kernels(w, args.implicit > 0, main_fp64),
             "peak_source": peak_kind,
             "algorithmic_bytes_per_cell_node": bytes_per_cn, "kernel_ms": kern_ms,
             "peak_spec_gbs": 8000.0, "frac_of_spec": achieved / 8000.0}
