@@ -13,9 +13,9 @@
 // one (see upwind_sure).  Shakhov's is in avs_step32.cu, Rykov's in avs_rykov.cu.
 // Measured on GB300, five steps of the sphere (36864 cells, 21372 nodes) and ten
 // of the cylinder (12288 cells, 3522 nodes), face and cell kernel: 24.0 + 14.5
-// and 2.74 + 2.42 ms; one face or cell per block with rows staged by bulk copies
+// and 2.63 + 2.42 ms; one face or cell per block with rows staged by bulk copies
 // or loaded directly, before: 31.3 + 21.2 and 4.20 + 2.91 ms.  The Rykov
-// cylinder (12288 cells, 3216 nodes, ten steps): 3.67 + 3.29 ms with 4.76 for the
+// cylinder (12288 cells, 3216 nodes, ten steps): 3.60 + 3.29 ms with 3.86 for the
 // foot values, against 10.3 + 4.7 and 3.5 for stored gradients that the face
 // kernel read.
 // Forming phi and its flux in the cell kernel instead, without storing them,
@@ -775,7 +775,7 @@ cudaError_t face32_t(avs_ctx* c, const double* Win, double dt, const typename G:
     // faces, 20 steps: 0.73 ms, one face 1.04 ms).  Slots of the ring: three, or
     // four in 3D and for long rows, again for L2 (12k nodes in 2D 10.9 against
     // 12.5 ms; 21k in 3D 24.0 against 25.7; 2D, 39 kB a row, 4.11 with four, 3.67
-    // with three).
+    // with three, in groups of 128).
     if (c->Nv <= 512 || (c->Nv <= 1024 && c->Nf >= 32 * c->nsm)) {
         if (c->Nf >= 16 * c->nsm) go(I2{}, N32{}, I4{}, I3{});
         else go(I1{}, N32{}, I4{}, I3{});
