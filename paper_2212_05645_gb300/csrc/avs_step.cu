@@ -1507,9 +1507,9 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
                       "static shared memory of the face block");
         if (axis_tables(c)) {
             const size_t smem = (size_t)c->tab_n * sizeof(AxisEq);
-            if (smem > 40 * 1024) {
-                const cudaError_t e =
-                    cudaFuncSetAttribute(k_face_tab<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (smem > 40 * 1024) {      // the most of any context: as k_cell32
+                const cudaError_t e = cudaFuncSetAttribute(k_face_tab<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)(AVS_TAB_MAX * sizeof(AxisEq)));
                 if (e != cudaSuccess) return e;
             }
             k_face_tab<D, NT><<<c->Nf, NT, smem, c->stream>>>(P, c->xtab, c->tix, c->xstride, c->tab_end[0], c->tab_end[1],
@@ -1580,8 +1580,9 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
         // node mapping, so that its sums equal the carried ones bit for bit
         if (axis_tables(c)) {
             const size_t smem = (size_t)c->tab_n * sizeof(AxisCell);
-            if (smem > 40 * 1024) {
-                e = cudaFuncSetAttribute(k_cell_tab<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (smem > 40 * 1024) {      // the most of any context: as k_cell32
+                e = cudaFuncSetAttribute(k_cell_tab<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(AVS_TAB_MAX * sizeof(AxisCell)));
                 if (e != cudaSuccess) return e;
             }
             k_cell_tab<D, NT><<<c->Nc, NT, smem, c->stream>>>(Q, c->xtab, c->tix, c->xstride, c->tab_end[0],

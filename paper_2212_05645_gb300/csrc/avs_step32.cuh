@@ -827,9 +827,13 @@ cudaError_t cell32_t(avs_ctx* c, const void* fin, void* fout)
     auto go = [&](auto nt) -> cudaError_t {
         constexpr int NT = decltype(nt)::value, STG = 3;
         const size_t smem = (size_t)STG * nrow * NT * 16;
-        if (smem > 40 * 1024) {
+        // the limit is a property of the kernel, shared by every context: always
+        // the most any mesh needs, never one mesh's own size, which another
+        // thread's smaller one could replace before the launch
+        constexpr size_t most = (size_t)STG * (D + 1 + G::NA * (1 + AVS_MAXS)) * NT * 16;
+        if constexpr (most > 40 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(k_cell32<G, NT, STG, RES>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
             if (e != cudaSuccess) return e;
         }
         k_cell32<G, NT, STG, RES><<<c->Nc, NT, smem, c->stream>>>(P, nrow);
