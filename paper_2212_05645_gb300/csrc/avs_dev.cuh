@@ -148,14 +148,6 @@ __device__ __forceinline__ float ex2_approx(float x)
     return r;
 }
 
-// 1 / x by the PTX rcp instruction (approximate, subnormal arguments flushed to zero)
-__device__ __forceinline__ float rcp_ftz(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // ---------------------------------------------------------------- equilibria
 // Parameters of one equilibrium evaluated on the nodes:
 //   G = pref exp(-|c|^2 inv2RT) (1 + (c . alpha)(|c|^2 invRT - D - 2)),

@@ -379,14 +379,17 @@ __device__ __forceinline__ void ext4(const float* v, float& mx, float& mn)
 
 // Venkatakrishnan ratio of venkat() in two lanes, uncapped: (d1^2 + eps2 +
 // 2 d1 d2) / (d1^2 + 2 d2^2 + d1 d2 + eps2).  All terms are >= 0 (d1 and d2 have
-// one sign).  The reciprocal flushes subnormal denominators, |f| below 1e-19,
-// where the ratio comes out infinite or NaN and limit2 takes 1.
+// one sign).  The division (a reciprocal and a product, like fdiv) keeps
+// subnormal denominators, so the ratio holds down to |f| of about 1e-20 and with
+// fewer bits to 1e-22, where the squares vanish and limit2 takes 1; it holds up to
+// 9e18.  (A reciprocal that flushes them, off from 1e-19 down, would save 0.8 % of
+// a step on the cylinder, 12288 cells x 3522 nodes: 8.35 against 8.42 ms for ten.)
 __device__ __forceinline__ float2 venkat2(float2 d1, float2 d2, float2 eps2)
 {
     const float2 u = fma2(d1, d1, eps2), v = mul2(d1, d2);
     const float2 num = fma2(bc2(2.0f), v, u);
     const float2 den = fma2(mul2(bc2(2.0f), d2), d2, add2(u, v));
-    return make_float2(num.x * rcp_ftz(den.x), num.y * rcp_ftz(den.y));
+    return make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
 }
 
 // Limiter of a node pair: the smaller of the two sides' ratios, capped at 1.
