@@ -24,6 +24,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "avs_dev.cuh"
 #include "avs_internal.h"
@@ -179,8 +180,15 @@ __device__ __forceinline__ void group_bar(int id)
 // it copied, so the loops have no barrier, and the copies of pass B are in
 // flight during the state.  The coordinates and weights are loaded once for the
 // FPT faces: at one face per load they were 32 of the 44 bytes that a face and
-// node moved from L2 to the SM in the two passes.  The moment basis about the
-// faces' common reference velocity is formed once too.
+// node moved from L2 to the SM in the two passes.  The moment basis is formed
+// once too, about the faces' common reference velocity, where their own (the mean
+// of the two cells') lie close together: within (1/16 of the least internal
+// energy)^(1/2), so that the mean is at most 0.16 sqrt(R T) from either and the
+// central moments cancel no large terms.  Elsewhere (a shock, the first cells at a
+// wall, faces far apart that follow each other in the order) each face has its own
+// basis: with a stream at 24 sqrt(R T) beside gas at rest, numbered at random, the
+// common one left an error of 9e-7 in the energy of the gas at rest after one step,
+// its own 8e-9.  (Two loops and not a choice within one, which spilled.)
 template <class G>
 struct Face32P {
     int Nv, Nvp, Nfi, Nf;
@@ -209,6 +217,7 @@ struct Face32S {
     double red[FPT * NM];
     float sw[(NT / 32) * FPT * NM];
     float V[FPT][3];
+    float e[FPT];            // least translational energy of the face's cells, 3/2 R T
     float An[FPT][4];
     typename G::Eq eq[FPT];
 };
@@ -358,13 +367,18 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ?
     for (int q = 0; q < STG - 1; ++q) fetch(q, q);
     if (t < FPT) {
         const int f = P.order[min(g * FPT + t, P.Nfi - 1)];
-        const int L = P.faceL[f], R = P.faceR[f];
+        const double *WL = P.Win + (size_t)P.faceL[f] * NW, *WR = P.Win + (size_t)P.faceR[f] * NW;
+        float eL = (float)(WL[D + 1] - (G::ROT ? WL[NW - 1] : 0.0)) / (float)WL[0];
+        float eR = (float)(WR[D + 1] - (G::ROT ? WR[NW - 1] : 0.0)) / (float)WR[0];
 #pragma unroll
         for (int d = 0; d < D; ++d) {
+            const float uL = (float)WL[1 + d] / (float)WL[0], uR = (float)WR[1 + d] / (float)WR[0];
             S.An[t][d] = P.An[(size_t)f * D + d];
-            S.V[t][d] = 0.5f * ((float)P.Win[(size_t)L * NW + 1 + d] / (float)P.Win[(size_t)L * NW] +
-                                (float)P.Win[(size_t)R * NW + 1 + d] / (float)P.Win[(size_t)R * NW]);
+            S.V[t][d] = 0.5f * (uL + uR);
+            eL -= 0.5f * uL * uL;
+            eR -= 0.5f * uR * uR;
         }
+        S.e[t] = fminf(eL, eR);
     }
     gsync();
     int slot = 0;
@@ -383,13 +397,20 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ?
         fetch(q + STG - 1, slot == 0 ? STG - 1 : slot - 1);
         slot = slot + 1 == STG ? 0 : slot + 1;
     };
-    float V[D];
+    float V[D];                                  // reference velocity: of the group, or of its first face
+    bool common = true;
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        V[d] = S.V[0][d];
+    for (int d = 0; d < D; ++d) V[d] = S.V[0][d];
+    if constexpr (FPT > 1) {
+        static_assert(FPT == 2, "two faces per group at most");
+        float dv = 0.0f;
 #pragma unroll
-        for (int j = 1; j < FPT; ++j) V[d] += S.V[j][d];
-        V[d] *= 1.0f / FPT;
+        for (int d = 0; d < D; ++d) dv = fmaf(S.V[1][d] - V[d], S.V[1][d] - V[d], dv);
+        common = dv <= 0.0625f * fminf(S.e[0], S.e[1]);
+        if (common) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) V[d] = 0.5f * (V[d] + S.V[1][d]);
+        }
     }
     // ---------------- pass A: raw moments about V
     {
@@ -398,36 +419,38 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ?
         for (int j = 0; j < FPT; ++j)
 #pragma unroll
             for (int q = 0; q < NM; ++q) m[j][q] = bc2(0.0f);
-        for (int q0 = 0; q0 < nq; ++q0) {        // pad nodes of the last quad carry w = 0
-            {
+        auto sums = [&](auto one) {              // one: the basis about V serves every face
+            for (int q0 = 0; q0 < nq; ++q0) {    // pad nodes of the last quad carry w = 0
                 float2 X[D][2], W2[2], F[FPT][NA][2];
                 next(q0, X, W2, F);
 #pragma unroll
                 for (int p = 0; p < 2; ++p) {
-                    float2 y[D], wy[D];
-#pragma unroll
-                    for (int d = 0; d < D; ++d) {
-                        y[d] = add2(X[d][p], bc2(-V[d]));
-                        wy[d] = mul2(W2[p], y[d]);
-                    }
-                    float2 s = mul2(y[0], y[0]);
-#pragma unroll
-                    for (int d = 1; d < D; ++d) s = fma2(y[d], y[d], s);
                     // basis in the order of raw_acc: 1, y, y y (upper triangle), y s
                     constexpr int NG = 1 + D + D * (D + 1) / 2 + D;
                     float2 b[NG];
-                    int q = 0;
-                    b[q++] = W2[p];
-#pragma unroll
-                    for (int d = 0; d < D; ++d) b[q++] = wy[d];
-#pragma unroll
-                    for (int d = 0; d < D; ++d)
-#pragma unroll
-                        for (int e = d; e < D; ++e) b[q++] = mul2(wy[d], y[e]);
-#pragma unroll
-                    for (int d = 0; d < D; ++d) b[q++] = mul2(wy[d], s);
 #pragma unroll
                     for (int j = 0; j < FPT; ++j) {
+                        if (j == 0 || !decltype(one)::value) {
+                            float2 y[D], wy[D];
+#pragma unroll
+                            for (int d = 0; d < D; ++d) {
+                                y[d] = add2(X[d][p], bc2(-(j == 0 ? V[d] : S.V[j][d])));
+                                wy[d] = mul2(W2[p], y[d]);
+                            }
+                            float2 s = mul2(y[0], y[0]);
+#pragma unroll
+                            for (int d = 1; d < D; ++d) s = fma2(y[d], y[d], s);
+                            int q = 0;
+                            b[q++] = W2[p];
+#pragma unroll
+                            for (int d = 0; d < D; ++d) b[q++] = wy[d];
+#pragma unroll
+                            for (int d = 0; d < D; ++d)
+#pragma unroll
+                                for (int e = d; e < D; ++e) b[q++] = mul2(wy[d], y[e]);
+#pragma unroll
+                            for (int d = 0; d < D; ++d) b[q++] = mul2(wy[d], s);
+                        }
 #pragma unroll
                         for (int z = 0; z < NG; ++z) m[j][z] = fma2(b[z], F[j][0][p], m[j][z]);
 #pragma unroll
@@ -440,7 +463,9 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ?
                     }
                 }
             }
-        }
+        };
+        if (FPT == 1 || common) sums(std::true_type{});
+        else if constexpr (FPT > 1) sums(std::false_type{});
         if constexpr (FPT * NM <= 32) {
             float v[FPT * NM];
 #pragma unroll
@@ -459,7 +484,8 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ?
         }
     }
     if (t < FPT) {
-        const double Vd[3] = {(double)V[0], (double)V[1], D == 3 ? (double)V[D - 1] : 0.0};
+        const float* Vt = common ? V : S.V[t];
+        const double Vd[3] = {(double)Vt[0], (double)Vt[1], D == 3 ? (double)Vt[D - 1] : 0.0};
         S.eq[t] = G::face_eq(P.g, P.hd, S.red + t * NM, Vd, P.err);
     }
     gsync();
