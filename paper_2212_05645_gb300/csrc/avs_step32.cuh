@@ -161,6 +161,53 @@ __device__ __forceinline__ void group_sum(float* v, int t, float* sw, double* ou
     gsync();
 }
 
+// The cell kernels' sums go in runs of kCellRun quads of a thread: FP32 over a
+// thread's quads of a run (two terms a quad and lane) and over the warp, FP64 over
+// the runs and the warps, so that an FP32 chain has at most 16 terms however long
+// the row.  As one run, a cell of one warp took 334 terms a lane for 21372 nodes;
+// with 1000 (64000 nodes, the first ones outweighing the rest) the lagged heat flux
+// came out 1.36 times too large, now 1.005.  The runs cost 0.5 % of a step of the
+// sphere (65.3 -> 65.6 ms for five; runs of 16 quads the same) and 2 % where the
+// rows are too short to have any (190 nodes, 12288 cells: 2.08 -> 2.12 ms for 20).
+constexpr int kCellRun = 8;
+// one run: lane pairs m, which are cleared, added to the warp's sums; a lane with
+// cnt > 0 holds that of value idx
+template <int N>
+__device__ __forceinline__ void run_sum(float2* m, double& sum, int& idx, int& cnt)
+{
+    static_assert(N <= 32, "one value per lane at most");
+    float v[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        v[q] = m[q].x + m[q].y;
+        m[q] = bc2(0.0f);
+    }
+    idx = 0;
+    cnt = N;
+    WarpSum<float, N, 16>::run(v, idx, cnt);
+    sum += to_double(v[0]);
+}
+// the last run, and the sums of all runs and warps into out[N]; sw: (NT / 32) * N doubles
+template <int N, int NT, typename Sync>
+__device__ __forceinline__ void run_sums(float2* m, double sum, int t, double* sw, double* out, Sync gsync)
+{
+    int idx, cnt;
+    run_sum<N>(m, sum, idx, cnt);
+    if constexpr (NT == 32) {
+        if (cnt > 0) out[idx] = sum;
+    } else {
+        if (cnt > 0) sw[(t >> 5) * N + idx] = sum;
+        gsync();
+        if (t < N) {
+            double s = sw[t];
+#pragma unroll
+            for (int w = 1; w < NT / 32; ++w) s += sw[w * N + t];
+            out[t] = s;
+        }
+    }
+    gsync();
+}
+
 template <int NT>
 __device__ __forceinline__ void group_bar(int id)
 {
@@ -594,8 +641,7 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<G> P, 
     __shared__ Par cp;
     __shared__ int fs[AVS_MAXS];
     __shared__ float sg[AVS_MAXS];
-    __shared__ float sw[(NT / 32) * NM];
-    __shared__ double red[NM];
+    __shared__ double sw[(NT / 32) * NM], red[NM];
     const int t = threadIdx.x;
     const int i = blockIdx.x;
     const int ns = P.nslot[i];
@@ -634,71 +680,77 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<G> P, 
 #pragma unroll
     for (int q = 0; q < STG - 1; ++q) fetch(q, q);
     float2 m[RES ? 1 : NM];
+    double sum = 0.0;
+    const int nall = (Nv + 3) / CH;              // quads that every thread has
     if constexpr (!RES) {
 #pragma unroll
         for (int q = 0; q < NM; ++q) m[q] = bc2(0.0f);
     }
     int slot = 0;
-    for (int q = 0; q < nq; ++q) {
-        const int k = q * CH + t * 4;
-        cp_wait<STG - 2>();
-        const float* src = my + (size_t)slot * nrow * RS;
-        float2 X[D][2], W2[2], f0[NA][2], N[NA][2], o[NA][2];
+    for (int q0 = 0; q0 < nq; q0 += kCellRun) {
+        for (int q = q0; q < min(nq, q0 + kCellRun); ++q) {
+            const int k = q * CH + t * 4;
+            cp_wait<STG - 2>();
+            const float* src = my + (size_t)slot * nrow * RS;
+            float2 X[D][2], W2[2], f0[NA][2], N[NA][2], o[NA][2];
 #pragma unroll
-        for (int d = 0; d < D; ++d) lds4(src + d * RS, X[d]);
-        if constexpr (!RES) lds4(src + D * RS, W2);
-#pragma unroll
-        for (int a = 0; a < NA; ++a) {
-            lds4(src + (D + 1 + a) * RS, f0[a]);
-            N[a][0] = N[a][1] = bc2(0.0f);
-        }
-#pragma unroll
-        for (int s = 0; s < AVS_MAXS; ++s) {
-            if (s >= ns) break;
-            const float2 g = bc2(sg[s]);
+            for (int d = 0; d < D; ++d) lds4(src + d * RS, X[d]);
+            if constexpr (!RES) lds4(src + D * RS, W2);
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
-                float2 F[2];
-                lds4(src + (D + 1 + NA * (1 + s) + a) * RS, F);
-#pragma unroll
-                for (int p = 0; p < 2; ++p) N[a][p] = fma2(g, F[p], N[a][p]);
+                lds4(src + (D + 1 + a) * RS, f0[a]);
+                N[a][0] = N[a][1] = bc2(0.0f);
             }
-        }
-        fetch(q + STG - 1, slot == 0 ? STG - 1 : slot - 1);
-        slot = slot + 1 == STG ? 0 : slot + 1;
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float2 x[D], y[D], g[NA];
+            for (int s = 0; s < AVS_MAXS; ++s) {
+                if (s >= ns) break;
+                const float2 g = bc2(sg[s]);
 #pragma unroll
-            for (int d = 0; d < D; ++d) x[d] = X[d][p];
-            G::cell_eq(cp, x, g);
+                for (int a = 0; a < NA; ++a) {
+                    float2 F[2];
+                    lds4(src + (D + 1 + NA * (1 + s) + a) * RS, F);
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) N[a][p] = fma2(g, F[p], N[a][p]);
+                }
+            }
+            fetch(q + STG - 1, slot == 0 ? STG - 1 : slot - 1);
+            slot = slot + 1 == STG ? 0 : slot + 1;
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                float2 x[D], y[D], g[NA];
+#pragma unroll
+                for (int d = 0; d < D; ++d) x[d] = X[d][p];
+                G::cell_eq(cp, x, g);
+#pragma unroll
+                for (int a = 0; a < NA; ++a)
+                    o[a][p] = mul2(fma2(N[a][p], bc2(cp.un), fma2(f0[a][p], bc2(cp.u0), mul2(g[a], bc2(cp.u1)))), bc2(cp.u3));
+                if (k + 4 > Nv) {                    // the last quad's pad nodes are stored as zero
+                    const bool r0 = k + 2 * p < Nv, r1 = k + 2 * p + 1 < Nv;
+#pragma unroll
+                    for (int a = 0; a < NA; ++a) o[a][p] = make_float2(r0 ? o[a][p].x : 0.0f, r1 ? o[a][p].y : 0.0f);
+                }
+                if constexpr (!RES) {
+                    float2 v[NA];
+#pragma unroll
+                    for (int a = 0; a < NA; ++a) v[a] = o[a][p];
+#pragma unroll
+                    for (int d = 0; d < D; ++d) y[d] = add2(x[d], bc2(-cp.V[d]));
+                    pair_moments<G>(m, y, W2[p], v);
+                }
+            }
 #pragma unroll
             for (int a = 0; a < NA; ++a)
-                o[a][p] = mul2(fma2(N[a][p], bc2(cp.un), fma2(f0[a][p], bc2(cp.u0), mul2(g[a], bc2(cp.u1)))), bc2(cp.u3));
-            if (k + 4 > Nv) {                    // the last quad's pad nodes are stored as zero
-                const bool r0 = k + 2 * p < Nv, r1 = k + 2 * p + 1 < Nv;
-#pragma unroll
-                for (int a = 0; a < NA; ++a) o[a][p] = make_float2(r0 ? o[a][p].x : 0.0f, r1 ? o[a][p].y : 0.0f);
-            }
-            if constexpr (!RES) {
-                float2 v[NA];
-#pragma unroll
-                for (int a = 0; a < NA; ++a) v[a] = o[a][p];
-#pragma unroll
-                for (int d = 0; d < D; ++d) y[d] = add2(x[d], bc2(-cp.V[d]));
-                pair_moments<G>(m, y, W2[p], v);
-            }
+                *reinterpret_cast<float4*>(fo + (size_t)a * Nvp + k) =
+                    make_float4(o[a][0].x, o[a][0].y, o[a][1].x, o[a][1].y);
         }
-#pragma unroll
-        for (int a = 0; a < NA; ++a)
-            *reinterpret_cast<float4*>(fo + (size_t)a * Nvp + k) =
-                make_float4(o[a][0].x, o[a][0].y, o[a][1].x, o[a][1].y);
+        if constexpr (!RES)
+            if (q0 + kCellRun <= nall) {
+                int idx, cnt;
+                run_sum<NM>(m, sum, idx, cnt);
+            }
     }
     if constexpr (!RES) {
-        float v[NM];
-#pragma unroll
-        for (int q = 0; q < NM; ++q) v[q] = m[q].x + m[q].y;
-        group_sum<NM, NT>(v, t, sw, red, [] { group_bar<NT>(1); });
+        run_sums<NM, NT>(m, sum, t, sw, red, [] { group_bar<NT>(1); });
         if (t < NM) P.mom[(size_t)i * NM + t] = red[t];
     }
 }
@@ -709,8 +761,7 @@ template <class G, int NT>
 __global__ void __launch_bounds__(NT) k_raw32(Cell32P<G> P)
 {
     constexpr int D = G::D, NA = G::NA, NM = G::NM, NW = G::NW;
-    __shared__ float sw[(NT / 32) * NM];
-    __shared__ double red[NM];
+    __shared__ double sw[(NT / 32) * NM], red[NM];
     const int t = threadIdx.x, i = blockIdx.x;
     float V[D];
 #pragma unroll
@@ -719,27 +770,33 @@ __global__ void __launch_bounds__(NT) k_raw32(Cell32P<G> P)
     float2 m[NM];
 #pragma unroll
     for (int q = 0; q < NM; ++q) m[q] = bc2(0.0f);
-    for (int k = t * 4; k < P.Nv; k += NT * 4) {
-        float2 X[D][2], W2[2], F[NA][2];
+    const int nq = (P.Nv - 4 * t + 4 * NT - 1) / (4 * NT), nall = (P.Nv + 3) / (4 * NT);
+    double sum = 0.0;
+    for (int q0 = 0; q0 < nq; q0 += kCellRun) {
+        for (int q = q0; q < min(nq, q0 + kCellRun); ++q) {
+            const int k = (q * NT + t) * 4;
+            float2 X[D][2], W2[2], F[NA][2];
 #pragma unroll
-        for (int d = 0; d < D; ++d) ld4(P.xs + d * P.xstride + k, X[d]);
-        ld4(P.w + k, W2);
+            for (int d = 0; d < D; ++d) ld4(P.xs + d * P.xstride + k, X[d]);
+            ld4(P.w + k, W2);
 #pragma unroll
-        for (int a = 0; a < NA; ++a) ld4cg(fi + (size_t)a * P.Nvp + k, F[a]);
+            for (int a = 0; a < NA; ++a) ld4cg(fi + (size_t)a * P.Nvp + k, F[a]);
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            float2 y[D], v[NA];
+            for (int p = 0; p < 2; ++p) {
+                float2 y[D], v[NA];
 #pragma unroll
-            for (int d = 0; d < D; ++d) y[d] = add2(X[d][p], bc2(-V[d]));
+                for (int d = 0; d < D; ++d) y[d] = add2(X[d][p], bc2(-V[d]));
 #pragma unroll
-            for (int a = 0; a < NA; ++a) v[a] = F[a][p];
-            pair_moments<G>(m, y, W2[p], v);
+                for (int a = 0; a < NA; ++a) v[a] = F[a][p];
+                pair_moments<G>(m, y, W2[p], v);
+            }
+        }
+        if (q0 + kCellRun <= nall) {
+            int idx, cnt;
+            run_sum<NM>(m, sum, idx, cnt);
         }
     }
-    float v[NM];
-#pragma unroll
-    for (int q = 0; q < NM; ++q) v[q] = m[q].x + m[q].y;
-    group_sum<NM, NT>(v, t, sw, red, [] { group_bar<NT>(1); });
+    run_sums<NM, NT>(m, sum, t, sw, red, [] { group_bar<NT>(1); });
     if (t < NM) P.mom[(size_t)i * NM + t] = red[t];
 }
 
