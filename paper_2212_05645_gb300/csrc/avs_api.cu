@@ -185,6 +185,30 @@ avs_status alloc_f(avs_ctx* c, int nodes, void** f0, void** f1)
     return AVS_OK;
 }
 
+}  // namespace
+
+// foot values, then (in place) the face flux; afterwards one f-sized array for
+// the implicit step's increment
+size_t avs::flux_need(const avs_ctx* c)
+{
+    const size_t rows = (size_t)std::max(c->fcap, c->Nvp);   // sized for the f capacity: no reallocation
+    return (size_t)std::max(c->Nf, c->Nc) * c->NA * rows * elem_size(c);
+}
+
+cudaError_t avs::ensure_flux(avs_ctx* c)
+{
+    const size_t need = flux_need(c);
+    if (c->flux_bytes >= need) return cudaSuccess;
+    if (c->flux) cudaFree(c->flux);
+    c->flux = nullptr;
+    c->flux_bytes = 0;
+    const cudaError_t e = cudaMalloc(&c->flux, need);
+    if (e == cudaSuccess) c->flux_bytes = need;
+    return e;
+}
+
+namespace {
+
 // He-uniform initial MLP weights from SplitMix64 (deterministic), zero biases.
 void mlp_default_params(std::vector<float>& P)
 {
@@ -637,6 +661,12 @@ avs_status avs_create(const avs_config* cfg, const avs_mesh* mesh, void* cuda_st
         st = alloc_f(c, c->fcap, &c->f[0], &c->f[1]);
         if (st != AVS_OK) goto bad;
     }
+    // the step's face buffer, where it is small: the first step would otherwise
+    // allocate it, which takes 80 us whenever the driver has to map memory, as
+    // long as a small step itself (266 triangles x 88 nodes: first step 138 us
+    // then, 60 without).  A larger one is left to the first step, whose own time
+    // hides it, as not every context steps.
+    if (flux_need(c) <= kFluxAtCreate && ensure_flux(c) != cudaSuccess) cudaGetLastError();   // the step tries again
     if (cudaMemsetAsync(c->W[0], 0, sizeof(double) * c->Nc * NW, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->W[1], 0, sizeof(double) * c->Nc * NW, c->stream) != cudaSuccess) {
         st = fail(c, AVS_ECUDA, "memset");

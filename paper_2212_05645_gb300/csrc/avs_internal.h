@@ -160,6 +160,11 @@ namespace avs {
 
 int round_up(int n, int m);
 
+// ---- the step's face buffer c->flux (avs_api.cu)
+constexpr size_t kFluxAtCreate = 32u << 20;      // bytes up to which avs_create allocates it
+size_t flux_need(const avs_ctx* c);
+cudaError_t ensure_flux(avs_ctx* c);             // allocates or grows it
+
 // ---- launchers (avs_step.cu)
 cudaError_t launch_step(avs_ctx* c, const void* fin, void* fout, const double* Win, double* Wout, double dt);
 // Rykov model (csrc/avs_rykov.cu)

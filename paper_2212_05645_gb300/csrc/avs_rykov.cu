@@ -1386,15 +1386,14 @@ template <int D, typename T>
 cudaError_t rk_face_stage(avs_ctx* c, const void* fin, const double* Win, double dt, RkP<T>& P)
 {
     constexpr int NA = RkNA<D>::v;
-    const size_t rows = (size_t)std::max(c->fcap, c->Nvp);
     const bool grad = c->cfg.limiter != 0 && sizeof(T) == 8;   // the FP32 form never stores gradients
     cudaError_t e;
     if (grad) {
+        const size_t rows = (size_t)std::max(c->fcap, c->Nvp);
         e = ensure_bytes(&c->grad, &c->grad_bytes, (size_t)c->Nc * NA * D * rows * sizeof(T));
         if (e != cudaSuccess) return e;
     }
-    // the face flux, and in the implicit step afterwards the per-cell dphi
-    e = ensure_bytes(&c->flux, &c->flux_bytes, (size_t)std::max(c->Nf, c->Nc) * NA * rows * sizeof(T));
+    e = ensure_flux(c);
     if (e != cudaSuccess) return e;
     P.Nv = c->Nv;
     P.Nvp = c->Nvp;

@@ -1435,20 +1435,8 @@ template <int D, typename T>
 static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, double dt)
 {
     const int NA = NArr<D>::v;
-    const size_t rows = (size_t)std::max(c->fcap, c->Nvp);   // sized for the f capacity: no reallocation
-    {
-        // foot values, then (in place) the face flux; afterwards one f-sized
-        // array for the implicit step's increment
-        const size_t need = (size_t)std::max(c->Nf, c->Nc) * NA * rows * sizeof(T);
-        if (c->flux_bytes < need) {
-            if (c->flux) cudaFree(c->flux);
-            c->flux = nullptr;
-            c->flux_bytes = 0;
-            cudaError_t e = cudaMalloc(&c->flux, need);
-            if (e != cudaSuccess) return e;
-            c->flux_bytes = need;
-        }
-    }
+    const cudaError_t ea = ensure_flux(c);
+    if (ea != cudaSuccess) return ea;
     const double hd = 0.5 * dt;
     {
         if constexpr (sizeof(T) == 4) {
