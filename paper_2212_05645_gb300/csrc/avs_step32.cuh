@@ -415,17 +415,24 @@ __global__ void __launch_bounds__(NT * HG, (NT * HG == 64 ? 8 : NT * HG == 128 ?
     if (t < FPT) {
         const int f = P.order[min(g * FPT + t, P.Nfi - 1)];
         const double *WL = P.Win + (size_t)P.faceL[f] * NW, *WR = P.Win + (size_t)P.faceR[f] * NW;
-        float eL = (float)(WL[D + 1] - (G::ROT ? WL[NW - 1] : 0.0)) / (float)WL[0];
-        float eR = (float)(WR[D + 1] - (G::ROT ? WR[NW - 1] : 0.0)) / (float)WR[0];
+        const float rL = (float)WL[0], rR = (float)WR[0];
+        float kL = 0.0f, kR = 0.0f;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
-            const float uL = (float)WL[1 + d] / (float)WL[0], uR = (float)WR[1 + d] / (float)WR[0];
+            const float uL = (float)WL[1 + d] / rL, uR = (float)WR[1 + d] / rR;
             S.An[t][d] = P.An[(size_t)f * D + d];
             S.V[t][d] = 0.5f * (uL + uR);
-            eL -= 0.5f * uL * uL;
-            eR -= 0.5f * uR * uR;
+            kL = fmaf(0.5f * uL, uL, kL);
+            kR = fmaf(0.5f * uR, uR, kR);
         }
-        S.e[t] = fminf(eL, eR);
+        if constexpr (FPT > 1) {
+            float eL = (float)WL[D + 1], eR = (float)WR[D + 1];
+            if constexpr (G::ROT) {
+                eL -= (float)WL[D + 2];
+                eR -= (float)WR[D + 2];
+            }
+            S.e[t] = fminf(fdiv(eL, rL) - kL, fdiv(eR, rR) - kR);
+        }
     }
     gsync();
     int slot = 0;
