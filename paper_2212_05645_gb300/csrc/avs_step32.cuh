@@ -167,8 +167,7 @@ __device__ __forceinline__ void group_sum(float* v, int t, float* sw, double* ou
 // the row.  As one run, a cell of one warp took 334 terms a lane for 21372 nodes;
 // with 1000 (64000 nodes, the first ones outweighing the rest) the lagged heat flux
 // came out 1.36 times too large, now 1.005.  The runs cost 0.5 % of a step of the
-// sphere (65.3 -> 65.6 ms for five; runs of 16 quads the same) and 2 % where the
-// rows are too short to have any (190 nodes, 12288 cells: 2.08 -> 2.12 ms for 20).
+// sphere (65.3 -> 65.6 ms for five; runs of 16 quads the same).
 constexpr int kCellRun = 8;
 // one run: lane pairs m, which are cleared, added to the warp's sums; a lane with
 // cnt > 0 holds that of value idx
@@ -187,16 +186,24 @@ __device__ __forceinline__ void run_sum(float2* m, double& sum, int& idx, int& c
     WarpSum<float, N, 16>::run(v, idx, cnt);
     sum += to_double(v[0]);
 }
-// the last run, and the sums of all runs and warps into out[N]; sw: (NT / 32) * N doubles
+// the last run, and the sums of all runs and warps into out[N]; sw: (NT / 32) * N
+// doubles.  one: there was no run before, so nothing is added (a branch of its own:
+// an FP64 addition is 16 cycles of an SM's pipe, predicated off or not; 190 nodes,
+// 12288 cells, 20 steps: 2.078 -> 2.055 ms).
 template <int N, int NT, typename Sync>
-__device__ __forceinline__ void run_sums(float2* m, double sum, int t, double* sw, double* out, Sync gsync)
+__device__ __forceinline__ void run_sums(float2* m, double sum, bool one, int t, double* sw, double* out, Sync gsync)
 {
+    double* const o = NT == 32 ? out : sw + (t >> 5) * N;
     int idx, cnt;
-    run_sum<N>(m, sum, idx, cnt);
-    if constexpr (NT == 32) {
-        if (cnt > 0) out[idx] = sum;
+    if (one) {
+        double s = -0.0;                         // x + -0 is x: no instruction
+        run_sum<N>(m, s, idx, cnt);
+        if (cnt > 0) o[idx] = s;
     } else {
-        if (cnt > 0) sw[(t >> 5) * N + idx] = sum;
+        run_sum<N>(m, sum, idx, cnt);
+        if (cnt > 0) o[idx] = sum;
+    }
+    if constexpr (NT > 32) {
         gsync();
         if (t < N) {
             double s = sw[t];
@@ -757,7 +764,7 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 16 : 4) k_cell32(Cell32P<G> P, 
             }
     }
     if constexpr (!RES) {
-        run_sums<NM, NT>(m, sum, t, sw, red, [] { group_bar<NT>(1); });
+        run_sums<NM, NT>(m, sum, nall < kCellRun, t, sw, red, [] { group_bar<NT>(1); });
         if (t < NM) P.mom[(size_t)i * NM + t] = red[t];
     }
 }
@@ -803,7 +810,7 @@ __global__ void __launch_bounds__(NT) k_raw32(Cell32P<G> P)
             run_sum<NM>(m, sum, idx, cnt);
         }
     }
-    run_sums<NM, NT>(m, sum, t, sw, red, [] { group_bar<NT>(1); });
+    run_sums<NM, NT>(m, sum, nall < kCellRun, t, sw, red, [] { group_bar<NT>(1); });
     if (t < NM) P.mom[(size_t)i * NM + t] = red[t];
 }
 
