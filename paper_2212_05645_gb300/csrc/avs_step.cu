@@ -413,11 +413,19 @@ __device__ __forceinline__ float2 limit2(float2 dmax, float2 dmin, float2 pp, fl
 // EXACT: the upwind choice is the FP64 one; only a quad with a normal velocity
 // within one bound of zero recomputes it (a bound per node cost the Rykov
 // cylinder 90 us more).
-// Warps per SM, by the vectors a quad loads (own and neighbours', every array):
-// the most that do not spill more than a few registers.
-constexpr int foot_warps(int D, int rows) { return D == 3 ? (rows <= 7 ? 36 : 16) : rows <= 10 ? 28 : rows <= 15 ? 24 - 4 * (rows < 15) : 16; }
+// Warps per SM, by arrays and face slots: the most of 16, 20, 24, 28, 32 and 36 at
+// which ptxas spills at most 24 bytes a thread.  One step further it spills 48 (2D,
+// two arrays, four slots), 120 (six slots), 100 and 128 (three arrays) and 112 bytes
+// (3D, two arrays).  2D, two arrays, four slots: 20 warps 322 us, 24 292, 28 270, 36
+// 369, 40 475.
+constexpr int foot_warps(int D, int NS, int NA)
+{
+    if (D == 3) return NA == 1 ? 36 : 16;
+    if (NS == 4) return NA == 2 ? 28 : 24;
+    return NA == 2 ? 20 : 16;
+}
 template <int D, int NS, int NA, bool EXACT>
-__global__ void __launch_bounds__(D == 3 ? 64 : 128, foot_warps(D, NA * (NS + 1)) / (D == 3 ? 2 : 4)) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
+__global__ void __launch_bounds__(D == 3 ? 64 : 128, foot_warps(D, NS, NA) / (D == 3 ? 2 : 4)) k_foot_f2(int Nv, int Nvp, int chunk, int limiter, float h,
                                                     const float* __restrict__ f, float* __restrict__ FB,
                                                     const float4* __restrict__ geo, const float* __restrict__ eps2,
                                                     const float* __restrict__ xs, size_t xstride,
