@@ -773,22 +773,14 @@ struct Rykov {
 static_assert(sizeof(Rykov<3>::Par) <= AVS_CELLPAR_BYTES, "cell parameter buffer");
 static_assert(RkNR<3>::v <= AVS_CMOM_MAX, "carried moments buffer size");
 
-constexpr int RK_VC = 2;     // nodes per thread per iteration of rk_moments32 (2 or 4)
+constexpr int RK_VC = 2;     // nodes per thread per iteration of rk_moments32
 
-// V = RK_VC consecutive nodes of an FP32 row in one vector load (L2 only).
+// two consecutive nodes of an FP32 row in one vector load (L2 only)
 __device__ __forceinline__ void rk_ldv(const float* p, float* o)
 {
-    if constexpr (RK_VC == 4) {
-        const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
-        o[0] = t.x;
-        o[1] = t.y;
-        o[2] = t.z;
-        o[3] = t.w;
-    } else {
-        const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
-        o[0] = t.x;
-        o[1] = t.y;
-    }
+    const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
+    o[0] = t.x;
+    o[1] = t.y;
 }
 
 // xi (D per node) and w of the RK_VC nodes from k0 (rows padded to 32 nodes;
@@ -1239,8 +1231,7 @@ __global__ void rk_imp_state32(RkP<float> P, const double* __restrict__ mom, typ
 // microscopic residual Res = V (g~ - phi^n) / tau~ - N of every array (written
 // over the f^{n+1} buffer); u0[i] = V/dt + V/tau~ for the sweeps.
 template <int D, typename T>
-__global__ void __launch_bounds__(RK_NT) rk_imp_res(RkP<T> P, const T* __restrict__ xiT,
-                                                    const T* __restrict__ wT, double* u0)
+__global__ void __launch_bounds__(RK_NT) rk_imp_res(RkP<T> P, const T* __restrict__ xiT, double* u0)
 {
     static_assert(sizeof(T) == 8, "the mixed form uses k_cell32");
     constexpr int NA = RkNA<D>::v, NW = D + 3;
@@ -1531,7 +1522,7 @@ cudaError_t rk_step_implicit_t(avs_ctx* c, const void* fin, void* fout, const do
         if (e == cudaSuccess) e = launch_micro32(c, fin, fout, u0, k_micro);
         if (e != cudaSuccess) return e;
     } else {
-        rk_imp_res<D, T><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_d, c->w_d, u0);
+        rk_imp_res<D, T><<<c->Nc, RK_NT, 0, c->stream>>>(P, c->xi_d, u0);
         c->launches += 1;
         T* dphi = (T*)c->flux;          // the face flux has been used
         e = cudaMemsetAsync(dphi, 0, (size_t)c->Nc * NA * c->Nvp * sizeof(T), c->stream);

@@ -233,8 +233,7 @@ __device__ __forceinline__ void ext_bits(const double* v, double& mx, double& mn
 template <int D, int NS, int NA>
 __global__ void __launch_bounds__(128) k_foot(int Nv, int Nvp, int chunk, int limiter, double h,
                                               const double* __restrict__ f, double* __restrict__ FB,
-                                              CellGeo<double> geo, const int* __restrict__ slot,
-                                              const double* __restrict__ An, const double* __restrict__ xi,
+                                              CellGeo<double> geo, const double* __restrict__ An, const double* __restrict__ xi,
                                               const float4* __restrict__ geo32, const float* __restrict__ xs,
                                               size_t xstride)
 {
@@ -354,8 +353,6 @@ __global__ void __launch_bounds__(128) k_foot(int Nv, int Nvp, int chunk, int li
 // thread as two pairs, each lane doing k_foot's operations (the same products
 // and fused multiply-adds in the same order, so the same foot values; the
 // limiter's two ratios are evaluated in both lanes and selected per lane).
-__device__ __forceinline__ float2 lo2(float4 a) { return make_float2(a.x, a.y); }
-__device__ __forceinline__ float2 hi2(float4 a) { return make_float2(a.z, a.w); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, bc2(-1.0f), a); }   // a - b, one rounding
 
 template <int NS>
@@ -620,35 +617,32 @@ __device__ __forceinline__ void load_nodes(const PP& P, int k0, T (*x)[D], T* w)
 }
 
 // ------------------------------------------------------------------ k_face
-template <int D, typename T>
+template <int D>
 struct FaceP {
     int Nv, Nvp;
     size_t cstride;          // elements per cell in f: NA * Nvp
-    T h;
     double hd;
     double R, Pr, omega, mu_ref, T_ref;
-    T* FB;                     // [face][array][Nvp]: foot values phi_bar (k_foot) in,
+    double* FB;                     // [face][array][Nvp]: foot values phi_bar (k_foot) in,
                                // per-node flux (xi . An) phi_ij out (pass B overwrites in place)
     double* __restrict__ AF;   // [face][D+2] area-weighted flux of W
     const double* __restrict__ Win;
-    const T* __restrict__ xi;
-    const T* __restrict__ w;
+    const double* __restrict__ xi;
+    const double* __restrict__ w;
     const int* __restrict__ order;
     const int* __restrict__ faceL;
     const int* __restrict__ faceR;
-    const T* __restrict__ An;
+    const double* __restrict__ An;
     const double* __restrict__ bc;
     int* err;
 };
 
-template <typename T>
 struct FaceSt {
     int kind, L, R;          // kind: 0 interior, 1 wall, 2 far field
-    T An[3];
+    double An[3];
     double V[3];             // reference velocity of the moment sums
-    T Vt[3];                 // the same in the element type
-    EqPar<T> eq;             // interface equilibrium / incoming Maxwellian
-    T wa, wb;
+    EqPar<double> eq;             // interface equilibrium / incoming Maxwellian
+    double wa, wb;
 };
 
 // The face stage in pieces.  One face, nodes [kb, ke) (thread t of NT owns
@@ -669,27 +663,26 @@ struct FaceSt {
 //                sum_k w (xi . An) psi phi_ij; boundary: outgoing foot value /
 //                incoming Maxwellian.
 // k_face runs them all in one block per face.
-template <int D, typename T>
-__device__ __forceinline__ void face_setup(const FaceP<D, T>& P, int f, FaceSt<T>& S)
+template <int D>
+__device__ __forceinline__ void face_setup(const FaceP<D>& P, int f, FaceSt& S)
 {
     constexpr int NW = D + 2;
     S.L = P.faceL[f];
     S.R = P.faceR[f];
     S.kind = S.R >= 0 ? 0 : (int)P.bc[(size_t)(-1 - S.R) * 6];
     for (int d = 0; d < 3; ++d) {
-        S.An[d] = d < D ? P.An[(size_t)f * D + d] : T(0);
-        T v = T(0);
+        S.An[d] = d < D ? P.An[(size_t)f * D + d] : 0.0;
+        double v = 0.0;
         if (d < D) {
-            v = (T)P.Win[(size_t)S.L * NW + 1 + d] / (T)P.Win[(size_t)S.L * NW];
-            if (S.R >= 0) v = T(0.5) * (v + (T)P.Win[(size_t)S.R * NW + 1 + d] / (T)P.Win[(size_t)S.R * NW]);
+            v = P.Win[(size_t)S.L * NW + 1 + d] / P.Win[(size_t)S.L * NW];
+            if (S.R >= 0) v = 0.5 * (v + P.Win[(size_t)S.R * NW + 1 + d] / P.Win[(size_t)S.R * NW]);
         }
-        S.V[d] = (double)v;
-        S.Vt[d] = v;
+        S.V[d] = v;
     }
     if (S.kind != 0) {
         const double* B = P.bc + (size_t)(-1 - S.R) * 6;
         const double Ub[3] = {B[2], B[3], B[4]};
-        S.eq = make_eq<D, T>(S.kind == 1 ? 1.0 : B[1], Ub, P.R * B[5], nullptr, P.Pr);
+        S.eq = make_eq<D, double>(S.kind == 1 ? 1.0 : B[1], Ub, P.R * B[5], nullptr, P.Pr);
     }
 }
 
@@ -701,69 +694,69 @@ struct FaceNR {
     static constexpr int v = (NM > 2 * NW) ? NM : 2 * NW;
 };
 
-template <int D, typename T, int NT, bool CACHE, int V>
-__device__ __forceinline__ void face_pass_a(const FaceP<D, T>& P, const FaceSt<T>& S, T* fc, int kb, int ke,
-                                            T* acc, int tid, int f)
+template <int D, int NT, bool CACHE, int V>
+__device__ __forceinline__ void face_pass_a(const FaceP<D>& P, const FaceSt& S, double* fc, int kb, int ke,
+                                            double* acc, int tid, int f)
 {
     constexpr int NA = NArr<D>::v, NW = D + 2;
     constexpr int NR = FaceNR<D>::v;
     const bool inter = S.kind == 0;
-    T An[D], Vt[D];
+    double An[D], Vt[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) {
         An[d] = S.An[d];
-        Vt[d] = S.Vt[d];
+        Vt[d] = S.V[d];
     }
     const int Nvp = P.Nvp;
-    const T* fb = P.FB + (size_t)f * NA * Nvp;          // the face's foot values
+    const double* fb = P.FB + (size_t)f * NA * Nvp;          // the face's foot values
 #pragma unroll
-    for (int m = 0; m < NR; ++m) acc[m] = T(0);
+    for (int m = 0; m < NR; ++m) acc[m] = 0.0;
     if (inter) {
 #pragma unroll 2
         for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
-            T x[V][D], wv[V];
+            double x[V][D], wv[V];
             load_nodes<D, V>(P, k0, x, wv);      // pad nodes carry w = 0 and contribute nothing
-            T fv[NA][V];
+            double fv[NA][V];
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
-                ldv<T, V>(fb + (size_t)a * Nvp + k0, fv[a]);
-                if constexpr (CACHE) stv<T, V>(fc + a * Nvp + k0, fv[a]);
+                ldv<double, V>(fb + (size_t)a * Nvp + k0, fv[a]);
+                if constexpr (CACHE) stv<double, V>(fc + a * Nvp + k0, fv[a]);
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                T xs[D];
+                double xs[D];
 #pragma unroll
                 for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vt[d];
-                raw_acc<D>(acc, xs, wv[v] * fv[0][v], NA == 2 ? wv[v] * fv[NA - 1][v] : T(0));
+                raw_acc<D>(acc, xs, wv[v] * fv[0][v], NA == 2 ? wv[v] * fv[NA - 1][v] : 0.0);
             }
         }
     } else {
 #pragma unroll 2
         for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
-            T x[V][D], wv[V], sn[V];
+            double x[V][D], wv[V], sn[V];
             load_nodes<D, V>(P, k0, x, wv);
-            T fv[NA][V];
+            double fv[NA][V];
 #pragma unroll
-            for (int a = 0; a < NA; ++a) ldv<T, V>(fb + (size_t)a * Nvp + k0, fv[a]);
+            for (int a = 0; a < NA; ++a) ldv<double, V>(fb + (size_t)a * Nvp + k0, fv[a]);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 sn[v] = dot_rn<D>(x[v], An);
-                const bool out = sn[v] >= T(0);
-                T g0 = fv[0][v], g1 = NA == 2 ? fv[NA - 1][v] : T(0);
+                const bool out = sn[v] >= 0.0;
+                double g0 = fv[0][v], g1 = NA == 2 ? fv[NA - 1][v] : 0.0;
                 if (!out) eq_eval<D>(S.eq, x[v], g0, g1);
-                const T t = wv[v] * sn[v];
-                T x2 = T(0);
+                const double t = wv[v] * sn[v];
+                double x2 = 0.0;
 #pragma unroll
                 for (int d = 0; d < D; ++d) x2 += x[v][d] * x[v][d];
-                T mm[NW];
+                double mm[NW];
                 mm[0] = t * g0;
 #pragma unroll
                 for (int d = 0; d < D; ++d) mm[1 + d] = t * g0 * x[v][d];
-                mm[D + 1] = t * T(0.5) * (x2 * g0 + g1);
+                mm[D + 1] = t * 0.5 * (x2 * g0 + g1);
 #pragma unroll
                 for (int c = 0; c < NW; ++c) {
-                    acc[c] += out ? mm[c] : T(0);
-                    acc[NW + c] += out ? T(0) : mm[c];
+                    acc[c] += out ? mm[c] : 0.0;
+                    acc[NW + c] += out ? 0.0 : mm[c];
                 }
             }
         }
@@ -772,20 +765,20 @@ __device__ __forceinline__ void face_pass_a(const FaceP<D, T>& P, const FaceSt<T
 
 // Interface state from the summed pass-A moments red[]; writes S.eq, S.wa,
 // S.wb and, for a boundary face, its area-weighted flux AF[0..D+1].
-template <int D, typename T>
-__device__ __forceinline__ void face_state(const FaceP<D, T>& P, FaceSt<T>& S, const double* red, double* AF)
+template <int D>
+__device__ __forceinline__ void face_state(const FaceP<D>& P, FaceSt& S, const double* red, double* AF)
 {
     constexpr int NW = D + 2;
     if (S.kind == 0) {
-        T rho, U[3], RT, qb[3];
-        state_from_raw<D, T>(red, S.V, rho, U, RT, qb);
-        if (!(rho > T(0)) || !(RT > T(0))) atomicOr(P.err, 1);
-        const T tau = tau_vhs<T>(rho, RT, (T)P.R, (T)P.mu_ref, (T)P.T_ref, (T)P.omega);
-        const T hh = (T)P.hd;
-        T qf[3] = {T(0), T(0), T(0)};
-        const T qs = fdiv(tau, tau + hh * (T)P.Pr);
+        double rho, U[3], RT, qb[3];
+        state_from_raw<D, double>(red, S.V, rho, U, RT, qb);
+        if (!(rho > 0.0) || !(RT > 0.0)) atomicOr(P.err, 1);
+        const double tau = tau_vhs<double>(rho, RT, P.R, P.mu_ref, P.T_ref, P.omega);
+        const double hh = P.hd;
+        double qf[3] = {0.0, 0.0, 0.0};
+        const double qs = fdiv(tau, tau + hh * P.Pr);
         for (int d = 0; d < D; ++d) qf[d] = qs * qb[d];
-        S.eq = make_eq_a<D, T, T>(rho, U, RT, qf, (T)P.Pr);
+        S.eq = make_eq_a<D, double, double>(rho, U, RT, qf, P.Pr);
         S.wa = fdiv(tau, tau + hh);
         S.wb = fdiv(hh, tau + hh);
     } else if (S.kind == 1) {
@@ -794,7 +787,7 @@ __device__ __forceinline__ void face_state(const FaceP<D, T>& P, FaceSt<T>& S, c
         for (int m = 0; m < NW; ++m) AF[m] = red[m] + rw * red[NW + m];
         const double* B = P.bc + (size_t)(-1 - S.R) * 6;
         const double Ub[3] = {B[2], B[3], B[4]};
-        S.eq = make_eq<D, T>(rw, Ub, P.R * B[5], nullptr, P.Pr);
+        S.eq = make_eq<D, double>(rw, Ub, P.R * B[5], nullptr, P.Pr);
     } else {
         for (int m = 0; m < NW; ++m) AF[m] = red[m] + red[NW + m];
     }
@@ -803,102 +796,102 @@ __device__ __forceinline__ void face_state(const FaceP<D, T>& P, FaceSt<T>& S, c
 // Pass B over nodes [kb, ke): writes the per-node flux over the face's foot
 // values in FB (in place) and, for an interior face, returns the per-thread
 // flux-moment partial sums in acc[D+2] (element type).
-template <int D, typename T, int NT, bool CACHE, int V>
-__device__ __forceinline__ void face_pass_b(const FaceP<D, T>& P, const FaceSt<T>& S, const T* fc, int kb, int ke,
-                                            T* acc, int tid, int f)
+template <int D, int NT, bool CACHE, int V>
+__device__ __forceinline__ void face_pass_b(const FaceP<D>& P, const FaceSt& S, const double* fc, int kb, int ke,
+                                            double* acc, int tid, int f)
 {
     constexpr int NA = NArr<D>::v, NW = D + 2;
     const bool inter = S.kind == 0;
-    T An[D];
+    double An[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) An[d] = S.An[d];
     const int Nvp = P.Nvp;
-    T* Fo = P.FB + (size_t)f * NA * Nvp;                // foot values in, flux out
+    double* Fo = P.FB + (size_t)f * NA * Nvp;                // foot values in, flux out
 #pragma unroll
-    for (int m = 0; m < NW; ++m) acc[m] = T(0);
+    for (int m = 0; m < NW; ++m) acc[m] = 0.0;
     if (inter) {
-        const T wa = S.wa, wb = S.wb;
+        const double wa = S.wa, wb = S.wb;
 #pragma unroll 2
         for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
-            T x[V][D], wv[V], sn[V];
+            double x[V][D], wv[V], sn[V];
             load_nodes<D, V>(P, k0, x, wv);
 #pragma unroll
             for (int v = 0; v < V; ++v) sn[v] = dot_rn<D>(x[v], An);
-            T fv[NA][V];
+            double fv[NA][V];
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
-                if constexpr (CACHE) ldv<T, V>(fc + a * Nvp + k0, fv[a]);
-                else ldv<T, V>(Fo + (size_t)a * Nvp + k0, fv[a]);
+                if constexpr (CACHE) ldv<double, V>(fc + a * Nvp + k0, fv[a]);
+                else ldv<double, V>(Fo + (size_t)a * Nvp + k0, fv[a]);
             }
-            T o[NA][V];
+            double o[NA][V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                T gG, gH;
+                double gG, gH;
                 eq_eval<D>(S.eq, x[v], gG, gH);
-                const T pG = wa * fv[0][v] + wb * gG;
-                const T pH = NA == 2 ? wa * fv[NA - 1][v] + wb * gH : T(0);
-                const T t = wv[v] * sn[v];
-                T x2 = T(0);
+                const double pG = wa * fv[0][v] + wb * gG;
+                const double pH = NA == 2 ? wa * fv[NA - 1][v] + wb * gH : 0.0;
+                const double t = wv[v] * sn[v];
+                double x2 = 0.0;
 #pragma unroll
                 for (int d = 0; d < D; ++d) x2 += x[v][d] * x[v][d];
                 acc[0] += t * pG;
 #pragma unroll
                 for (int d = 0; d < D; ++d) acc[1 + d] += t * pG * x[v][d];
-                acc[D + 1] += t * T(0.5) * (x2 * pG + pH);
+                acc[D + 1] += t * 0.5 * (x2 * pG + pH);
                 o[0][v] = sn[v] * pG;
                 if (NA == 2) o[NA - 1][v] = sn[v] * pH;
             }
 #pragma unroll
-            for (int a = 0; a < NA; ++a) stv<T, V>(Fo + (size_t)a * Nvp + k0, o[a]);
+            for (int a = 0; a < NA; ++a) stv<double, V>(Fo + (size_t)a * Nvp + k0, o[a]);
         }
     } else {
 #pragma unroll 2
         for (int k0 = kb + tid * V; k0 < ke; k0 += NT * V) {
-            T x[V][D], wv[V], sn[V];
+            double x[V][D], wv[V], sn[V];
             load_nodes<D, V>(P, k0, x, wv);
-            T fv[NA][V];
+            double fv[NA][V];
 #pragma unroll
-            for (int a = 0; a < NA; ++a) ldv<T, V>(Fo + (size_t)a * Nvp + k0, fv[a]);
-            T o[NA][V];
+            for (int a = 0; a < NA; ++a) ldv<double, V>(Fo + (size_t)a * Nvp + k0, fv[a]);
+            double o[NA][V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 sn[v] = dot_rn<D>(x[v], An);
-                T g0 = fv[0][v], g1 = NA == 2 ? fv[NA - 1][v] : T(0);
-                if (sn[v] < T(0)) eq_eval<D>(S.eq, x[v], g0, g1);
+                double g0 = fv[0][v], g1 = NA == 2 ? fv[NA - 1][v] : 0.0;
+                if (sn[v] < 0.0) eq_eval<D>(S.eq, x[v], g0, g1);
                 o[0][v] = sn[v] * g0;
                 if (NA == 2) o[NA - 1][v] = sn[v] * g1;
             }
 #pragma unroll
-            for (int a = 0; a < NA; ++a) stv<T, V>(Fo + (size_t)a * Nvp + k0, o[a]);
+            for (int a = 0; a < NA; ++a) stv<double, V>(Fo + (size_t)a * Nvp + k0, o[a]);
         }
     }
 }
 
 // One block per face, all nodes: setup, pass A, state, pass B.
-template <int D, typename T, int NT, bool CACHE, int VF>
-__global__ void __launch_bounds__(NT, 4) k_face(FaceP<D, T> P)
+template <int D, int NT, bool CACHE, int VF>
+__global__ void __launch_bounds__(NT, 4) k_face(FaceP<D> P)
 {
     constexpr int NW = D + 2;
     constexpr int NR = FaceNR<D>::v;
-    __shared__ FaceSt<T> S;
+    __shared__ FaceSt S;
     __shared__ double sw[(NT / 32) * NR];
     __shared__ double red[NR];
     extern __shared__ __align__(16) unsigned char face_dsm[];
-    T* fc = reinterpret_cast<T*>(face_dsm);     // [array][Nvp] foot values (CACHE)
+    double* fc = reinterpret_cast<double*>(face_dsm);     // [array][Nvp] foot values (CACHE)
 
     const int tid = threadIdx.x;
     const int f = P.order[blockIdx.x];
-    if (tid == 0) face_setup<D, T>(P, f, S);
+    if (tid == 0) face_setup<D>(P, f, S);
     __syncthreads();
     {
-        T acc[NR];
-        face_pass_a<D, T, NT, CACHE, VF>(P, S, fc, 0, P.Nv, acc, tid, f);
+        double acc[NR];
+        face_pass_a<D, NT, CACHE, VF>(P, S, fc, 0, P.Nv, acc, tid, f);
         block_sum_t<NR, NT>(acc, sw, red);
     }
-    if (tid == 0) face_state<D, T>(P, S, red, P.AF + (size_t)f * NW);
+    if (tid == 0) face_state<D>(P, S, red, P.AF + (size_t)f * NW);
     __syncthreads();
-    T acc[NW];
-    face_pass_b<D, T, NT, CACHE, VF>(P, S, fc, 0, P.Nv, acc, tid, f);
+    double acc[NW];
+    face_pass_b<D, NT, CACHE, VF>(P, S, fc, 0, P.Nv, acc, tid, f);
     if (S.kind == 0) {
         block_sum_t<NW, NT>(acc, sw, red);
         if (tid < NW) P.AF[(size_t)f * NW + tid] = red[tid];
@@ -919,7 +912,7 @@ struct AxisEq {
 };
 
 template <int D, int NT>
-__global__ void __launch_bounds__(NT) k_face_tab(FaceP<D, double> P, const double* __restrict__ xtab,
+__global__ void __launch_bounds__(NT) k_face_tab(FaceP<D> P, const double* __restrict__ xtab,
                                                  const unsigned short* __restrict__ tix, size_t xstride, int n0,
                                                  int n1, int nt)
 {
@@ -927,23 +920,23 @@ __global__ void __launch_bounds__(NT) k_face_tab(FaceP<D, double> P, const doubl
     constexpr int NR = FaceNR<D>::v;
     extern __shared__ __align__(16) unsigned char tab_dsm[];
     AxisEq* tab = reinterpret_cast<AxisEq*>(tab_dsm);
-    __shared__ FaceSt<double> S;
+    __shared__ FaceSt S;
     __shared__ double sw[(NT / 32) * NR];
     __shared__ double red[NR];
     const int tid = threadIdx.x;
     const int f = P.order[blockIdx.x];
-    if (tid == 0) face_setup<D, double>(P, f, S);
+    if (tid == 0) face_setup<D>(P, f, S);
     __syncthreads();
     {
         double acc[NR];
-        face_pass_a<D, double, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
+        face_pass_a<D, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
         block_sum_t<NR, NT>(acc, sw, red);
     }
-    if (tid == 0) face_state<D, double>(P, S, red, P.AF + (size_t)f * NW);
+    if (tid == 0) face_state<D>(P, S, red, P.AF + (size_t)f * NW);
     __syncthreads();
     double acc[NW];
     if (S.kind != 0) {
-        face_pass_b<D, double, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
+        face_pass_b<D, NT, false, 2>(P, S, nullptr, 0, P.Nv, acc, tid, f);
         return;
     }
     for (int e = tid; e < nt; e += NT) {
@@ -1041,28 +1034,28 @@ struct CellP {
 
 // Raw moments of the own f^n of cell i about its U(W^n) over nodes [kb, ke):
 // per-thread partial sums in acc[NM].
-template <int D, typename T, int NT, int VC>
-__device__ __forceinline__ void cell_raw_moments(const CellP<D, T>& P, int i, int kb, int ke, T* acc)
+template <int D, int NT, int VC>
+__device__ __forceinline__ void cell_raw_moments(const CellP<D, double>& P, int i, int kb, int ke, double* acc)
 {
     constexpr int NA = NArr<D>::v, NM = NMom<D>::v, NW = D + 2;
     constexpr int V = VC;
-    T Vct[D];
+    double Vct[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) Vct[d] = (T)P.Win[(size_t)i * NW + 1 + d] / (T)P.Win[(size_t)i * NW];
-    const T* fi = P.fin + (size_t)i * P.cstride;
+    for (int d = 0; d < D; ++d) Vct[d] = P.Win[(size_t)i * NW + 1 + d] / P.Win[(size_t)i * NW];
+    const double* fi = P.fin + (size_t)i * P.cstride;
 #pragma unroll
-    for (int m = 0; m < NM; ++m) acc[m] = T(0);
+    for (int m = 0; m < NM; ++m) acc[m] = 0.0;
     for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
-        T x[V][D], wv[V], f0[V], f1[V];
+        double x[V][D], wv[V], f0[V], f1[V];
         load_nodes<D, V>(P, k0, x, wv);
-        ldv<T, V>(fi + k0, f0);
-        if (NA == 2) ldv<T, V>(fi + P.Nvp + k0, f1);
+        ldv<double, V>(fi + k0, f0);
+        if (NA == 2) ldv<double, V>(fi + P.Nvp + k0, f1);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            T xs[D];
+            double xs[D];
 #pragma unroll
             for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vct[d];
-            raw_acc<D>(acc, xs, wv[v] * f0[v], NA == 2 ? wv[v] * f1[v] : T(0));
+            raw_acc<D>(acc, xs, wv[v] * f0[v], NA == 2 ? wv[v] * f1[v] : 0.0);
         }
     }
 }
@@ -1070,15 +1063,15 @@ __device__ __forceinline__ void cell_raw_moments(const CellP<D, T>& P, int i, in
 // Raw moments of the own f^n of every cell about its U(W^n) (one block per
 // cell); used when the previous step did not leave them (after init, set_f,
 // set_W or an adaptation).
-template <int D, typename T, int NT, int VC>
-__global__ void __launch_bounds__(NT) k_raw_moments(CellP<D, T> P)
+template <int D, int NT, int VC>
+__global__ void __launch_bounds__(NT) k_raw_moments(CellP<D, double> P)
 {
     constexpr int NM = NMom<D>::v;
     __shared__ double sw[(NT / 32) * NM];
     __shared__ double red[NM];
     const int i = blockIdx.x;
-    T acc[NM];
-    cell_raw_moments<D, T, NT, VC>(P, i, 0, P.Nv, acc);
+    double acc[NM];
+    cell_raw_moments<D, NT, VC>(P, i, 0, P.Nv, acc);
     block_sum_t<NM, NT>(acc, sw, red);
     if (threadIdx.x < NM) P.mom[(size_t)i * NM + threadIdx.x] = red[threadIdx.x];
 }
@@ -1181,71 +1174,71 @@ __global__ void k_cell_state(CellP<D, T> P)
 // (per-thread partials in acc[NM], same nodes per thread and order as
 // cell_raw_moments).  fs, sg: the cell's face indices and signs; cp its
 // collision parameters (shared memory).
-template <int D, typename T, int NT, int VC>
-__device__ __forceinline__ void cell_update(const CellP<D, T>& P, int i, int ns, const int* fs, const T* sg,
-                                            const CellPar<T>& cp, int kb, int ke, T* acc)
+template <int D, int NT, int VC>
+__device__ __forceinline__ void cell_update(const CellP<D, double>& P, int i, int ns, const int* fs, const double* sg,
+                                            const CellPar<double>& cp, int kb, int ke, double* acc)
 {
     constexpr int NA = NArr<D>::v, NM = NMom<D>::v;
     constexpr int V = VC;
-    const T* fi = P.fin + (size_t)i * P.cstride;
-    T* fo = P.fout + (size_t)i * P.cstride;
-    const T u0 = cp.upd[0], u1 = cp.upd[1], u2 = cp.upd[2], u3 = cp.upd[3];
-    T Vnt[D];
+    const double* fi = P.fin + (size_t)i * P.cstride;
+    double* fo = P.fout + (size_t)i * P.cstride;
+    const double u0 = cp.upd[0], u1 = cp.upd[1], u2 = cp.upd[2], u3 = cp.upd[3];
+    double Vnt[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) Vnt[d] = cp.Vn[d];
 #pragma unroll
-    for (int m = 0; m < NM; ++m) acc[m] = T(0);
+    for (int m = 0; m < NM; ++m) acc[m] = 0.0;
     for (int k0 = kb + threadIdx.x * V; k0 < ke; k0 += NT * V) {
-        T x[V][D], wv[V];
+        double x[V][D], wv[V];
         load_nodes<D, V>(P, k0, x, wv);
-        T Nn[NA][V], fv[NA][V], out[NA][V];
+        double Nn[NA][V], fv[NA][V], out[NA][V];
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
-            ldv_cg<T, V>(fi + (size_t)a * P.Nvp + k0, fv[a]);
+            ldv_cg<double, V>(fi + (size_t)a * P.Nvp + k0, fv[a]);
 #pragma unroll
-            for (int v = 0; v < V; ++v) Nn[a][v] = T(0);
+            for (int v = 0; v < V; ++v) Nn[a][v] = 0.0;
         }
 #pragma unroll
         for (int s = 0; s < AVS_MAXS; ++s) {
             if (s >= ns) break;
-            const T* Fs = P.F + (size_t)fs[s] * NA * P.Nvp + k0;
-            const T g = sg[s];
+            const double* Fs = P.F + (size_t)fs[s] * NA * P.Nvp + k0;
+            const double g = sg[s];
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
-                T t[V];
-                ldv_cg<T, V>(Fs + (size_t)a * P.Nvp, t);
+                double t[V];
+                ldv_cg<double, V>(Fs + (size_t)a * P.Nvp, t);
 #pragma unroll
                 for (int v = 0; v < V; ++v) Nn[a][v] += g * t[v];
             }
         }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            T gG, gH;
+            double gG, gH;
             eq_eval<D>(cp.eq, x[v], gG, gH);
             const bool real = k0 + v < P.Nv;
-            out[0][v] = real ? (fv[0][v] * u0 + gG * u1 - Nn[0][v] * u2) * u3 : T(0);
+            out[0][v] = real ? (fv[0][v] * u0 + gG * u1 - Nn[0][v] * u2) * u3 : 0.0;
             if (NA == 2)
-                out[NA - 1][v] = real ? (fv[NA - 1][v] * u0 + gH * u1 - Nn[NA - 1][v] * u2) * u3 : T(0);
-            T xs[D];
+                out[NA - 1][v] = real ? (fv[NA - 1][v] * u0 + gH * u1 - Nn[NA - 1][v] * u2) * u3 : 0.0;
+            double xs[D];
 #pragma unroll
             for (int d = 0; d < D; ++d) xs[d] = x[v][d] - Vnt[d];
-            raw_acc<D>(acc, xs, wv[v] * out[0][v], NA == 2 ? wv[v] * out[NA - 1][v] : T(0));
+            raw_acc<D>(acc, xs, wv[v] * out[0][v], NA == 2 ? wv[v] * out[NA - 1][v] : 0.0);
         }
 #pragma unroll
-        for (int a = 0; a < NA; ++a) stv<T, V>(fo + (size_t)a * P.Nvp + k0, out[a]);
+        for (int a = 0; a < NA; ++a) stv<double, V>(fo + (size_t)a * P.Nvp + k0, out[a]);
     }
 }
 
 // One block per cell, all nodes; the raw moments of f^{n+1} to P.mom.
-template <int D, typename T, int NT, int VC>
-__global__ void __launch_bounds__(NT, 4) k_cell(CellP<D, T> P)
+template <int D, int NT, int VC>
+__global__ void __launch_bounds__(NT, 4) k_cell(CellP<D, double> P)
 {
     constexpr int NM = NMom<D>::v;
     __shared__ int fs[AVS_MAXS];
-    __shared__ T sg[AVS_MAXS];
+    __shared__ double sg[AVS_MAXS];
     __shared__ double sw[(NT / 32) * NM];
     __shared__ double red[NM];
-    __shared__ CellPar<T> cp;
+    __shared__ CellPar<double> cp;
 
     const int tid = threadIdx.x;
     const int i = blockIdx.x;
@@ -1253,12 +1246,12 @@ __global__ void __launch_bounds__(NT, 4) k_cell(CellP<D, T> P)
     if (tid < ns) {
         const int sl = P.slot[i * AVS_MAXS + tid];
         fs[tid] = sl >> 1;
-        sg[tid] = (sl & 1) ? T(-1) : T(1);
+        sg[tid] = (sl & 1) ? -1.0 : 1.0;
     }
     if (tid == 32 % NT) cp = P.par[i];
     __syncthreads();
-    T acc[NM];
-    cell_update<D, T, NT, VC>(P, i, ns, fs, sg, cp, 0, P.Nv, acc);
+    double acc[NM];
+    cell_update<D, NT, VC>(P, i, ns, fs, sg, cp, 0, P.Nv, acc);
     block_sum_t<NM, NT>(acc, sw, red);
     if (tid < NM) P.mom[(size_t)i * NM + tid] = red[tid];
 }
@@ -1460,10 +1453,11 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
             const int chunk = (npair + ny - 1) / ny * 2;
             auto go = [&](auto ns) {
                 k_foot<D, decltype(ns)::value, NArr<D>::v><<<dim3(c->Nc, ny), nt, 0, c->stream>>>(
-                    c->Nv, c->Nvp, chunk, c->cfg.limiter, hd, (const double*)fin, (double*)c->flux, geo, c->slot,
+                    c->Nv, c->Nvp, chunk, c->cfg.limiter, hd, (const double*)fin, (double*)c->flux, geo,
                     c->An_d, c->xi_d, (const float4*)c->geo32, c->xi_s, c->xstride);
             };
-            if (D == 2 && c->max_ns <= 4) go(std::integral_constant<int, 4>{});
+            using Four = std::integral_constant<int, D == 2 ? 4 : AVS_MAXS>;      // 3D: six slots always
+            if (c->max_ns <= 4) go(Four{});
             else go(std::integral_constant<int, AVS_MAXS>{});
             c->launches += 1;
         }
@@ -1471,18 +1465,17 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
     if constexpr (sizeof(T) == 4) {
         return launch_face32(c, Win, dt);
     } else {
-        FaceP<D, T> P;
+        FaceP<D> P;
         P.Nv = c->Nv;
         P.Nvp = c->Nvp;
         P.cstride = (size_t)NA * c->Nvp;
         P.hd = hd;
-        P.h = (T)P.hd;
         P.R = c->cfg.R;
         P.Pr = c->cfg.Pr;
         P.omega = c->cfg.omega;
         P.mu_ref = c->mu_ref;
         P.T_ref = c->cfg.T_ref;
-        P.FB = (T*)c->flux;
+        P.FB = (double*)c->flux;
         P.AF = c->AFf;
         P.Win = Win;
         P.xi = c->xi_d;
@@ -1502,7 +1495,7 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
         // the default allowance covers static and dynamic shared memory together:
         // the block's own arrays (state, reductions: under 2 KB) come first
         constexpr size_t kStaticFace = 2048;
-        static_assert(sizeof(FaceSt<T>) + (NT / 32 + 1) * FaceNR<D>::v * sizeof(double) <= kStaticFace,
+        static_assert(sizeof(FaceSt) + (NT / 32 + 1) * FaceNR<D>::v * sizeof(double) <= kStaticFace,
                       "static shared memory of the face block");
         if (axis_tables(c)) {
             const size_t smem = (size_t)c->tab_n * sizeof(AxisEq);
@@ -1514,9 +1507,9 @@ static cudaError_t face_stage_t(avs_ctx* c, const void* fin, const double* Win, 
             k_face_tab<D, NT><<<c->Nf, NT, smem, c->stream>>>(P, c->xtab, c->tix, c->xstride, c->tab_end[0], c->tab_end[1],
                                                              c->tab_n);
         } else if (cache_bytes + kStaticFace <= 48 * 1024)
-            k_face<D, T, NT, true, VF><<<c->Nf, NT, cache_bytes, c->stream>>>(P);
+            k_face<D, NT, true, VF><<<c->Nf, NT, cache_bytes, c->stream>>>(P);
         else
-            k_face<D, T, NT, false, VF><<<c->Nf, NT, 0, c->stream>>>(P);
+            k_face<D, NT, false, VF><<<c->Nf, NT, 0, c->stream>>>(P);
         c->launches += 1;
 
         return cudaGetLastError();
@@ -1565,7 +1558,7 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
             e = launch_raw32(c, fin, Win);
             if (e != cudaSuccess) return e;
         } else {
-            k_raw_moments<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+            k_raw_moments<D, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
             c->launches += 1;
         }
     }
@@ -1587,7 +1580,7 @@ static cudaError_t launch_step_t(avs_ctx* c, const void* fin, void* fout, const 
             k_cell_tab<D, NT><<<c->Nc, NT, smem, c->stream>>>(Q, c->xtab, c->tix, c->xstride, c->tab_end[0],
                                                              c->tab_end[1], c->tab_n);
         } else {
-            k_cell<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+            k_cell<D, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
         }
         c->launches += 1;
     }
@@ -2187,7 +2180,7 @@ static cudaError_t launch_step_implicit_t(avs_ctx* c, const void* fin, void* fou
             e = launch_raw32(c, fin, Win);
             if (e != cudaSuccess) return e;
         } else {
-            k_raw_moments<D, T, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
+            k_raw_moments<D, NT, VW<T>::v><<<c->Nc, NT, 0, c->stream>>>(Q);
             c->launches += 1;
         }
     }

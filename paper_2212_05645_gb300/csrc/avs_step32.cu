@@ -290,7 +290,7 @@ static cudaError_t micro32_t(avs_ctx* c, const void* fin, void* fout, const doub
         P.clist = c->clist;
         P.colour = c->colour;
         seen[col] = 1;
-        if (D == 2 && c->max_ns <= 4) k_micro32<D, 4, NA><<<dim3(cells, ny), nt, 0, c->stream>>>(P);
+        if (c->max_ns <= 4) k_micro32<D, D == 2 ? 4 : AVS_MAXS, NA><<<dim3(cells, ny), nt, 0, c->stream>>>(P);
         else k_micro32<D, AVS_MAXS, NA><<<dim3(cells, ny), nt, 0, c->stream>>>(P);
         c->launches += 1;
     }

@@ -36,8 +36,6 @@ namespace {
 
 constexpr float kTwoLn2 = 1.3862943611198906f;     // 2 ln 2
 
-__device__ __forceinline__ float2 lo2(float4 a) { return make_float2(a.x, a.y); }
-__device__ __forceinline__ float2 hi2(float4 a) { return make_float2(a.z, a.w); }
 
 // four nodes k..k+3 (k a multiple of 4) of a planar array as two lane pairs
 __device__ __forceinline__ void ld4(const float* __restrict__ p, float2 (&o)[2])
