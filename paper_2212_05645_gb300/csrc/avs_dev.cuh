@@ -1,8 +1,9 @@
 // Device-side building blocks of the UGKS/AVS kernels (sm_103a).
 //
 // Element type T is double (FP64 form) or float (mixed form: f, reconstruction,
-// flux and collision in FP32; every velocity-space sum is carried into FP64
-// through short FP32 partials flushed into double accumulators).
+// flux and collision in FP32; velocity-space sums in FP32 over a thread's nodes and a
+// warp, in FP64 beyond; the monatomic moments that are handed out or decide on the
+// adaptation compensated, see raw_acc_c).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -9,8 +9,8 @@
 //
 // The FP64 form takes one block per face or cell and sums over the nodes in
 // FP64 directly.  The FP32 (mixed) form is the gas Rykov<D> of the kernels in
-// avs_step32.cuh: raw moments in FP32 per thread and in FP64 across warps.  The
-// equilibrium is evaluated in the element type.
+// avs_step32.cuh, with their sums.  The equilibrium is evaluated in the element
+// type.
 #include <algorithm>
 
 #include "avs_dev.cuh"
@@ -472,10 +472,11 @@ __global__ void __launch_bounds__(RK_NT) rk_cell(RkP<T> P)
 }
 
 // ---------------------------------------------------------------- mixed form
-// The FP32 form sums over the nodes in FP32 per thread (FP64 across warps),
-// as raw moments about a reference velocity V near the local mean velocity
-// (the upwind-side cell's carried U), so that no per-node FP64 arithmetic is
-// left: on GB300 an FP64 operation costs about as much as 70 FP32 ones.
+// The FP32 form sums over the nodes in FP32 per thread and warp and in FP64 beyond
+// (avs_step.cu says where), as raw moments about a reference velocity V near the
+// local mean velocity (the mean of the face's cells, the cell's carried U), so that
+// no per-node FP64 arithmetic is left: on GB300 an FP64 operation costs about as
+// much as 70 FP32 ones.
 
 template <int D>
 struct RkNR {
@@ -1118,7 +1119,7 @@ __device__ __forceinline__ void rk_imp_cell(const RkImpP<A>& P, int q)
     A rhs[NW];
 #pragma unroll
     for (int c = 0; c < NW; ++c) rhs[c] = P.rhs[(size_t)q * NW + c];
-    // loads before the arithmetic, as imp_macro_cell
+    // all neighbours' loads before the arithmetic, as ImpCell (avs_step.cu)
     int j[AVS_MAXS];
     A Wj[AVS_MAXS][NW], dWj[AVS_MAXS][NW];
 #pragma unroll

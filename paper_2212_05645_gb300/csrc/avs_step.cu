@@ -24,10 +24,13 @@
 //
 // Every face is evaluated once, so the two cells of a face see the same flux
 // and W telescopes exactly.  f^n and W^n are read-only during the step; no
-// block waits on another.  Sums: per-thread and warp sums in the element
-// type, FP64 across warps and in every per-cell / per-face formula.  The
-// limited-gradient kernel k_grad (gradients stored next to f) serves the
-// Rykov model's face kernels.
+// block waits on another.  Sums in the FP32 form: FP32 over a thread's nodes
+// and over the warp; FP64 over the warps of a block and, in the cell kernels, over
+// runs of eight quads of a thread (a face group of one warp sums its row, of 1024
+// nodes at most, in FP32; a face's FP32 chains are a 1/128 of rows to 48 KB, a 1/256
+// of longer ones).  Interface and cell states: FP32 formulas on these sums, the
+// balance of W in FP64.  The limited-gradient kernel k_grad (gradients stored next
+// to f) serves the FP64 form of the Rykov model.
 #include <algorithm>
 #include <type_traits>
 
@@ -349,10 +352,10 @@ __global__ void __launch_bounds__(128) k_foot(int Nv, int Nvp, int chunk, int li
     }
 }
 
-// k_foot for the FP32 form in packed two-lane arithmetic: four nodes per
-// thread as two pairs, each lane doing k_foot's operations (the same products
-// and fused multiply-adds in the same order, so the same foot values; the
-// limiter's two ratios are evaluated in both lanes and selected per lane).
+// The FP32 form of the reconstruction, in packed two-lane arithmetic: four nodes
+// per thread as two pairs.  Each lane rounds as the scalar operation would; the
+// upwind choice is the sign of the FP32 xi . An, the same for both cells of a face
+// (or, EXACT, the FP64 one), and both sides of the limiter are evaluated always.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, bc2(-1.0f), a); }   // a - b, one rounding
 
 template <int NS>

@@ -47,7 +47,7 @@ def test_two_threads_step_their_contexts(pair):
                 dt = g.dt()
                 if not alone:
                     both.wait()
-                for _ in range(100):
+                for _ in range(25):
                     g.step(50, dt=dt)
                 W = g.moments()[0]
                 g.close()
