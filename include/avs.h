@@ -328,10 +328,10 @@ avs_status avs_grid_barrier_check(avs_ctx *ctx, int blocks, int rounds, int shor
  * bulk copy into shared memory that completes it, with arrive = 0 nothing ever
  * does, so the wait gives up after its limit (about a second), sets the error
  * bit of such copies and the call returns AVS_ETIMEOUT with the context still
- * usable.  (The step kernels' copies are waited for by the copying thread
- * itself and need no such wait.)  *completed (host) = 1 when the copy arrived
- * and its 128 bytes equal the source's.  Blocking.  Errors: EINVAL, ENOMEM,
- * ECUDA, ETIMEOUT. */
+ * usable.  No other kernel of the library waits this way: the step kernels'
+ * copies are waited for by the copying thread itself.  *completed (host) = 1
+ * when the copy arrived and its 128 bytes equal the source's.  Blocking.
+ * Errors: EINVAL, ENOMEM, ECUDA, ETIMEOUT. */
 avs_status avs_stage_wait_check(avs_ctx *ctx, int arrive, int *completed);
 
 /* Measured FMA throughput of the current GPU (GFLOP/s, 2 flops per FMA):
