@@ -12,10 +12,10 @@
 // equilibria (face_eq, face_phi, cell_eq); EXACT: the upwind choice is the FP64
 // one (see upwind_sure).  Shakhov's is in avs_step32.cu, Rykov's in avs_rykov.cu.
 // Measured on GB300, five steps of the sphere (36864 cells, 21372 nodes) and ten
-// of the cylinder (12288 cells, 3522 nodes), face and cell kernel: 24.0 + 14.5
-// and 2.63 + 2.42 ms; one face or cell per block with rows staged by bulk copies
+// of the cylinder (12288 cells, 3522 nodes), face and cell kernel: 24.0 + 15.1
+// and 2.62 + 2.43 ms; one face or cell per block with rows staged by bulk copies
 // or loaded directly, before: 31.3 + 21.2 and 4.20 + 2.91 ms.  The Rykov
-// cylinder (12288 cells, 3216 nodes, ten steps): 3.60 + 3.29 ms with 3.86 for the
+// cylinder (12288 cells, 3216 nodes, ten steps): 3.59 + 3.39 ms with 4.01 for the
 // foot values, against 10.3 + 4.7 and 3.5 for stored gradients that the face
 // kernel read.
 // Forming phi and its flux in the cell kernel instead, without storing them,
@@ -35,7 +35,6 @@ namespace avs {
 namespace {
 
 constexpr float kTwoLn2 = 1.3862943611198906f;     // 2 ln 2
-
 
 // four nodes k..k+3 (k a multiple of 4) of a planar array as two lane pairs
 __device__ __forceinline__ void ld4(const float* __restrict__ p, float2 (&o)[2])
