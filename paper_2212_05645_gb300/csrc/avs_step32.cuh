@@ -877,10 +877,8 @@ cudaError_t face32_t(avs_ctx* c, const double* Win, double dt, const typename G:
         go(I1{}, N128{}, I1{}, I3{});
     } else if ((size_t)NA * c->Nvp * sizeof(float) > 49152) {
         go(I2{}, N128{}, I1{}, I4{});
-    } else if (D == 3) {
-        go(I2{}, N64{}, I1{}, I4{});
     } else {
-        go(I2{}, N64{}, I1{}, I3{});
+        go(I2{}, N64{}, I1{}, integral_constant<int, D == 3 ? 4 : 3>{});
     }
     if (e != cudaSuccess) return e;
     c->launches += 1;
