@@ -7,8 +7,6 @@ again after f was changed must give the same bits in every form the launch rules
 choose: one warp or 128 threads per cell, rows of several runs, either gas, and in
 the FP64 form with tables of the axes and without.
 """
-import dataclasses
-
 import numpy as np
 import pytest
 
